@@ -291,7 +291,8 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
     const int cw = p.stage_cw;  // columns per staging pass (<= 64)
     const int pitch = cw * 2 + 16;
     float* wstat = reinterpret_cast<float*>(stg + (size_t)2 * TC_BM * pitch);  // per team [4 warps][2][its columns of every n-tile]: warp-private channel sums
-    uint64_t* bars = reinterpret_cast<uint64_t*>(wstat + ((STATS || EPI) ? 8 * p.ldo : 0));  // EPI: wstat holds [ldo] (scale, shift) pairs
+    const int cols_pad = p.n_tiles * p.BN;  // columns of all n-tiles (>= ldo: the last tile may reach past the channel count)
+    uint64_t* bars = reinterpret_cast<uint64_t*>(wstat + ((STATS || EPI) ? 8 * cols_pad : 0));  // EPI: wstat holds [cols_pad] (scale, shift) pairs
     uint64_t* full = bars;                // [stages]
     uint64_t* empty = bars + p.stages;    // [stages]
     uint64_t* tfull = empty + p.stages;   // [2]
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                 if (p.out_w[i]) ptx::prefetch_tmap(&p.tmOut[i]);
     }
     if (STATS) {
-        for (int c = threadIdx.x; c < 8 * p.ldo; c += IG_THREADS) wstat[c] = 0.f;
+        for (int c = threadIdx.x; c < 8 * cols_pad; c += IG_THREADS) wstat[c] = 0.f;
     }
     if (warp == 1) {
         if (CG2) {
@@ -356,9 +357,9 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
         pdl_wait();
         // per-channel coefficients of the fused epilogue, in fp64 like the training-mode finalize
         // (stored per channel pair as scale, scale, shift, shift: the operands of the packed fp32 multiply-add)
-        for (int c = threadIdx.x; c < p.ldo; c += IG_THREADS) {
-            double sc, sh;
-            bn_eval_coef(p.fin_gamma, p.fin_beta, p.fin_rmean, p.fin_rvar, p.fin_eps, c, sc, sh);
+        for (int c = threadIdx.x; c < cols_pad; c += IG_THREADS) {
+            double sc = 0.0, sh = 0.0;  // padding columns: zero, so that they cannot count as saturated stores
+            if (c < p.ldo) bn_eval_coef(p.fin_gamma, p.fin_beta, p.fin_rmean, p.fin_rvar, p.fin_eps, c, sc, sh);
             wstat[4 * (c >> 1) + (c & 1)] = (float)sc;
             wstat[4 * (c >> 1) + 2 + (c & 1)] = (float)sh;
         }
@@ -621,6 +622,10 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                         };
                         const CUtensorMap* tm = npass == p.out_w[0] ? &p.tmOut[0] : npass == p.out_w[1] ? &p.tmOut[1] : &p.tmOut[2];
                         const int col = n_tile * p.BN + c_lo + cb, grow = (int)(m0 + lane_group * 32);
+                        if (col >= p.ldo) {  // a piece that lies wholly in the padding columns of the last tile
+                            release();
+                            continue;
+                        }
                         float* ss = my_stat + n_tile * ncol + cb;
                         float* sq = ss + st_ld;
                         const uint32_t ta = taddr + (uint32_t)cb;
@@ -676,8 +681,11 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                             const long long t1 = pixrow / p.Wq;
                             const int i = (int)(t1 % p.Hq);
                             const long long n = t1 / p.Hq;
-                            pixrow = (n * p.Hout + (long long)i * p.os + p.cls_oa[cls]) * p.Wout + (long long)j * p.os + p.cls_ob[cls];
+                            const int oi = i * p.os + p.cls_oa[cls], oj = j * p.os + p.cls_ob[cls];
+                            // (odd extents: the grid of an odd parity is one row or column longer than the image)
+                            pixrow = oi < p.Hout && oj < p.Wout ? (n * p.Hout + oi) * p.Wout + oj : -1;
                         }
+                        const int cvalid = (p.ldo - (n_tile * p.BN + c_lo + cb)) / 8;  // pieces of a row before the padding columns
                         // byte offset of staged row `lane` in the output (-1: not stored); pieces are handled four (or two) at
                         // a time so that their shuffle -> shared load -> global store chains overlap
                         const long long rowbyte = pixrow < 0 ? -1 : pixrow * (long long)(p.ldo * 2) + (n_tile * p.BN + c_lo + cb) * 2;
@@ -707,10 +715,10 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                             const uint4 v1 = *reinterpret_cast<const uint4*>(wrows + r1 * pitch + c1 * 16);
                             const uint4 v2 = *reinterpret_cast<const uint4*>(wrows + r2 * pitch + c2 * 16);
                             const uint4 v3 = *reinterpret_cast<const uint4*>(wrows + r3 * pitch + c3 * 16);
-                            if (o0 >= 0) *reinterpret_cast<uint4*>(outb + o0 + c0 * 16) = v0;
-                            if (o1 >= 0) *reinterpret_cast<uint4*>(outb + o1 + c1 * 16) = v1;
-                            if (o2 >= 0) *reinterpret_cast<uint4*>(outb + o2 + c2 * 16) = v2;
-                            if (o3 >= 0) *reinterpret_cast<uint4*>(outb + o3 + c3 * 16) = v3;
+                            if (o0 >= 0 && c0 < cvalid) *reinterpret_cast<uint4*>(outb + o0 + c0 * 16) = v0;
+                            if (o1 >= 0 && c1 < cvalid) *reinterpret_cast<uint4*>(outb + o1 + c1 * 16) = v1;
+                            if (o2 >= 0 && c2 < cvalid) *reinterpret_cast<uint4*>(outb + o2 + c2 * 16) = v2;
+                            if (o3 >= 0 && c3 < cvalid) *reinterpret_cast<uint4*>(outb + o3 + c3 * 16) = v3;
                         }
                         for (; it < cpr; it += 2) {  // cpr is even
                             int r0 = rr, c0 = cc, r1 = r0, c1 = c0;
@@ -720,8 +728,8 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                             const long long o0 = __shfl_sync(0xffffffffu, rowbyte, r0), o1 = __shfl_sync(0xffffffffu, rowbyte, r1);
                             const uint4 v0 = *reinterpret_cast<const uint4*>(wrows + r0 * pitch + c0 * 16);
                             const uint4 v1 = *reinterpret_cast<const uint4*>(wrows + r1 * pitch + c1 * 16);
-                            if (o0 >= 0) *reinterpret_cast<uint4*>(outb + o0 + c0 * 16) = v0;
-                            if (o1 >= 0) *reinterpret_cast<uint4*>(outb + o1 + c1 * 16) = v1;
+                            if (o0 >= 0 && c0 < cvalid) *reinterpret_cast<uint4*>(outb + o0 + c0 * 16) = v0;
+                            if (o1 >= 0 && c1 < cvalid) *reinterpret_cast<uint4*>(outb + o1 + c1 * 16) = v1;
                         }
                     }
                     __syncwarp();  // staged rows consumed before the next pass overwrites them
@@ -868,13 +876,30 @@ inline int igemm_stage_cw(int BN) {
     const int nc = igemm_team_cols(BN), passes = (nc + 63) / 64;
     return ((nc + passes - 1) / passes + 15) / 16 * 16;
 }
-inline size_t igemm_fixed_smem(int BN, int ldo) {
-    return 1024 /*alignment slack*/ + (size_t)2 * TC_BM * (igemm_stage_cw(BN) * 2 + 16) + (size_t)8 * ldo * 4 + 512;
+inline size_t igemm_fixed_smem(int BN, int n_tiles) {
+    return 1024 /*alignment slack*/ + (size_t)2 * TC_BM * (igemm_stage_cw(BN) * 2 + 16) + (size_t)8 * BN * n_tiles * 4 + 512;
 }
-inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int ldo, int sm_count, int nclasses) {
+// Columns of an N tile.  The widest divisor of the channel count is the best choice where it is wide (fewer shared-memory
+// bytes per flop).  Channel counts that are not multiples of 16, or have no wide divisor (304 = 16 x 19), take the fewest
+// tiles of at most 256 columns, balanced and rounded up to 16: TMA fills the filter rows past the channel count with zeros
+// and clips the stores, so at most 15 columns per tile are computed for nothing.
+// Measured, training step of 72 -> 136 channels 3x3 on 3 x 53 x 75 pixels: 1325 us on the CUDA cores, 68 us padded to 144.
+inline int igemm_tile_cols(int rowsB, int most = 256) {
+    const int tiles = (rowsB + most - 1) / most;
+    const int padded = ((rowsB + tiles - 1) / tiles + 15) / 16 * 16;
+    for (int bn = std::min(most, rowsB) / 16 * 16; 4 * bn >= 3 * padded; bn -= 16)
+        if (rowsB % bn == 0) return bn;
+    return padded;
+}
+// Channel counts the tensor-core kernels take: whole 16-byte vectors (TMA strides and starts), and at least 16 on the N side.
+// Tiny layers (fewer than two 128-row tiles) whose channel counts also need padding stay on the CUDA-core kernels.
+inline bool igemm_channels_ok(int Ca, int rowsB, long long M) {
+    return Ca % 8 == 0 && rowsB % 8 == 0 && rowsB >= 16 && ((Ca % 16 == 0 && rowsB % 16 == 0) || M >= 2 * TC_BM);
+}
+inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int sm_count, int nclasses) {
     IgemmCfg c;
     c.Ca = Ca; c.rowsB = rowsB; c.ntaps = ntaps; c.M = M;
-    if (Ca % 16 || rowsB % 16 || M < 1) return c;
+    if (M < 1) return c;
     // 64-channel k-blocks in the 128-byte swizzle (the narrower swizzles make tcgen05.mma 1.6-2.1x slower per
     // instruction); when Ca is not a multiple of 64 the last k-block of every tap reads past the channel extent and
     // TMA fills A with zeros there (whatever finite filter values B holds at those positions are multiplied by zero).
@@ -890,9 +915,9 @@ inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int l
     // count wins everywhere (fewer shared-memory bytes written and read per flop); pairing two 128-row blocks per tile
     // (mh = 2) pays only while two accumulator sets still fit in TMEM (N <= 128) and there are enough tiles for every SM;
     // a pipeline stage should hold about 450 tensor cycles of work.
-    for (int bn = std::min(256, rowsB) / 16 * 16; bn >= 16 && !c.BN; bn -= 16) {
-        if (rowsB % bn) continue;
-        if (force_bn && bn != force_bn && rowsB % force_bn == 0) continue;
+    for (int bn = force_bn ? force_bn : igemm_tile_cols(rowsB), next = bn; bn >= 16 && !c.BN; bn = next) {
+        next = bn - 16 < 16 ? 0 : igemm_tile_cols(rowsB, bn - 16);  // (a narrower tile only where two stages of this one do not fit)
+        const int n_tiles = (rowsB + bn - 1) / bn;
         const int acc_stride = bn <= 32 ? 32 : bn <= 64 ? 64 : bn <= 128 ? 128 : 256;
         // CTA pairs (one tcgen05.mma over 256 rows whose B tile is split between two CTAs): a pair's MMA of 256 x N x 16
         // runs at N/2 cycles even for small N where a single CTA's 128 x N x 16 never drops below 97, and each CTA reads
@@ -905,14 +930,14 @@ inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int l
         int mh = 1;
         if (4 * acc_stride <= 512) {
             const long long rows_tile = 2LL * TC_BM * (cg2 ? 2 : 1);
-            const long long tiles2 = ((M + rows_tile - 1) / rows_tile) * (rowsB / bn) * nclasses;
+            const long long tiles2 = ((M + rows_tile - 1) / rows_tile) * n_tiles * nclasses;
             if (tiles2 >= (cg2 ? sm_count / 2 : sm_count)) mh = 2;
         }
         if (force_mh && force_mh * acc_stride <= 512) mh = force_mh;
         const int acc_bufs = (2 * mh * acc_stride <= 512) ? 2 : 1;
         const uint32_t a_sub = (uint32_t)(TC_BM * mh * c.KC * 2);
         const uint32_t b_sub = (uint32_t)(((cg2 ? bn / 2 : bn) * c.KC * 2 + 1023) / 1024 * 1024);
-        const size_t fixed = igemm_fixed_smem(bn, ldo);
+        const size_t fixed = igemm_fixed_smem(bn, n_tiles);
         if (fixed + 2 * (size_t)(a_sub + b_sub) > kMaxSmem) continue;
         const double mma_kb = mh * 4.0 * std::max(97.0, bn / 2.0);  // tensor cycles per k-block
         int kpb = std::max(1, std::min(kblocks, (int)((450.0 + mma_kb - 1) / mma_kb)));
@@ -929,13 +954,13 @@ inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int l
         c.m_tiles = (int)((M + TC_BM * mh * (cg2 ? 2 : 1) - 1) / (TC_BM * mh * (cg2 ? 2 : 1)));
     }
     if (!c.BN) return c;
-    c.n_tiles = rowsB / c.BN;
+    c.n_tiles = (rowsB + c.BN - 1) / c.BN;
     c.stage_cols = igemm_team_cols(c.BN);
     c.tmem_cols = std::max(32, c.acc_bufs * c.mh * c.acc_stride);
     c.a_stage = c.a_sub * c.kpb;
     c.b_stage = c.b_sub * c.kpb;
     c.stages = std::max(2, std::min(c.stages, std::max(2, (kblocks + c.kpb - 1) / c.kpb)));
-    c.smem_bytes = std::max<size_t>(igemm_fixed_smem(c.BN, ldo) + (size_t)c.stages * (c.a_stage + c.b_stage), 120 * 1024);  // > half an SM: one CTA per SM
+    c.smem_bytes = std::max<size_t>(igemm_fixed_smem(c.BN, c.n_tiles) + (size_t)c.stages * (c.a_stage + c.b_stage), 120 * 1024);  // > half an SM: one CTA per SM
     c.grid = (int)std::min<long long>((long long)c.m_tiles * c.n_tiles * nclasses, c.cg2 ? sm_count / 2 : sm_count);
     if (c.cg2) c.grid *= 2;  // two CTAs per pair
     c.ok = true;
@@ -1088,10 +1113,9 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
     if (!enable) return NB_OK;
     DriverFns& d = driver();
     if (!d.tiled || !d.im2col) return NB_OK;  // no TMA descriptors from this driver: stay on the CUDA-core kernels
-    const bool even = (g.h % 2 == 0) && (g.w % 2 == 0);
     // ---- fprop: A = x (im2col), B = w [Cout][k*k*Cin]
-    if (g.c_in % 16 == 0 && g.c_out % 16 == 0) {
-        const IgemmCfg c = igemm_configure(g.m, g.c_in, g.c_out, g.k * g.k, g.c_out, sm_count, 1);
+    if (igemm_channels_ok(g.c_in, g.c_out, g.m)) {
+        const IgemmCfg c = igemm_configure(g.m, g.c_in, g.c_out, g.k * g.k, sm_count, 1);
         if (c.ok) {
             tc->fp.cfg = c;
             IgemmParams& P = tc->fp.prm;
@@ -1115,7 +1139,7 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
     }
     // ---- dgrad: A = dy (im2col), B = rearranged filter [Cin][taps*Cout]; stride 2 splits dx into four output-parity
     // classes, numbered heaviest (four taps) first; the order in which their tiles are visited is igemm_tile_class's
-    if (g.c_in % 16 == 0 && g.c_out % 16 == 0 && (g.stride == 1 || (g.k == 3 && even))) {
+    if (igemm_channels_ok(g.c_out, g.c_in, g.m) && g.c_out >= 16 && (g.stride == 1 || g.k == 3)) {
         WtParams& W = tc->wtp;
         memset(&W, 0, sizeof W);
         W.c_in = g.c_in; W.c_out = g.c_out; W.k = g.k;
@@ -1160,10 +1184,10 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
             P.Hq = g.h; P.Wq = g.w; P.ts = 1; P.lo_w = P.lo_h = -(g.k - 1 - g.pad);
             P.Hout = g.h; P.Wout = g.w; P.os = 1;
         } else {
-            P.Hq = g.h / 2; P.Wq = g.w / 2; P.ts = 1; P.lo_w = P.lo_h = 0;
+            P.Hq = g.ho; P.Wq = g.wo; P.ts = 1; P.lo_w = P.lo_h = 0;
             P.Hout = g.h; P.Wout = g.w; P.os = 2;
         }
-        const IgemmCfg c = igemm_configure((long long)g.n * P.Hq * P.Wq, g.c_out, g.c_in, max_taps, g.c_in, sm_count, ncls);
+        const IgemmCfg c = igemm_configure((long long)g.n * P.Hq * P.Wq, g.c_out, g.c_in, max_taps, sm_count, ncls);
         if (c.ok) {
             tc->dg.cfg = c;
             fill_params(P, c);  // sets only the tiling fields; the geometry written above stays
@@ -1176,7 +1200,7 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
         }
     }
     // ---- wgrad: A = x (im2col, MN-major), B = dy (MN-major), reduction over pixels with split-K
-    if (g.c_in % 16 == 0 && g.c_out % 16 == 0) {
+    if (igemm_channels_ok(g.c_in, g.c_out, g.m)) {
         WgradParams& P = tc->wg;
         memset(&P, 0, sizeof P);
         P.M = g.m; P.Hq = g.ho; P.Wq = g.wo; P.ts = g.stride; P.lo_w = P.lo_h = -g.pad;
@@ -1189,16 +1213,8 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
         P.cblk_per_tap = (g.c_in + 63) / 64;
         P.nblk_total = g.k * g.k * P.cblk_per_tap;
         P.m_tiles = (P.nblk_total + 1) / 2;
-        double best = 1e30;
-        for (int bn = 16; bn <= 256 && bn <= g.c_out; bn += 16) {
-            if (g.c_out % bn) continue;
-            const double cost = (double)(g.c_out / bn) * std::max(97.0, bn / 2.0);  // tensor cycles per K = 16 step
-            if (cost < best - 1e-9 || (cost < best + 1e-9 && bn > P.BN)) {
-                best = cost;
-                P.BN = bn;
-            }
-        }
-        P.n_tiles = g.c_out / P.BN;
+        P.BN = igemm_tile_cols(g.c_out);  // (the fewest passes over x)
+        P.n_tiles = (g.c_out + P.BN - 1) / P.BN;
         P.nblkB = (P.BN + 63) / 64;
         // One or two 128-row accumulator blocks per CTA.  With two, four x boxes share every dy stage (a third less
         // shared-memory traffic per MMA: measured 1.6x the time of a one-block stage for twice the work) but there are half

@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
             const int kidx = tap * p.c_in + c;  // position inside dw[c'][:]
             const uint32_t taddr = tmem_base + ((uint32_t)(lane_group * 32) << 16) + (uint32_t)(h * p.acc_stride);
             float* dst = p.out + (size_t)split * p.c_out * p.kdim;
-            for (int c0 = 0; c0 < p.BN; c0 += 16) {
+            for (int c0 = 0; c0 < p.BN && n_tile * p.BN + c0 < p.c_out; c0 += 16) {  // (the last tile may reach past the channel count)
                 uint32_t r[16];
                 if (nchunks > 0) {
                     ptx::tmem_ld_32x32b_x16(taddr + (uint32_t)c0, r);
@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
                 }
                 if (valid) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) dst[(size_t)(n_tile * p.BN + c0 + j) * p.kdim + kidx] = __uint_as_float(r[j]);
+                    for (int j = 0; j < 16; ++j)
+                        if (j < 8 || n_tile * p.BN + c0 + 8 < p.c_out) dst[(size_t)(n_tile * p.BN + c0 + j) * p.kdim + kidx] = __uint_as_float(r[j]);
                 }
             }
         }
@@ -437,7 +438,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_rows_kernel(const __gr
             const int kidx = (r * 3 + sft) * p.c_in + c;
             const uint32_t taddr = tmem_base + ((uint32_t)(lane_group * 32) << 16) + (uint32_t)(a * p.acc_stride);
             float* dst = p.out + (size_t)split * p.c_out * p.kdim;
-            for (int c0 = 0; c0 < p.BN; c0 += 16) {
+            for (int c0 = 0; c0 < p.BN && n_tile * p.BN + c0 < p.c_out; c0 += 16) {  // (the last tile may reach past the channel count)
                 uint32_t rr[16];
                 if (nrows > 0) {
                     ptx::tmem_ld_32x32b_x16(taddr + (uint32_t)c0, rr);
@@ -448,7 +449,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_rows_kernel(const __gr
                 }
                 if (valid) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) dst[(size_t)(n_tile * p.BN + c0 + j) * p.kdim + kidx] = __uint_as_float(rr[j]);
+                    for (int j = 0; j < 16; ++j)
+                        if (j < 8 || n_tile * p.BN + c0 + 8 < p.c_out) dst[(size_t)(n_tile * p.BN + c0 + j) * p.kdim + kidx] = __uint_as_float(rr[j]);
                 }
             }
         }
