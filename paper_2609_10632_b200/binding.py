@@ -134,28 +134,36 @@ def _ptr(t):
     """Device (or host) address of a torch tensor / numpy array / int / None."""
     if t is None:
         return None
+    try:  # (a tensor in nearly every call: no tests before the address is taken)
+        return t.data_ptr()
+    except AttributeError:
+        pass
     if isinstance(t, int):
         return t
-    if hasattr(t, "data_ptr"):
-        return t.data_ptr()
     if hasattr(t, "ctypes"):
         return t.ctypes.data
     raise TypeError(type(t))
 
 
 def _nbytes(t) -> int:
-    if t is None:
-        return 0
-    if hasattr(t, "element_size"):
-        return t.numel() * t.element_size()
-    return t.nbytes
+    return 0 if t is None else t.nbytes  # (torch tensors and numpy arrays alike)
+
+
+_raw_stream = _raw_device = None
 
 
 def _stream(stream):
+    """cudaStream_t of `stream`: an address, a torch stream, or None for the current stream of the current device.  The
+    current stream is read as a plain address: torch.cuda.current_stream() builds a Stream object, which alone takes
+    3.2 us -- more than a kernel launch -- against 0.1 us."""
     if stream is None:
-        import torch
+        global _raw_stream, _raw_device
+        if _raw_stream is None:
+            import torch
 
-        return torch.cuda.current_stream().cuda_stream
+            torch.cuda.init()
+            _raw_stream, _raw_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        return _raw_stream(_raw_device())
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
