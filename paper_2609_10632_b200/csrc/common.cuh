@@ -181,7 +181,7 @@ typedef __nv_bfloat16 WtTileBuf[32][WT_PITCH];
 struct WtTile {
     int cls, tap, r0, c0;
 };
-__device__ __forceinline__ int wt_num_tiles(const WtParams& P) {
+__host__ __device__ __forceinline__ int wt_num_tiles(const WtParams& P) {
     int taps = 0;
     for (int cls = 0; cls < P.nclasses; ++cls) taps += P.cls[cls].ntaps;
     return taps * ((P.c_out + 31) / 32) * ((P.c_in + 63) / 64);

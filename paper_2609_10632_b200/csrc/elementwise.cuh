@@ -503,7 +503,8 @@ __global__ void __launch_bounds__(288, 3) bn_silu_bwd_reduce_kernel(const AT* __
         }
     }
     const int R = blockDim.x / cgs;
-    for (int pass = 0; pass < 2; ++pass) {
+    const bool has_rows = (long long)blockIdx.x * blockDim.x < total_vecs;  // (the grid may be larger than the tensor: filter tiles)
+    for (int pass = 0; pass < 2 && has_rows; ++pass) {
 #pragma unroll
         for (int j = 0; j < V / 2; ++j) *reinterpret_cast<float2*>(&red[tid * V + 2 * j]) = pass ? sy[j] : sb[j];
         __syncthreads();

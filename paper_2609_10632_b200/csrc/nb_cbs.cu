@@ -55,6 +55,7 @@ struct EwCfg {  // launch geometry of the [M][C] passes
     long long total_vecs;
     int blocks_reduce, blocks_map;  // stats / backward-reduce grids (they size the partial buffers) and apply / dy grids
     int blocks_stats, blocks_apply, blocks_dy;
+    int wave_reduce;  // resident blocks of the backward-reduce kernel on the whole device
 };
 
 }  // namespace
@@ -218,8 +219,13 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
             fb.w = static_cast<const __nv_bfloat16*>(w); fb.wt = wtp ? static_cast<__nv_bfloat16*>(wt) : nullptr;
         }
         const size_t red_smem = (size_t)e.tpb * e.vec * sizeof(float);
+        // A small activation needs few blocks, a large filter many: every block takes two filter tiles, blocks without
+        // rows of their own take nothing else (288 -> 288 3x3 on one 20 x 20 image has 405 tiles and 8 blocks of rows:
+        // 61 us when those 8 rearranged the filter alone).
+        int blocks = e.blocks_reduce;
+        if (fb.wt) blocks = std::max(blocks, std::min(e.wave_reduce, (wt_num_tiles(*wtp) + 1) / 2));
         auto go = [&](auto kernel, long long ld) {
-            launch_k(kernel, dim3(e.blocks_reduce), dim3(e.tpb), red_smem, st, 1, static_cast<const AT*>(g), static_cast<const YT*>(y), e.total_vecs, C, mean, invstd,
+            launch_k(kernel, dim3(blocks), dim3(e.tpb), red_smem, st, 1, static_cast<const AT*>(g), static_cast<const YT*>(y), e.total_vecs, C, mean, invstd,
                      gamma, beta, partials, fb, wtp ? *wtp : none, ld);
         };
         if (p->ld_g) go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true>, p->ld_g);
@@ -358,38 +364,41 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     e.tpb = e.cgs * R;
     e.total_vecs = g.m * e.cgs;
     const long long max_blocks = (e.total_vecs + e.tpb - 1) / e.tpb;
-    // enough blocks to fill the machine, but at least ~8 (reductions) / ~4 (maps) vectors per thread so that the
-    // per-thread parameter loads and the block epilogue are amortised on small tensors
-    // Grids are one wave of resident blocks (occupancy queried per kernel), but never so many that a thread sees fewer
-    // than ~8 (reductions) / ~4 (maps) vectors: the per-thread parameter loads and block epilogues must be amortised.
+    // Grids are one wave of resident blocks (occupancy queried per kernel).  A tensor smaller than that gets as many blocks
+    // as it has work for: four vectors per thread in the reductions (a block also adds 2*C sums to the accumulators), one
+    // in the maps.  A thread's vectors are a serial chain of memory latencies, and on small tensors that chain is the
+    // kernel: with 8 and 4 vectors the five passes of a 16 -> 32 layer on 2 x 32 x 32 pixels took 4.9 us longer (36.3 ->
+    // 31.4 us for the step's kernels), 72 -> 136 on 3 x 53 x 75 pixels 4.0 us (60.9 -> 56.9).
     {
-        auto wave = [&](const void* fn, size_t dyn_smem, int min_vecs) {
+        e.wave_reduce = 0;
+        auto wave = [&](const void* fn, size_t dyn_smem, int min_vecs, int* resident = nullptr) {
             int occ = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, e.tpb, dyn_smem) != cudaSuccess || occ < 1) {
                 cudaGetLastError();
                 occ = 1;
             }
             const long long cap = (long long)p->sm_count * occ;
+            if (resident) *resident = (int)cap;
             return (int)std::max<long long>(1, std::min<long long>((max_blocks + min_vecs - 1) / min_vecs, cap));
         };
         const size_t red_smem = (size_t)e.tpb * vec * sizeof(float);
         // the passes that derive their coefficients from the accumulators keep them in dynamic shared memory
         const size_t apply_smem = p->fuse_finalize ? (size_t)2 * g.c_out * sizeof(float) : 0, dy_smem = p->fuse_finalize ? (size_t)4 * g.c_out * sizeof(float) : 0;
         if (d->mode == NB_MODE_F32_REF) {
-            e.blocks_stats = wave((const void*)bn_stats_partial_kernel<float>, red_smem, 8);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, red_smem, 8);
-            e.blocks_apply = wave((const void*)bn_silu_apply_kernel<float, float, false>, 0, 4);
-            e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<float, float, false>, 0, 4);
+            e.blocks_stats = wave((const void*)bn_stats_partial_kernel<float>, red_smem, 4);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, red_smem, 4, &e.wave_reduce);
+            e.blocks_apply = wave((const void*)bn_silu_apply_kernel<float, float, false>, 0, 1);
+            e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<float, float, false>, 0, 1);
         } else if (d->mode == NB_MODE_F16_TC) {
-            e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 8);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, red_smem, 8);
-            e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __half, true, true, false, false, true>, apply_smem, 4);
-            e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __half, true, false, true>, dy_smem, 4);
+            e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, red_smem, 4, &e.wave_reduce);
+            e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __half, true, true, false, false, true>, apply_smem, 1);
+            e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __half, true, false, true>, dy_smem, 1);
         } else {
-            e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 8);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, red_smem, 8);
-            e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __nv_bfloat16, true, true, false, false, true>, apply_smem, 4);
-            e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __nv_bfloat16, true, false, true>, dy_smem, 4);
+            e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, red_smem, 4, &e.wave_reduce);
+            e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __nv_bfloat16, true, true, false, false, true>, apply_smem, 1);
+            e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __nv_bfloat16, true, false, true>, dy_smem, 1);
         }
         e.blocks_map = std::max(e.blocks_apply, e.blocks_dy);
     }
