@@ -78,7 +78,7 @@ typedef enum { NB_MODE_BF16_TC = 0, NB_MODE_F32_REF = 1, NB_MODE_F16_TC = 2 } nb
 #define NB_CBS_FLAG_SEPARATE_FINALIZE 2u /* the BatchNorm statistics are finished by separate small kernels that add
                                      per-block partial sums in a fixed order, so that they come out bit-identical from
                                      run to run (a few microseconds more per call).  By default the kernels that sum
-                                     (the tensor-core forward convolution, the backward reduce pass) add their block
+                                     (the forward convolution, the backward reduce pass) add their block
                                      sums to fp64 accumulators with atomics and the pass that follows derives its
                                      coefficients from the totals: the same values, except that a total may differ
                                      in its last fp64 bit with the order of the additions (seen in an fp32 result

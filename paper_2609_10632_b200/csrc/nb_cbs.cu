@@ -60,6 +60,13 @@ struct EwCfg {  // launch geometry of the [M][C] passes
 
 }  // namespace
 
+struct SgCfg {  // launch of one CUDA-core convolution
+    int bm, bn, splits;
+    long long kchunk;
+    dim3 grid;
+    size_t partial_bytes;  // slices as fp32 (0: one slice)
+};
+
 constexpr size_t kStatusBytes = 256;  // ST_WORDS ints, padded so that what follows in the same allocation is 256-byte aligned
 static_assert(ST_WORDS * sizeof(int) <= kStatusBytes, "status block");
 
@@ -71,8 +78,7 @@ struct nb_cbs_plan_s {
     int* status;  // device, ST_WORDS ints
     EwCfg ew;
     int nparts;      // rows of the partial-sum buffers
-    int wg_splits;   // split-K slices of the CUDA-core wgrad
-    long long wg_chunk;
+    SgCfg sg[3];     // CUDA-core convolutions: fprop, dgrad, wgrad
     TcPlan tc;       // tensor-core kernel choices (all disabled when unsupported or forced off)
     long long ld_a = 0, ld_g = 0;  // row pitch (elements) of a_out in the forward call and of g in the backward call (set by nb_cbs_plan_set_pitches; default c_out)
     const void* fwd_res = nullptr;  // residual added to the forward call's output (nb_cbs_plan_set_fwd_residual) and its row pitch
@@ -100,7 +106,8 @@ struct nb_cbs_plan_s {
     double prof_ms[SITE_COUNT] = {};
     long long prof_n[SITE_COUNT] = {};
     size_t fwd_bytes, bwd_bytes;
-    size_t infer_bytes, off_iy;  // evaluation-mode forward: scale and shift at the forward offsets, then the convolution output when not fused
+    size_t off_sgpart;           // slices of a split CUDA-core forward convolution
+    size_t infer_bytes, off_iy, off_isg;  // evaluation-mode forward: scale and shift at the forward offsets, then the convolution output when not fused
     // workspace offsets
     size_t off_scale, off_shift, off_fpart;                  // forward
     size_t off_coef, off_bpart, off_wt, off_wgpart;          // backward
@@ -205,7 +212,7 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
                               float* coef, cudaStream_t st, const void* w = nullptr, void* wt = nullptr, const WtParams* wtp = nullptr) {
     const EwCfg& e = p->ew;
     const int C = p->g.c_out;
-    const bool fuse = p->fuse_finalize && !std::is_same<YT, float>::value;
+    const bool fuse = p->fuse_finalize;
     WtParams none;
     if (!wtp) memset(&none, 0, sizeof none);
     const ChanAcc ca{fuse ? p->acc + (size_t)p->acc_copies_f * 2 * C : nullptr, p->status + ST_READERS_BWD, p->acc_copies_b};
@@ -265,42 +272,118 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
 }
 
 // ---------------------------------------------------------------- CUDA-core convolutions
+// Tile and slices.  64 x 64 where such tiles give every SM two blocks, else 32 x 64; 64 x 32 for at most 32 columns and for
+// the 16-bit fallback.  One block alone on an SM waits for its ring (0.5 us per 16-k stage, half of it latency), so where
+// the tiles give an SM fewer than two blocks the k range is cut into slices of at least eight stages, at most four blocks
+// per SM (one more than fits a wave is worse than one fewer); that costs a reduce launch and the slices' trip through L2
+// (3 to 4 us), hence not below 16 stages.
+// Measured (step): 64 -> 64 3x3 at 2 x 40 x 40, one slice 75 us, five slices 59 us; 16 -> 32 at 2 x 32 x 32, 46 -> 39 us.
+SgCfg sg_configure(const Geom& g, int kind, bool f32, int sm_count) {
+    SgCfg c{};
+    const int cols = kind == 0 ? g.c_out : kind == 1 ? g.c_in : g.kdim;
+    const int taps = (g.k + g.stride - 1) / g.stride;  // data gradient: the most taps per axis that reach an input pixel
+    const long long KK = kind == 2 ? g.m : kind == 0 ? (long long)g.kdim : (long long)taps * taps * g.c_out;
+    c.bn = (!f32 || cols <= 32) ? 32 : 64;
+    auto row_tiles = [&](int bm) {
+        if (kind != 1) return ((kind == 0 ? g.m : (long long)g.c_out) + bm - 1) / bm;
+        long long t = 0;
+        for (int cls = 0; cls < g.stride * g.stride; ++cls) t += (sg_class(g, cls).rows + bm - 1) / bm;
+        return t;
+    };
+    const long long col_tiles = (cols + c.bn - 1) / c.bn;
+    c.bm = c.bn == 64 && row_tiles(64) * col_tiles < 2 * sm_count ? 32 : 64;
+    const long long tiles = row_tiles(c.bm) * col_tiles;
+    long long splits = 1;
+    if (tiles <= 2 * sm_count && KK >= 16 * SG_BK) splits = std::max<long long>(1, std::min<long long>(4LL * sm_count / tiles, KK / (8 * SG_BK)));
+    c.kchunk = ((KK + splits - 1) / splits + SG_BK - 1) / SG_BK * SG_BK;
+    c.splits = (int)((KK + c.kchunk - 1) / c.kchunk);
+    c.grid = dim3((unsigned)row_tiles(c.bm), (unsigned)col_tiles, (unsigned)c.splits);
+    const size_t out = kind == 0 ? (size_t)g.m * g.c_out : kind == 1 ? (size_t)g.n * g.h * g.w * g.c_in : (size_t)g.c_out * g.kdim;
+    c.partial_bytes = c.splits > 1 ? (size_t)c.splits * out * 4 : 0;
+    return c;
+}
+
+template <int KIND, typename TIN, typename TO, int BM, int BN, int V>
+nb_status launch_sg_tile(const nb_cbs_plan_s* p, const SgCfg& c, const void* a, const void* b, void* out, const SgArgs& args, cudaStream_t st) {
+    using T = SgTile<KIND, BM, BN>;
+    const size_t flush = (size_t)T::TM * 4 * SG_THREADS * sizeof(double);
+    // Blocks become resident while the previous kernel still runs, wherever it leaves room: with room for five on an SM, 100
+    // blocks of a small layer pile up on a few of them (measured: 28 us alone, 50 us behind the passes of the block).
+    // Enough shared memory is asked for that an SM takes no more than its share.
+    const long long blocks = (long long)c.grid.x * c.grid.y * c.grid.z;
+    const long long share = (blocks + p->sm_count - 1) / p->sm_count;
+    const size_t smem = std::max(T::stage_bytes(sizeof(TIN)) + (c.kchunk > 1024 ? flush : 0), share <= 4 ? (size_t)(233472 / (share + 1)) : (size_t)0);
+    static std::atomic<unsigned long long> attr_set{0};  // one bit per device ordinal
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(attr_set.load(std::memory_order_acquire) & bit)) {
+        NB_CUDA_CHECK(cudaFuncSetAttribute(simt_gemm_kernel<KIND, TIN, TO, BM, BN, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024));
+        attr_set.fetch_or(bit, std::memory_order_release);
+    }
+    launch_k(simt_gemm_kernel<KIND, TIN, TO, BM, BN, V>, c.grid, dim3(SG_THREADS), smem, st, 1, static_cast<const TIN*>(a), static_cast<const TIN*>(b), static_cast<TO*>(out), args);
+    return launch_ok("simt convolution");
+}
+template <int KIND, typename TIN, typename TO>
+nb_status launch_sg(const nb_cbs_plan_s* p, const void* a, const void* b, void* out, const SgArgs& args, cudaStream_t st) {
+    const SgCfg& c = p->sg[KIND];
+    const bool vec = p->g.c_in % 4 == 0;
+    if constexpr (std::is_same<TIN, float>::value) {
+        if (c.bn == 64 && c.bm == 64) return vec ? launch_sg_tile<KIND, TIN, TO, 64, 64, 4>(p, c, a, b, out, args, st) : launch_sg_tile<KIND, TIN, TO, 64, 64, 1>(p, c, a, b, out, args, st);
+        if (c.bn == 64) return vec ? launch_sg_tile<KIND, TIN, TO, 32, 64, 4>(p, c, a, b, out, args, st) : launch_sg_tile<KIND, TIN, TO, 32, 64, 1>(p, c, a, b, out, args, st);
+    }
+    return vec ? launch_sg_tile<KIND, TIN, TO, 64, 32, 4>(p, c, a, b, out, args, st) : launch_sg_tile<KIND, TIN, TO, 64, 32, 1>(p, c, a, b, out, args, st);
+}
+
+// `sums`: with a default plan the channel sums of y go to the plan's accumulators (false: y only, or separate statistics).
 template <typename TIN, typename TOUT>
-nb_status run_simt_fprop(nb_cbs_plan_s* p, const void* x, const void* w, void* y, cudaStream_t st) {
-    FpropProblem<TIN, TIN> prob{static_cast<const TIN*>(x), static_cast<const TIN*>(w), p->g};
-    dim3 grid((unsigned)((p->g.m + SIMT_BM - 1) / SIMT_BM), (unsigned)((p->g.c_out + SIMT_BN - 1) / SIMT_BN), 1);
-    SiteTimer tm(p, SITE_FPROP, st);
-    launch_k(simt_gemm_kernel<FpropProblem<TIN, TIN>, TOUT>, grid, dim3(256), 0, st, 1, prob, static_cast<TOUT*>(y), (long long)p->g.kdim);
-    return launch_ok("simt fprop");
+nb_status run_simt_fprop(nb_cbs_plan_s* p, const void* x, const void* w, void* y, void* partial, bool sums, cudaStream_t st) {
+    const SgCfg& c = p->sg[0];
+    const ChanAcc ca{sums ? p->acc : nullptr, nullptr, sums ? p->acc_copies_f : 1};
+    const SgArgs args{p->g, c.kchunk, sums && c.splits == 1, ca};
+    {
+        SiteTimer tm(p, SITE_FPROP, st);
+        if (c.splits == 1) return launch_sg<0, TIN, TOUT>(p, x, w, y, args, st);
+        NB_TRY((launch_sg<0, TIN, float>(p, x, w, partial, args, st)));
+    }
+    SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
+    const int cgs = p->g.c_out / 4, tpb = cgs >= 256 ? cgs : 256 / cgs * cgs;
+    const long long vecs = p->g.m * cgs;
+    const long long blocks = std::min<long long>((vecs + tpb - 1) / tpb, (long long)p->sm_count * 4);
+    launch_k(splitk_fwd_reduce_kernel<TOUT>, dim3((unsigned)blocks), dim3(tpb), (size_t)tpb * 16, st, 1, static_cast<const float*>(partial), c.splits, vecs, p->g.c_out,
+             static_cast<TOUT*>(y), ca);
+    return launch_ok("splitk_fwd_reduce");
 }
 
 template <typename TIN>
-nb_status run_simt_dgrad(nb_cbs_plan_s* p, const void* dy, const void* w, void* dx, cudaStream_t st) {
-    DgradProblem<TIN, TIN> prob{static_cast<const TIN*>(dy), static_cast<const TIN*>(w), p->g};
-    const long long I = (long long)p->g.n * p->g.h * p->g.w;
-    dim3 grid((unsigned)((I + SIMT_BM - 1) / SIMT_BM), (unsigned)((p->g.c_in + SIMT_BN - 1) / SIMT_BN), 1);
-    SiteTimer tm(p, SITE_DGRAD, st);
-    launch_k(simt_gemm_kernel<DgradProblem<TIN, TIN>, TIN>, grid, dim3(256), 0, st, 1, prob, static_cast<TIN*>(dx), (long long)p->g.k * p->g.k * p->g.c_out);
-    return launch_ok("simt dgrad");
+nb_status run_simt_dgrad(nb_cbs_plan_s* p, const void* dy, const void* w, void* dx, void* partial, cudaStream_t st) {
+    const SgCfg& c = p->sg[1];
+    const SgArgs args{p->g, c.kchunk, false, ChanAcc{nullptr, nullptr, 1}};
+    {
+        SiteTimer tm(p, SITE_DGRAD, st);
+        if (c.splits == 1) return launch_sg<1, TIN, TIN>(p, dy, w, dx, args, st);
+        NB_TRY((launch_sg<1, TIN, float>(p, dy, w, partial, args, st)));
+    }
+    const size_t elems = (size_t)p->g.n * p->g.h * p->g.w * p->g.c_in;
+    SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
+    const unsigned blocks = (unsigned)std::min<size_t>((elems / 4 + 255) / 256 + 1, (size_t)p->sm_count * 8);
+    launch_k(splitk_reduce_kernel<TIN>, dim3(blocks), dim3(256), 0, st, 1, static_cast<const float*>(partial), c.splits, elems, static_cast<TIN*>(dx));
+    return launch_ok("splitk_reduce");
 }
 
 template <typename TIN>
 nb_status run_simt_wgrad(nb_cbs_plan_s* p, const void* x, const void* dy, float* dw, float* partial, cudaStream_t st) {
-    WgradProblem<TIN, TIN> prob{static_cast<const TIN*>(dy), static_cast<const TIN*>(x), p->g};
-    dim3 grid((unsigned)((p->g.c_out + SIMT_BM - 1) / SIMT_BM), (unsigned)((p->g.kdim + SIMT_BN - 1) / SIMT_BN), (unsigned)p->wg_splits);
-    if (p->wg_splits == 1) {
-        SiteTimer tm(p, SITE_WGRAD, st);
-        launch_k(simt_gemm_kernel<WgradProblem<TIN, TIN>, float>, grid, dim3(256), 0, st, 1, prob, dw, p->g.m);
-        return launch_ok("simt wgrad");
-    }
+    const SgCfg& c = p->sg[2];
+    const SgArgs args{p->g, c.kchunk, false, ChanAcc{nullptr, nullptr, 1}};
     {
         SiteTimer tm(p, SITE_WGRAD, st);
-        launch_k(simt_gemm_kernel<WgradProblem<TIN, TIN>, float>, grid, dim3(256), 0, st, 1, prob, partial, p->wg_chunk);
-        NB_LAUNCH_OK("simt wgrad (split-K)");
+        NB_TRY((launch_sg<2, TIN, float>(p, dy, x, c.splits == 1 ? dw : partial, args, st)));
+        if (c.splits == 1) return NB_OK;
     }
     const size_t elems = (size_t)p->g.c_out * p->g.kdim;
     SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
-    launch_k(splitk_reduce_kernel, dim3((unsigned)((elems + 255) / 256)), dim3(256), 0, st, 1, partial, p->wg_splits, elems, dw);
+    if (c.splits >= 96) launch_k(splitk_reduce_tall_kernel, dim3((unsigned)((elems + 31) / 32)), dim3(1024), 0, st, 1, partial, c.splits, elems, dw);
+    else launch_k(splitk_reduce_kernel<float>, dim3((unsigned)std::min<size_t>((elems / 4 + 255) / 256 + 1, (size_t)p->sm_count * 8)), dim3(256), 0, st, 1, partial, c.splits, elems, dw);
     return launch_ok("splitk_reduce");
 }
 
@@ -355,7 +438,7 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     p->g = g;
     p->device = device;
     p->sm_count = prop.multiProcessorCount;
-    p->fuse_finalize = !(d->flags & NB_CBS_FLAG_SEPARATE_FINALIZE) && d->mode != NB_MODE_F32_REF;
+    p->fuse_finalize = !(d->flags & NB_CBS_FLAG_SEPARATE_FINALIZE);
 
     EwCfg& e = p->ew;
     e.vec = vec;
@@ -387,8 +470,8 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
         if (d->mode == NB_MODE_F32_REF) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<float>, red_smem, 4);
             e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, red_smem, 4, &e.wave_reduce);
-            e.blocks_apply = wave((const void*)bn_silu_apply_kernel<float, float, false>, 0, 1);
-            e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<float, float, false>, 0, 1);
+            e.blocks_apply = wave((const void*)bn_silu_apply_kernel<float, float, false, true, false, false, true>, apply_smem, 1);
+            e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<float, float, false, false, true>, dy_smem, 1);
         } else if (d->mode == NB_MODE_F16_TC) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
             e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, red_smem, 4, &e.wave_reduce);
@@ -403,18 +486,7 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
         e.blocks_map = std::max(e.blocks_apply, e.blocks_dy);
     }
 
-    // CUDA-core wgrad split-K: enough slices to fill the machine, at least 512 rows each.
-    {
-        const long long tiles = (long long)((g.c_out + SIMT_BM - 1) / SIMT_BM) * ((g.kdim + SIMT_BN - 1) / SIMT_BN);
-        long long splits = (4LL * p->sm_count + tiles - 1) / tiles;
-        const long long max_splits = std::max<long long>(1, g.m / 512);
-        splits = std::max<long long>(1, std::min(splits, max_splits));
-        long long chunk = (g.m + splits - 1) / splits;
-        chunk = (chunk + SIMT_BK - 1) / SIMT_BK * SIMT_BK;
-        splits = (g.m + chunk - 1) / chunk;
-        p->wg_splits = (int)splits;
-        p->wg_chunk = chunk;
-    }
+    for (int kind = 0; kind < 3; ++kind) p->sg[kind] = sg_configure(g, kind, d->mode == NB_MODE_F32_REF, p->sm_count);
 
     int cur = 0;
     NB_CUDA_CHECK(cudaGetDevice(&cur));
@@ -471,16 +543,19 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     p->off_scale = off; off = align_up(off + C * 4, 256);
     p->off_shift = off; off = align_up(off + C * 4, 256);
     p->off_fpart = off; off = align_up(off + (size_t)p->nparts * 2 * C * 4, 256);
+    const bool simt_fwd = !p->stem && !p->tc.fprop, simt_dg = !p->stem && !p->tc.dgrad, simt_wg = !p->stem && !p->tc.wgrad;
+    p->off_sgpart = off; off = align_up(off + (simt_fwd ? p->sg[0].partial_bytes : 0), 256);
     p->fwd_bytes = off;
     p->off_iy = p->off_fpart;
-    p->infer_bytes = infer_fused(p) ? p->off_fpart : align_up(p->off_iy + (size_t)g.m * C * (is_f32(p) ? 4 : 2), 256);
+    p->off_isg = align_up(p->off_iy + (size_t)g.m * C * (is_f32(p) ? 4 : 2), 256);
+    p->infer_bytes = infer_fused(p) ? p->off_fpart : align_up(p->off_isg + p->sg[0].partial_bytes, 256);
     off = 0;
     p->off_coef = off; off = align_up(off + 4 * C * 4, 256);
     p->off_bpart = off; off = align_up(off + (size_t)p->nparts * 2 * C * 4, 256);
     p->off_wt = off; off = align_up(off + p->tc.wt_bytes, 256);
     p->off_wgpart = off;
     {
-        size_t simt = p->wg_splits > 1 ? (size_t)p->wg_splits * C * g.kdim * 4 : 0;
+        const size_t simt = std::max(simt_wg ? p->sg[2].partial_bytes : 0, simt_dg ? p->sg[1].partial_bytes : 0);
         size_t stem = p->stem ? (size_t)p->stem_blocks * C * g.kdim * 4 : 0;
         off = align_up(off + std::max(std::max(simt, stem), p->tc.wgrad_partial_bytes), 256);
     }
@@ -562,7 +637,7 @@ nb_status nb_cbs_plan_set_bwd_residual(nb_cbs_plan p, void* gres, int64_t ld_gre
     if (ld_gres == p->g.c_out) ld_gres = 0;
     if (gres && ld_gres != 0 && (ld_gres < p->g.c_out || ld_gres % 8 != 0))
         return fail(NB_ERR_INVALID_ARG, "ld_gres must be 0 (dense) or at least c_out and a multiple of 8 elements");
-    if (gres && !p->fuse_finalize)
+    if (gres && (!p->fuse_finalize || is_f32(p)))
         return fail(NB_ERR_UNSUPPORTED, "the shortcut's gradient rides in the dy pass of the default 16-bit plans only (not fp32 mode, not NB_CBS_FLAG_SEPARATE_FINALIZE)");
     p->bwd_gres = gres;
     p->ld_gres = gres ? ld_gres : 0;
@@ -659,8 +734,9 @@ nb_status nb_conv_bn_silu_fwd(nb_cbs_plan p, const void* x, const void* w, const
     int nparts = p->ew.blocks_stats;
     bool finalized = false;
     if (is_f32(p)) {
-        NB_TRY((run_simt_fprop<float, float>(p, x, w, y_saved, st)));
-        NB_TRY(run_stats_partial<float>(p, y_saved, part, st));
+        NB_TRY((run_simt_fprop<float, float>(p, x, w, y_saved, ws + p->off_sgpart, p->fuse_finalize, st)));
+        finalized = p->fuse_finalize;
+        if (!finalized) NB_TRY(run_stats_partial<float>(p, y_saved, part, st));
     } else if (p->stem) {
         // the first layer's kernel sums the statistics of the values it stores itself (one partial slice per block)
         SiteTimer tm(p, SITE_FPROP, st);
@@ -689,15 +765,16 @@ nb_status nb_conv_bn_silu_fwd(nb_cbs_plan p, const void* x, const void* w, const
         nparts = p->tc.fprop_parts;
         finalized = fuse;
     } else {
-        NB_TRY(NB_WITH_AT(p, run_simt_fprop<AT, __half>(p, x, w, y_saved, st)));
-        NB_TRY(run_stats_partial<__half>(p, y_saved, part, st));
+        NB_TRY(NB_WITH_AT(p, run_simt_fprop<AT, __half>(p, x, w, y_saved, ws + p->off_sgpart, p->fuse_finalize, st)));
+        finalized = p->fuse_finalize;
+        if (!finalized) NB_TRY(run_stats_partial<__half>(p, y_saved, part, st));
     }
     if (!finalized)
         NB_TRY(run_finalize(p, part, nparts, gamma, beta, save_mean, save_invstd, scale, shift, running_mean, running_var, nullptr, nullptr, st));
-    if (is_f32(p)) return run_apply<float, float, false>(p, y_saved, a_out, scale, shift, st, p->ld_a, p->fwd_res, p->ld_res);
-    // after the tensor-core kernel the pass derives mean, invstd, scale and shift from the accumulators itself
+    // when the convolution has left its sums in the accumulators the pass derives mean, invstd, scale and shift from them itself
     const double M = (double)p->g.m;
     const FwdFin fin{1.0 / M, M / (M - 1.0), p->desc.eps, p->desc.momentum, gamma, beta, save_mean, save_invstd, running_mean, running_var};
+    if (is_f32(p)) return run_apply<float, float, false>(p, y_saved, a_out, scale, shift, st, p->ld_a, p->fwd_res, p->ld_res, finalized ? &fin : nullptr);
     return NB_WITH_AT(p, run_apply<__half, AT, true>(p, y_saved, a_out, scale, shift, st, p->ld_a, p->fwd_res, p->ld_res, finalized ? &fin : nullptr));
 }
 
@@ -731,9 +808,9 @@ nb_status run_infer(nb_cbs_plan_s* p, const void* x, const void* w, const float*
     float* shift = reinterpret_cast<float*>(ws + p->off_shift);
     void* y = ws + p->off_iy;
     if (is_f32(p)) {
-        NB_TRY((run_simt_fprop<float, float>(p, x, w, y, st)));
+        NB_TRY((run_simt_fprop<float, float>(p, x, w, y, ws + p->off_isg, false, st)));
     } else {
-        NB_TRY(NB_WITH_AT(p, run_simt_fprop<AT, __half>(p, x, w, y, st)));
+        NB_TRY(NB_WITH_AT(p, run_simt_fprop<AT, __half>(p, x, w, y, ws + p->off_isg, false, st)));
     }
     {
         SiteTimer tm(p, SITE_EVAL_COEF, st);
@@ -834,7 +911,7 @@ nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan p, const void* g, const void* y_s
     float* part = reinterpret_cast<float*>(ws + p->off_bpart);
     if (is_f32(p)) {
         NB_TRY((run_bwd_elementwise<float, float, false>(p, g, y_saved, save_mean, save_invstd, gamma, beta, dgamma, dbeta, dy_out, part, coef, st)));
-        if (dx) NB_TRY(run_simt_dgrad<float>(p, dy_out, w, dx, st));
+        if (dx) NB_TRY(run_simt_dgrad<float>(p, dy_out, w, dx, ws + p->off_wgpart, st));
         return NB_OK;
     }
     const bool tc_dg = dx && !p->stem && p->tc.dgrad;  // the finalize kernel also rearranges the filter for the tensor-core dgrad
@@ -855,7 +932,7 @@ nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan p, const void* g, const void* y_s
         if (ts != NB_OK) return fail(ts, "%s", tc_last_error());
         return NB_OK;
     }
-    return NB_WITH_AT(p, run_simt_dgrad<AT>(p, dy_out, w, dx, st));
+    return NB_WITH_AT(p, run_simt_dgrad<AT>(p, dy_out, w, dx, ws + p->off_wgpart, st));
 }
 
 nb_status nb_conv_bias_bwd(nb_cbs_plan p, const void* x, const void* w, const void* dout, void* dx, float* dw, float* dbias, void* workspace,
@@ -878,7 +955,7 @@ nb_status nb_conv_bias_bwd(nb_cbs_plan p, const void* x, const void* w, const vo
         }
         if (dx) {
             if (is_f32(p)) {
-                NB_TRY(run_simt_dgrad<float>(p, dout, w, dx, st));
+                NB_TRY(run_simt_dgrad<float>(p, dout, w, dx, ws + p->off_wgpart, st));
             } else if (p->stem) {
                 SiteTimer tm(p, SITE_DGRAD, st);
                 NB_WITH_AT(p, launch_k(stem_dgrad_mma_kernel<48, AT>, dim3(p->stem_dgrad_blocks), dim3(128), 0, st, 1, static_cast<const AT*>(dout), static_cast<const AT*>(w),
@@ -891,7 +968,7 @@ nb_status nb_conv_bias_bwd(nb_cbs_plan p, const void* x, const void* w, const vo
                 g_launches.fetch_add((unsigned long long)(p->tc.launches - l0), std::memory_order_relaxed);
                 if (ts != NB_OK) return fail(ts, "%s", tc_last_error());
             } else {
-                NB_TRY(NB_WITH_AT(p, run_simt_dgrad<AT>(p, dout, w, dx, st)));
+                NB_TRY(NB_WITH_AT(p, run_simt_dgrad<AT>(p, dout, w, dx, ws + p->off_wgpart, st)));
             }
         }
     }

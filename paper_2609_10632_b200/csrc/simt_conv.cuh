@@ -1,166 +1,453 @@
-// CUDA-core implicit GEMMs for the three convolutions (fprop, dgrad, wgrad): any shape, fp32 or bf16 inputs,
+// CUDA-core implicit GEMMs for the three convolutions (fprop, dgrad, wgrad): any shape, fp32 or 16-bit inputs,
 // fp32 accumulation flushed into fp64 every 1024 terms.  They carry the fp32 reference mode and every shape
-// the tensor-core kernels do not take; they are not tuned.
+// the tensor-core kernels do not take.
 #pragma once
 #include "common.cuh"
+#include "elementwise.cuh"
 
 namespace nbcbs {
 
-// out[i][j] = sum_kk A(i,kk) * B(kk,j).  A policy supplies the extents and element loaders.
-template <typename TX, typename TW> struct FpropProblem {
-    const TX* x;
-    const TW* w;
-    Geom g;
-    static constexpr bool A_KCONTIG = true, B_KCONTIG = true;
-    __device__ long long I() const { return g.m; }
-    __device__ int J() const { return g.c_out; }
-    __device__ long long KK() const { return g.kdim; }
-    __device__ float loadA(long long i, long long kk) const {
-        const int q = (int)(i % g.wo);
-        const long long t1 = i / g.wo;
-        const int p = (int)(t1 % g.ho), n = (int)(t1 / g.ho);
-        const int c = (int)(kk % g.c_in);
-        const int t2 = (int)(kk / g.c_in);
-        const int t = t2 % g.k, r = t2 / g.k;
-        const int h = p * g.stride - g.pad + r, ww = q * g.stride - g.pad + t;
-        if (h < 0 || h >= g.h || ww < 0 || ww >= g.w) return 0.f;
-        return to_f32(x[(((size_t)n * g.h + h) * g.w + ww) * g.c_in + c]);
+// out[i][j] = sum_kk A(i,kk) * B(kk,j) on plain FMA units.  Bound: FMA issue on large problems (a thread's 8 x 4 tile takes
+// 12 16-byte shared loads per 128 multiply-adds), memory latency on small ones.  A block is 128 threads on a
+// [BM x BN] tile; both operand tiles travel global -> shared memory by cp.async through a ring of four stages of 16 k
+// (element-wise loads into registers, two block barriers per 16 k and an index decode by 64-bit divisions per element
+// are what the previous version spent its time on: 64 -> 64 channels 3x3 on 2 x 40 x 40 pixels, step 445 -> 59 us;
+// 96 -> 96 at 2 x 80 x 80, 990 -> 275 us, 24 TFLOP/s in the convolutions; 31 with the idle columns of the second tile).
+//   KIND 0 (fprop): rows = output pixels, cols = c_out, k = (tap, c_in).   A, B tiles [row][k], [col][k]
+//   KIND 1 (dgrad): rows = input pixels, cols = c_in, k = (tap, c_out).    A tile [row][k], B tile [k][col]
+//   KIND 2 (wgrad): rows = c_out, cols = (tap, c_in), k = output pixels.   A, B tiles [k][row], [k][col]
+// A stride-2 data gradient walks the parity classes of the input pixels one after the other, each with the taps that
+// reach it (a quarter of the products of the undivided sum).
+// V = 4: channels come as vectors of four (c_in % 4 == 0); V = 1: element by element (c_in = 3).
+constexpr int SG_BK = 16, SG_STAGES = 4, SG_THREADS = 128, SG_KPITCH = SG_BK + 4, SG_FLUSH = 1024 / SG_BK;
+
+template <typename T> __device__ __forceinline__ float4 sg_ld4(const T* p);
+template <> __device__ __forceinline__ float4 sg_ld4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
+template <> __device__ __forceinline__ float4 sg_ld4<__nv_bfloat16>(const __nv_bfloat16* p) {
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+template <> __device__ __forceinline__ float4 sg_ld4<__half>(const __half* p) {
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+// four elements global -> shared, zeros when !ok (src is then any valid address)
+template <typename T> __device__ __forceinline__ void sg_copy4(T* dst, const T* src, bool ok) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if (sizeof(T) == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+template <typename T> __device__ __forceinline__ void sg_copy1(T* dst, const T* src, bool ok) {
+    if (sizeof(T) == 4) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 4 : 0) : "memory");
+    } else {
+        *dst = ok ? *src : from_f32<T>(0.f);  // (cp.async moves at least four bytes)
     }
-    __device__ float loadB(long long kk, int j) const { return to_f32(w[(size_t)j * g.kdim + kk]); }
+}
+
+template <int KIND, int BM, int BN> struct SgTile {
+    static constexpr int A_ELEMS = KIND == 2 ? SG_BK * (BM + 4) : BM * SG_KPITCH;
+    static constexpr int B_ELEMS = KIND == 0 ? BN * SG_KPITCH : SG_BK * (BN + 4);
+    static constexpr int NTX = BN / 4, NTY = SG_THREADS / NTX, TM = BM / NTY;
+    static __host__ __device__ constexpr size_t stage_bytes(size_t elem) { return SG_STAGES * (size_t)(A_ELEMS + B_ELEMS) * elem; }
 };
 
-template <typename TD, typename TW> struct DgradProblem {
-    const TD* dy;
-    const TW* w;
+struct SgArgs {
     Geom g;
-    static constexpr bool A_KCONTIG = true, B_KCONTIG = false;
-    __device__ long long I() const { return (long long)g.n * g.h * g.w; }
-    __device__ int J() const { return g.c_in; }
-    __device__ long long KK() const { return (long long)g.k * g.k * g.c_out; }
-    __device__ float loadA(long long i, long long kk) const {
-        const int ww = (int)(i % g.w);
-        const long long t1 = i / g.w;
-        const int h = (int)(t1 % g.h), n = (int)(t1 / g.h);
-        const int co = (int)(kk % g.c_out);
-        const int t2 = (int)(kk / g.c_out);
-        const int t = t2 % g.k, r = t2 / g.k;
-        const int hp = h + g.pad - r, wq = ww + g.pad - t;
-        if (hp < 0 || wq < 0 || (hp % g.stride) != 0 || (wq % g.stride) != 0) return 0.f;
-        const int p = hp / g.stride, q = wq / g.stride;
-        if (p >= g.ho || q >= g.wo) return 0.f;
-        return to_f32(dy[(((size_t)n * g.ho + p) * g.wo + q) * g.c_out + co]);
-    }
-    __device__ float loadB(long long kk, int j) const {
-        const int co = (int)(kk % g.c_out);
-        const int rt = (int)(kk / g.c_out);
-        return to_f32(w[((size_t)co * g.k * g.k + rt) * g.c_in + j]);
-    }
+    long long kchunk;  // k per slice (blockIdx.z), a multiple of SG_BK
+    bool stats;        // KIND 0 with one slice: add the channel sums of the stored values to `acc`
+    ChanAcc acc;
 };
 
-template <typename TD, typename TX> struct WgradProblem {
-    const TD* dy;
-    const TX* x;
-    Geom g;
-    static constexpr bool A_KCONTIG = false, B_KCONTIG = false;
-    __device__ long long I() const { return g.c_out; }
-    __device__ int J() const { return g.kdim; }
-    __device__ long long KK() const { return g.m; }
-    __device__ float loadA(long long i, long long kk) const { return to_f32(dy[(size_t)kk * g.c_out + i]); }
-    __device__ float loadB(long long kk, int j) const {
-        const int q = (int)(kk % g.wo);
-        const long long t1 = kk / g.wo;
-        const int p = (int)(t1 % g.ho), n = (int)(t1 / g.ho);
-        const int c = j % g.c_in;
-        const int t2 = j / g.c_in;
-        const int t = t2 % g.k, r = t2 / g.k;
-        const int h = p * g.stride - g.pad + r, ww = q * g.stride - g.pad + t;
-        if (h < 0 || h >= g.h || ww < 0 || ww >= g.w) return 0.f;
-        return to_f32(x[(((size_t)n * g.h + h) * g.w + ww) * g.c_in + c]);
-    }
+// rows of parity class `cls` of a data gradient, and the grid that covers all classes (host and device)
+struct SgClass {
+    int pa, pb, hc, wc;  // parities, rows and columns of the class's pixel grid
+    long long rows;
 };
+__host__ __device__ __forceinline__ SgClass sg_class(const Geom& g, int cls) {
+    SgClass c;
+    c.pa = cls / g.stride;
+    c.pb = cls % g.stride;
+    c.hc = (g.h - c.pa + g.stride - 1) / g.stride;
+    c.wc = (g.w - c.pb + g.stride - 1) / g.stride;
+    c.rows = (long long)g.n * c.hc * c.wc;
+    return c;
+}
 
-constexpr int SIMT_BM = 64, SIMT_BN = 64, SIMT_BK = 16, SIMT_FLUSH = 64;
-
-// grid (ceil(I/64), ceil(J/64), splits); block 256.  With splits > 1, `out` is a float partial buffer
-// [splits][I][J] and slice z covers kk in [z*kchunk, (z+1)*kchunk).
-template <class P, typename TO>
-__global__ void __launch_bounds__(256) simt_gemm_kernel(P prob, TO* __restrict__ out, long long kchunk) {
+// grid (row tiles, column tiles, slices).  With several slices `out` is a float buffer [slices][rows][cols].
+template <int KIND, typename TIN, typename TO, int BM, int BN, int V>
+__global__ void __launch_bounds__(SG_THREADS) simt_gemm_kernel(const TIN* __restrict__ asrc, const TIN* __restrict__ bsrc, TO* __restrict__ out, const SgArgs p) {
     pdl_launch_dependents();
-    pdl_wait();
-    __shared__ float As[SIMT_BK][SIMT_BM + 4];
-    __shared__ float Bs[SIMT_BK][SIMT_BN + 4];
-    const long long I = prob.I();
-    const int J = prob.J();
-    const long long KK = prob.KK();
-    const long long i0 = (long long)blockIdx.x * SIMT_BM;
-    const int j0 = blockIdx.y * SIMT_BN;
-    const long long kbeg = (long long)blockIdx.z * kchunk;
-    const long long kend = (kbeg + kchunk < KK) ? kbeg + kchunk : KK;
-    const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-    float acc[4][4];
-    double dacc[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            acc[a][b] = 0.f;
-            dacc[a][b] = 0.0;
+    using T = SgTile<KIND, BM, BN>;
+    constexpr int TM = T::TM, NTX = T::NTX, NTY = T::NTY;
+    extern __shared__ __align__(16) uint8_t sg_smem[];
+    TIN* const sA = reinterpret_cast<TIN*>(sg_smem);
+    TIN* const sB = sA + SG_STAGES * T::A_ELEMS;
+    double* const flushed = reinterpret_cast<double*>(sg_smem + T::stage_bytes(sizeof(TIN)));  // [TM * 4][128 threads], slices longer than 1024 only
+    const Geom& g = p.g;
+    const int tid = threadIdx.x, tx = tid % NTX, ty = tid / NTX;
+    const int j0 = blockIdx.y * BN;
+    const int cols = KIND == 0 ? g.c_out : KIND == 1 ? g.c_in : g.kdim;
+
+    // ---- the row tile: its class (data gradient), first row, taps
+    long long i0 = (long long)blockIdx.x * BM, rows = KIND == 0 ? g.m : KIND == 1 ? 0 : g.c_out;
+    SgClass cl{0, 0, g.h, g.w, 0};
+    int r_first = 0, r_step = 1, nr = g.k, t_first = 0, nt = g.k;
+    if (KIND == 1) {
+        long long tile = blockIdx.x;
+        int cls = 0;
+        cl = sg_class(g, 0);
+        while (tile >= (cl.rows + BM - 1) / BM) {
+            tile -= (cl.rows + BM - 1) / BM;
+            cl = sg_class(g, ++cls);
         }
-    int since = 0;
-    for (long long k0 = kbeg; k0 < kend; k0 += SIMT_BK) {
+        i0 = tile * BM;
+        rows = cl.rows;
+        r_step = g.stride;
+        r_first = (cl.pa + g.pad) % g.stride;
+        t_first = (cl.pb + g.pad) % g.stride;
+        nr = (g.k - r_first + r_step - 1) / r_step;
+        nt = (g.k - t_first + r_step - 1) / r_step;
+    }
+    const int ntd = nt > 0 ? nt : 1;  // (no tap reaches the odd pixels of a 1x1 stride-2 layer: K = 0, zeros are stored)
+    const int kch = KIND == 1 ? g.c_out : g.c_in;  // channels per tap on the k side (KIND 0, 1)
+    const long long KK = KIND == 2 ? g.m : (long long)nr * nt * kch;
+    const long long kbeg = (long long)blockIdx.z * p.kchunk;
+    const long long kend = kbeg + p.kchunk < KK ? kbeg + p.kchunk : KK;
+    const int nsteps = kend > kbeg ? (int)((kend - kbeg + SG_BK - 1) / SG_BK) : 0;
+
+    // ---- loader state (advanced by one stage per call)
+    // [row][k] tiles: a thread copies four k (kv) of rows tid / 4 + 32 i
+    constexpr int AP = KIND == 2 ? BM * SG_BK / 4 / SG_THREADS : BM / 32;  // copies of four per thread and stage
+    constexpr int BP = KIND == 0 ? BN / 32 : BN * SG_BK / 4 / SG_THREADS;
+    const int kv = (tid & 3) * 4;
+    int a_h[AP > 0 ? AP : 1], a_w[AP > 0 ? AP : 1];
+    long long a_base[AP > 0 ? AP : 1];
+    bool a_ok[AP > 0 ? AP : 1];
+    int tap_r = 0, tap_t = 0, ch = 0;  // tap and channel of this thread's four k (V = 4, or KIND 1)
+    if (KIND != 2) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int idx = tid + e * 256;
-            int il, kl;
-            if (P::A_KCONTIG) { kl = idx % SIMT_BK; il = idx / SIMT_BK; } else { il = idx % SIMT_BM; kl = idx / SIMT_BM; }
-            As[kl][il] = (i0 + il < I && k0 + kl < kend) ? prob.loadA(i0 + il, k0 + kl) : 0.f;
-            int jl, kb;
-            if (P::B_KCONTIG) { kb = idx % SIMT_BK; jl = idx / SIMT_BK; } else { jl = idx % SIMT_BN; kb = idx / SIMT_BN; }
-            Bs[kb][jl] = (j0 + jl < J && k0 + kb < kend) ? prob.loadB(k0 + kb, j0 + jl) : 0.f;
+        for (int i = 0; i < AP; ++i) {
+            const long long row = i0 + (tid >> 2) + 32 * i;
+            a_ok[i] = row < rows;
+            const long long rr = a_ok[i] ? row : 0;
+            if (KIND == 0) {
+                const int q = (int)(rr % g.wo);
+                const long long t1 = rr / g.wo;
+                const int pp = (int)(t1 % g.ho);
+                a_base[i] = (t1 / g.ho) * g.h * g.w;
+                a_h[i] = pp * g.stride - g.pad;
+                a_w[i] = q * g.stride - g.pad;
+            } else {  // dy row and column of tap (r, t): (h + pad - r) / stride
+                const int j = (int)(rr % cl.wc);
+                const long long t1 = rr / cl.wc;
+                const int ii = (int)(t1 % cl.hc);
+                a_base[i] = (t1 / cl.hc) * g.ho * g.wo;
+                a_h[i] = (ii * g.stride + cl.pa + g.pad - r_first) / g.stride;
+                a_w[i] = (j * g.stride + cl.pb + g.pad - t_first) / g.stride;
+            }
         }
-        __syncthreads();
+        const long long k0 = kbeg + kv;
+        const int tap = (int)(k0 / kch);
+        ch = (int)(k0 - (long long)tap * kch);
+        tap_r = tap / ntd;
+        tap_t = tap - tap_r * ntd;
+    }
+    // [k][..] tiles: a thread copies four neighbouring rows / columns of k rows kr + i * step
+    const int a_mv = (tid % (BM / 4)) * 4, a_kr = tid / (BM / 4);
+    constexpr int A_KSTEP = SG_THREADS / (BM / 4), B_KSTEP = SG_THREADS / (BN / 4);
+    const int b_nv = (tid % (BN / 4)) * 4, b_kr = tid / (BN / 4);
+    int px_n[KIND == 2 ? BP : 1], px_p[KIND == 2 ? BP : 1], px_q[KIND == 2 ? BP : 1];  // pixel of each k row (weight gradient)
+    int b_r[KIND == 2 ? 4 : 1], b_t[KIND == 2 ? 4 : 1], b_c[KIND == 2 ? 4 : 1];        // tap and channel of this thread's columns
+    if (KIND == 2) {
 #pragma unroll
-        for (int kk = 0; kk < SIMT_BK; ++kk) {
-            float a[4], b[4];
+        for (int i = 0; i < BP; ++i) {
+            const long long px = kbeg + b_kr + i * B_KSTEP;
+            const long long t1 = px / g.wo;
+            px_q[i] = (int)(px - t1 * g.wo);
+            px_n[i] = (int)(t1 / g.ho);
+            px_p[i] = (int)(t1 - (long long)px_n[i] * g.ho);
+        }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = As[kk][ty * 4 + u];
-                b[u] = Bs[kk][tx * 4 + u];
+        for (int e = 0; e < (V == 4 ? 1 : 4); ++e) {
+            const int j = j0 + b_nv + e < cols ? j0 + b_nv + e : 0;
+            const int tap = j / g.c_in;
+            b_c[e] = j - tap * g.c_in;
+            b_r[e] = tap / g.k;
+            b_t[e] = tap - b_r[e] * g.k;
+        }
+    }
+    long long kload = kbeg;  // first k of the next stage to load
+    auto load_stage = [&](int s) {
+        TIN* const a_s = sA + s * T::A_ELEMS;
+        TIN* const b_s = sB + s * T::B_ELEMS;
+        if (KIND == 0 && V == 1) {  // element by element, k decoded per element
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const long long kk = kload + kv + e;
+                const int tap = (int)(kk / kch), c = (int)(kk - (long long)tap * kch), r = tap / g.k, t = tap - r * g.k;
+#pragma unroll
+                for (int i = 0; i < AP; ++i) {
+                    const int h = a_h[i] + r, w = a_w[i] + t;
+                    const bool ok = a_ok[i] && kk < kend && h >= 0 && h < g.h && w >= 0 && w < g.w;
+                    sg_copy1(a_s + ((tid >> 2) + 32 * i) * SG_KPITCH + kv + e, ok ? asrc + (a_base[i] + (long long)h * g.w + w) * g.c_in + c : asrc, ok);
+                }
+#pragma unroll
+                for (int i = 0; i < BP; ++i) {
+                    const int col = j0 + (tid >> 2) + 32 * i;
+                    const bool ok = col < cols && kk < kend;
+                    sg_copy1(b_s + ((tid >> 2) + 32 * i) * SG_KPITCH + kv + e, ok ? bsrc + (long long)col * g.kdim + kk : bsrc, ok);
+                }
+            }
+            kload += SG_BK;
+            return;
+        }
+        if (KIND != 2) {
+            const bool kok = kload + kv < kend;
+#pragma unroll
+            for (int i = 0; i < AP; ++i) {
+                const int h = KIND == 0 ? a_h[i] + tap_r : a_h[i] - tap_r, w = KIND == 0 ? a_w[i] + tap_t : a_w[i] - tap_t;
+                const int hh = KIND == 0 ? g.h : g.ho, ww = KIND == 0 ? g.w : g.wo;
+                const bool ok = kok && a_ok[i] && h >= 0 && h < hh && w >= 0 && w < ww;
+                sg_copy4(a_s + ((tid >> 2) + 32 * i) * SG_KPITCH + kv, ok ? asrc + (a_base[i] + (long long)h * ww + w) * kch + ch : asrc, ok);
+            }
+            if (KIND == 0) {
+#pragma unroll
+                for (int i = 0; i < BP; ++i) {
+                    const int col = j0 + (tid >> 2) + 32 * i;
+                    const bool ok = kok && col < cols;
+                    sg_copy4(b_s + ((tid >> 2) + 32 * i) * SG_KPITCH + kv, ok ? bsrc + (long long)col * g.kdim + kload + kv : bsrc, ok);
+                }
+            } else {  // filter rows k = (tap, c_out), c_in contiguous
+#pragma unroll
+                for (int i = 0; i < BP; ++i) {
+                    const int kr = b_kr + i * B_KSTEP;
+                    const long long kk = kload + kr;
+                    const int tap = (int)kk / kch, co = (int)kk - tap * kch, ri = tap / ntd, ti = tap - ri * ntd;
+                    const TIN* src = bsrc + ((long long)co * g.k * g.k + (r_first + ri * r_step) * g.k + t_first + ti * r_step) * g.c_in + j0 + b_nv;
+                    if (V == 4) {
+                        const bool ok = kk < kend && j0 + b_nv < cols;
+                        sg_copy4(b_s + kr * (BN + 4) + b_nv, ok ? src : bsrc, ok);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const bool ok = kk < kend && j0 + b_nv + e < cols;
+                            sg_copy1(b_s + kr * (BN + 4) + b_nv + e, ok ? src + e : bsrc, ok);
+                        }
+                    }
+                }
+            }
+            ch += SG_BK;
+            while (ch >= kch) {
+                ch -= kch;
+                if (++tap_t == nt) {
+                    tap_t = 0;
+                    ++tap_r;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < AP; ++i) {
+                const int kr = a_kr + i * A_KSTEP;
+                const bool ok = kload + kr < kend && i0 + a_mv < rows;
+                sg_copy4(a_s + kr * (BM + 4) + a_mv, ok ? asrc + (kload + kr) * g.c_out + i0 + a_mv : asrc, ok);
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int i = 0; i < BP; ++i) {
+                const int kr = b_kr + i * B_KSTEP;
+                const bool kok = kload + kr < kend;
+                const int hb = px_p[i] * g.stride - g.pad, wb = px_q[i] * g.stride - g.pad;
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+                for (int e = 0; e < (V == 4 ? 1 : 4); ++e) {
+                    const int h = hb + b_r[e], w = wb + b_t[e];
+                    const bool ok = kok && j0 + b_nv + e < cols && h >= 0 && h < g.h && w >= 0 && w < g.w;
+                    const TIN* src = ok ? bsrc + (((long long)px_n[i] * g.h + h) * g.w + w) * g.c_in + b_c[e] : bsrc;
+                    if (V == 4) sg_copy4(b_s + kr * (BN + 4) + b_nv, src, ok);
+                    else sg_copy1(b_s + kr * (BN + 4) + b_nv + e, src, ok);
+                }
+                px_q[i] += SG_BK;
+                while (px_q[i] >= g.wo) {
+                    px_q[i] -= g.wo;
+                    if (++px_p[i] == g.ho) {
+                        px_p[i] = 0;
+                        ++px_n[i];
+                    }
+                }
+            }
         }
+        kload += SG_BK;
+    };
+
+    float acc[TM][4];
+#pragma unroll
+    for (int u = 0; u < TM; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+    const bool flush = p.kchunk > 1024;
+    if (flush) {
+#pragma unroll
+        for (int e = 0; e < TM * 4; ++e) flushed[e * SG_THREADS + tid] = 0.0;
+    }
+    pdl_wait();
+#pragma unroll
+    for (int s = 0; s < SG_STAGES - 1; ++s) {
+        if (s < nsteps) load_stage(s);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    int since = 0;
+    for (int it = 0; it < nsteps; ++it) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(SG_STAGES - 2) : "memory");
         __syncthreads();
-        if (++since == SIMT_FLUSH) {
+        if (it + SG_STAGES - 1 < nsteps) load_stage((it + SG_STAGES - 1) % SG_STAGES);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const TIN* const a_s = sA + (it % SG_STAGES) * T::A_ELEMS;
+        const TIN* const b_s = sB + (it % SG_STAGES) * T::B_ELEMS;
+        if (KIND != 2) {
+#pragma unroll
+            for (int kq = 0; kq < SG_BK; kq += 4) {
+                float4 a[TM], b[4];
+#pragma unroll
+                for (int u = 0; u < TM; ++u) a[u] = sg_ld4(a_s + (ty + u * NTY) * SG_KPITCH + kq);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) b[v] = KIND == 0 ? sg_ld4(b_s + (tx + v * NTX) * SG_KPITCH + kq) : sg_ld4(b_s + (kq + v) * (BN + 4) + tx * 4);
+#pragma unroll
+                for (int u = 0; u < TM; ++u) {
+                    const float au[4] = {a[u].x, a[u].y, a[u].z, a[u].w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            const float4 bb = KIND == 0 ? b[v] : b[e];  // KIND 0: column v at k e; KIND 1: k e at column v
+                            const int at = KIND == 0 ? e : v;
+                            acc[u][v] = fmaf(au[e], at == 0 ? bb.x : at == 1 ? bb.y : at == 2 ? bb.z : bb.w, acc[u][v]);
+                        }
+                }
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < SG_BK; ++k) {
+                float a[TM];
+#pragma unroll
+                for (int u = 0; u < TM; u += 4) {
+                    const float4 t = sg_ld4(a_s + k * (BM + 4) + ty * TM + u);
+                    a[u] = t.x; a[u + 1] = t.y; a[u + 2] = t.z; a[u + 3] = t.w;
+                }
+                const float4 b = sg_ld4(b_s + k * (BN + 4) + tx * 4);
+#pragma unroll
+                for (int u = 0; u < TM; ++u) {
+                    acc[u][0] = fmaf(a[u], b.x, acc[u][0]);
+                    acc[u][1] = fmaf(a[u], b.y, acc[u][1]);
+                    acc[u][2] = fmaf(a[u], b.z, acc[u][2]);
+                    acc[u][3] = fmaf(a[u], b.w, acc[u][3]);
+                }
+            }
+        }
+        if (flush && ++since == SG_FLUSH) {
             since = 0;
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < TM; ++u)
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
-                    dacc[u][v] += (double)acc[u][v];
+                    flushed[(u * 4 + v) * SG_THREADS + tid] += (double)acc[u][v];
                     acc[u][v] = 0.f;
                 }
         }
     }
-    TO* o = out + (size_t)blockIdx.z * (size_t)I * (size_t)J;
+
+    // ---- store, and the channel sums of what is stored
+    const long long out_rows = KIND == 0 ? g.m : KIND == 1 ? (long long)g.n * g.h * g.w : g.c_out;
+    TO* const o = out + (size_t)blockIdx.z * (size_t)out_rows * (size_t)cols;
+    float cs[4] = {0.f, 0.f, 0.f, 0.f}, cq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const long long i = i0 + ty * 4 + u;
-        if (i >= I) continue;
+    for (int u = 0; u < TM; ++u) {
+        const long long i = i0 + (KIND == 2 ? ty * TM + u : ty + u * NTY);
+        if (i >= rows) continue;
+        long long orow = i;
+        if (KIND == 1 && g.stride > 1) {
+            const int j = (int)(i % cl.wc);
+            const long long t1 = i / cl.wc;
+            orow = ((t1 / cl.hc) * g.h + (t1 % cl.hc) * g.stride + cl.pa) * g.w + (long long)j * g.stride + cl.pb;
+        }
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const int j = j0 + tx * 4 + v;
-            if (j < J) o[(size_t)i * J + j] = from_f32<TO>((float)(dacc[u][v] + (double)acc[u][v]));
+            const int j = j0 + (KIND == 0 ? tx + v * NTX : tx * 4 + v);
+            if (j >= cols) continue;
+            const float val = flush ? (float)(flushed[(u * 4 + v) * SG_THREADS + tid] + (double)acc[u][v]) : acc[u][v];
+            const TO st = from_f32<TO>(val);
+            o[(size_t)orow * cols + j] = st;
+            if (KIND == 0) {
+                const float f = to_f32(st);
+                cs[v] += f;
+                cq[v] = fmaf(f, f, cq[v]);
+            }
         }
+    }
+    if (KIND == 0 && p.stats) {
+        float* const red = reinterpret_cast<float*>(sg_smem);  // [NTY][2][BN]
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            red[(ty * 2) * BN + tx + v * NTX] = cs[v];
+            red[(ty * 2 + 1) * BN + tx + v * NTX] = cq[v];
+        }
+        __syncthreads();
+        for (int e = tid; e < 2 * BN; e += SG_THREADS) {
+            const int which = e / BN, c = e - which * BN;
+            if (j0 + c >= cols) continue;
+            float sum = 0.f;
+            for (int r = 0; r < NTY; ++r) sum += red[(r * 2 + which) * BN + c];
+            chan_acc_add(p.acc, g.c_out, which, j0 + c, sum);
+        }
+    }
+}
+
+// out = sum over the slices of a split forward convolution (fp64, slice order), rounded to YT, and with acc.acc != NULL the
+// channel sums of the stored values (a thread keeps one group of four channels, like the elementwise passes).
+template <typename YT>
+__global__ void __launch_bounds__(256) splitk_fwd_reduce_kernel(const float* __restrict__ partial, int splits, long long vecs, int C, YT* __restrict__ out, ChanAcc acc) {
+    pdl_launch_dependents();
+    pdl_wait();
+    extern __shared__ float red[];  // [blockDim.x][4]
+    const int tid = threadIdx.x, cgs = C / 4;
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, q[4] = {0.f, 0.f, 0.f, 0.f};
+    const float4* p4 = reinterpret_cast<const float4*>(partial);
+    for (long long v = (long long)blockIdx.x * blockDim.x + tid; v < vecs; v += (long long)gridDim.x * blockDim.x) {
+        double d[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+        for (int z = 0; z < splits; ++z) {
+            const float4 a = p4[(size_t)z * vecs + v];
+            d[0] += (double)a.x; d[1] += (double)a.y; d[2] += (double)a.z; d[3] += (double)a.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const YT y = from_f32<YT>((float)d[i]);
+            out[v * 4 + i] = y;
+            const float f = to_f32(y);
+            s[i] += f;
+            q[i] = fmaf(f, f, q[i]);
+        }
+    }
+    if (!acc.acc) return;
+    for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) red[tid * 4 + i] = pass ? q[i] : s[i];
+        __syncthreads();
+        for (int c = tid; c < C; c += blockDim.x) {
+            float sum = 0.f;
+            for (int r = c / 4; r < (int)blockDim.x; r += cgs) sum += red[r * 4 + (c & 3)];
+            chan_acc_add(acc, C, pass, c, sum);
+        }
+        __syncthreads();
     }
 }
 
 // out[e] = sum_z partial[z][e], summed in fp64 in slice order (four elements per thread when the count allows).
 // Eight slices are loaded before any is added so that a thread keeps eight independent 16-byte loads in flight:
 // the kernel is tiny and otherwise bound by one memory latency per slice.
-__global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restrict__ partial, int splits, size_t elems, float* __restrict__ out) {
+template <typename TO>
+__global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restrict__ partial, int splits, size_t elems, TO* __restrict__ out) {
     pdl_launch_dependents();
     pdl_wait();
     const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -183,13 +470,18 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
                         s3 += (double)a[u].w;
                     }
             }
-            reinterpret_cast<float4*>(out)[v] = make_float4((float)s0, (float)s1, (float)s2, (float)s3);
+            if constexpr (sizeof(TO) == 4) {
+                reinterpret_cast<float4*>(out)[v] = make_float4((float)s0, (float)s1, (float)s2, (float)s3);
+            } else {
+                TO o[4] = {from_f32<TO>((float)s0), from_f32<TO>((float)s1), from_f32<TO>((float)s2), from_f32<TO>((float)s3)};
+                reinterpret_cast<uint2*>(out)[v] = *reinterpret_cast<const uint2*>(o);
+            }
         }
     } else {
         for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < elems; e += stride) {
             double s = 0.0;
             for (int z = 0; z < splits; ++z) s += (double)partial[(size_t)z * elems + e];
-            out[e] = (float)s;
+            out[e] = from_f32<TO>((float)s);
         }
     }
 }

@@ -1483,7 +1483,7 @@ inline nb_status tc_wgrad(TcPlan* tc, const Geom& g, const void* x, const void* 
                 launch_k(splitk_reduce_tall_kernel, dim3((unsigned)((elems + 31) / 32)), dim3(1024), 0, st, 1, partial, R.splits, elems, dw);
             } else {
                 const int blocks = (int)std::min<size_t>((elems / 4 + 127) / 128 + 1, (size_t)tc->sm_count * 8);
-                launch_k(splitk_reduce_kernel, dim3(blocks), dim3(128), 0, st, 1, partial, R.splits, elems, dw);
+                launch_k(splitk_reduce_kernel<float>, dim3(blocks), dim3(128), 0, st, 1, partial, R.splits, elems, dw);
             }
             if (cudaGetLastError() != cudaSuccess) { err() = "launch of splitk_reduce_kernel failed"; return NB_ERR_CUDA; }
             tc->launches += 1;
@@ -1517,7 +1517,7 @@ inline nb_status tc_wgrad(TcPlan* tc, const Geom& g, const void* x, const void* 
     if (P.splits > 1) {
         const size_t elems = (size_t)g.c_out * g.kdim;
         const int blocks = (int)std::min<size_t>((elems / 4 + 127) / 128 + 1, (size_t)tc->sm_count * 8);
-        launch_k(splitk_reduce_kernel, dim3(blocks), dim3(128), 0, st, 1, partial, P.splits, elems, dw);
+        launch_k(splitk_reduce_kernel<float>, dim3(blocks), dim3(128), 0, st, 1, partial, P.splits, elems, dw);
         if (cudaGetLastError() != cudaSuccess) { err() = "launch of splitk_reduce_kernel failed"; return NB_ERR_CUDA; }
         tc->launches += 1;
     }
