@@ -612,6 +612,8 @@ nb_status nb_cbs_plan_set_pitches(nb_cbs_plan p, int64_t ld_x, int64_t ld_a, int
     // tensor maps cached for the previous layout are stale
     p->tc.fp.a_ptr = nullptr;
     p->tc.inf.a_ptr = nullptr;
+    p->tc.fps.a_ptr = nullptr;
+    p->tc.infs.a_ptr = nullptr;
     p->tc.wg_a_ptr = nullptr;
     return NB_OK;
 }

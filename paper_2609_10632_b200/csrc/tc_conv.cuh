@@ -70,6 +70,8 @@ struct IgemmParams {
     int ldo;                     // channels per output pixel
     int Hout, Wout, os;          // GEMM row (n,i,j) -> output pixel (n, i*os+oa, j*os+ob) of an Hout x Wout image
     void* out;
+    int split;         // CTAs (a cluster) that share the K range of a tile in tc_split_kernel
+    long long ld_out;  // its output row pitch in elements
     float* partials;  // [gridDim.x][2][ldo] per-CTA channel sums and sums of squares (statistics variant only)
     int* status;
     uint16_t off_w[4][9], off_h[4][9];
@@ -774,6 +776,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
 
 }  // namespace nbcbs
 #include "tc_wgrad.cuh"
+#include "tc_split.cuh"
 namespace nbcbs {
 
 // ------------------------------------------------------------------------------------------ host side
@@ -786,6 +789,7 @@ struct IgemmCfg {
     uint32_t a_stage = 0, b_stage = 0, a_sub = 0, b_sub = 0;
     size_t smem_bytes = 0;
     long long M = 0;
+    int split = 0;  // > 0: tc_split_kernel with this many CTAs per tile
 };
 
 struct TcGemmSlot {  // one launch: configuration plus the tensor maps encoded for the pointers last seen
@@ -810,6 +814,7 @@ struct TcPlan {
     bool infer = false;  // the forward configuration also runs with the fused per-channel epilogue (its own slot: own output maps)
     TcGemmSlot inf;
     TcGemmSlot dg;  // one launch covers all output-parity classes
+    TcGemmSlot fps, infs, dgs;  // the same three as split launches (cfg.ok only where the layer has few tiles)
     WtParams wtp;
     // wgrad
     WgradParams wg;
@@ -984,6 +989,76 @@ inline void fill_params(IgemmParams& P, const IgemmCfg& c) {
     P.idesc = ptx::make_idesc_bf16(c.cg2 ? 2 * TC_BM : TC_BM, c.BN, 0, 0);
 }
 
+// The split form of a launch (tc_split_kernel), where it is the faster one; cfg.ok stays false elsewhere.  `min_taps`: taps of
+// the lightest parity class.  Times in us, fitted to measurements on B200 over the detector's layers at batch 1 (640 x 640)
+// and 2 (320 x 320): a CTA fetches a k-block at about 55 bytes per cycle and the tensor pipe needs max(45, BN / 2) cycles per
+// K = 16 step, whichever is longer; then the hand-over and the stores, which the persistent kernel does with TMA and, in the
+// training calls, behind a predecessor that still drains (`eval`: the evaluation-mode call, whose persistent form derives
+// every channel's coefficients in every CTA instead).
+// Measured, evaluation-mode forward of the 77 layers, one image: 1190 -> 590 us; single layers: 288 -> 288 3x3 at 20 x 20
+// 20.6 -> 7.5 us (8 tiles of 45 k-blocks -> 28 of 9), 192 -> 192 3x3 at 40 x 40 15.1 -> 7.8, 384 -> 384 1x1 at 40 x 40
+// 9.5 -> 5.5; data gradient of 288 -> 288 at 20 x 20 (the whole call) 28.6 -> 16.2.
+inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_taps, bool eval, int sm_count) {
+    out = full;
+    out.cfg = IgemmCfg();
+    out.a_ptr = out.b_ptr = out.out_ptr = nullptr;
+    const IgemmCfg& f = full.cfg;
+    const int kc_per_tap = (f.Ca + f.KC - 1) / f.KC, kblocks = f.ntaps * kc_per_tap, min_kb = min_taps * kc_per_tap, ncls = full.prm.nclasses;
+    if (getenv("NB_TC_SPLIT") && atoi(getenv("NB_TC_SPLIT")) == 0) return;
+    const long long m_tiles = (f.M + TC_BM - 1) / TC_BM;
+    if (m_tiles * ncls > sm_count) return;
+    auto kb_time = [](int bn) { return std::max(4.0 * std::max(45.0, bn / 2.0), (TC_BM + bn) * 128 / 55.0) / 1900.0; };
+    const double workers = f.cg2 ? sm_count / 2 : sm_count;
+    const double full_waves = (double)(((long long)f.m_tiles * f.n_tiles * ncls + (long long)workers - 1) / (long long)workers);
+    double best = 4.5 + full_waves * (kblocks * f.mh * kb_time(f.BN) + 0.8);
+    const int force_s = getenv("NB_TC_SPLIT_S") ? atoi(getenv("NB_TC_SPLIT_S")) : 0, force_bn = getenv("NB_TC_SPLIT_BN") ? atoi(getenv("NB_TC_SPLIT_BN")) : 0;
+    if (force_s || force_bn) best = 1e30;
+    int best_bn = 0, best_s = 0;
+    for (int nt = (f.rowsB + 127) / 128; nt <= (f.rowsB + 15) / 16; ++nt) {
+        const int bn = ((f.rowsB + nt - 1) / nt + 15) / 16 * 16;
+        if ((f.rowsB + bn - 1) / bn != nt || (force_bn && bn != force_bn)) continue;
+        for (int s = 1; s <= 8 && s <= min_kb; s *= 2) {
+            const long long ctas = m_tiles * nt * ncls * s;
+            if (ctas > (s == 8 ? sm_count * 6 / 7 : s == 4 ? sm_count * 9 / 10 : sm_count) || (force_s && s != force_s)) continue;
+            const double t = 3.5 + ((kblocks + s - 1) / s) * kb_time(bn) + 0.012 * bn + (s > 1 ? 1.2 : 0.0) + (eval ? 0.0 : 0.5 + 0.023 * bn / s);
+            if (t < best) {
+                best = t;
+                best_bn = bn;
+                best_s = s;
+            }
+        }
+    }
+    if (!best_bn) return;
+    IgemmCfg c = f;
+    c.BN = best_bn;
+    c.n_tiles = (f.rowsB + best_bn - 1) / best_bn;
+    c.m_tiles = (int)m_tiles;
+    c.mh = 1; c.cg2 = false; c.kpb = 1; c.acc_bufs = 1;
+    c.split = best_s;
+    c.a_sub = c.a_stage = TC_BM * 128;
+    c.b_sub = c.b_stage = (uint32_t)((best_bn * 128 + 1023) / 1024 * 1024);
+    c.tmem_cols = 32;
+    while (c.tmem_cols < best_bn) c.tmem_cols *= 2;
+    c.acc_stride = c.tmem_cols;
+    c.stages = std::max(2, std::min(8, (kblocks + best_s - 1) / best_s));
+    const size_t part = (size_t)TC_BM * (best_bn + 4) * 4, fixed = 1024 + 64 + (size_t)2 * SP_THREADS * 16 + 512;
+    while (c.stages > 2 && fixed + (size_t)c.stages * (c.a_stage + c.b_stage) > kMaxSmem) --c.stages;
+    c.smem_bytes = std::max<size_t>(fixed + std::max(part, (size_t)c.stages * (c.a_stage + c.b_stage)), 120 * 1024);  // > half an SM: one CTA per SM
+    c.grid = (int)(m_tiles * c.n_tiles * ncls * best_s);
+    IgemmParams& P = out.prm;
+    P.BN = c.BN; P.n_tiles = c.n_tiles; P.m_tiles = c.m_tiles; P.tiles_per_class = c.m_tiles * c.n_tiles;
+    P.stages = c.stages; P.acc_stride = c.acc_stride; P.tmem_cols = c.tmem_cols;
+    P.a_stage_bytes = P.a_sub_bytes = c.a_stage; P.b_stage_bytes = P.b_sub_bytes = c.b_stage;
+    P.kpb = 1; P.mh = 1; P.acc_bufs = 1; P.tma_store = 0;
+    P.split = c.split;
+    P.idesc = ptx::make_idesc_bf16(TC_BM, c.BN, 0, 0);
+    c.ok = true;
+    out.cfg = c;
+    if (getenv("NB_TC_VERBOSE"))
+        fprintf(stderr, "[nb_cbs] split igemm M=%lld Ca=%d rowsB=%d taps=%d classes=%d: BN=%d S=%d stages=%d tiles=%dx%d grid=%d est %.1f us\n", c.M, c.Ca, c.rowsB, c.ntaps, ncls,
+                c.BN, c.split, c.stages, c.m_tiles, c.n_tiles, c.grid, best);
+}
+
 // im2col map over a bf16 NHWC tensor [N][H][W][C]: traversal starts at (lo, lo), steps `ts`, and ends `up` short of the far edge.
 // ld = pixel pitch in elements (0: dense, = C); channels past C read as zeros whatever lies behind them in memory.
 inline bool encode_im2col(CUtensorMap* m, const void* base, int N, int H, int W, int C, int lo, int up, int ts, int KC, int pixels = TC_BM, long long ld = 0) {
@@ -1054,6 +1129,19 @@ inline bool encode_out_maps(IgemmParams& P, const IgemmCfg& c, void* out, long l
     return true;
 }
 
+// Input and filter maps of a forward launch (the evaluation-mode one included), when the pointers are not those last seen.
+inline bool encode_forward_inputs(TcGemmSlot& S, const Geom& g, const void* x, const void* w, long long ld_x) {
+    if (S.a_ptr == x && S.b_ptr == w) return true;
+    const int up = g.pad - (g.k - 1), rows = TC_BM * S.cfg.mh, cols = S.cfg.cg2 ? S.cfg.BN / 2 : S.cfg.BN;
+    auto input = [&](CUtensorMap* m, int KC) {
+        return S.prm.a_tiled ? encode_tiled_2d(m, x, g.m, g.c_in, KC, rows, ld_x) : encode_im2col(m, x, g.n, g.h, g.w, g.c_in, -g.pad, up, g.stride, KC, rows, ld_x);
+    };
+    if (!input(&S.prm.tmA, S.cfg.KC) || !encode_tiled_2d(&S.prm.tmB[0], w, g.c_out, (long long)g.kdim, S.cfg.KC, cols)) return false;
+    if (S.cfg.tail32 && (!input(&S.prm.tmA_t, 32) || !encode_tiled_2d(&S.prm.tmB_t[0], w, g.c_out, (long long)g.kdim, 32, cols))) return false;
+    S.a_ptr = x; S.b_ptr = w;
+    return true;
+}
+
 // Raises the dynamic shared-memory limit of one kernel instantiation once per device.
 template <typename OutT, bool STATS, bool CG2, int EPI, bool CLS4> inline bool igemm_allow_smem() {
     // the attribute belongs to the (function, device) pair: one bit per device ordinal that already has it
@@ -1087,6 +1175,25 @@ template <typename OutT, bool STATS> inline nb_status launch_igemm(const TcGemmS
     }
     return s.cfg.cg2 ? launch_igemm_impl<OutT, STATS, true>(s, st) : launch_igemm_impl<OutT, STATS, false>(s, st);
 }
+template <typename OutT, int MODE> inline nb_status launch_split(const TcGemmSlot& s, cudaStream_t st) {
+    static std::atomic<unsigned long long> attr_set{0};  // one bit per device ordinal
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(attr_set.load(std::memory_order_acquire) & bit)) {
+        if (cudaFuncSetAttribute(tc_split_kernel<OutT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess) {
+            err() = "cannot raise the dynamic shared memory limit of the split implicit-GEMM kernel";
+            return NB_ERR_CUDA;
+        }
+        attr_set.fetch_or(bit, std::memory_order_release);
+    }
+    const cudaError_t e = launch_k(tc_split_kernel<OutT, MODE>, dim3((unsigned)s.cfg.grid), dim3(SP_THREADS), s.cfg.smem_bytes, st, s.cfg.split, s.prm);
+    if (e != cudaSuccess) {
+        err() = std::string("launch of tc_split_kernel failed: ") + cudaGetErrorString(e);
+        return NB_ERR_CUDA;
+    }
+    return NB_OK;
+}
 }  // namespace tcdetail
 
 inline const char* tc_last_error() { return tcdetail::err().c_str(); }
@@ -1099,6 +1206,9 @@ inline nb_status tc_plan_init(TcPlan* tc, const Geom& g, bool enable, int sm_cou
     if (st == NB_OK && f16) {  // A and B formats of the instruction descriptors: bits 7 and 10 set = bf16, clear = f16
         const uint32_t fmt = (1u << 7) | (1u << 10);
         tc->fp.prm.idesc &= ~fmt;
+        tc->fps.prm.idesc &= ~fmt;
+        tc->infs.prm.idesc &= ~fmt;
+        tc->dgs.prm.idesc &= ~fmt;
         tc->inf.prm.idesc &= ~fmt;
         tc->dg.prm.idesc &= ~fmt;
         tc->wg.idesc &= ~fmt;
@@ -1134,6 +1244,8 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
             tc->fprop = true;
             tc->fprop_parts = c.grid;
             tc->inf = tc->fp;
+            split_configure(tc->fps, tc->fp, g.k * g.k, false, sm_count);
+            split_configure(tc->infs, tc->inf, g.k * g.k, true, sm_count);
             tc->infer = true;
         }
     }
@@ -1197,6 +1309,7 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
             W.nclasses = ncls;
             tc->wt_bytes = off * 2;
             tc->dgrad = true;
+            split_configure(tc->dgs, tc->dg, ncls == 4 ? 1 : g.k * g.k, false, sm_count);
         }
     }
     // ---- wgrad: A = x (im2col, MN-major), B = dy (MN-major), reduction over pixels with split-K
@@ -1332,24 +1445,14 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
 inline nb_status tc_fprop(TcPlan* tc, const Geom& g, const void* x, const void* w, void* y, float* partials, int* status, cudaStream_t st,
                           const ChanAcc& acc) {
     using namespace tcdetail;
-    TcGemmSlot& S = tc->fp;
-    if (S.a_ptr != x || S.b_ptr != w) {
-        const int up = g.pad - (g.k - 1);
-        if (S.prm.a_tiled) {
-            if (!encode_tiled_2d(&S.prm.tmA, x, g.m, g.c_in, S.cfg.KC, TC_BM * S.cfg.mh, tc->ld_x)) return NB_ERR_CUDA;
-        } else if (!encode_im2col(&S.prm.tmA, x, g.n, g.h, g.w, g.c_in, -g.pad, up, g.stride, S.cfg.KC, TC_BM * S.cfg.mh, tc->ld_x)) {
-            return NB_ERR_CUDA;
-        }
-        if (!encode_tiled_2d(&S.prm.tmB[0], w, g.c_out, (long long)g.kdim, S.cfg.KC, S.cfg.cg2 ? S.cfg.BN / 2 : S.cfg.BN)) return NB_ERR_CUDA;
-        if (S.cfg.tail32) {
-            if (S.prm.a_tiled) {
-                if (!encode_tiled_2d(&S.prm.tmA_t, x, g.m, g.c_in, 32, TC_BM * S.cfg.mh, tc->ld_x)) return NB_ERR_CUDA;
-            } else if (!encode_im2col(&S.prm.tmA_t, x, g.n, g.h, g.w, g.c_in, -g.pad, g.pad - (g.k - 1), g.stride, 32, TC_BM * S.cfg.mh, tc->ld_x)) {
-                return NB_ERR_CUDA;
-            }
-            if (!encode_tiled_2d(&S.prm.tmB_t[0], w, g.c_out, (long long)g.kdim, 32, S.cfg.cg2 ? S.cfg.BN / 2 : S.cfg.BN)) return NB_ERR_CUDA;
-        }
-        S.a_ptr = x; S.b_ptr = w;
+    const bool split = tc->fps.cfg.ok && acc.acc;  // (the split kernel has no per-CTA partial sums)
+    TcGemmSlot& S = split ? tc->fps : tc->fp;
+    if (!encode_forward_inputs(S, g, x, w, tc->ld_x)) return NB_ERR_CUDA;
+    if (split) {
+        S.prm.acc = acc;
+        S.prm.out = y; S.prm.ld_out = g.c_out; S.prm.status = status;
+        tc->launches += 1;
+        return launch_split<__half, 1>(S, st);
     }
     S.prm.tma_store = 1;
     if (S.out_ptr != y) {
@@ -1371,23 +1474,16 @@ struct EpiAffine {
 };
 inline nb_status tc_infer(TcPlan* tc, const Geom& g, const void* x, const void* w, void* out, const EpiAffine& e, int* status, cudaStream_t st) {
     using namespace tcdetail;
-    TcGemmSlot& S = tc->inf;
-    if (S.a_ptr != x || S.b_ptr != w) {
-        if (S.prm.a_tiled) {
-            if (!encode_tiled_2d(&S.prm.tmA, x, g.m, g.c_in, S.cfg.KC, TC_BM * S.cfg.mh)) return NB_ERR_CUDA;
-        } else if (!encode_im2col(&S.prm.tmA, x, g.n, g.h, g.w, g.c_in, -g.pad, g.pad - (g.k - 1), g.stride, S.cfg.KC, TC_BM * S.cfg.mh)) {
-            return NB_ERR_CUDA;
-        }
-        if (!encode_tiled_2d(&S.prm.tmB[0], w, g.c_out, (long long)g.kdim, S.cfg.KC, S.cfg.cg2 ? S.cfg.BN / 2 : S.cfg.BN)) return NB_ERR_CUDA;
-        if (S.cfg.tail32) {
-            if (S.prm.a_tiled) {
-                if (!encode_tiled_2d(&S.prm.tmA_t, x, g.m, g.c_in, 32, TC_BM * S.cfg.mh, 0)) return NB_ERR_CUDA;
-            } else if (!encode_im2col(&S.prm.tmA_t, x, g.n, g.h, g.w, g.c_in, -g.pad, g.pad - (g.k - 1), g.stride, 32, TC_BM * S.cfg.mh, 0)) {
-                return NB_ERR_CUDA;
-            }
-            if (!encode_tiled_2d(&S.prm.tmB_t[0], w, g.c_out, (long long)g.kdim, 32, S.cfg.cg2 ? S.cfg.BN / 2 : S.cfg.BN)) return NB_ERR_CUDA;
-        }
-        S.a_ptr = x; S.b_ptr = w;
+    TcGemmSlot& S = tc->infs.cfg.ok ? tc->infs : tc->inf;
+    if (!encode_forward_inputs(S, g, x, w, 0)) return NB_ERR_CUDA;
+    S.prm.fin_gamma = e.gamma; S.prm.fin_beta = e.beta;
+    S.prm.fin_rmean = e.rmean; S.prm.fin_rvar = e.rvar;
+    S.prm.fin_eps = e.eps; S.prm.epi_act = e.act;
+    S.prm.out = out; S.prm.partials = nullptr; S.prm.status = status;
+    tc->launches += 1;
+    if (S.cfg.split) {
+        S.prm.ld_out = g.c_out;
+        return tc->f16 ? launch_split<__half, 2>(S, st) : launch_split<__nv_bfloat16, 2>(S, st);
     }
     S.prm.tma_store = 1;  // the fused epilogue exists only on the TMA-store path
     if (S.out_ptr != out) {
@@ -1395,11 +1491,6 @@ inline nb_status tc_infer(TcPlan* tc, const Geom& g, const void* x, const void* 
         S.out_ptr = out;
     }
     S.prm.acc = ChanAcc{nullptr, nullptr, 1};
-    S.prm.fin_gamma = e.gamma; S.prm.fin_beta = e.beta;
-    S.prm.fin_rmean = e.rmean; S.prm.fin_rvar = e.rvar;
-    S.prm.fin_eps = e.eps; S.prm.epi_act = e.act;
-    S.prm.out = out; S.prm.partials = nullptr; S.prm.status = status;
-    tc->launches += 1;
     if (tc->f16) return S.cfg.cg2 ? launch_igemm_impl<__half, false, true, 1>(S, st) : launch_igemm_impl<__half, false, false, 1>(S, st);
     return S.cfg.cg2 ? launch_igemm_impl<__nv_bfloat16, false, true, 1>(S, st) : launch_igemm_impl<__nv_bfloat16, false, false, 1>(S, st);
 }
@@ -1418,7 +1509,7 @@ inline nb_status tc_dgrad(TcPlan* tc, const Geom& g, const void* dy, const void*
         if (cudaGetLastError() != cudaSuccess) { err() = "launch of dgrad_weight_transform_kernel failed"; return NB_ERR_CUDA; }
         tc->launches += 1;
     }
-    TcGemmSlot& S = tc->dg;
+    TcGemmSlot& S = tc->dgs.cfg.ok ? tc->dgs : tc->dg;
     if (S.a_ptr != dy || S.b_ptr != wt) {
         // stride 1: window start runs over [-(k-1-P), W-1-(k-1-P)], i.e. W positions; stride-2 classes: over [0, Wo-1]
         const int lo = g.stride == 1 ? -(g.k - 1 - g.pad) : 0;
@@ -1431,6 +1522,16 @@ inline nb_status tc_dgrad(TcPlan* tc, const Geom& g, const void* dy, const void*
                 return NB_ERR_CUDA;
         }
         S.a_ptr = dy; S.b_ptr = wt;
+    }
+    if (S.cfg.split) {
+        if (g.stride != 1 && (ld_dx || accumulate)) {
+            err() = "a pitched or accumulating data gradient needs a stride-1 layer";
+            return NB_ERR_UNSUPPORTED;
+        }
+        S.prm.out_accumulate = accumulate ? 1 : 0;
+        S.prm.out = dx; S.prm.ld_out = ld_dx ? ld_dx : g.c_in; S.prm.status = status;
+        tc->launches += 1;
+        return tc->f16 ? launch_split<__half, 0>(S, st) : launch_split<__nv_bfloat16, 0>(S, st);
     }
     S.prm.tma_store = g.stride == 1 ? 1 : 0;  // the parity classes of a stride-2 layer write every other output pixel
     if (!S.prm.tma_store && (ld_dx || accumulate)) {

@@ -1,0 +1,55 @@
+"""The split-K cluster form of the implicit GEMM (layers with few output tiles) with every cluster size forced: k-blocks that
+do not divide evenly, a 32-channel tail k-block, ragged rows, padded columns, the parity classes of a stride-2 data gradient
+with odd extents, and a data gradient added into a channel slice."""
+import pytest
+
+from paper_2609_10632_b200 import workloads as wl
+from tests import parity
+from tests.test_gpu_parity import EPS, _compare, _oracle, _run_block
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    (1, 20, 20, 192, 192, 3, 1),  # 27 k-blocks, four row tiles
+    (2, 13, 11, 96, 80, 3, 1),    # 18 k-blocks of 64 and 32 channels, 286 rows
+    (3, 11, 9, 72, 136, 3, 1),    # padded columns, tail of 8 channels
+    (1, 17, 19, 128, 64, 3, 2),   # parity classes of 1, 2, 2 and 4 taps, odd height and width
+    (2, 12, 14, 512, 48, 1, 1),   # tiled A map
+]
+
+
+@pytest.mark.parametrize("split", [1, 2, 4, 8])
+@pytest.mark.parametrize("dims", SHAPES, ids=lambda d: "x".join(map(str, d)))
+def test_split_launches_match_oracle(dims, split, monkeypatch):
+    import oracle
+    import torch
+
+    from paper_2609_10632_b200 import binding as nb
+    from paper_2609_10632_b200.block import CbsBlock
+
+    monkeypatch.setenv("NB_TC_SPLIT_S", str(split))
+    shape = wl.ConvShape("split", *dims)
+    mode = nb.NB_MODE_F16_TC if split == 2 else nb.NB_MODE_BF16_TC
+    inp, blk, out = _run_block(shape, mode, cfg_id=43, layer_id=SHAPES.index(dims), affine="random")
+    _compare(out, _oracle(inp), 0)
+    again = CbsBlock(shape, mode=mode, eps=EPS)
+    again.upload(inp)
+    again.step()
+    assert torch.equal(again.y, blk.y) and torch.equal(again.dx, blk.dx)  # rank order: the same bits every run
+    rm, rv, _ = wl.make_eval_stats(shape, 43, SHAPES.index(dims))
+    up = lambda a: torch.from_numpy(a).to(blk.dev)
+    o = torch.empty_like(blk.a)
+    ws = torch.empty(max(blk.plan.infer_bytes, 256), dtype=torch.uint8, device=blk.dev)
+    nb.nb_conv_bn_silu_infer(blk.plan, blk.x, blk.w, blk.gamma, blk.beta, up(rm), up(rv), o, ws)
+    torch.cuda.synchronize()
+    assert blk.poll() == ""
+    parity.check("a_eval", o.double().cpu().numpy(), oracle.cbs_infer(inp.x, inp.w, inp.gamma, inp.beta, rm, rv, shape.stride, EPS), "bf16")
+    if shape.stride == 1:  # round(old + dx) in a channel slice, nothing beside it
+        wide = torch.randn(shape.n, shape.h, shape.w, shape.c_in + 24, device=blk.dev).to(blk.dx.dtype)
+        want = wide.clone()
+        want[..., 8:8 + shape.c_in] = (wide[..., 8:8 + shape.c_in].float() + blk.dx.float()).to(wide.dtype)
+        blk.plan.set_dx_target(ld_dx=shape.c_in + 24, accumulate=True)
+        blk.dx = wide[..., 8:8 + shape.c_in]
+        blk.backward_data()
+        torch.cuda.synchronize()
+        assert torch.equal(wide, want)
