@@ -178,6 +178,8 @@ class Plan:
         self.desc = nb_cbs_desc(ctypes.sizeof(nb_cbs_desc), n, h, w, c_in, c_out, ksize, stride, eps, momentum, mode, flags)
         self.handle = c_void_p()
         self.device = device
+        self.revision = 0       # counts the setter calls: what was recorded from calls of this plan is stale after one
+        self.profiling = False  # nb_cbs_profile_enable
         _check(load().nb_cbs_plan_create(byref(self.desc), device, byref(self.handle)))
         ho, wo = c_int32(), c_int32()
         _check(load().nb_cbs_out_shape(self.handle, byref(ho), byref(wo)))
@@ -194,18 +196,22 @@ class Plan:
 
     def set_pitches(self, ld_x=0, ld_a=0, ld_g=0):
         """x, a_out, g of the training calls are channel slices with these row pitches in elements (0 = dense)."""
+        self.revision += 1
         _check(load().nb_cbs_plan_set_pitches(self.handle, int(ld_x), int(ld_a), int(ld_g)))
 
     def set_fwd_residual(self, res=None, ld_res=0):
         """The forward call adds `res` (a tensor of the output's shape; row pitch ld_res elements, 0 = dense) to its output."""
+        self.revision += 1
         _check(load().nb_cbs_plan_set_fwd_residual(self.handle, _ptr(res), int(ld_res)))
 
     def set_bwd_residual(self, gres=None, ld_gres=0, accumulate=True):
         """The data-gradient call also adds (accumulate) or copies its incoming gradient g into `gres` (row pitch ld_gres, 0 = dense)."""
+        self.revision += 1
         _check(load().nb_cbs_plan_set_bwd_residual(self.handle, _ptr(gres), int(ld_gres), 1 if accumulate else 0))
 
     def set_dx_target(self, ld_dx=0, accumulate=False):
         """dx of the data-gradient call is a channel slice with this row pitch (0 = dense) and is added to, not overwritten."""
+        self.revision += 1
         _check(load().nb_cbs_plan_set_dx_target(self.handle, int(ld_dx), 1 if accumulate else 0))
 
     @classmethod
@@ -233,11 +239,15 @@ class Plan:
             pass
 
 
+replayed_launches = 0  # kernels of this library that went out as nodes of a CUDA graph this package recorded (GraphRunner)
+
+
 def nb_cbs_launch_count() -> int:
-    return int(load().nb_cbs_launch_count())
+    return int(load().nb_cbs_launch_count()) + replayed_launches
 
 
 def nb_cbs_profile_enable(plan: Plan, enable: bool):
+    plan.profiling = bool(enable)
     _check(load().nb_cbs_profile_enable(plan.handle, 1 if enable else 0))
 
 

@@ -4,6 +4,12 @@ Sec. 6, from the image to the raw head outputs) on the GPU, forward and backward
 Only wiring happens here: every arithmetic step is a C-ABI call (block calls of nb_cbs.h, glue calls of nb_glue.h);
 torch allocates the buffers, zeroes gradient accumulators where needed and owns the streams.
 
+A pass is some 200 to 400 kernel launches whose arguments do not change from step to step, and issuing them one by one (2.4 us
+each, plus 2 us for every call's way through Python) takes longer than a small batch takes on the GPU.  From the second pass
+with unchanged arguments on, forward() and backward() therefore replay a CUDA graph recorded from the same calls.  Measured,
+one training iteration at batch 2, 320 x 320: 2.94 ms issued one by one, of which the host alone needs 2.81 ms, and 2.57 ms
+as graphs; at batch 16, 640 x 640: 9.94 and 9.66 ms.
+
 Every named tensor is an NHWC bf16 tensor, dense or -- with views=True -- a CHANNEL SLICE of a wider buffer (a torch
 view: data_ptr() is the slice's first channel, stride(-2) its row pitch), which the block calls accept through
 nb_cbs_plan_set_pitches and the glue calls through their pitch arguments:
@@ -19,12 +25,29 @@ from the order of the backward pass; zeroed beforehand only if the overwriting c
 """
 from __future__ import annotations
 
+from operator import attrgetter
+
 import torch
 
 from . import binding as nb
 from .block import CbsBlock
 
 _PITCH_IN = ("slice", "add", "concat", "upsample", "maxpool")  # glue ops that read pitched operands (blocks do when their plan says so)
+
+
+_FORWARD_TENSORS = attrgetter("x", "w", "gamma", "beta", "running_mean", "running_var", "y", "mean", "invstd", "a", "ws")
+_BACKWARD_TENSORS = attrgetter("g", "y", "mean", "invstd", "gamma", "beta", "w", "dx", "dgamma", "dbeta", "dy", "ws", "x", "dw")
+
+
+def _address(t):
+    return 0 if t is None else t.data_ptr()
+
+
+class _Recording:
+    """One pass of a runner: the arguments it was last issued with and, from the second time on, a CUDA graph of its calls."""
+
+    def __init__(self, key):
+        self.key, self.graph, self.launches = key, None, 0
 
 
 class GraphRunner:
@@ -44,6 +67,8 @@ class GraphRunner:
         self.dev = torch.device("cuda", device)
         self.plain, self.idx = [], {}
         self.glue_fwd = self.glue_bwd = 0
+        self._recordings = {}        # pass -> _Recording
+        self._record_streams = None  # the streams that graphs are recorded on
         new = lambda shp, dtype=torch.bfloat16: torch.empty(shp, dtype=dtype, device=self.dev)
         prod = {o["out"]: (i, o) for i, o in enumerate(ops)}
         cons = {}
@@ -297,8 +322,68 @@ class GraphRunner:
     def _sadd(self, out, a, rows, channels, b=None, accumulate=False, stream=None):
         nb.nb_slice_add(nb.NB_DTYPE_BF16, rows, channels, out, out.stride(-2), a, a.stride(-2), b, b.stride(-2) if b is not None else 0, accumulate, stream)
 
+    # ------------------------------------------------------------------ recorded passes
+    def _arguments(self, tensors_of, extra):
+        """Everything the calls of a pass are issued with: addresses of the blocks', glue calls' and plain convolutions' tensors
+        and the revision of every plan.  None while a plan is being profiled (its calls wait for their kernels)."""
+        if any(b.plan.profiling for b in self.blocks) or any(pl["plan"].profiling for pl in self.plain):
+            return None
+        key = [t if isinstance(t, int) else _address(t) for b in self.blocks for t in tensors_of(b)]
+        key += [b.plan.revision for b in self.blocks]
+        for pl in self.plain:
+            key.append(pl["plan"].revision)
+            key += [_address(t) for t in pl.values() if isinstance(t, torch.Tensor)]
+        for tensors in (self.buf, self.grad, self.idx):
+            key += [_address(t) for t in tensors.values()]
+        return key + extra
+
+    def _run(self, name, tensors_of, issue, stream, side=None, side_workspace=None):
+        """issue(stream, side) -- or, once it has been issued with the same arguments before, a replay of its recording."""
+        if stream is not None and not isinstance(stream, torch.cuda.Stream):
+            return issue(stream, side)  # a bare stream address
+        with torch.cuda.stream(stream):
+            if torch.cuda.is_current_stream_capturing():
+                return issue(stream, side)  # the caller records a graph of its own
+        name = (name, side is not None)
+        key = self._arguments(tensors_of, [] if side_workspace is None else [_address(side_workspace), side_workspace.nbytes])
+        rec = self._recordings.get(name)
+        if key is None or rec is None or rec.key != key:
+            self._recordings[name] = _Recording(key)
+            return issue(stream, side)
+        if rec.graph is None:
+            self._record(rec, issue, side is not None)
+        main = torch.cuda.current_stream(self.dev) if stream is None else stream
+        if side is not None:  # the recording's weight gradients run behind what the caller queued on `side`, and before what follows there
+            main.wait_stream(side)
+        with torch.cuda.stream(main):
+            rec.graph.replay()
+        if side is not None:
+            side.wait_stream(main)
+        nb.replayed_launches += rec.launches
+
+    def _record(self, rec, issue, with_side):
+        if self._record_streams is None:
+            self._record_streams = torch.cuda.Stream(self.dev), torch.cuda.Stream(self.dev)
+        main, side = self._record_streams
+        graph = torch.cuda.CUDAGraph()
+        before = nb.nb_cbs_launch_count()
+        with torch.cuda.stream(main):
+            graph.capture_begin(capture_error_mode="thread_local")  # (other threads may go on using the GPU)
+            try:
+                issue(main, side if with_side else None)
+                if with_side:
+                    main.wait_stream(side)
+            finally:
+                graph.capture_end()
+        rec.launches = nb.nb_cbs_launch_count() - before
+        nb.replayed_launches -= rec.launches  # recorded, not launched
+        rec.graph = graph
+
     # ------------------------------------------------------------------ passes
     def forward(self, stream=None):
+        self._run("forward", _FORWARD_TENSORS, lambda st, _: self._forward(st), stream)
+
+    def _forward(self, stream):
         B, n_glue = self.buf, 0
         for o in self.ops:
             kind, out, ins = o["op"], o["out"], o["ins"]
@@ -339,6 +424,9 @@ class GraphRunner:
         block's dw, dgamma, dbeta in the block.  With wgrad_stream (and a workspace for it) every weight gradient is queued
         on that stream behind an event that follows the block's data-gradient call (it only reads the block's input
         activations and dy, which nothing overwrites during the backward pass); the caller joins the streams."""
+        self._run("backward", _BACKWARD_TENSORS, lambda st, side: self._backward(st, side, wgrad_workspace), stream, wgrad_stream, wgrad_workspace)
+
+    def _backward(self, stream, wgrad_stream, wgrad_workspace):
         G, n_glue = self.grad, 0
         for name in self.zeroed:
             G[name].zero_()

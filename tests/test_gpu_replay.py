@@ -1,0 +1,78 @@
+"""GraphRunner replays a recording of its passes from the second call with unchanged arguments on: the same bits as issuing
+the calls, with new values in the same tensors, after a tensor or a plan option was replaced, on streams of the caller, and
+inside a graph that the caller records."""
+import pytest
+
+from paper_2609_10632_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("side", [False, True], ids=["one stream", "weight gradients on a second stream"])
+def test_replayed_passes_give_the_issued_bits(side):
+    import torch
+
+    from paper_2609_10632_b200 import binding as nb
+    from paper_2609_10632_b200.detector import GraphRunner
+
+    ops, layers, outs, plain = wl.detector_graph(1, 64, plain_head=True)
+    run = GraphRunner(ops, layers, outs, plain_layers=plain)
+    run.fill_parameters(seed=3)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    for pl in run.plain:
+        pl["w"].normal_(0.0, 0.05, generator=gen)
+        pl["bias"].normal_(0.0, 0.5, generator=gen)
+    second = torch.cuda.Stream() if side else None
+    ws = torch.empty(max(b.plan.bwd_bytes for b in run.blocks), dtype=torch.uint8, device="cuda") if side else None
+
+    def inputs(seed):
+        gen.manual_seed(seed)
+        run.buf["img"].uniform_(0.0, 1.0, generator=gen)
+        for name in outs:
+            run.grad[name].normal_(generator=gen)
+
+    def results():
+        torch.cuda.synchronize()
+        run.poll()
+        return [t.clone() for t in [run.buf[o] for o in outs] + [run.grad["img"]] + [b.dw for b in run.blocks] + [b.dgamma for b in run.blocks]]
+
+    def step(stream=None):
+        before = nb.nb_cbs_launch_count()
+        run.forward(stream)
+        run.backward(stream, wgrad_stream=second, wgrad_workspace=ws)
+        return nb.nb_cbs_launch_count() - before
+
+    def issued(seed):  # the calls themselves
+        inputs(seed)
+        run._forward(None)
+        torch.cuda.synchronize()
+        run._backward(None, second, ws)
+        return results()
+
+    def same(seed, stream=None):
+        want = issued(seed)
+        inputs(seed)
+        torch.cuda.synchronize()
+        n = step(stream)
+        assert all(torch.equal(a, b) for a, b in zip(results(), want))
+        return n
+
+    counts = [same(seed) for seed in (1, 2, 3, 4)]  # issued, recorded and replayed, replayed, replayed
+    assert len(set(counts)) == 1 and counts[0] > 400
+    run.blocks[5].dw = torch.zeros_like(run.blocks[5].dw)  # another tensor: issued again, then recorded again
+    assert [same(seed) for seed in (5, 6, 7)] == counts[:3]
+    mine = torch.cuda.Stream()
+    assert [same(seed, mine) for seed in (8, 9)] == counts[:2]
+    want = issued(10)
+    inputs(10)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        if side:
+            second.wait_stream(torch.cuda.current_stream())
+        step()
+        if side:
+            torch.cuda.current_stream().wait_stream(second)
+    graph.replay()
+    assert all(torch.equal(a, b) for a, b in zip(results(), want))
