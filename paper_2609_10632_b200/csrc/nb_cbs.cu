@@ -233,10 +233,11 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
         if (fb.wt) blocks = std::max(blocks, std::min(e.wave_reduce, (wt_num_tiles(*wtp) + 1) / 2));
         auto go = [&](auto kernel, long long ld) {
             launch_k(kernel, dim3(blocks), dim3(e.tpb), red_smem, st, 1, static_cast<const AT*>(g), static_cast<const YT*>(y), e.total_vecs, C, mean, invstd,
-                     gamma, beta, partials, fb, wtp ? *wtp : none, ld);
+                     gamma, beta, partials, fb, wtp ? *wtp : none, ld, e.blocks_reduce);
         };
-        if (p->ld_g) go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true>, p->ld_g);
-        else go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false>, (long long)C);
+        const bool deep = 2 * e.blocks_reduce <= p->sm_count;  // at most every second SM has rows
+        if (p->ld_g) deep ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true, true>, p->ld_g) : go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true>, p->ld_g);
+        else deep ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false, true>, (long long)C) : go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false>, (long long)C);
         NB_LAUNCH_OK("bn_silu_bwd_reduce");
     }
     if (!fuse) {
@@ -448,10 +449,9 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     e.total_vecs = g.m * e.cgs;
     const long long max_blocks = (e.total_vecs + e.tpb - 1) / e.tpb;
     // Grids are one wave of resident blocks (occupancy queried per kernel).  A tensor smaller than that gets as many blocks
-    // as it has work for: four vectors per thread in the reductions (a block also adds 2*C sums to the accumulators), one
-    // in the maps.  A thread's vectors are a serial chain of memory latencies, and on small tensors that chain is the
-    // kernel: with 8 and 4 vectors the five passes of a 16 -> 32 layer on 2 x 32 x 32 pixels took 4.9 us longer (36.3 ->
-    // 31.4 us for the step's kernels), 72 -> 136 on 3 x 53 x 75 pixels 4.0 us (60.9 -> 56.9).
+    // as it has work for: eight vectors per thread in the backward reduction (a block also adds 2*C sums to the accumulators;
+    // the grouping of the additions is part of the results' last bits, and stays), one in the maps, whose threads would
+    // otherwise chain memory latencies: 16 -> 32 on 2 x 32 x 32 pixels, 36.3 -> 34.0 us for the step's kernels against four.
     {
         e.wave_reduce = 0;
         auto wave = [&](const void* fn, size_t dyn_smem, int min_vecs, int* resident = nullptr) {
@@ -469,17 +469,17 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
         const size_t apply_smem = p->fuse_finalize ? (size_t)2 * g.c_out * sizeof(float) : 0, dy_smem = p->fuse_finalize ? (size_t)4 * g.c_out * sizeof(float) : 0;
         if (d->mode == NB_MODE_F32_REF) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<float>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, red_smem, 4, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, red_smem, 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<float, float, false, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<float, float, false, false, true>, dy_smem, 1);
         } else if (d->mode == NB_MODE_F16_TC) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, red_smem, 4, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, red_smem, 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __half, true, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __half, true, false, true>, dy_smem, 1);
         } else {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, red_smem, 4, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, red_smem, 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __nv_bfloat16, true, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __nv_bfloat16, true, false, true>, dy_smem, 1);
         }

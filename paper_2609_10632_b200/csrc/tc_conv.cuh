@@ -72,6 +72,7 @@ struct IgemmParams {
     void* out;
     int split;         // CTAs (a cluster) that share the K range of a tile in tc_split_kernel
     long long ld_out;  // its output row pitch in elements
+    int full_rows, full_bn, full_n_tiles, full_workers;  // tiling and workers of the persistent form of the same launch
     float* partials;  // [gridDim.x][2][ldo] per-CTA channel sums and sums of squares (statistics variant only)
     int* status;
     uint16_t off_w[4][9], off_h[4][9];
@@ -1008,8 +1009,8 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     const long long m_tiles = (f.M + TC_BM - 1) / TC_BM;
     if (m_tiles * ncls > sm_count) return;
     auto kb_time = [](int bn) { return std::max(4.0 * std::max(45.0, bn / 2.0), (TC_BM + bn) * 128 / 55.0) / 1900.0; };
-    const double workers = f.cg2 ? sm_count / 2 : sm_count;
-    const double full_waves = (double)(((long long)f.m_tiles * f.n_tiles * ncls + (long long)workers - 1) / (long long)workers);
+    const int workers = f.cg2 ? f.grid / 2 : f.grid;
+    const double full_waves = (double)(((long long)f.m_tiles * f.n_tiles * ncls + workers - 1) / workers);
     double best = 4.5 + full_waves * (kblocks * f.mh * kb_time(f.BN) + 0.8);
     const int force_s = getenv("NB_TC_SPLIT_S") ? atoi(getenv("NB_TC_SPLIT_S")) : 0, force_bn = getenv("NB_TC_SPLIT_BN") ? atoi(getenv("NB_TC_SPLIT_BN")) : 0;
     if (force_s || force_bn) best = 1e30;
@@ -1017,7 +1018,8 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     for (int nt = (f.rowsB + 127) / 128; nt <= (f.rowsB + 15) / 16; ++nt) {
         const int bn = ((f.rowsB + nt - 1) / nt + 15) / 16 * 16;
         if ((f.rowsB + bn - 1) / bn != nt || (force_bn && bn != force_bn)) continue;
-        for (int s = 1; s <= 8 && s <= min_kb; s *= 2) {
+        if (!eval && f.BN % bn) continue;  // a tile lies within one tile of the persistent form
+        for (int s = 1; s <= (eval ? 8 : 1) && s <= min_kb; s *= 2) {
             const long long ctas = m_tiles * nt * ncls * s;
             if (ctas > (s == 8 ? sm_count * 6 / 7 : s == 4 ? sm_count * 9 / 10 : sm_count) || (force_s && s != force_s)) continue;
             const double t = 3.5 + ((kblocks + s - 1) / s) * kb_time(bn) + 0.012 * bn + (s > 1 ? 1.2 : 0.0) + (eval ? 0.0 : 0.5 + 0.023 * bn / s);
@@ -1041,7 +1043,7 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     while (c.tmem_cols < best_bn) c.tmem_cols *= 2;
     c.acc_stride = c.tmem_cols;
     c.stages = std::max(2, std::min(8, (kblocks + best_s - 1) / best_s));
-    const size_t part = (size_t)TC_BM * (best_bn + 4) * 4, fixed = 1024 + 64 + (size_t)2 * SP_THREADS * 16 + 512;
+    const size_t part = (size_t)TC_BM * (best_bn + 4) * 4, fixed = 1024 + 64 + (size_t)8 * 128 * 4 + 512;
     while (c.stages > 2 && fixed + (size_t)c.stages * (c.a_stage + c.b_stage) > kMaxSmem) --c.stages;
     c.smem_bytes = std::max<size_t>(fixed + std::max(part, (size_t)c.stages * (c.a_stage + c.b_stage)), 120 * 1024);  // > half an SM: one CTA per SM
     c.grid = (int)(m_tiles * c.n_tiles * ncls * best_s);
@@ -1051,6 +1053,7 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     P.a_stage_bytes = P.a_sub_bytes = c.a_stage; P.b_stage_bytes = P.b_sub_bytes = c.b_stage;
     P.kpb = 1; P.mh = 1; P.acc_bufs = 1; P.tma_store = 0;
     P.split = c.split;
+    P.full_rows = TC_BM * f.mh * (f.cg2 ? 2 : 1); P.full_bn = f.BN; P.full_n_tiles = f.n_tiles; P.full_workers = workers;
     P.idesc = ptx::make_idesc_bf16(TC_BM, c.BN, 0, 0);
     c.ok = true;
     out.cfg = c;
@@ -1244,7 +1247,8 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
             tc->fprop = true;
             tc->fprop_parts = c.grid;
             tc->inf = tc->fp;
-            split_configure(tc->fps, tc->fp, g.k * g.k, false, sm_count);
+            // (a training forward whose persistent form has one 128-row tile per CTA: its channel sums are one tile's)
+            if (c.mh == 1 && (long long)c.m_tiles * c.n_tiles <= (c.cg2 ? c.grid / 2 : c.grid)) split_configure(tc->fps, tc->fp, g.k * g.k, false, sm_count);
             split_configure(tc->infs, tc->inf, g.k * g.k, true, sm_count);
             tc->infer = true;
         }

@@ -4,6 +4,10 @@
 // K range of a tile is cut over a CLUSTER of 1, 2, 4 or 8 CTAs.  Every CTA accumulates its share in TMEM, leaves it as fp32
 // in its own shared memory, and after one cluster barrier CTA r sums rows [128 r / S, 128 (r + 1) / S) of all S partial
 // tiles through distributed shared memory, in rank order (the same bits every run), applies the epilogue and stores.
+// The training calls use clusters of one (narrow tiles only): the sum of an element then runs over the k-blocks in the order
+// in which the persistent kernel would add them (the same starting k-block), and the channel sums are formed as there, so
+// that the results of a training step do not depend on which of the two kernels a layer gets -- a deep network in training
+// mode turns a difference in the last bit of one layer into percents a few dozen layers on.
 // No block waits for a block outside its cluster.  Bound: latency -- operand fetch to first MMA, the k-blocks of one CTA
 // (a k-block is (128 + BN) 128-byte rows through TMA), accumulator -> shared memory -> peers -> rounding -> store.
 // The narrow tiles (BN <= 128, often 32 to 64) are part of the same idea: more CTAs, and less to hand over.
@@ -35,8 +39,8 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
     float* part = reinterpret_cast<float*>(smem);  // [128][BN + 4] this CTA's share, over the operand stages once they are consumed
     const int S = p.split, pitch = p.BN + 4;
     const size_t stage_total = (size_t)p.stages * (p.a_stage_bytes + p.b_stage_bytes), part_total = (size_t)TC_BM * pitch * 4;
-    float* red = reinterpret_cast<float*>(smem + ((stage_total > part_total ? stage_total : part_total) + 15) / 16 * 16);  // MODE 1: [256 / (BN / 4)][2][BN]; MODE 2: scale, shift [2][BN]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(red + 2 * SP_THREADS * 4);
+    float* red = reinterpret_cast<float*>(smem + ((stage_total > part_total ? stage_total : part_total) + 15) / 16 * 16);  // MODE 1: channel sums [4][2][BN]; MODE 2: scale, shift [2][BN]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(red + 8 * 128);
     uint64_t* full = bars;
     uint64_t* empty = bars + p.stages;
     uint64_t* tfull = empty + p.stages;
@@ -51,6 +55,16 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
     const int m_tile = lt / p.n_tiles, n_tile = lt - m_tile * p.n_tiles;
     const int kblocks = p.cls_ntaps[cls] * p.kc_per_tap;
     const int kb0 = kblocks * rank / S, kb1 = kblocks * (rank + 1) / S;  // this CTA's share of the K range
+    // MODE 0, 1: first k-block of the tile of the persistent kernel that contains this one
+    int rot = 0;
+    if (MODE != 2) {
+        int full_tile = (m_tile * TC_BM / p.full_rows) * p.full_n_tiles + n_tile * p.BN / p.full_bn;
+        if (p.nclasses == 4) {  // igemm_tile_class, solved for the tile
+            const int round = full_tile * 4 / p.full_workers;
+            full_tile = full_tile * 4 + ((cls - ((p.full_workers & 1) ? 0 : round)) & 3);
+        }
+        rot = (int)(((unsigned)(full_tile % p.full_workers) * 7u) % (unsigned)kblocks);
+    }
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
@@ -66,7 +80,8 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
         ptx::prefetch_tmap(&p.tmB[cls]);
         // this CTA's filter tiles start for L2 while the previous kernel still runs (a hint: L2 stays coherent whoever
         // writes the filter in the meantime)
-        for (int kb = kb0; kb < kb1 && kb < kb0 + 16; ++kb) {
+        for (int i = kb0; i < kb1 && i < kb0 + 16; ++i) {
+            const int kb = i + rot < kblocks ? i + rot : i + rot - kblocks;
             const int tap = kb / p.kc_per_tap, kc = kb - tap * p.kc_per_tap;
             prefetch_tile_2d(&p.tmB[cls], tap * p.Ca + kc * p.KC, n_tile * p.BN);
         }
@@ -99,7 +114,8 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
             cw0 = p.lo_w + j0 * p.ts;
             ch0 = p.lo_h + i0 * p.ts;
         }
-        int tap = kb0 / p.kc_per_tap, kc = kb0 - tap * p.kc_per_tap, s = 0, issued = 0;
+        const int first = (kb0 + rot) % kblocks, ntaps = p.cls_ntaps[cls];
+        int tap = first / p.kc_per_tap, kc = first - tap * p.kc_per_tap, s = 0, issued = 0;
         uint32_t ph = 0;
         bool ok = true;
         pdl_wait();
@@ -117,7 +133,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
             else ptx::tma_load_im2col_4d_u32_if(leader, dst, tm, bar, kc * p.KC, cw0, ch0, n0, p.off_w[cls][tap], p.off_h[cls][tap]);
             if (++kc == p.kc_per_tap) {
                 kc = 0;
-                ++tap;
+                if (++tap == ntaps) tap = 0;
             }
             ++issued;
             if (++s == p.stages) {
@@ -142,7 +158,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
         const uint64_t da0 = ptx::make_smem_desc(ptx::smem_u32(sA), 16, p.sbo, p.umma_swizzle), db0 = ptx::make_smem_desc(ptx::smem_u32(sB), 16, p.sbo, p.umma_swizzle);
         const uint64_t a_stage16 = (uint64_t)(p.a_stage_bytes >> 4), b_stage16 = (uint64_t)(p.b_stage_bytes >> 4);
         const uint32_t empty_u32 = ptx::smem_u32(empty);
-        int kc = kb0 % p.kc_per_tap, s = 0;
+        int kc = (kb0 + rot) % kblocks % p.kc_per_tap, s = 0;
         uint32_t ph = 0, accumulate = 0;
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
@@ -223,7 +239,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
         const int col = n_tile * p.BN + gi * 4;
         const bool live = r0 < rp && col < p.ldo;
         const uint32_t part_u32 = ptx::smem_u32(part);
-        float4 cs = make_float4(0.f, 0.f, 0.f, 0.f), cq = cs, sc = cs, sh = cs;
+        float4 sc = make_float4(0.f, 0.f, 0.f, 0.f), sh = sc;
         if (MODE == 2) {
             sc = *reinterpret_cast<const float4*>(red + gi * 4);
             sh = *reinterpret_cast<const float4*>(red + p.BN + gi * 4);
@@ -276,27 +292,39 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
                 o = sum;
             }
             *reinterpret_cast<uint2*>(dst) = o;
-            if (MODE == 1) {
-                const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&o.x)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&o.y));
-                cs.x += f0.x; cs.y += f0.y; cs.z += f1.x; cs.w += f1.y;
-                cq.x = fmaf(f0.x, f0.x, cq.x); cq.y = fmaf(f0.y, f0.y, cq.y); cq.z = fmaf(f1.x, f1.x, cq.z); cq.w = fmaf(f1.y, f1.y, cq.w);
-            }
         }
-        if (sat_bits & (int)0x80008000u) atomicAdd(p.status + ST_SAT, 1);
+        int sat = sat_bits & (int)0x80008000u ? 1 : 0;
         if (MODE == 1) {
-            if (r0 < rp) {
-                *reinterpret_cast<float4*>(red + (size_t)(r0 * 2) * p.BN + gi * 4) = cs;
-                *reinterpret_cast<float4*>(red + (size_t)(r0 * 2 + 1) * p.BN + gi * 4) = cq;
+            // channel sums of the rounded values: a thread takes two channels of 32 rows, even and odd rows apart, then the
+            // four row groups are added in order (the persistent kernel's grouping; rows past the last pixel are zeros)
+            const int c2 = (int)threadIdx.x % (p.BN / 2), grp = (int)threadIdx.x / (p.BN / 2);
+            if (grp < 4) {
+                float2 sa = make_float2(0.f, 0.f), sb = sa, qa = sa, qb = sa;
+                const float* src = part + (size_t)grp * 32 * pitch + 2 * c2;
+#pragma unroll 8
+                for (int rr = 0; rr < 32; rr += 2) {
+                    const float2 a0 = *reinterpret_cast<const float2*>(src + (size_t)rr * pitch), a1 = *reinterpret_cast<const float2*>(src + (size_t)(rr + 1) * pitch);
+                    const uint32_t h0 = pack2<__half>(a0.x, a0.y, nullptr), h1 = pack2<__half>(a1.x, a1.y, nullptr);
+                    const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&h0)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&h1));
+                    sa = add2(sa, f0);
+                    sb = add2(sb, f1);
+                    qa = fma2(f0, f0, qa);
+                    qb = fma2(f1, f1, qb);
+                }
+                const float qx = qa.x + qb.x, qy = qa.y + qb.y;
+                float* dst = red + (size_t)grp * 2 * p.BN + 2 * c2;
+                *reinterpret_cast<float2*>(dst) = make_float2(sa.x + sb.x, sa.y + sb.y);
+                *reinterpret_cast<float2*>(dst + p.BN) = make_float2(qx, qy);
             }
             __syncthreads();
             for (int e = threadIdx.x; e < 2 * p.BN; e += SP_THREADS) {
-                const int which = e >= p.BN ? 1 : 0, c = e - which * p.BN;
+                const int c = e >= p.BN ? e - p.BN : e;
                 if (n_tile * p.BN + c >= p.ldo) continue;
-                float t = 0.f;
-                for (int r = 0; r < rp && r < rows; ++r) t += red[(size_t)(r * 2 + which) * p.BN + c];
-                chan_acc_add(p.acc, p.ldo, which, n_tile * p.BN + c, t);
+                const float* b = red + e;
+                chan_acc_add(p.acc, p.ldo, e >= p.BN ? 1 : 0, n_tile * p.BN + c, ((b[0] + b[2 * p.BN]) + b[4 * p.BN]) + b[6 * p.BN]);
             }
         }
+        if (sat) atomicAdd(p.status + ST_SAT, sat);
     }
     if (S > 1) ptx::cluster_sync_all();  // no CTA leaves while a peer may still read its rows
 }
