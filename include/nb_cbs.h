@@ -222,8 +222,8 @@ nb_status nb_conv_bn_silu_bwd_weight(nb_cbs_plan plan, const void* x, const void
  * Workspace size of the three calls below and whether they run as ONE kernel: `*fused` (may be NULL) is 1 when the
  * convolution runs on the tensor-core kernel with the per-channel scale/shift and the activation applied to the fp32
  * accumulators in its epilogue (16-bit modes, c_in % 8 == 0, c_out % 8 == 0, c_out >= 16 -- with fewer than 256 output
- * pixels both counts multiples of 16; also the 3 -> 48 channel 3x3 stride-2 first layer, whose own kernel has the same
- * epilogue); 0 when the plan falls back to
+ * pixels both counts multiples of 16; also 3x3 stride-2 first layers of even extents with 3 input and 16, 32, 48, 64 or
+ * 80 output channels, whose own kernel has the same epilogue); 0 when the plan falls back to
  * convolution -> coefficient kernel -> elementwise pass, whose workspace also holds the convolution output. */
 nb_status nb_cbs_infer_workspace_bytes(nb_cbs_plan plan, size_t* bytes, int32_t* fused);
 

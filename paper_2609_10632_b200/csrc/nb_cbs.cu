@@ -272,6 +272,60 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
     return launch_ok("bn_silu_bwd_dy");
 }
 
+// ---------------------------------------------------------------- first layer
+// f(integral_constant) with the plan's output channel count (one of stem_cout_ok's)
+template <class F> nb_status with_stem_cout(int c_out, F f) {
+    switch (c_out) {
+        case 16: return f(std::integral_constant<int, 16>{});
+        case 32: return f(std::integral_constant<int, 32>{});
+        case 48: return f(std::integral_constant<int, 48>{});
+        case 64: return f(std::integral_constant<int, 64>{});
+        default: return f(std::integral_constant<int, 80>{});
+    }
+}
+template <typename OutT, typename AT, bool EPI>
+nb_status run_stem_fprop(nb_cbs_plan_s* p, const void* x, const void* w, void* y, const StemEpi& ep, float* part, double* acc, cudaStream_t st) {
+    return with_stem_cout(p->g.c_out, [&](auto co) {
+        auto go = [&](auto kernel) {
+            launch_k(kernel, dim3(p->stem_fprop_blocks), dim3(128), 0, st, 1, static_cast<const AT*>(x), static_cast<const AT*>(w), static_cast<OutT*>(y), p->g, ep, part, acc,
+                     acc ? p->acc_copies_f : 1);
+        };
+        if (p->stem_wide) go(stem_fprop_mma_kernel<decltype(co)::value, OutT, EPI, AT, STEM_TQ_WIDE>);
+        else go(stem_fprop_mma_kernel<decltype(co)::value, OutT, EPI, AT, STEM_TQ>);
+        return launch_ok("stem_fprop");
+    });
+}
+template <typename AT> nb_status run_stem_dgrad(nb_cbs_plan_s* p, const void* dy, const void* w, void* dx, cudaStream_t st) {
+    return with_stem_cout(p->g.c_out, [&](auto co) {
+        launch_k(stem_dgrad_mma_kernel<decltype(co)::value, AT>, dim3(p->stem_dgrad_blocks), dim3(128), 0, st, 1, static_cast<const AT*>(dy), static_cast<const AT*>(w),
+                 static_cast<AT*>(dx), p->g, p->stem_dgrad_rows);
+        return launch_ok("stem_dgrad");
+    });
+}
+template <typename AT> nb_status run_stem_wgrad(nb_cbs_plan_s* p, const void* x, const void* dy, float* partial, cudaStream_t st) {
+    return with_stem_cout(p->g.c_out, [&](auto co) {
+        constexpr int CO = decltype(co)::value;
+        auto go = [&](auto kernel, size_t smem) {
+            launch_k(kernel, dim3(p->stem_wgrad_blocks), dim3(128), smem, st, 1, static_cast<const AT*>(x), static_cast<const AT*>(dy), partial, p->g);
+        };
+        if (p->stem_wide) go(stem_wgrad_mma_kernel<CO, AT, STEM_TQ_WGRAD>, stem_wgrad_smem_bytes<CO, AT, STEM_TQ_WGRAD>());
+        else go(stem_wgrad_mma_kernel<CO, AT, STEM_TQ>, stem_wgrad_smem_bytes<CO, AT, STEM_TQ>());
+        return launch_ok("stem_wgrad");
+    });
+}
+// More dynamic shared memory than the 48 KB a kernel gets without asking (the weight gradient's ring), with the device current.
+template <typename AT> cudaError_t stem_allow_smem(int c_out) {
+    cudaError_t e = cudaSuccess;
+    with_stem_cout(c_out, [&](auto co) {
+        constexpr int CO = decltype(co)::value;
+        e = cudaFuncSetAttribute(stem_wgrad_mma_kernel<CO, AT, STEM_TQ_WGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stem_wgrad_smem_bytes<CO, AT, STEM_TQ_WGRAD>());
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(stem_wgrad_mma_kernel<CO, AT, STEM_TQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stem_wgrad_smem_bytes<CO, AT, STEM_TQ>());
+        return NB_OK;
+    });
+    return e;
+}
+
 // ---------------------------------------------------------------- CUDA-core convolutions
 // Tile and slices.  64 x 64 where such tiles give every SM two blocks, else 32 x 64; 64 x 32 for at most 32 columns and for
 // the 16-bit fallback.  One block alone on an SM waits for its ring (0.5 us per 16-k stage, half of it latency), so where
@@ -429,16 +483,18 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     int count = 0;
     NB_CUDA_CHECK(cudaGetDeviceCount(&count));
     if (device < 0 || device >= count) return fail(NB_ERR_INVALID_ARG, "device %d out of range (%d devices)", device, count);
-    cudaDeviceProp prop;
-    NB_CUDA_CHECK(cudaGetDeviceProperties(&prop, device));
-    if (prop.major != 10) return fail(NB_ERR_ARCH, "device %d is sm_%d%d; this library is built for sm_100a only", device, prop.major, prop.minor);
+    int major = 0, minor = 0, sms = 0;  // (attributes: cudaGetDeviceProperties takes 2.5 ms)
+    NB_CUDA_CHECK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device));
+    NB_CUDA_CHECK(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device));
+    NB_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+    if (major != 10) return fail(NB_ERR_ARCH, "device %d is sm_%d%d; this library is built for sm_100a only", device, major, minor);
 
     nb_cbs_plan_s* p = new (std::nothrow) nb_cbs_plan_s();
     if (!p) return fail(NB_ERR_INTERNAL, "out of host memory");
     p->desc = *d;
     p->g = g;
     p->device = device;
-    p->sm_count = prop.multiProcessorCount;
+    p->sm_count = sms;
     p->fuse_finalize = !(d->flags & NB_CBS_FLAG_SEPARATE_FINALIZE);
 
     EwCfg& e = p->ew;
@@ -507,7 +563,7 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     if (ce == cudaSuccess && acc_bytes) p->acc = reinterpret_cast<double*>(reinterpret_cast<char*>(p->status) + kStatusBytes);
     nb_status tcs = NB_OK;
     if (ce == cudaSuccess)
-        tcs = tc_plan_init(&p->tc, g, d->mode != NB_MODE_F32_REF && !(d->flags & NB_CBS_FLAG_FORCE_SIMT), p->sm_count, prop, d->mode == NB_MODE_F16_TC);
+        tcs = tc_plan_init(&p->tc, g, d->mode != NB_MODE_F32_REF && !(d->flags & NB_CBS_FLAG_FORCE_SIMT), p->sm_count, d->mode == NB_MODE_F16_TC);
     cudaSetDevice(cur);
     if (ce != cudaSuccess || tcs != NB_OK) {
         if (p->status) cudaFree(p->status);
@@ -517,24 +573,18 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     }
 
     p->stem = d->mode != NB_MODE_F32_REF && !(d->flags & NB_CBS_FLAG_FORCE_SIMT) && g.c_in == 3 && g.k == 3 && g.stride == 2 &&
-              g.c_out == 48 && g.h % 2 == 0 && g.w % 2 == 0 && g.m < (1LL << 31) && (long long)g.n * g.h * g.w * 3 < (1LL << 31);
-    p->stem_blocks = (int)std::min<long long>(stem_num_strips(g), (long long)p->sm_count * 4);  // grid of the three first-layer kernels: one wave of four resident blocks per SM
-    p->stem_dgrad_blocks = stem_dgrad_grid(g, p->sm_count * 5, &p->stem_dgrad_rows);
+              stem_cout_ok(g.c_out) && g.h % 2 == 0 && g.w % 2 == 0 && g.m < (1LL << 31) && (long long)g.n * g.h * g.w * 3 < (1LL << 31);
+    p->stem_blocks = (int)std::min<long long>(stem_num_strips(g), (long long)p->sm_count * stem_occ(g.c_out));  // grid of the first-layer kernels: one wave of resident blocks
+    p->stem_dgrad_blocks = stem_dgrad_grid(g, p->sm_count * stem_dgrad_occ(g.c_out), &p->stem_dgrad_rows);
     p->stem_wide = g.wo >= STEM_TQ_WIDE / 2;  // (a strip of a narrower row would leave most of its tile slots empty)
     if (const char* e2 = getenv("NB_STEM_WIDE")) p->stem_wide = atoi(e2) != 0;
-    p->stem_fprop_blocks = p->stem_wide ? (int)std::min<long long>(stem_num_strips(g, STEM_TQ_WIDE), (long long)p->sm_count * 4) : p->stem_blocks;
-    p->stem_wgrad_blocks = p->stem_wide ? (int)std::min<long long>(stem_num_strips(g, STEM_TQ_WGRAD), (long long)p->sm_count * 4) : p->stem_blocks;
-    if (p->stem && p->stem_wide) {  // (more than the 48 KB a kernel gets without asking)
+    p->stem_fprop_blocks = p->stem_wide ? (int)std::min<long long>(stem_num_strips(g, STEM_TQ_WIDE), (long long)p->sm_count * stem_occ(g.c_out)) : p->stem_blocks;
+    p->stem_wgrad_blocks = p->stem_wide ? (int)std::min<long long>(stem_num_strips(g, STEM_TQ_WGRAD), (long long)p->sm_count * stem_occ(g.c_out)) : p->stem_blocks;
+    if (p->stem) {
         DeviceGuard on_device(p->device);
-        cudaError_t ae = cudaFuncSetAttribute(stem_wgrad_mma_kernel<48, __nv_bfloat16, STEM_TQ_WGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)stem_wgrad_smem_bytes<48, __nv_bfloat16, STEM_TQ_WGRAD>());
-        if (ae == cudaSuccess)
-            ae = cudaFuncSetAttribute(stem_wgrad_mma_kernel<48, __half, STEM_TQ_WGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)stem_wgrad_smem_bytes<48, __half, STEM_TQ_WGRAD>());
-        if (ae != cudaSuccess) {
-            p->stem_wide = false;
-            p->stem_fprop_blocks = p->stem_wgrad_blocks = p->stem_blocks;
+        if (NB_WITH_AT(p, stem_allow_smem<AT>(g.c_out)) != cudaSuccess) {
             (void)cudaGetLastError();
+            p->stem = false;  // the CUDA-core kernels take any shape
         }
     }
     p->nparts = std::max(std::max(std::max(e.blocks_reduce, e.blocks_stats), p->tc.fprop_parts), p->stem ? p->stem_blocks : 0);
@@ -743,16 +793,7 @@ nb_status nb_conv_bn_silu_fwd(nb_cbs_plan p, const void* x, const void* w, const
         // the first layer's kernel sums the statistics of the values it stores itself (one partial slice per block)
         SiteTimer tm(p, SITE_FPROP, st);
         const bool fuse = p->fuse_finalize;  // sums into the plan's accumulators; the normalise + SiLU pass finalizes
-        if (p->stem_wide) {
-            NB_WITH_AT(p, launch_k(stem_fprop_mma_kernel<48, __half, false, AT, STEM_TQ_WIDE>, dim3(p->stem_fprop_blocks), dim3(128), 0, st, 1,
-                                   static_cast<const AT*>(x), static_cast<const AT*>(w), static_cast<__half*>(y_saved), p->g, StemEpi{},
-                                   fuse ? static_cast<float*>(nullptr) : part, fuse ? p->acc : static_cast<double*>(nullptr), fuse ? p->acc_copies_f : 1));
-        } else {
-            NB_WITH_AT(p, launch_k(stem_fprop_mma_kernel<48, __half, false, AT, STEM_TQ>, dim3(p->stem_fprop_blocks), dim3(128), 0, st, 1,
-                                   static_cast<const AT*>(x), static_cast<const AT*>(w), static_cast<__half*>(y_saved), p->g, StemEpi{},
-                                   fuse ? static_cast<float*>(nullptr) : part, fuse ? p->acc : static_cast<double*>(nullptr), fuse ? p->acc_copies_f : 1));
-        }
-        NB_LAUNCH_OK("stem_fprop");
+        NB_TRY(NB_WITH_AT(p, run_stem_fprop<__half, AT, false>(p, x, w, y_saved, StemEpi{}, fuse ? nullptr : part, fuse ? p->acc : nullptr, st)));
         nparts = p->stem_fprop_blocks;
         finalized = fuse;
     } else if (p->tc.fprop) {
@@ -795,16 +836,7 @@ nb_status run_infer(nb_cbs_plan_s* p, const void* x, const void* w, const float*
     }
     if (!is_f32(p) && p->stem) {  // the first layer's own kernel applies the coefficients and the activation itself
         SiteTimer tm(p, SITE_INFER, st);
-        if (p->stem_wide) {
-            NB_WITH_AT(p, launch_k(stem_fprop_mma_kernel<48, AT, true, AT, STEM_TQ_WIDE>, dim3(p->stem_fprop_blocks), dim3(128), 0, st, 1, static_cast<const AT*>(x),
-                                   static_cast<const AT*>(w), static_cast<AT*>(out), p->g, StemEpi{gamma, beta, rmean, rvar, p->desc.eps, act},
-                                   static_cast<float*>(nullptr), static_cast<double*>(nullptr), 1));
-        } else {
-            NB_WITH_AT(p, launch_k(stem_fprop_mma_kernel<48, AT, true, AT, STEM_TQ>, dim3(p->stem_fprop_blocks), dim3(128), 0, st, 1, static_cast<const AT*>(x),
-                                   static_cast<const AT*>(w), static_cast<AT*>(out), p->g, StemEpi{gamma, beta, rmean, rvar, p->desc.eps, act},
-                                   static_cast<float*>(nullptr), static_cast<double*>(nullptr), 1));
-        }
-        return launch_ok("stem_fprop (fused epilogue)");
+        return NB_WITH_AT(p, run_stem_fprop<AT, AT, true>(p, x, w, out, StemEpi{gamma, beta, rmean, rvar, p->desc.eps, act}, nullptr, nullptr, st));
     }
     float* scale = reinterpret_cast<float*>(ws + p->off_scale);
     float* shift = reinterpret_cast<float*>(ws + p->off_shift);
@@ -922,9 +954,7 @@ nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan p, const void* g, const void* y_s
     if (!dx) return NB_OK;
     if (p->stem) {
         SiteTimer tm(p, SITE_DGRAD, st);
-        NB_WITH_AT(p, launch_k(stem_dgrad_mma_kernel<48, AT>, dim3(p->stem_dgrad_blocks), dim3(128), 0, st, 1, static_cast<const AT*>(dy_out), static_cast<const AT*>(w),
-                               static_cast<AT*>(dx), p->g, p->stem_dgrad_rows));
-        return launch_ok("stem_dgrad");
+        return NB_WITH_AT(p, run_stem_dgrad<AT>(p, dy_out, w, dx, st));
     }
     if (p->tc.dgrad) {
         SiteTimer tm(p, SITE_DGRAD, st);
@@ -960,9 +990,7 @@ nb_status nb_conv_bias_bwd(nb_cbs_plan p, const void* x, const void* w, const vo
                 NB_TRY(run_simt_dgrad<float>(p, dout, w, dx, ws + p->off_wgpart, st));
             } else if (p->stem) {
                 SiteTimer tm(p, SITE_DGRAD, st);
-                NB_WITH_AT(p, launch_k(stem_dgrad_mma_kernel<48, AT>, dim3(p->stem_dgrad_blocks), dim3(128), 0, st, 1, static_cast<const AT*>(dout), static_cast<const AT*>(w),
-                                       static_cast<AT*>(dx), p->g, p->stem_dgrad_rows));
-                NB_LAUNCH_OK("stem_dgrad");
+                NB_TRY(NB_WITH_AT(p, run_stem_dgrad<AT>(p, dout, w, dx, st)));
             } else if (p->tc.dgrad) {
                 SiteTimer tm(p, SITE_DGRAD, st);
                 const long long l0 = p->tc.launches;
@@ -990,14 +1018,7 @@ nb_status nb_conv_bn_silu_bwd_weight(nb_cbs_plan p, const void* x, const void* d
     if (p->stem) {
         {
             SiteTimer tm(p, SITE_WGRAD, st);
-            if (p->stem_wide) {
-                NB_WITH_AT(p, launch_k(stem_wgrad_mma_kernel<48, AT, STEM_TQ_WGRAD>, dim3(p->stem_wgrad_blocks), dim3(128),
-                                       stem_wgrad_smem_bytes<48, AT, STEM_TQ_WGRAD>(), st, 1, static_cast<const AT*>(x), static_cast<const AT*>(dy), partial, p->g));
-            } else {
-                NB_WITH_AT(p, launch_k(stem_wgrad_mma_kernel<48, AT, STEM_TQ>, dim3(p->stem_wgrad_blocks), dim3(128), stem_wgrad_smem_bytes<48, AT, STEM_TQ>(), st, 1,
-                                       static_cast<const AT*>(x), static_cast<const AT*>(dy), partial, p->g));
-            }
-            NB_LAUNCH_OK("stem_wgrad");
+            NB_TRY(NB_WITH_AT(p, run_stem_wgrad<AT>(p, x, dy, partial, st)));
         }
         const size_t elems = (size_t)p->g.c_out * p->g.kdim;
         SiteTimer tm(p, SITE_SPLITK_REDUCE, st);

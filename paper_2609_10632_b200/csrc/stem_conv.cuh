@@ -6,7 +6,8 @@
 // from global memory but cut out of input rows staged in shared memory.
 // Work unit of every kernel: a STRIP of up to 64 consecutive output pixels of one output row (16 per warp); the forward
 // kernel takes strips of up to 320 pixels on wide images (five tiles per warp).
-// COUT is a template parameter (48 for the detector's stem).
+// COUT is a template parameter: 48 for the detector's stem, also 16, 32, 64 and 80 (first layers of narrower and wider
+// networks, which the CUDA-core kernels ran at a few TFLOP/s: 3 -> 32 on 4 x 384 x 212 pixels, step 1400 -> 55 us).
 #pragma once
 #include "common.cuh"
 
@@ -15,6 +16,11 @@ namespace nbcbs {
 constexpr int STEM_CIN = 3, STEM_K = 3, STEM_TAPS = 9, STEM_KDIM = 27;
 constexpr int STEM_TQ = 64;        // output pixels per strip (data and weight gradient; forward of narrow images)
 constexpr int STEM_TQ_WIDE = 320;  // the forward kernel's strip on wide images: per-strip work is shared by 20 tiles instead of 4
+// Resident blocks per SM of the forward and weight-gradient kernels, and of the data gradient (registers: the filter
+// fragments and running sums of 64 and 80 channels need more than a quarter / a fifth of the register file).
+constexpr int stem_occ(int cout) { return cout <= 48 ? 4 : 2; }
+constexpr int stem_dgrad_occ(int cout) { return cout <= 48 ? 5 : 3; }
+constexpr bool stem_cout_ok(int cout) { return cout == 16 || cout == 32 || cout == 48 || cout == 64 || cout == 80; }
 __host__ __device__ constexpr int stem_xchunks(int tq) {  // 16-byte chunks per staged input row: columns 2*q0-1 .. 2*q0+2*tq-1, plus the alignment shift (<= 7)
     return ((2 * tq + 1) * STEM_CIN + 7 + 7) / 8;
 }
@@ -164,7 +170,7 @@ struct StemEpi {
 // without a second pass over y; fixed order, bitwise reproducible).  EPI = true: OutT = activations, see StemEpi.
 // InT = the 16-bit type of x and w (bf16, or IEEE fp16).
 template <int COUT, typename OutT = __half, bool EPI = false, typename InT = __nv_bfloat16, int TQ = STEM_TQ>
-__global__ void __launch_bounds__(128, 4) stem_fprop_mma_kernel(const InT* __restrict__ x, const InT* __restrict__ w, OutT* __restrict__ y, Geom g,
+__global__ void __launch_bounds__(128, stem_occ(COUT)) stem_fprop_mma_kernel(const InT* __restrict__ x, const InT* __restrict__ w, OutT* __restrict__ y, Geom g,
                                                                 StemEpi ep, float* __restrict__ partials, double* __restrict__ acc, int acc_copies) {
     pdl_launch_dependents();
     pdl_wait();
@@ -355,10 +361,9 @@ __global__ void __launch_bounds__(128, 4) stem_fprop_mma_kernel(const InT* __res
 //   parity b = 0:  dy[i][j] x [w11 | w21],  dy[i+1][j] x [0 | w01]
 //   parity b = 1:  dy[i][j] x [w12 | w22],  dy[i][j+1] x [w10 | w20],  dy[i+1][j] x [0 | w02],  dy[i+1][j+1] x [0 | w00].
 // A block stages rows i and i+1 of a 64-position strip (plus one column) in shared memory with 16-byte loads (pixel
-// pitch 112 bytes: conflict-free ldmatrix), the 18 filter fragments stay in registers, and the 2 x 32 output pixels of a
+// pitch 112 bytes at 48 channels: conflict-free ldmatrix), the 18 filter fragments stay in registers, and the 2 x 32 output pixels of a
 // warp are staged and written as 4-byte words (coalesced).  Five blocks are resident per SM (96 registers, a ring of four
 // staged rows of 7.3 KB per block).  Grid: stem_dgrad_grid().
-constexpr int STEM_DYPITCH = 56;  // elements per staged dy pixel (48 channels + padding)
 // Blocks and rows per block of the data-gradient kernel: the bands (image x 64-column strip) are cut into as many row
 // segments as keep the grid within one wave of `slots` resident blocks; more bands than slots: whole bands, several waves.
 inline int stem_dgrad_grid(const Geom& g, int slots, int* seg_rows) {
@@ -369,10 +374,11 @@ inline int stem_dgrad_grid(const Geom& g, int slots, int* seg_rows) {
     return (int)(bands * segs);
 }
 template <int COUT, typename T = __nv_bfloat16>
-__global__ void __launch_bounds__(128, 5) stem_dgrad_mma_kernel(const T* __restrict__ dy, const T* __restrict__ w, T* __restrict__ dx, Geom g, int seg_rows) {
+__global__ void __launch_bounds__(128, stem_dgrad_occ(COUT)) stem_dgrad_mma_kernel(const T* __restrict__ dy, const T* __restrict__ w, T* __restrict__ dx, Geom g, int seg_rows) {
     pdl_launch_dependents();
     pdl_wait();
-    static_assert(COUT % 16 == 0 && COUT + 8 <= STEM_DYPITCH, "whole k-steps; pitch holds a pixel");
+    static_assert(COUT % 16 == 0, "whole k-steps");
+    constexpr int STEM_DYPITCH = COUT + 8;  // elements per staged dy pixel: rows of 16 x odd bytes, conflict-free for ldmatrix
     constexpr int KS = COUT / 16;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gq = lane >> 2, tq = lane & 3;
     const unsigned short* wsrc = reinterpret_cast<const unsigned short*>(w);
@@ -510,7 +516,7 @@ template <int COUT, typename T, int TQ> constexpr size_t stem_wgrad_smem_bytes()
     return sizeof(StemWgradRing<COUT, T, TQ>) > 4 * sizeof(float[COUT][33]) ? sizeof(StemWgradRing<COUT, T, TQ>) : 4 * sizeof(float[COUT][33]);
 }
 template <int COUT, typename T = __nv_bfloat16, int TQ = STEM_TQ>
-__global__ void __launch_bounds__(128, 4) stem_wgrad_mma_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ partial, Geom g) {
+__global__ void __launch_bounds__(128, stem_occ(COUT)) stem_wgrad_mma_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ partial, Geom g) {
     pdl_launch_dependents();
     pdl_wait();
     static_assert(COUT % 16 == 0, "whole m-blocks");

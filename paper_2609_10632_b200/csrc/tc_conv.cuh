@@ -1203,7 +1203,7 @@ inline const char* tc_last_error() { return tcdetail::err().c_str(); }
 
 // Decide which convolutions of this shape run on the tensor-core kernels and size their scratch.
 inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int sm_count);
-inline nb_status tc_plan_init(TcPlan* tc, const Geom& g, bool enable, int sm_count, const cudaDeviceProp&, bool f16 = false) {
+inline nb_status tc_plan_init(TcPlan* tc, const Geom& g, bool enable, int sm_count, bool f16 = false) {
     const nb_status st = tc_plan_init_impl(tc, g, enable, sm_count);
     tc->f16 = f16;
     if (st == NB_OK && f16) {  // A and B formats of the instruction descriptors: bits 7 and 10 set = bf16, clear = f16
