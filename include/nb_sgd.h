@@ -104,7 +104,7 @@ nb_status nb_sgd_clip_nesterov_step(nb_sgd_plan plan, void* workspace, size_t wo
  * the step is SKIPPED: parameters, momentum and working copies stay untouched.  Then the state is advanced:
  *   skipped:  scale = max(scale * backoff_factor, floor_scale), growth_tracker = 0, skipped = 1
  *   otherwise growth_tracker += 1; when it reaches growth_interval: scale *= growth_factor, growth_tracker = 0; skipped = 0
- * Three launches (norm partials; clip + update; scaler state), no host readback; `state` is a device pointer, 16-byte
+ * Two launches (norm partials; clip + update + scaler state), no host readback; `state` is a device pointer, 16-byte
  * aligned.  Errors as nb_sgd_clip_nesterov_step, plus NB_ERR_INVALID_ARG for a NULL state or scaler. */
 nb_status nb_sgd_clip_nesterov_step_scaled(nb_sgd_plan plan, void* workspace, size_t workspace_bytes, const nb_sgd_hyper* hyper,
                                            const nb_scaler_hyper* scaler, nb_loss_scaler* state, float* total_norm, void* stream);

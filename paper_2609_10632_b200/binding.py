@@ -359,6 +359,7 @@ class SgdPlan:
             copy_dtype = NB_DTYPE_F16 if (lp is not None and hasattr(lp, "dtype") and "float16" in str(lp.dtype) and "bfloat16" not in str(lp.dtype)) else 0
             arr[i] = nb_sgd_tensor(_ptr(grad), _ptr(param), _ptr(mom), _ptr(lp), int(numel), int(group), copy_dtype)
         self.count = len(items)
+        self._hyper = self._scaler = (None, None)  # (values, structure) of the last step: they seldom change
         self.handle = c_void_p()
         _check(load().nb_sgd_plan_create(arr, self.count, device, byref(self.handle)))
         b = c_size_t()
@@ -368,16 +369,26 @@ class SgdPlan:
     def upload(self, workspace, stream=None):
         _check(load().nb_sgd_upload(self.handle, _ptr(workspace), _nbytes(workspace), _stream(stream)))
 
+    def _hyper_struct(self, lr, weight_decay, momentum, max_norm, first_step):
+        values = (*lr, *weight_decay, momentum, max_norm, bool(first_step))
+        if self._hyper[0] != values:
+            h = nb_sgd_hyper(ctypes.sizeof(nb_sgd_hyper), momentum, max_norm, (c_float * 3)(*lr), (c_float * 3)(*weight_decay), 1 if first_step else 0)
+            self._hyper = values, h, byref(h)
+        return self._hyper[2]
+
     def step(self, workspace, lr, weight_decay, momentum, max_norm, first_step, total_norm=None, stream=None):
-        h = nb_sgd_hyper(ctypes.sizeof(nb_sgd_hyper), momentum, max_norm, (c_float * 3)(*lr), (c_float * 3)(*weight_decay), 1 if first_step else 0)
-        _check(load().nb_sgd_clip_nesterov_step(self.handle, _ptr(workspace), _nbytes(workspace), byref(h), _ptr(total_norm), _stream(stream)))
+        h = self._hyper_struct(lr, weight_decay, momentum, max_norm, first_step)
+        _check(load().nb_sgd_clip_nesterov_step(self.handle, _ptr(workspace), _nbytes(workspace), h, _ptr(total_norm), _stream(stream)))
 
     def step_scaled(self, workspace, state, lr, weight_decay, momentum, max_norm, first_step, growth_factor=2.0, backoff_factor=0.5, floor_scale=0.0,
                     growth_interval=2000, total_norm=None, stream=None):
         """`state`: a 16-byte device buffer laid out as nb_loss_scaler (float scale, int32 growth_tracker, int32 skipped, int32 reserved)."""
-        h = nb_sgd_hyper(ctypes.sizeof(nb_sgd_hyper), momentum, max_norm, (c_float * 3)(*lr), (c_float * 3)(*weight_decay), 1 if first_step else 0)
-        sc = nb_scaler_hyper(ctypes.sizeof(nb_scaler_hyper), growth_factor, backoff_factor, floor_scale, growth_interval)
-        _check(load().nb_sgd_clip_nesterov_step_scaled(self.handle, _ptr(workspace), _nbytes(workspace), byref(h), byref(sc), _ptr(state), _ptr(total_norm),
+        h = self._hyper_struct(lr, weight_decay, momentum, max_norm, first_step)
+        values = (growth_factor, backoff_factor, floor_scale, growth_interval)
+        if self._scaler[0] != values:
+            sc = nb_scaler_hyper(ctypes.sizeof(nb_scaler_hyper), growth_factor, backoff_factor, floor_scale, growth_interval)
+            self._scaler = values, sc, byref(sc)
+        _check(load().nb_sgd_clip_nesterov_step_scaled(self.handle, _ptr(workspace), _nbytes(workspace), h, self._scaler[2], _ptr(state), _ptr(total_norm),
                                                        _stream(stream)))
 
     def close(self):

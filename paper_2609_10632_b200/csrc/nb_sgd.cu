@@ -132,16 +132,14 @@ nb_status sgd_step_impl(nb_sgd_plan p, void* workspace, size_t workspace_bytes, 
     SgdScalars s;
     s.momentum = hyper->momentum; s.max_norm = hyper->max_norm; s.first_step = hyper->first_step;
     s.scaler = state;
+    s.growth_factor = s.backoff_factor = 1.f; s.floor_scale = 0.f; s.growth_interval = 1;
+    if (sc) { s.growth_factor = sc->growth_factor; s.backoff_factor = sc->backoff_factor; s.floor_scale = sc->floor_scale; s.growth_interval = sc->growth_interval; }
     for (int i = 0; i < NB_SGD_GROUPS; ++i) { s.lr[i] = hyper->lr[i]; s.wd[i] = hyper->weight_decay[i]; }
-    const uint8_t* ws = static_cast<const uint8_t*>(workspace);
-    launch_k(sgd_sqnorm_kernel, dim3((unsigned)p->h.grid), dim3(SGD_THREADS), 0, st, 1, ws);
+    uint8_t* ws = static_cast<uint8_t*>(workspace);
+    launch_k(sgd_sqnorm_kernel, dim3((unsigned)p->h.grid), dim3(SGD_THREADS), 0, st, 1, static_cast<const uint8_t*>(ws));
     NB_LAUNCH_OK("sgd_sqnorm");
     launch_k(sgd_update_kernel, dim3((unsigned)p->h.grid), dim3(SGD_THREADS), 0, st, 1, ws, s, total_norm);
     NB_LAUNCH_OK("sgd_update");
-    if (state) {
-        launch_k(sgd_scaler_kernel, dim3(1), dim3(32), 0, st, 1, ws, state, sc->growth_factor, sc->backoff_factor, sc->floor_scale, (int)sc->growth_interval);
-        NB_LAUNCH_OK("sgd_scaler");
-    }
     return NB_OK;
 }
 }  // namespace
