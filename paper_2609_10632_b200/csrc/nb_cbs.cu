@@ -103,6 +103,8 @@ struct nb_cbs_plan_s {
     int stem_dgrad_rows = 0;    // output row pairs per block
     bool profiling = false;  // when set, every kernel site is bracketed by events and the call waits for it
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    cudaStream_t copy_in = nullptr, copy_out = nullptr;  // nb_conv_bn_silu_step_host: its copies in either direction, created on first use
+    cudaEvent_t copy_ev[4] = {};
     double prof_ms[SITE_COUNT] = {};
     long long prof_n[SITE_COUNT] = {};
     size_t fwd_bytes, bwd_bytes;
@@ -624,6 +626,10 @@ nb_status nb_cbs_plan_destroy(nb_cbs_plan p) {
         cudaFree(p->status);
         if (p->ev0) cudaEventDestroy(p->ev0);
         if (p->ev1) cudaEventDestroy(p->ev1);
+        if (p->copy_in) cudaStreamDestroy(p->copy_in);  // (work still queued completes first)
+        if (p->copy_out) cudaStreamDestroy(p->copy_out);
+        for (cudaEvent_t e : p->copy_ev)
+            if (e) cudaEventDestroy(e);
         cudaSetDevice(cur);
     }
     delete p;
@@ -1162,25 +1168,45 @@ nb_status nb_conv_bn_silu_step_host(nb_cbs_plan p, const void* host_x, const voi
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char* d = static_cast<char*>(device_scratch);
     const size_t cb = (size_t)p->g.c_out * 4;
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.x, host_x, L.nx, cudaMemcpyHostToDevice, st));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.w, host_w, L.nw, cudaMemcpyHostToDevice, st));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.gamma, host_gamma, cb, cudaMemcpyHostToDevice, st));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.beta, host_beta, cb, cudaMemcpyHostToDevice, st));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.g, host_g, L.ny_act, cudaMemcpyHostToDevice, st));
+    // PCIe moves data both ways at once: the copies run on two streams of the plan, so that g travels in while a travels
+    // out, and dx goes out while the weight gradient is computed.  On one stream every byte of either direction waits for
+    // every other.  Measured: 384 -> 384 1x1 on 16 x 40 x 40 pixels (40 MB each way) 1548 -> 1230 us (x in, then a and dx out
+    // is what the data dependence leaves), 64 -> 64 3x3 on 2 x 20 x 20 pixels (200 KB) 101 -> 83 us.
+    if (!p->copy_in) NB_CUDA_CHECK(cudaStreamCreateWithFlags(&p->copy_in, cudaStreamNonBlocking));
+    if (!p->copy_out) NB_CUDA_CHECK(cudaStreamCreateWithFlags(&p->copy_out, cudaStreamNonBlocking));
+    for (cudaEvent_t& e : p->copy_ev)
+        if (!e) NB_CUDA_CHECK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    const cudaStream_t in = p->copy_in, out = p->copy_out;
+    // `to` continues behind everything queued on `from` so far
+    auto order = [&](int event, cudaStream_t from, cudaStream_t to) {
+        const cudaError_t e = cudaEventRecord(p->copy_ev[event], from);
+        return e != cudaSuccess ? e : cudaStreamWaitEvent(to, p->copy_ev[event], 0);
+    };
+    NB_CUDA_CHECK(order(0, st, in));
+    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.w, host_w, L.nw, cudaMemcpyHostToDevice, in));
+    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.gamma, host_gamma, cb, cudaMemcpyHostToDevice, in));
+    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.beta, host_beta, cb, cudaMemcpyHostToDevice, in));
+    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.x, host_x, L.nx, cudaMemcpyHostToDevice, in));
+    NB_CUDA_CHECK(order(1, in, st));
+    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.g, host_g, L.ny_act, cudaMemcpyHostToDevice, in));
     float* gam = reinterpret_cast<float*>(d + L.gamma);
     float* bet = reinterpret_cast<float*>(d + L.beta);
     float* mean = reinterpret_cast<float*>(d + L.mean);
     float* invstd = reinterpret_cast<float*>(d + L.invstd);
     NB_TRY(nb_conv_bn_silu_fwd(p, d + L.x, d + L.w, gam, bet, nullptr, nullptr, d + L.y, mean, invstd, d + L.a, d + L.ws_fwd, p->fwd_bytes, stream));
+    NB_CUDA_CHECK(order(2, st, out));
+    NB_CUDA_CHECK(cudaMemcpyAsync(host_a, d + L.a, L.ny_act, cudaMemcpyDeviceToHost, out));
+    NB_CUDA_CHECK(order(3, in, st));
     NB_TRY(nb_conv_bn_silu_bwd_data(p, d + L.g, d + L.y, mean, invstd, gam, bet, d + L.w, host_dx ? d + L.dx : nullptr,
                                     reinterpret_cast<float*>(d + L.dgamma), reinterpret_cast<float*>(d + L.dbeta), d + L.dy,
                                     d + L.ws_bwd, p->bwd_bytes, stream));
+    NB_CUDA_CHECK(order(0, st, out));
+    if (host_dx) NB_CUDA_CHECK(cudaMemcpyAsync(host_dx, d + L.dx, L.nx, cudaMemcpyDeviceToHost, out));
+    NB_CUDA_CHECK(cudaMemcpyAsync(host_dgamma, d + L.dgamma, cb, cudaMemcpyDeviceToHost, out));
+    NB_CUDA_CHECK(cudaMemcpyAsync(host_dbeta, d + L.dbeta, cb, cudaMemcpyDeviceToHost, out));
     NB_TRY(nb_conv_bn_silu_bwd_weight(p, d + L.x, d + L.dy, reinterpret_cast<float*>(d + L.dw), d + L.ws_bwd, p->bwd_bytes, stream));
-    NB_CUDA_CHECK(cudaMemcpyAsync(host_a, d + L.a, L.ny_act, cudaMemcpyDeviceToHost, st));
-    if (host_dx) NB_CUDA_CHECK(cudaMemcpyAsync(host_dx, d + L.dx, L.nx, cudaMemcpyDeviceToHost, st));
     NB_CUDA_CHECK(cudaMemcpyAsync(host_dw, d + L.dw, L.ndw, cudaMemcpyDeviceToHost, st));
-    NB_CUDA_CHECK(cudaMemcpyAsync(host_dgamma, d + L.dgamma, cb, cudaMemcpyDeviceToHost, st));
-    NB_CUDA_CHECK(cudaMemcpyAsync(host_dbeta, d + L.dbeta, cb, cudaMemcpyDeviceToHost, st));
+    NB_CUDA_CHECK(order(1, out, st));
     return NB_OK;
 }
 
