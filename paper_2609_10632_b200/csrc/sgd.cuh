@@ -88,7 +88,7 @@ __device__ __forceinline__ void sgd_one(float g, float& p, float& b, float coef,
 // Bound: memory.  Chunks are taken last first: the norm kernel has just read all gradients in ascending order, so what is
 // left of them in L2 (126 MB) is their end; parameters and momentum pass through L2 as streams so that they do not push it
 // out, and a chunk's table entries are fetched behind the previous chunk's data.  Measured, the detector's 243 tensors with
-// fp16 copies and the scaler: 162 -> 115 us for the step (5.9 TB/s of 26 bytes per parameter; without the scaler 114 -> 113).
+// fp16 copies and the scaler: 162 -> 115 us for the step (5.9 TB/s of 26 bytes per parameter).
 // With a scaler the last block to have read its state writes the state for the next step (no block waits for another);
 // a kernel of its own, whose one thread summed the norm's partials once more, took 30 us after this one.
 __global__ void __launch_bounds__(SGD_THREADS) sgd_update_kernel(uint8_t* __restrict__ ws, SgdScalars hs, float* __restrict__ total_norm_out) {

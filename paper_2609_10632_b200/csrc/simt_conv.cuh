@@ -59,6 +59,7 @@ struct SgArgs {
     long long kchunk;  // k per slice (blockIdx.z), a multiple of SG_BK
     bool stats;        // KIND 0 with one slice: add the channel sums of the stored values to `acc`
     ChanAcc acc;
+    int overlap;       // KIND 2: runs beside the data gradient in front of it (see the end of common.cuh)
 };
 
 // rows of parity class `cls` of a data gradient, and the grid that covers all classes (host and device)
@@ -79,7 +80,7 @@ __host__ __device__ __forceinline__ SgClass sg_class(const Geom& g, int cls) {
 // grid (row tiles, column tiles, slices).  With several slices `out` is a float buffer [slices][rows][cols].
 template <int KIND, typename TIN, typename TO, int BM, int BN, int V>
 __global__ void __launch_bounds__(SG_THREADS) simt_gemm_kernel(const TIN* __restrict__ asrc, const TIN* __restrict__ bsrc, TO* __restrict__ out, const SgArgs p) {
-    pdl_launch_dependents();
+    if (KIND != 1) pdl_launch_dependents();
     using T = SgTile<KIND, BM, BN>;
     constexpr int TM = T::TM, NTX = T::NTX, NTY = T::NTY;
     extern __shared__ __align__(16) uint8_t sg_smem[];
@@ -290,7 +291,8 @@ __global__ void __launch_bounds__(SG_THREADS) simt_gemm_kernel(const TIN* __rest
 #pragma unroll
         for (int e = 0; e < TM * 4; ++e) flushed[e * SG_THREADS + tid] = 0.0;
     }
-    pdl_wait();
+    if (KIND != 2 || !p.overlap) pdl_wait();
+    if (KIND == 1) pdl_launch_dependents();  // (behind its own wait: see the end of common.cuh)
 #pragma unroll
     for (int s = 0; s < SG_STAGES - 1; ++s) {
         if (s < nsteps) load_stage(s);
@@ -401,6 +403,7 @@ __global__ void __launch_bounds__(SG_THREADS) simt_gemm_kernel(const TIN* __rest
             chan_acc_add(p.acc, g.c_out, which, j0 + c, sum);
         }
     }
+    if (KIND == 2 && p.overlap) pdl_wait();
 }
 
 // out = sum over the slices of a split forward convolution (fp64, slice order), rounded to YT, and with acc.acc != NULL the
@@ -446,10 +449,12 @@ __global__ void __launch_bounds__(256) splitk_fwd_reduce_kernel(const float* __r
 // out[e] = sum_z partial[z][e], summed in fp64 in slice order (four elements per thread when the count allows).
 // Eight slices are loaded before any is added so that a thread keeps eight independent 16-byte loads in flight:
 // the kernel is tiny and otherwise bound by one memory latency per slice.
-template <typename TO>
+// LATE: the last launch of a data gradient (it signals its dependents behind its own wait: see the end of common.cuh).
+template <typename TO, bool LATE = false>
 __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restrict__ partial, int splits, size_t elems, TO* __restrict__ out) {
-    pdl_launch_dependents();
+    if (!LATE) pdl_launch_dependents();
     pdl_wait();
+    if (LATE) pdl_launch_dependents();
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     if ((elems & 3) == 0) {
         const size_t nv = elems >> 2;

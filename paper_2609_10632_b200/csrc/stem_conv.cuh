@@ -375,8 +375,8 @@ inline int stem_dgrad_grid(const Geom& g, int slots, int* seg_rows) {
 }
 template <int COUT, typename T = __nv_bfloat16>
 __global__ void __launch_bounds__(128, stem_dgrad_occ(COUT)) stem_dgrad_mma_kernel(const T* __restrict__ dy, const T* __restrict__ w, T* __restrict__ dx, Geom g, int seg_rows) {
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();  // (behind its own wait: see the end of common.cuh)
     static_assert(COUT % 16 == 0, "whole k-steps");
     constexpr int STEM_DYPITCH = COUT + 8;  // elements per staged dy pixel: rows of 16 x odd bytes, conflict-free for ldmatrix
     constexpr int KS = COUT / 16;
@@ -516,9 +516,9 @@ template <int COUT, typename T, int TQ> constexpr size_t stem_wgrad_smem_bytes()
     return sizeof(StemWgradRing<COUT, T, TQ>) > 4 * sizeof(float[COUT][33]) ? sizeof(StemWgradRing<COUT, T, TQ>) : 4 * sizeof(float[COUT][33]);
 }
 template <int COUT, typename T = __nv_bfloat16, int TQ = STEM_TQ>
-__global__ void __launch_bounds__(128, stem_occ(COUT)) stem_wgrad_mma_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ partial, Geom g) {
+__global__ void __launch_bounds__(128, stem_occ(COUT)) stem_wgrad_mma_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ partial, Geom g, int overlap) {
     pdl_launch_dependents();
-    pdl_wait();
+    if (!overlap) pdl_wait();
     static_assert(COUT % 16 == 0, "whole m-blocks");
     static_assert(TQ % 64 == 0, "whole 16-pixel tiles for each of the four warps");
     constexpr int MB = COUT / 16, NBK = 4;  // accumulator blocks: MB x 16 channels by NBK x 8 filter positions (27 padded to 32)
@@ -648,6 +648,7 @@ __global__ void __launch_bounds__(128, stem_occ(COUT)) stem_wgrad_mma_kernel(con
         const int c = e / STEM_KDIM, k = e - c * STEM_KDIM;
         o[e] = ((red[0][c][k] + red[1][c][k]) + red[2][c][k]) + red[3][c][k];
     }
+    if (overlap) pdl_wait();
 }
 
 }  // namespace nbcbs

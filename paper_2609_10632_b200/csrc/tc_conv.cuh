@@ -304,8 +304,9 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    // the next kernel of the stream may become resident and run its prologue right away
-    pdl_launch_dependents();
+    // the next kernel of the stream may become resident and run its prologue right away (behind a data gradient: once this
+    // kernel's own wait is over, see WgradOverlap)
+    if (STATS || EPI) pdl_launch_dependents();
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // warp index in a form the compiler knows to be uniform
     const int total_tiles = p.nclasses * p.tiles_per_class;
     const int mh = p.mh;          // 128-row sub-tiles per tile (1 or 2); both share every B stage
@@ -389,6 +390,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
         const uint32_t base_u32 = ptx::smem_u32(isA ? sA : sB);
         const uint32_t full_u32 = CG2 ? ptx::mapa_u32(ptx::smem_u32(full), 0u) : ptx::smem_u32(full);
         pdl_wait();
+        if (!STATS && !EPI && isA) pdl_launch_dependents();
         for (int tile = worker; ok && tile < total_tiles; tile += nworkers) {
             int cls, lt;
             igemm_tile_class<CLS4>(p, tile, nworkers, cls, lt);
@@ -1555,7 +1557,8 @@ inline nb_status tc_dgrad(TcPlan* tc, const Geom& g, const void* dy, const void*
     return NB_OK;
 }
 
-inline nb_status tc_wgrad(TcPlan* tc, const Geom& g, const void* x, const void* dy, float* dw, float* partial, int* status, cudaStream_t st) {
+// `overlap`: the previous launch on the stream is this layer's data gradient (see the end of common.cuh).
+inline nb_status tc_wgrad(TcPlan* tc, const Geom& g, const void* x, const void* dy, float* dw, float* partial, int* status, cudaStream_t st, bool overlap) {
     using namespace tcdetail;
     if (tc->wgrad_rows) {
         WgradRowsParams& R = tc->wr;
@@ -1566,6 +1569,7 @@ inline nb_status tc_wgrad(TcPlan* tc, const Geom& g, const void* x, const void* 
         }
         R.out = R.splits > 1 ? partial : dw;
         R.status = status;
+        R.overlap = overlap ? 1 : 0;
         static std::atomic<unsigned long long> rows_attr_set{0};  // one bit per device ordinal (see launch_igemm_impl)
         int dev = 0;
         cudaGetDevice(&dev);
@@ -1604,6 +1608,7 @@ inline nb_status tc_wgrad(TcPlan* tc, const Geom& g, const void* x, const void* 
     }
     P.out = P.splits > 1 ? partial : dw;
     P.status = status;
+    P.overlap = overlap ? 1 : 0;
     static std::atomic<unsigned long long> attr_set{0};  // one bit per device ordinal (see launch_igemm_impl)
     int dev = 0;
     cudaGetDevice(&dev);

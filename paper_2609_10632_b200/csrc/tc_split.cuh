@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    pdl_launch_dependents();
+    if (MODE != 0) pdl_launch_dependents();
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int rank = (int)blockIdx.x % S, tile = (int)blockIdx.x / S;
     const int cls = tile / p.tiles_per_class, lt = tile - cls * p.tiles_per_class;
@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
         uint32_t ph = 0;
         bool ok = true;
         pdl_wait();
+        if (MODE == 0 && isA) pdl_launch_dependents();  // (behind its own wait: see the end of common.cuh)
         for (int kb = kb0; kb < kb1; ++kb) {
             if (!wait_bar_fast(empty + s, ph ^ 1u, abort_flag, p.status, isA ? 1 : 5)) {
                 ok = false;

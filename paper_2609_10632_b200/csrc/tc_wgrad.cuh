@@ -28,6 +28,7 @@ struct WgradParams {
     uint32_t a_stage_bytes, b_stage_bytes, blk_bytes, idesc;
     float* out;  // [splits][c_out][kdim] (or dw itself when splits == 1)
     int* status;
+    int overlap;  // runs beside the data gradient in front of it (see the end of common.cuh)
     uint16_t off_w[9], off_h[9];
 };
 
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();  // everything above touched only shared memory, TMEM and kernel parameters
+    if (!p.overlap) pdl_wait();  // everything above touched only shared memory, TMEM and kernel parameters
 
     if (warp == 0 || warp == 6) {
         // ------------------------------------------------------------------ TMA producers: warp 0 feeds x, warp 6 feeds dy
@@ -228,6 +229,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
             }
         }
     }
+    if (p.overlap) pdl_wait();
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -262,6 +264,7 @@ struct WgradRowsParams {
     uint32_t a_box_bytes, b_box_bytes, a_stage_bytes, b_stage_bytes, idesc;
     float* out;
     int* status;
+    int overlap;  // see WgradParams
 };
 
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_rows_kernel(const __grid_constant__ WgradRowsParams p) {
@@ -309,7 +312,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_rows_kernel(const __gr
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();  // everything above touched only shared memory, TMEM and kernel parameters
+    if (!p.overlap) pdl_wait();  // everything above touched only shared memory, TMEM and kernel parameters
 
     if (warp == 0 || warp == 6) {
         // ------------------------------------------------------------------ TMA producers: warp 0 feeds x, warp 6 feeds dy
@@ -455,6 +458,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_rows_kernel(const __gr
             }
         }
     }
+    if (p.overlap) pdl_wait();
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 1) {
