@@ -307,7 +307,10 @@ template <int V> __device__ __forceinline__ void load_params_shared(const float*
 // RES: a = SiLU(...) + res with res a (possibly pitched) tensor of the output's type -- the residual connection of a
 // bottleneck performed by the block that feeds it; the sum is formed in fp32 and rounded once.
 // FIN: scale and shift are derived here from the totals in `ca` (dynamic shared memory: 2*C floats); else they are read.
-template <typename YT, typename AT, bool FAST, bool ACT = true, bool PITCHED = false, bool RES = false, bool FIN = false>
+// ONE (with FIN): the grid has a thread for every vector.  The thread asks for its vector before the coefficients are
+// derived, so that the two memory latencies of a small tensor's pass overlap (with more vectors per thread the registers
+// that stay live across the fp64 arithmetic cost more than that).
+template <typename YT, typename AT, bool FAST, bool ACT = true, bool PITCHED = false, bool RES = false, bool FIN = false, bool ONE = false>
 __global__ void __launch_bounds__(288, 3) bn_silu_apply_kernel(const YT* __restrict__ y, AT* __restrict__ a,
                                                              long long total_vecs, int C, const float* __restrict__ scale,
                                                              const float* __restrict__ shift, long long ld_a, const AT* __restrict__ res, long long ld_r,
@@ -321,6 +324,15 @@ __global__ void __launch_bounds__(288, 3) bn_silu_apply_kernel(const YT* __restr
     extern __shared__ __align__(16) float s_coef[];
     __shared__ int s_last;
     int readers_before = 0;
+    Vec16<YT> q1;
+    Vec16<AT> r1;
+    if (ONE) {
+        const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (v < total_vecs) {
+            q1 = ld16(y + v * V);
+            if (RES) r1 = ld16(res + (v / (C / V)) * ld_r + (long long)cg * V);
+        }
+    }
     if (FIN) {
         fwd_coef_from_acc(ca, fin, C, s_coef);
         __syncthreads();
@@ -341,10 +353,10 @@ __global__ void __launch_bounds__(288, 3) bn_silu_apply_kernel(const YT* __restr
     long long orr = RES ? (v0 / cgs) * ld_r + (long long)cg * V : 0;
     const long long or_step = RES ? (stride / cgs) * ld_r : 0;
     for (long long v = v0; v < total_vecs; v += stride, oa += oa_step, orr += or_step) {
-        if (v + 2 * stride < total_vecs) asm volatile("prefetch.global.L2 [%0];" ::"l"(y + (v + 2 * stride) * V));  // see the reduce kernel
-        const Vec16<YT> q = ld16(y + v * V);
+        if (!ONE && v + 2 * stride < total_vecs) asm volatile("prefetch.global.L2 [%0];" ::"l"(y + (v + 2 * stride) * V));  // see the reduce kernel
+        const Vec16<YT> q = ONE ? q1 : ld16(y + v * V);
         Vec16<AT> o, r;
-        if (RES) r = ld16(res + orr);
+        if (RES) r = ONE ? r1 : ld16(res + orr);
 #pragma unroll
         for (int j = 0; j < V / 2; ++j) {
             const float2 z = fma2(pair_to_f32(q.v + 2 * j), sc[j], sh[j]);
@@ -353,6 +365,7 @@ __global__ void __launch_bounds__(288, 3) bn_silu_apply_kernel(const YT* __restr
             pair_from_f32(o.v + 2 * j, out);
         }
         st16(a + oa, o);
+        if (ONE) break;
     }
     if (FIN) {
         if (threadIdx.x == 0) s_last = readers_before == (int)gridDim.x - 1;
@@ -442,9 +455,9 @@ struct BwdFused {
     __nv_bfloat16* wt;
 };
 // `row_blocks` blocks walk the tensor (the sums are grouped by them); blocks past those only rearrange filter tiles.
-// DEEP: for small tensors, whose threads have a few vectors each and whose blocks do not fill the device: four vectors of
-// each tensor are on their way before the first is used (a small tensor's pass is one memory latency per step of this
-// loop), with the registers that take; the additions and their order are the same.
+// DEEP: for small tensors, whose threads have at most eight vectors each and whose blocks do not fill the device: all of them
+// are on their way before the parameters are used (a small tensor's pass is one memory latency per step of this loop), with
+// the registers that takes; the additions and their order are the same.
 template <typename YT, typename AT, bool FAST, bool PITCHED = false, bool DEEP = false>
 __global__ void __launch_bounds__(288, DEEP ? 1 : 3) bn_silu_bwd_reduce_kernel(const AT* __restrict__ g, const YT* __restrict__ y,
                                                                   long long total_vecs, int C, const float* __restrict__ mean,
@@ -470,6 +483,23 @@ __global__ void __launch_bounds__(288, DEEP ? 1 : 3) bn_silu_bwd_reduce_kernel(c
             if (t < wt_tiles) wt_tile_load_async(fb.w, wtp, wt_tile_decode(wtp, t), wtile[k]);
         }
     }
+    const bool has_rows = (int)blockIdx.x < row_blocks;
+    const long long stride = (long long)row_blocks * blockDim.x;
+    // g may be a channel slice of a wider tensor (row pitch ld_g elements); the stride is a whole number of rows
+    const long long v0 = (long long)blockIdx.x * blockDim.x + tid;
+    long long og = PITCHED ? (v0 / cgs) * ld_g + (long long)cg * V : v0 * V;  // (dense: the flat offset)
+    const long long og_step = PITCHED ? (stride / cgs) * ld_g : stride * V;
+    constexpr int D = DEEP ? 8 : 1;
+    Vec16<YT> qyd[D];
+    Vec16<AT> qgd[D];
+    if (DEEP && has_rows) {
+#pragma unroll
+        for (int u = 0; u < D; ++u)
+            if (v0 + u * stride < total_vecs) {
+                qyd[u] = ld16(y + (v0 + u * stride) * V);
+                qgd[u] = ld16(g + og + u * og_step);
+            }
+    }
     float2 a[V / 2], b[V / 2], sb[V / 2], sy[V / 2];
     {
         float mu[V], is[V], ga[V], be[V];
@@ -484,12 +514,6 @@ __global__ void __launch_bounds__(288, DEEP ? 1 : 3) bn_silu_bwd_reduce_kernel(c
             sb[j] = sy[j] = splat2(0.f);
         }
     }
-    const bool has_rows = (int)blockIdx.x < row_blocks;
-    const long long stride = (long long)row_blocks * blockDim.x;
-    // g may be a channel slice of a wider tensor (row pitch ld_g elements); the stride is a whole number of rows
-    const long long v0 = (long long)blockIdx.x * blockDim.x + tid;
-    long long og = PITCHED ? (v0 / cgs) * ld_g + (long long)cg * V : v0 * V;  // (dense: the flat offset)
-    const long long og_step = PITCHED ? (stride / cgs) * ld_g : stride * V;
     auto add_vec = [&](const Vec16<YT>& qy, const Vec16<AT>& qg) {
 #pragma unroll
         for (int j = 0; j < V / 2; ++j) {
@@ -500,18 +524,10 @@ __global__ void __launch_bounds__(288, DEEP ? 1 : 3) bn_silu_bwd_reduce_kernel(c
         }
     };
     if (DEEP) {
-        for (long long v = v0; has_rows && v < total_vecs; v += 4 * stride, og += 4 * og_step) {
-            Vec16<YT> qy[4];
-            Vec16<AT> qg[4];
+        if (has_rows) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (v + u * stride < total_vecs) {
-                    qy[u] = ld16(y + (v + u * stride) * V);
-                    qg[u] = ld16(g + og + u * og_step);
-                }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (v + u * stride < total_vecs) add_vec(qy[u], qg[u]);
+            for (int u = 0; u < D; ++u)
+                if (v0 + u * stride < total_vecs) add_vec(qyd[u], qgd[u]);
         }
     } else {
         for (long long v = v0; has_rows && v < total_vecs; v += stride, og += og_step) {
@@ -527,19 +543,22 @@ __global__ void __launch_bounds__(288, DEEP ? 1 : 3) bn_silu_bwd_reduce_kernel(c
         }
     }
     const int R = blockDim.x / cgs;
-    for (int pass = 0; pass < 2 && has_rows; ++pass) {
+    if (has_rows) {  // both sums of every channel at once: red holds [2][blockDim.x][V]
+        float* const red1 = red + (size_t)blockDim.x * V;
 #pragma unroll
-        for (int j = 0; j < V / 2; ++j) *reinterpret_cast<float2*>(&red[tid * V + 2 * j]) = pass ? sy[j] : sb[j];
+        for (int j = 0; j < V / 2; ++j) {
+            *reinterpret_cast<float2*>(&red[tid * V + 2 * j]) = sb[j];
+            *reinterpret_cast<float2*>(&red1[tid * V + 2 * j]) = sy[j];
+        }
         __syncthreads();
-        for (int c = tid; c < C; c += blockDim.x) {
-            const int gq = c / V, e = c % V;
+        for (int e = tid; e < 2 * C; e += blockDim.x) {
+            const int pass = e >= C ? 1 : 0, c = e - pass * C;  // pass 0: sum dz, pass 1: sum dz*y
+            const float* const src = (pass ? red1 : red) + c;  // element c of row r: ((r * cgs + c / V) * V + c % V) = r * C + c
             float acc = 0.f;
-            for (int r = 0; r < R; ++r) acc += red[(r * cgs + gq) * V + e];
-            // pass 0: sum dz, pass 1: sum dz*y
+            for (int r = 0; r < R; ++r) acc += src[r * C];
             if (fb.acc.acc) chan_acc_add(fb.acc, C, pass, c, acc);
             else partials[((size_t)blockIdx.x * 2 + pass) * C + c] = acc;
         }
-        __syncthreads();
     }
     if (wt_tiles > 0) {
         wt_async_wait();
@@ -610,7 +629,8 @@ __device__ __forceinline__ void bwd_coef_from_acc(const ChanAcc& ca, const BwdFi
 // GRES: the incoming gradient g is also the gradient of a residual connection's shortcut: the pass adds it to (or, with
 // gres_add = 0, copies it into) `gres`, a tensor of g's shape with pixels ld_gres elements apart -- the backward
 // counterpart of the RES form of the normalise + SiLU pass (fp32 sum, rounded once, like a separate accumulation pass).
-template <typename YT, typename AT, bool FAST, bool PITCHED = false, bool FIN = false, bool GRES = false>
+// ONE (with FIN): a thread for every vector, asked for before the coefficients are derived (see the normalise + SiLU pass).
+template <typename YT, typename AT, bool FAST, bool PITCHED = false, bool FIN = false, bool GRES = false, bool ONE = false>
 __global__ void __launch_bounds__(288, 3) bn_silu_bwd_dy_kernel(const AT* __restrict__ g, const YT* __restrict__ y,
                                                               AT* __restrict__ dy, long long total_vecs, int C,
                                                               const float* __restrict__ coef, long long ld_g, ChanAcc ca, BwdFin fin,
@@ -623,6 +643,15 @@ __global__ void __launch_bounds__(288, 3) bn_silu_bwd_dy_kernel(const AT* __rest
     extern __shared__ __align__(16) float s_coef[];
     __shared__ int s_last;
     int readers_before = 0;
+    Vec16<YT> qy1;
+    Vec16<AT> qg1;
+    if (ONE) {
+        const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (v < total_vecs) {
+            qy1 = ld16(y + v * V);
+            qg1 = ld16(g + (PITCHED ? (v / (C / V)) * ld_g + (long long)cg * V : v * V));
+        }
+    }
     if (FIN) {
         bwd_coef_from_acc(ca, fin, C, s_coef);
         __syncthreads();
@@ -647,12 +676,12 @@ __global__ void __launch_bounds__(288, 3) bn_silu_bwd_dy_kernel(const AT* __rest
     long long ogr = GRES ? (v0 / cgs) * ld_gres + (long long)cg * V : 0;
     const long long ogr_step = GRES ? (stride / cgs) * ld_gres : 0;
     for (long long v = v0; v < total_vecs; v += stride, og += og_step, ogr += ogr_step) {
-        if (v + 2 * stride < total_vecs) {  // L2 prefetch two iterations ahead (see the reduce kernel)
+        if (!ONE && v + 2 * stride < total_vecs) {  // L2 prefetch two iterations ahead (see the reduce kernel)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(y + (v + 2 * stride) * V));
             asm volatile("prefetch.global.L2 [%0];" ::"l"(g + og + 2 * og_step));
         }
-        const Vec16<YT> qy = ld16(y + v * V);
-        const Vec16<AT> qg = ld16(g + og);
+        const Vec16<YT> qy = ONE ? qy1 : ld16(y + v * V);
+        const Vec16<AT> qg = ONE ? qg1 : ld16(g + og);
         if (GRES) {
             Vec16<AT> r = qg;
             if (gres_add) {
@@ -670,6 +699,7 @@ __global__ void __launch_bounds__(288, 3) bn_silu_bwd_dy_kernel(const AT* __rest
             pair_from_f32(o.v + 2 * j, fma2(a[j], dz, fma2(np1[j], yv, p0[j])));
         }
         st16(dy + v * V, o);
+        if (ONE) break;
     }
     if (FIN) {
         if (threadIdx.x == 0) s_last = readers_before == (int)gridDim.x - 1;

@@ -222,9 +222,10 @@ nb_status run_apply(nb_cbs_plan_s* p, const void* y, void* a, const float* scale
         if (fin) {
             const ChanAcc ca{p->acc, p->status + ST_READERS_FWD, p->acc_copies_f};
             const size_t smem = (size_t)2 * C * sizeof(float);
-            if (res) go(bn_silu_apply_kernel<YT, AT, FAST, true, true, true, true>, ca, *fin, smem);
-            else if (ld_a) go(bn_silu_apply_kernel<YT, AT, FAST, true, true, false, true>, ca, *fin, smem);
-            else go(bn_silu_apply_kernel<YT, AT, FAST, true, false, false, true>, ca, *fin, smem);
+            const bool one = (long long)e.blocks_apply * e.tpb >= e.total_vecs;
+            if (res) one ? go(bn_silu_apply_kernel<YT, AT, FAST, true, true, true, true, true>, ca, *fin, smem) : go(bn_silu_apply_kernel<YT, AT, FAST, true, true, true, true>, ca, *fin, smem);
+            else if (ld_a) one ? go(bn_silu_apply_kernel<YT, AT, FAST, true, true, false, true, true>, ca, *fin, smem) : go(bn_silu_apply_kernel<YT, AT, FAST, true, true, false, true>, ca, *fin, smem);
+            else one ? go(bn_silu_apply_kernel<YT, AT, FAST, true, false, false, true, true>, ca, *fin, smem) : go(bn_silu_apply_kernel<YT, AT, FAST, true, false, false, true>, ca, *fin, smem);
             return launch_ok("bn_silu_apply (statistics from the accumulators)");
         }
         if (res) {
@@ -256,7 +257,7 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
         if (fuse) {
             fb.w = static_cast<const __nv_bfloat16*>(w); fb.wt = wtp ? static_cast<__nv_bfloat16*>(wt) : nullptr;
         }
-        const size_t red_smem = (size_t)e.tpb * e.vec * sizeof(float);
+        const size_t red_smem = (size_t)2 * e.tpb * e.vec * sizeof(float);
         // A small activation needs few blocks, a large filter many: every block takes two filter tiles, blocks without
         // rows of their own take nothing else (288 -> 288 3x3 on one 20 x 20 image has 405 tiles and 8 blocks of rows:
         // 61 us when those 8 rearranged the filter alone).
@@ -290,12 +291,13 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
                  p->ld_g ? p->ld_g : (long long)C, ca, bf, static_cast<AT*>(p->bwd_gres), p->ld_gres ? p->ld_gres : (long long)C, p->gres_add ? 1 : 0);
     };
     const size_t coef_smem = (size_t)4 * C * sizeof(float);
+    const bool one = (long long)e.blocks_dy * e.tpb >= e.total_vecs;
     if (fuse && p->bwd_gres) {  // (the setter admits this only on plans that take this path)
-        if (p->ld_g) go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true, true>, coef_smem);
-        else go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true, true>, coef_smem);
+        if (p->ld_g) one ? go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true, true, true>, coef_smem) : go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true, true>, coef_smem);
+        else one ? go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true, true, true>, coef_smem) : go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true, true>, coef_smem);
     } else if (fuse) {
-        if (p->ld_g) go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true>, coef_smem);
-        else go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true>, coef_smem);
+        if (p->ld_g) one ? go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true, false, true>, coef_smem) : go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true>, coef_smem);
+        else one ? go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true, false, true>, coef_smem) : go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true>, coef_smem);
     } else {
         if (p->ld_g) go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, false>, 0);
         else go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, false>, 0);
@@ -556,17 +558,17 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
         const size_t apply_smem = p->fuse_finalize ? (size_t)2 * g.c_out * sizeof(float) : 0, dy_smem = p->fuse_finalize ? (size_t)4 * g.c_out * sizeof(float) : 0;
         if (d->mode == NB_MODE_F32_REF) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<float>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, red_smem, 8, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, 2 * red_smem, 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<float, float, false, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<float, float, false, false, true>, dy_smem, 1);
         } else if (d->mode == NB_MODE_F16_TC) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, red_smem, 8, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, 2 * red_smem, 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __half, true, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __half, true, false, true>, dy_smem, 1);
         } else {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, red_smem, 8, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, 2 * red_smem, 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __nv_bfloat16, true, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __nv_bfloat16, true, false, true>, dy_smem, 1);
         }
