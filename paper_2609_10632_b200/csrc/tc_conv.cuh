@@ -1392,8 +1392,12 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
         tc->wgrad_partial_bytes = P.splits > 1 ? (size_t)P.splits * g.c_out * g.kdim * 4 : 0;
         tc->wgrad = true;
         // the row-tile form: 3x3, stride 1, pad 1, image width a multiple of 16 (a stage is one output row: whole K = 16 steps)
-        // (layers with more than 128 output columns per tile are not bound by x traffic in the other kernel: measured equal)
-        const bool rows_wanted = getenv("NB_WG_ROWS") ? atoi(getenv("NB_WG_ROWS")) != 0 : P.acc_stride <= 128;
+        // (layers with more than 128 output columns per tile are not bound by x traffic in the other kernel: measured equal; nor
+        // are those with three channel blocks: 192 -> 64 at 16 x 80 x 80, 39 us by rows, 35 us; and a layer that the other
+        // kernel does in fewer than 50 stage units -- about 25 us -- is better off there, because the row form needs one long
+        // stage per image row and a slice per SM: 64 -> 64 at 80 x 80 14 us by rows, 7.4 us; at 4 x 80 x 80 20 and 11 us; 96 -> 96
+        // at 16 x 80 x 80, 55 units, 31.6 and 33.2; at 16 x 160 x 160, 187 units, 80 and 105)
+        const bool rows_wanted = getenv("NB_WG_ROWS") ? atoi(getenv("NB_WG_ROWS")) != 0 : P.acc_stride <= 128 && g.c_in <= 128 && best_cost >= 50.0;
         if (g.k == 3 && g.stride == 1 && g.pad == 1 && g.w % 16 == 0 && g.w + 2 <= 256 && g.wo == g.w && g.ho == g.h && rows_wanted) {
             WgradRowsParams& R = tc->wr;
             memset(&R, 0, sizeof R);
