@@ -360,12 +360,14 @@ template <typename AT> cudaError_t stem_allow_smem(int c_out) {
 }
 
 // ---------------------------------------------------------------- CUDA-core convolutions
-// Tile and slices.  64 x 64 where such tiles give every SM two blocks, else 32 x 64; 64 x 32 for at most 32 columns and for
-// the 16-bit fallback.  One block alone on an SM waits for its ring (0.5 us per 16-k stage, half of it latency), so where
-// the tiles give an SM fewer than two blocks the k range is cut into slices of at least eight stages, at most four blocks
-// per SM (one more than fits a wave is worse than one fewer); that costs a reduce launch and the slices' trip through L2
-// (3 to 4 us), hence not below 16 stages.
-// Measured (step): 64 -> 64 3x3 at 2 x 40 x 40, one slice 75 us, five slices 59 us; 16 -> 32 at 2 x 32 x 32, 46 -> 39 us.
+// Tile and slices.  64 x 64; 32 x 64 where even eight-stage slices of such tiles would leave an SM fewer than two blocks;
+// 64 x 32 for at most 32 columns and for the 16-bit fallback.  One block
+// alone on an SM waits for its ring (0.5 us per 16-k stage, half of it latency), so where an SM has two tiles or fewer the k
+// range is cut into slices of at least eight stages until it has up to six blocks (one more than fits a wave is worse than one fewer), and into slices
+// of at most 1024 products where the slices fit 128 MB: such a slice needs no fp64 flush, whose shared memory leaves three
+// blocks per SM, and evens out the last wave.  Slices cost a reduce launch and a trip through L2 (3 to 4 us), hence not
+// below 16 stages.  Measured (step): 64 -> 64 3x3 at 2 x 40 x 40, one slice 75 us, five slices 59 us; 288 -> 288 3x3 at
+// 4 x 20 x 20, 348 -> 262 us against at most four blocks per SM; 272 -> 304 stride 2 on 7 x 44 x 84, 1265 -> 982 us.
 SgCfg sg_configure(const Geom& g, int kind, bool f32, int sm_count) {
     SgCfg c{};
     const int cols = kind == 0 ? g.c_out : kind == 1 ? g.c_in : g.kdim;
@@ -379,14 +381,20 @@ SgCfg sg_configure(const Geom& g, int kind, bool f32, int sm_count) {
         return t;
     };
     const long long col_tiles = (cols + c.bn - 1) / c.bn;
-    c.bm = c.bn == 64 && row_tiles(64) * col_tiles < 2 * sm_count ? 32 : 64;
+    const size_t out = kind == 0 ? (size_t)g.m * g.c_out : kind == 1 ? (size_t)g.n * g.h * g.w * g.c_in : (size_t)g.c_out * g.kdim;
+    const long long most = std::max<long long>(1, KK / (8 * SG_BK));
+    c.bm = 64;
+    if (c.bn == 64 && row_tiles(64) * col_tiles * most < 2 * sm_count) c.bm = 32;
     const long long tiles = row_tiles(c.bm) * col_tiles;
     long long splits = 1;
-    if (tiles <= 2 * sm_count && KK >= 16 * SG_BK) splits = std::max<long long>(1, std::min<long long>(4LL * sm_count / tiles, KK / (8 * SG_BK)));
+    if (KK >= 16 * SG_BK) {
+        if (tiles <= 2 * sm_count) splits = std::max<long long>(1, std::min<long long>(6LL * sm_count / tiles, most));
+        const long long flush_free = (KK + 1023) / 1024;
+        if (splits < flush_free && (size_t)flush_free * out * 4 <= (size_t)128 << 20) splits = flush_free;
+    }
     c.kchunk = ((KK + splits - 1) / splits + SG_BK - 1) / SG_BK * SG_BK;
     c.splits = (int)((KK + c.kchunk - 1) / c.kchunk);
     c.grid = dim3((unsigned)row_tiles(c.bm), (unsigned)col_tiles, (unsigned)c.splits);
-    const size_t out = kind == 0 ? (size_t)g.m * g.c_out : kind == 1 ? (size_t)g.n * g.h * g.w * g.c_in : (size_t)g.c_out * g.kdim;
     c.partial_bytes = c.splits > 1 ? (size_t)c.splits * out * 4 : 0;
     return c;
 }

@@ -180,6 +180,16 @@ __global__ void __launch_bounds__(SG_THREADS) simt_gemm_kernel(const TIN* __rest
             b_t[e] = tap - b_r[e] * g.k;
         }
     }
+    int f_co[KIND == 1 ? BP : 1], f_r[KIND == 1 ? BP : 1], f_t[KIND == 1 ? BP : 1];  // channel and tap of each k row of the filter tile (data gradient)
+    if (KIND == 1) {
+#pragma unroll
+        for (int i = 0; i < BP; ++i) {
+            const int kk = (int)kbeg + b_kr + i * B_KSTEP, tap = kk / kch;
+            f_co[i] = kk - tap * kch;
+            f_r[i] = tap / ntd;
+            f_t[i] = tap - f_r[i] * ntd;
+        }
+    }
     long long kload = kbeg;  // first k of the next stage to load
     auto load_stage = [&](int s) {
         TIN* const a_s = sA + s * T::A_ELEMS;
@@ -226,8 +236,15 @@ __global__ void __launch_bounds__(SG_THREADS) simt_gemm_kernel(const TIN* __rest
                 for (int i = 0; i < BP; ++i) {
                     const int kr = b_kr + i * B_KSTEP;
                     const long long kk = kload + kr;
-                    const int tap = (int)kk / kch, co = (int)kk - tap * kch, ri = tap / ntd, ti = tap - ri * ntd;
-                    const TIN* src = bsrc + ((long long)co * g.k * g.k + (r_first + ri * r_step) * g.k + t_first + ti * r_step) * g.c_in + j0 + b_nv;
+                    const TIN* src = bsrc + ((long long)f_co[i] * g.k * g.k + (r_first + f_r[i] * r_step) * g.k + t_first + f_t[i] * r_step) * g.c_in + j0 + b_nv;
+                    f_co[i] += SG_BK;
+                    while (f_co[i] >= kch) {
+                        f_co[i] -= kch;
+                        if (++f_t[i] == ntd) {
+                            f_t[i] = 0;
+                            ++f_r[i];
+                        }
+                    }
                     if (V == 4) {
                         const bool ok = kk < kend && j0 + b_nv < cols;
                         sg_copy4(b_s + kr * (BN + 4) + b_nv, ok ? src : bsrc, ok);
