@@ -257,7 +257,8 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
         if (fuse) {
             fb.w = static_cast<const __nv_bfloat16*>(w); fb.wt = wtp ? static_cast<__nv_bfloat16*>(wt) : nullptr;
         }
-        const size_t red_smem = (size_t)2 * e.tpb * e.vec * sizeof(float);
+        const bool deep = 2 * e.blocks_reduce <= p->sm_count;  // at most every second SM has rows
+        const size_t red_smem = std::max((size_t)2 * e.tpb * e.vec * sizeof(float), deep ? (size_t)0 : (size_t)EW_RING * 2 * e.tpb * 16);
         // A small activation needs few blocks, a large filter many: every block takes two filter tiles, blocks without
         // rows of their own take nothing else (288 -> 288 3x3 on one 20 x 20 image has 405 tiles and 8 blocks of rows:
         // 61 us when those 8 rearranged the filter alone).
@@ -267,7 +268,6 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
             launch_k(kernel, dim3(blocks), dim3(e.tpb), red_smem, st, 1, static_cast<const AT*>(g), static_cast<const YT*>(y), e.total_vecs, C, mean, invstd,
                      gamma, beta, partials, fb, wtp ? *wtp : none, ld, e.blocks_reduce);
         };
-        const bool deep = 2 * e.blocks_reduce <= p->sm_count;  // at most every second SM has rows
         if (p->ld_g) deep ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true, true>, p->ld_g) : go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true>, p->ld_g);
         else deep ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false, true>, (long long)C) : go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false>, (long long)C);
         NB_LAUNCH_OK("bn_silu_bwd_reduce");
@@ -566,17 +566,17 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
         const size_t apply_smem = p->fuse_finalize ? (size_t)2 * g.c_out * sizeof(float) : 0, dy_smem = p->fuse_finalize ? (size_t)4 * g.c_out * sizeof(float) : 0;
         if (d->mode == NB_MODE_F32_REF) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<float>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, 2 * red_smem, 8, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, std::max(2 * red_smem, (size_t)EW_RING * 2 * e.tpb * 16), 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<float, float, false, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<float, float, false, false, true>, dy_smem, 1);
         } else if (d->mode == NB_MODE_F16_TC) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, 2 * red_smem, 8, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, std::max(2 * red_smem, (size_t)EW_RING * 2 * e.tpb * 16), 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __half, true, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __half, true, false, true>, dy_smem, 1);
         } else {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, 2 * red_smem, 8, &e.wave_reduce);
+            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, std::max(2 * red_smem, (size_t)EW_RING * 2 * e.tpb * 16), 8, &e.wave_reduce);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __nv_bfloat16, true, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __nv_bfloat16, true, false, true>, dy_smem, 1);
         }
