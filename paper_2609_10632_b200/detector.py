@@ -8,7 +8,7 @@ A pass is some 200 to 400 kernel launches whose arguments do not change from ste
 each, plus 2 us for every call's way through Python) takes longer than a small batch takes on the GPU.  From the second pass
 with unchanged arguments on, forward() and backward() therefore replay a CUDA graph recorded from the same calls.  Measured,
 one training iteration at batch 2, 320 x 320: 2.94 ms issued one by one, of which the host alone needs 2.81 ms, and 2.57 ms
-as graphs; at batch 16, 640 x 640: 9.94 and 9.66 ms.
+as graphs; at batch 16, 640 x 640: 9.94 and 9.66 ms.  The recording has the dataflow's branches (_Lanes): 2.29 and 9.31 ms.
 
 Every named tensor is an NHWC bf16 tensor, dense or -- with views=True -- a CHANNEL SLICE of a wider buffer (a torch
 view: data_ptr() is the slice's first channel, stride(-2) its row pitch), which the block calls accept through
@@ -38,6 +38,11 @@ _PITCH_IN = ("slice", "add", "concat", "upsample", "maxpool")  # glue ops that r
 _FORWARD_TENSORS = attrgetter("x", "w", "gamma", "beta", "running_mean", "running_var", "y", "mean", "invstd", "a", "ws")
 _BACKWARD_TENSORS = attrgetter("g", "y", "mean", "invstd", "gamma", "beta", "w", "dx", "dgamma", "dbeta", "dy", "ws", "x", "dw")
 
+# what the calls of a block read and what they write (its tensors, its workspace, its plan)
+_FORWARD_READS, _FORWARD_WRITES = attrgetter("x", "w", "gamma", "beta"), attrgetter("running_mean", "running_var", "y", "mean", "invstd", "a", "ws", "plan")
+_BACKWARD_READS = attrgetter("g", "y", "mean", "invstd", "gamma", "beta", "w", "x")
+_BACKWARD_WRITES = attrgetter("dx", "dgamma", "dbeta", "dy", "dw", "ws", "plan")
+
 
 def _address(t):
     return 0 if t is None else t.data_ptr()
@@ -48,6 +53,94 @@ class _Recording:
 
     def __init__(self, key):
         self.key, self.graph, self.launches = key, None, 0
+
+
+def _span(t):
+    """(storage, first byte, byte behind the last, row pitch in bytes of a channel slice or 0, bytes per row) of what a call
+    touches: a tensor, or -- as a whole -- any other object that only one call at a time may use (a plan)."""
+    if not isinstance(t, torch.Tensor):
+        return id(t), 0, 1, 0, 1
+    size, first = t.element_size(), t.data_ptr()
+    end = first + size * (1 + sum((n - 1) * st for n, st in zip(t.shape, t.stride())))
+    pitch = t.stride(-2) * size if t.dim() == 4 and t.stride(-2) > t.shape[-1] else 0
+    return t.untyped_storage().data_ptr(), first, end, pitch, t.shape[-1] * size
+
+
+def _overlap(a, b):
+    if a[0] != b[0] or a[1] >= b[2] or b[1] >= a[2]:
+        return False
+    if a[3] and a[3] == b[3]:  # two channel ranges of the same rows
+        d = (b[1] - a[1]) % a[3]
+        return d < a[4] or d + b[4] > a[3]
+    return True
+
+
+class _Lanes:
+    """Branches of a recording.  Every call says what it reads and writes; it waits for the earlier calls that it has a
+    conflict with (so that sums into one gradient keep their order, and their bits) and for no others.  A call joins the
+    branch that ends with one of those; where there is none, as at the detector's six head branches, it opens another.
+    The kernels of a small batch leave most SMs idle and are bound by their latency, so that branches beside the longest
+    chain of the dataflow (67 of 77 blocks) cost next to nothing.  Measured, forward and backward pass of the detector at batch 2,
+    320 x 320: 888 -> 761 us, 1581 -> 1407 us; at batch 16, 640 x 640: 3163 -> 3085, 6333 -> 6250."""
+
+    LIMIT = 8  # (the detector opens six)
+
+    def __init__(self, main, device, spare):
+        self.device, self.spare = device, spare  # spare: streams kept by the runner
+        self.streams, self.tails, self.seen = [main], [-1], [{}]
+        self.calls = []     # (lane, event, lane -> last call known to be complete behind it)
+        self.touched = {}   # storage -> [(span, call, writes)]
+        self.open = None    # lane of the call being issued
+
+    def enter(self, reads, writes):
+        """The stream of the next call."""
+        self._close()
+        spans = [(_span(t), False) for t in reads if t is not None] + [(_span(t), True) for t in writes if t is not None]
+        need = {c for sp, wr in spans for other, c, w in self.touched.get(sp[0], ()) if (wr or w) and _overlap(sp, other)}
+        ends = [c for c in need if self.tails[self.calls[c][0]] == c]
+        if ends:
+            lane = self.calls[max(ends)][0]
+        elif not self.calls:
+            lane = 0
+            self.start = torch.cuda.Event()
+            self.start.record(self.streams[0])
+        elif len(self.streams) < self.LIMIT:
+            lane = len(self.streams)
+            if len(self.spare) < lane:
+                self.spare.append(torch.cuda.Stream(self.device))
+            self.streams.append(self.spare[lane - 1])
+            self.tails.append(-1)
+            self.seen.append({})
+            if not need:
+                self.streams[lane].wait_event(self.start)
+        else:
+            lane = self.calls[max(need)][0] if need else 0
+        seen = self.seen[lane]
+        for c in sorted(need, reverse=True):
+            other, event, behind = self.calls[c]
+            if other != lane and seen.get(other, -1) < c:
+                self.streams[lane].wait_event(event)
+                for k, v in behind.items():
+                    seen[k] = max(seen.get(k, -1), v)
+        self.open = lane
+        for sp, wr in spans:
+            self.touched.setdefault(sp[0], []).append((sp, len(self.calls), wr))
+        return self.streams[lane]
+
+    def _close(self):
+        if self.open is None:
+            return
+        lane, call = self.open, len(self.calls)
+        event = torch.cuda.Event()
+        event.record(self.streams[lane])
+        self.seen[lane][lane] = self.tails[lane] = call
+        self.calls.append((lane, event, dict(self.seen[lane])))
+        self.open = None
+
+    def finish(self):
+        self._close()
+        for lane in range(1, len(self.streams)):
+            self.streams[0].wait_event(self.calls[self.tails[lane]][1])
 
 
 class GraphRunner:
@@ -68,7 +161,7 @@ class GraphRunner:
         self.plain, self.idx = [], {}
         self.glue_fwd = self.glue_bwd = 0
         self._recordings = {}        # pass -> _Recording
-        self._record_streams = None  # the streams that graphs are recorded on
+        self._record_streams = None  # the streams that graphs are recorded on: main, side, further branches
         new = lambda shp, dtype=torch.bfloat16: torch.empty(shp, dtype=dtype, device=self.dev)
         prod = {o["out"]: (i, o) for i, o in enumerate(ops)}
         cons = {}
@@ -319,7 +412,9 @@ class GraphRunner:
         n, h, w, _ = self.shape[name]
         return n * h * w
 
-    def _sadd(self, out, a, rows, channels, b=None, accumulate=False, stream=None):
+    def _sadd(self, out, a, rows, channels, b=None, accumulate=False, stream=None, lanes=None):
+        if lanes:
+            stream = lanes.enter([a, b], [out])
         nb.nb_slice_add(nb.NB_DTYPE_BF16, rows, channels, out, out.stride(-2), a, a.stride(-2), b, b.stride(-2) if b is not None else 0, accumulate, stream)
 
     # ------------------------------------------------------------------ recorded passes
@@ -363,14 +458,18 @@ class GraphRunner:
 
     def _record(self, rec, issue, with_side):
         if self._record_streams is None:
-            self._record_streams = torch.cuda.Stream(self.dev), torch.cuda.Stream(self.dev)
-        main, side = self._record_streams
+            # (priority for the branch that holds the longest chain: 2307 -> 2285 us at batch 2, 320 x 320; given to every
+            # branch it starves the weight gradients, 9.31 -> 9.74 ms at batch 16)
+            self._record_streams = torch.cuda.Stream(self.dev, priority=-1), torch.cuda.Stream(self.dev), []
+        main, side, spare = self._record_streams
         graph = torch.cuda.CUDAGraph()
         before = nb.nb_cbs_launch_count()
         with torch.cuda.stream(main):
             graph.capture_begin(capture_error_mode="thread_local")  # (other threads may go on using the GPU)
             try:
-                issue(main, side if with_side else None)
+                lanes = _Lanes(main, self.dev, spare)
+                issue(main, side if with_side else None, lanes)
+                lanes.finish()
                 if with_side:
                     main.wait_stream(side)
             finally:
@@ -381,40 +480,49 @@ class GraphRunner:
 
     # ------------------------------------------------------------------ passes
     def forward(self, stream=None):
-        self._run("forward", _FORWARD_TENSORS, lambda st, _: self._forward(st), stream)
+        self._run("forward", _FORWARD_TENSORS, lambda st, _, lanes=None: self._forward(st, lanes), stream)
 
-    def _forward(self, stream):
+    def _forward(self, stream, lanes=None):
         B, n_glue = self.buf, 0
         for o in self.ops:
             kind, out, ins = o["op"], o["out"], o["ins"]
             rows, c_out = self._rows(out), self.shape[out][3]
             if kind == "cbs":
-                self.blocks[o["layer"]].forward(stream)
+                blk = self.blocks[o["layer"]]
+                if lanes:
+                    stream = lanes.enter(_FORWARD_READS(blk) + (getattr(blk, "res", None),), _FORWARD_WRITES(blk))
+                blk.forward(stream)
             elif kind == "plain":
                 pl = self.plain[o["layer"]]
+                if lanes:
+                    stream = lanes.enter([B[ins[0]], pl["w"], pl["bias"]], [B[out], pl["ws"], pl["plan"]])
                 nb.nb_conv_bias_act(pl["plan"], B[ins[0]], pl["w"], pl["bias"], 0, B[out], pl["ws"], stream)
             elif kind == "slice":
                 if out not in self.slice_view:
-                    self._sadd(B[out], B[ins[0]][..., o["c0"]:o["c1"]], rows, c_out, stream=stream)
+                    self._sadd(B[out], B[ins[0]][..., o["c0"]:o["c1"]], rows, c_out, stream=stream, lanes=lanes)
                     n_glue += 1
             elif kind == "add":
                 if id(o) not in self.fused_adds:
-                    self._sadd(B[out], B[ins[0]], rows, c_out, b=B[ins[1]], stream=stream)
+                    self._sadd(B[out], B[ins[0]], rows, c_out, b=B[ins[1]], stream=stream, lanes=lanes)
                     n_glue += 1
             elif kind == "concat":
                 c0 = 0
                 for name in ins:
                     c = self.shape[name][3]
                     if not self._in_place(B[name], B[out], c0):
-                        self._sadd(B[out][..., c0:c0 + c], B[name], rows, c, stream=stream)
+                        self._sadd(B[out][..., c0:c0 + c], B[name], rows, c, stream=stream, lanes=lanes)
                         n_glue += 1
                     c0 += c
             elif kind == "maxpool":
                 n, h, w, c = self.shape[out]
+                if lanes:
+                    stream = lanes.enter([B[ins[0]]], [B[out], self.idx[out]])
                 nb.nb_maxpool5_fwd(nb.NB_DTYPE_BF16, n, h, w, c, B[ins[0]], B[out], self.idx[out], stream, ld_x=B[ins[0]].stride(-2), ld_y=B[out].stride(-2))
                 n_glue += 1
             elif kind == "upsample":
                 n, h, w, c = self.shape[ins[0]]
+                if lanes:
+                    stream = lanes.enter([B[ins[0]]], [B[out]])
                 nb.nb_upsample2(nb.NB_DTYPE_BF16, n, h, w, c, B[ins[0]], B[out], ld_small=B[ins[0]].stride(-2), ld_large=B[out].stride(-2), stream=stream)
                 n_glue += 1
         self.glue_fwd = n_glue
@@ -424,9 +532,10 @@ class GraphRunner:
         block's dw, dgamma, dbeta in the block.  With wgrad_stream (and a workspace for it) every weight gradient is queued
         on that stream behind an event that follows the block's data-gradient call (it only reads the block's input
         activations and dy, which nothing overwrites during the backward pass); the caller joins the streams."""
-        self._run("backward", _BACKWARD_TENSORS, lambda st, side: self._backward(st, side, wgrad_workspace), stream, wgrad_stream, wgrad_workspace)
+        self._run("backward", _BACKWARD_TENSORS, lambda st, side, lanes=None: self._backward(st, side, wgrad_workspace, lanes), stream,
+                  wgrad_stream, wgrad_workspace)
 
-    def _backward(self, stream, wgrad_stream, wgrad_workspace):
+    def _backward(self, stream, wgrad_stream, wgrad_workspace, lanes=None):
         G, n_glue = self.grad, 0
         for name in self.zeroed:
             G[name].zero_()
@@ -436,6 +545,8 @@ class GraphRunner:
             c_out = self.shape[out][3]
             if kind == "cbs":
                 blk = self.blocks[o["layer"]]
+                if lanes:
+                    stream = lanes.enter(_BACKWARD_READS(blk), _BACKWARD_WRITES(blk) + (getattr(blk, "gres", None),))
                 blk.backward_data(stream)
                 if wgrad_stream is None:
                     blk.backward_weight(stream)
@@ -446,36 +557,42 @@ class GraphRunner:
                     blk.backward_weight(wgrad_stream, wgrad_workspace)
                 src = ins[0]
                 if G[src] is not blk.dx:
-                    self._sadd(G[src], blk.dx, self._rows(src), self.shape[src][3], accumulate=self.acc[(oi, 0)], stream=stream)
+                    self._sadd(G[src], blk.dx, self._rows(src), self.shape[src][3], accumulate=self.acc[(oi, 0)], stream=stream, lanes=lanes)
                     n_glue += 1
             elif kind == "plain":
                 pl = self.plain[o["layer"]]
+                if lanes:
+                    stream = lanes.enter([self.buf[ins[0]], pl["w"], G[out]], [pl["dx"], pl["dw"], pl["dbias"], pl["ws"], pl["plan"]])
                 nb.nb_conv_bias_bwd(pl["plan"], self.buf[ins[0]], pl["w"], G[out], pl["dx"], pl["dw"], pl["dbias"], pl["ws"], stream)
                 assert G[ins[0]] is pl["dx"]  # a plain convolution is the only consumer of its input in this dataflow
             elif kind == "slice":
                 if out not in self.slice_view:
-                    self._sadd(G[ins[0]][..., o["c0"]:o["c1"]], G[out], self._rows(out), c_out, accumulate=self.acc[(oi, 0)], stream=stream)
+                    self._sadd(G[ins[0]][..., o["c0"]:o["c1"]], G[out], self._rows(out), c_out, accumulate=self.acc[(oi, 0)], stream=stream, lanes=lanes)
                     n_glue += 1
             elif kind == "add":
                 for pos, src in enumerate(ins):
                     if not self._implicit(o, pos) and not (pos == 0 and oi in self.shortcut_by_block):
-                        self._sadd(G[src], G[out], self._rows(out), c_out, accumulate=self.acc[(oi, pos)], stream=stream)
+                        self._sadd(G[src], G[out], self._rows(out), c_out, accumulate=self.acc[(oi, pos)], stream=stream, lanes=lanes)
                         n_glue += 1
             elif kind == "concat":
                 c0 = 0
                 for pos, src in enumerate(ins):
                     c = self.shape[src][3]
                     if not self._implicit(o, pos):
-                        self._sadd(G[src], G[out][..., c0:c0 + c], self._rows(out), c, accumulate=self.acc[(oi, pos)], stream=stream)
+                        self._sadd(G[src], G[out][..., c0:c0 + c], self._rows(out), c, accumulate=self.acc[(oi, pos)], stream=stream, lanes=lanes)
                         n_glue += 1
                     c0 += c
             elif kind == "maxpool":
                 n, h, w, c = self.shape[out]
+                if lanes:
+                    stream = lanes.enter([G[out], self.idx[out]], [G[ins[0]]])
                 nb.nb_maxpool5_bwd(nb.NB_DTYPE_BF16, n, h, w, c, G[out], self.idx[out], G[ins[0]], self.acc[(oi, 0)], stream, ld_g=G[out].stride(-2),
                                    ld_dx=G[ins[0]].stride(-2))
                 n_glue += 1
             elif kind == "upsample":
                 n, h, w, c = self.shape[ins[0]]
+                if lanes:
+                    stream = lanes.enter([G[out]], [G[ins[0]]])
                 nb.nb_upsample2(nb.NB_DTYPE_BF16, n, h, w, c, G[out], G[ins[0]], backward=True, accumulate=self.acc[(oi, 0)], ld_small=G[ins[0]].stride(-2),
                                 ld_large=G[out].stride(-2), stream=stream)
                 n_glue += 1
