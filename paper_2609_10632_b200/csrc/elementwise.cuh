@@ -5,6 +5,7 @@
 // (bitwise reproducible run to run: no floating-point atomics anywhere).
 #pragma once
 #include "common.cuh"
+#include "ptx_sm100.cuh"
 
 namespace nbcbs {
 
@@ -626,6 +627,16 @@ struct BwdFin {
     const float *mean, *invstd, *gamma, *beta;
     float *dgamma, *dbeta;
 };
+struct BwdCoef {
+    float a, b, p1, p0, dgamma;
+};
+__device__ __forceinline__ BwdCoef bwd_coef_channel(float mu_f, float is_f, float ga, float be, double s0, double s1, double inv_m) {
+    const double mu = (double)mu_f, is = (double)is_f;
+    const double dg = is * (s1 - mu * s0);
+    const double a = (double)ga * is;
+    const double p1 = a * is * dg * inv_m;
+    return {(float)a, (float)((double)be - mu * a), (float)p1, (float)(p1 * mu - a * s0 * inv_m), (float)dg};
+}
 __device__ __forceinline__ void bwd_coef_from_acc(const ChanAcc& ca, const BwdFin& f, int C, float* s_coef /*[4][C] shared*/) {
     const bool writer = blockIdx.x == 0;
 #pragma unroll 1
@@ -636,18 +647,15 @@ __device__ __forceinline__ void bwd_coef_from_acc(const ChanAcc& ca, const BwdFi
         chan_acc_total2(ca, C, c, t0, t1);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const double mu = (double)(j ? mu_f.y : mu_f.x), is = (double)(j ? is_f.y : is_f.x);
             const double s0 = j ? t0.y : t0.x, s1 = j ? t1.y : t1.x;
-            const double dg = is * (s1 - mu * s0);
-            const double a = (double)(j ? ga.y : ga.x) * is;
-            const double p1 = a * is * dg * f.inv_m;
-            s_coef[c + j] = (float)a;
-            s_coef[C + c + j] = (float)((double)(j ? be.y : be.x) - mu * a);
-            s_coef[2 * C + c + j] = (float)p1;
-            s_coef[3 * C + c + j] = (float)(p1 * mu - a * s0 * f.inv_m);
+            const BwdCoef k = bwd_coef_channel(j ? mu_f.y : mu_f.x, j ? is_f.y : is_f.x, j ? ga.y : ga.x, j ? be.y : be.x, s0, s1, f.inv_m);
+            s_coef[c + j] = k.a;
+            s_coef[C + c + j] = k.b;
+            s_coef[2 * C + c + j] = k.p1;
+            s_coef[3 * C + c + j] = k.p0;
             if (writer) {
                 f.dbeta[c + j] = (float)s0;
-                f.dgamma[c + j] = (float)dg;
+                f.dgamma[c + j] = k.dgamma;
             }
         }
     }
@@ -733,6 +741,166 @@ __global__ void __launch_bounds__(288, 3) bn_silu_bwd_dy_kernel(const AT* __rest
         __syncthreads();
         chan_acc_reset_if(ca, C, s_last != 0);
     }
+}
+
+// ------------------------------------------------------------------ both backward passes in one launch, for small tensors
+// Where the reduction's threads have at most eight vectors each and few blocks, the two passes are two memory latencies, a
+// launch and a trip of the sums through the fp64 accumulators, with nothing busy.  Here g and y stay in registers between
+// them and the sums travel through distributed shared memory: the channels are cut into `slabs` (clusters of at most eight
+// CTAs that need nothing from one another), and CTA q of a slab's cluster does the slab's share of the `slabs` row blocks
+// from q * slabs on.  The additions and their grouping in fp32 are those of the reduce kernel, the block sums are added in
+// fp64 as there, and dz is computed anew from the same coefficients as in the dy kernel, so the results are too.
+// CTAs past the slabs rearrange filter tiles.
+// Bound: latency (loads, two cluster barriers, the fp64 chain of a channel).  Measured (step): 336 -> 392 3x3 on 21 x 18 pixels
+// 46.0 -> 43.5 us, 248 -> 208 3x3 on 60 x 19 48.1 -> 46.2, 16 -> 32 3x3 on 4 x 13 x 82 27.5 -> 26.7; more at e.slabs in nb_cbs.cu.
+__device__ __forceinline__ double ld_dsmem_f64(uint32_t cluster_addr) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
+// Dynamic shared memory: fp64 sums [2][C / slabs], coefficients [4][C / slabs], then red [2][blockDim.x * V] and part [2 C].
+inline size_t bwd_small_smem(int C, int slabs, int tpb, int vec) { return (size_t)(C / slabs) * 32 + ((size_t)2 * tpb * vec + 2 * C) * 4; }
+template <typename YT, typename AT, bool FAST, bool PITCHED, bool GRES>
+__global__ void __launch_bounds__(288, 1) bn_silu_bwd_small_kernel(const AT* __restrict__ g, const YT* __restrict__ y, AT* __restrict__ dy, long long rows,
+                                                                   int C, BwdFin fin, const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wt,
+                                                                   WtParams wtp, long long ld_g, AT* __restrict__ gres, long long ld_gres, int gres_add,
+                                                                   int slabs, int cluster, int row_blocks) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int slab = (int)blockIdx.x / cluster, q = (int)blockIdx.x % cluster;
+    if (slab >= slabs) {
+        wt_transform_blocks(w, wt, wtp, (int)blockIdx.x - slabs * cluster, (int)gridDim.x - slabs * cluster);
+        return;
+    }
+    constexpr int V = Vec16<YT>::N, D = 8;
+    static_assert(V == Vec16<AT>::N, "g and y must have the same element size");
+    extern __shared__ __align__(16) float small_smem[];
+    const int tid = threadIdx.x, tpb = blockDim.x;
+    const int cgs = C / V, R = tpb / cgs, wv = cgs / slabs, wc = wv * V;  // vectors and channels of the slab
+    double* const s_tot = reinterpret_cast<double*>(small_smem);          // [2][wc]
+    float* const s_coef = small_smem + 4 * wc;                            // [4][wc]
+    float* const red = s_coef + 4 * wc;                                   // [2][tpb * V]
+    float* const part = red + 2 * tpb * V;                                // [2][slabs][wc]
+    const int jl = tid / (R * wv), rem = tid % (R * wv), cg = rem % wv;
+    const int block = q * slabs + jl;                                     // of the reduce kernel's grid
+    const long long row0 = (long long)block * R + rem / wv, row_step = (long long)row_blocks * R;
+    const int ch = (slab * wv + cg) * V;
+    auto has = [&](int u) { return block < row_blocks && row0 + u * row_step < rows; };
+    Vec16<YT> qy[D];
+    Vec16<AT> qg[D];
+#pragma unroll
+    for (int u = 0; u < D; ++u)
+        if (has(u)) {
+            qy[u] = ld16(y + (row0 + u * row_step) * C + ch);
+            qg[u] = ld16(g + (row0 + u * row_step) * (PITCHED ? ld_g : (long long)C) + ch);
+        }
+    float2 a[V / 2], b[V / 2];
+    {
+        float2 sb[V / 2], sy[V / 2];
+        float mu[V], is[V], ga[V], be[V];
+        load_params<V>(fin.mean, slab * wv + cg, mu);
+        load_params<V>(fin.invstd, slab * wv + cg, is);
+        load_params<V>(fin.gamma, slab * wv + cg, ga);
+        load_params<V>(fin.beta, slab * wv + cg, be);
+#pragma unroll
+        for (int j = 0; j < V / 2; ++j) {
+            a[j] = make_float2(ga[2 * j] * is[2 * j], ga[2 * j + 1] * is[2 * j + 1]);
+            b[j] = make_float2(fmaf(-mu[2 * j], a[j].x, be[2 * j]), fmaf(-mu[2 * j + 1], a[j].y, be[2 * j + 1]));
+            sb[j] = sy[j] = splat2(0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < D; ++u)
+            if (has(u)) {
+#pragma unroll
+                for (int j = 0; j < V / 2; ++j) {
+                    const float2 yv = pair_to_f32(qy[u].v + 2 * j);
+                    const float2 dz = silu_bwd_dz2<FAST>(fma2(yv, a[j], b[j]), pair_to_f32(qg[u].v + 2 * j));
+                    sb[j] = add2(sb[j], dz);
+                    sy[j] = fma2(dz, yv, sy[j]);
+                }
+            }
+#pragma unroll
+        for (int j = 0; j < V / 2; ++j) {
+            *reinterpret_cast<float2*>(&red[tid * V + 2 * j]) = sb[j];
+            *reinterpret_cast<float2*>(&red[(tpb + tid) * V + 2 * j]) = sy[j];
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < 2 * C; e += tpb) {  // the sums of every row block of this CTA (zero past the last)
+        const int pass = e >= C ? 1 : 0, k = e - pass * C, bl = k / wc, c = k - bl * wc;
+        const float* const src = red + (pass * tpb + bl * R * wv) * V + c;
+        float acc = 0.f;
+        for (int r = 0; r < R; ++r) acc += src[r * wc];
+        part[e] = q * slabs + bl < row_blocks ? acc : 0.f;
+    }
+    __syncthreads();
+    for (int e = tid; e < 2 * wc; e += tpb) {
+        const int pass = e >= wc ? 1 : 0;
+        const float* const src = part + pass * C + (e - pass * wc);
+        double t = 0.0;
+        for (int bl = 0; bl < slabs; ++bl) t += (double)src[bl * wc];
+        s_tot[e] = t;
+    }
+    __syncthreads();  // (the cluster barrier wants whole warps)
+    if (cluster > 1) ptx::cluster_sync_all();
+    const uint32_t tot = ptx::smem_u32(s_tot);
+    for (int c = tid; c < wc; c += tpb) {
+        double s0 = 0.0, s1 = 0.0;
+        if (cluster > 1) {
+            for (int k = 0; k < cluster; ++k) {
+                const uint32_t peer = ptx::mapa_u32(tot, (uint32_t)k);
+                s0 += ld_dsmem_f64(peer + 8u * (uint32_t)c);
+                s1 += ld_dsmem_f64(peer + 8u * (uint32_t)(wc + c));
+            }
+        } else {
+            s0 = s_tot[c];
+            s1 = s_tot[wc + c];
+        }
+        const int cc = slab * wc + c;
+        const BwdCoef k = bwd_coef_channel(fin.mean[cc], fin.invstd[cc], fin.gamma[cc], fin.beta[cc], s0, s1, fin.inv_m);
+        s_coef[c] = k.a;
+        s_coef[wc + c] = k.b;
+        s_coef[2 * wc + c] = k.p1;
+        s_coef[3 * wc + c] = k.p0;
+        if (q == 0) {
+            fin.dbeta[cc] = (float)s0;
+            fin.dgamma[cc] = k.dgamma;
+        }
+    }
+    __syncthreads();
+    // behind its own reads a CTA tells its peers that they may leave
+    if (cluster > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    float2 np1[V / 2], p0[V / 2];
+    load_params_shared<V>(s_coef, cg, a);
+    load_params_shared<V>(s_coef + wc, cg, b);
+    load_params_shared<V>(s_coef + 2 * wc, cg, np1);
+    load_params_shared<V>(s_coef + 3 * wc, cg, p0);
+#pragma unroll
+    for (int j = 0; j < V / 2; ++j) np1[j] = make_float2(-np1[j].x, -np1[j].y);
+#pragma unroll
+    for (int u = 0; u < D; ++u)
+        if (has(u)) {
+            const long long row = row0 + u * row_step;
+            if (GRES) {
+                Vec16<AT> r = qg[u];
+                if (gres_add) {
+                    const Vec16<AT> old = ld16(gres + row * ld_gres + ch);
+#pragma unroll
+                    for (int j = 0; j < V / 2; ++j) pair_from_f32(r.v + 2 * j, add2(pair_to_f32(old.v + 2 * j), pair_to_f32(qg[u].v + 2 * j)));
+                }
+                st16(gres + row * ld_gres + ch, r);
+            }
+            Vec16<AT> o;
+#pragma unroll
+            for (int j = 0; j < V / 2; ++j) {
+                const float2 yv = pair_to_f32(qy[u].v + 2 * j);
+                const float2 dz = silu_bwd_dz2<FAST>(fma2(yv, a[j], b[j]), pair_to_f32(qg[u].v + 2 * j));
+                pair_from_f32(o.v + 2 * j, fma2(a[j], dz, fma2(np1[j], yv, p0[j])));
+            }
+            st16(dy + row * C + ch, o);
+        }
+    __syncwarp();
+    if (cluster > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 }  // namespace nbcbs
