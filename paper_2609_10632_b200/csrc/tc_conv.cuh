@@ -46,6 +46,7 @@ struct IgemmParams {
     int BN, n_tiles, m_tiles;
     int mh;                      // 128-row sub-tiles per tile (1 or 2): the tile is [128*mh x BN]
     int acc_bufs;                // accumulator sets in TMEM (2 when 2*mh*acc_stride <= 512)
+    int rot_workers;             // igemm_first_kblock: workers of the tiling that decides where a tile's K loop starts
     int ncol_a;                  // columns of a tile that epilogue team 0 handles (team 1: the other BN - ncol_a)
     int stage_cw;                // columns per staging pass of a team (<= 64)
     // When GEMM row == output row (everything but a stride-2 dgrad) a warp hands each staged [32 x width] piece
@@ -98,6 +99,12 @@ template <bool CLS4> __device__ __forceinline__ void igemm_tile_class(const Igem
         cls = tile / p.tiles_per_class;
         lt = tile - cls * p.tiles_per_class;
     }
+}
+// The k-block with which a tile starts its K loop: one per worker -- HALF: of the tiling with twice as many rows per tile
+// (IgemmCfg::rot_div; an instantiation of its own, because the divisions cost every other layer 1 %).
+template <bool HALF> __device__ __forceinline__ int igemm_first_kblock(const IgemmParams& p, int worker, int lt, int kblocks) {
+    if (HALF) worker = (lt / p.n_tiles / 2 * p.n_tiles + lt % p.n_tiles) % p.rot_workers;
+    return (int)(((unsigned)worker * 7u) % (unsigned)kblocks);
 }
 
 constexpr int TC_BM = 128;
@@ -282,7 +289,7 @@ __device__ __forceinline__ void epi_pass_tma(uint32_t taddr, uint8_t* wrows, int
 // EPI = 1: the epilogue applies a per-channel scale and shift (evaluation-mode BN or a bias) and optionally SiLU to the
 // accumulators, so the kernel writes the block's final activations (no statistics, no second pass); TMA stores only.
 // STATS (forward of a training block): TMA stores only; the epilogue also sums every channel's values and squares.
-template <typename OutT, bool STATS, bool CG2, int EPI = 0, bool CLS4 = false>
+template <typename OutT, bool STATS, bool CG2, int EPI = 0, bool CLS4 = false, bool HALF = false>
 __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_constant__ IgemmParams p) {
     static_assert(!CLS4 || (!STATS && !EPI), "four classes: the stride-2 data gradient only");
     static_assert(!EPI || !STATS, "the fused per-channel epilogue is a forward-only variant without statistics");
@@ -411,7 +418,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
             // each CTA starts its K loop at a different k-block so that the CTAs do not all ask L2 for the same
             // filter lines at the same moment
             const int ntaps_c = p.cls_ntaps[cls];
-            const int rot = (int)(((unsigned)worker * 7u) % (unsigned)kblocks);
+            const int rot = igemm_first_kblock<HALF>(p, worker, lt, kblocks);
             int tap = rot / kc_per_tap, kc = rot - tap * kc_per_tap;
             for (int kb0 = 0; kb0 < kblocks; kb0 += kpb) {
                 const int nkb = (kblocks - kb0 < kpb) ? kblocks - kb0 : kpb;
@@ -497,7 +504,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * mh) * acc_stride;
                 uint32_t accumulate = 0;
-                int kc = (int)(((unsigned)worker * 7u) % (unsigned)kblocks) % kc_per_tap;  // the producers' starting k-block
+                int kc = igemm_first_kblock<HALF>(p, worker, lt_mma, kblocks) % kc_per_tap;  // the producers' starting k-block
                 for (int kb0 = 0; kb0 < kblocks; kb0 += kpb) {
                     const int nkb = (kblocks - kb0 < kpb) ? kblocks - kb0 : kpb;
                     if (!wait_bar_fast(full + s, ph, abort_flag, p.status, 3)) {
@@ -786,7 +793,7 @@ namespace nbcbs {
 struct IgemmCfg {
     bool ok = false;
     int Ca = 0, rowsB = 0, ntaps = 0;
-    int KC = 0, BN = 0, n_tiles = 0, m_tiles = 0, stages = 0, acc_stride = 0, tmem_cols = 0, grid = 0, kpb = 1, mh = 1, acc_bufs = 2, stage_cols = 0;
+    int KC = 0, BN = 0, n_tiles = 0, m_tiles = 0, stages = 0, acc_stride = 0, tmem_cols = 0, grid = 0, kpb = 1, mh = 1, rot_div = 1, rot_workers = 1, acc_bufs = 2, stage_cols = 0;
     bool cg2 = false;  // CTA pairs (tcgen05 cta_group::2)
     bool tail32 = false;  // the last k-block of every tap is 32 channels wide
     uint32_t a_stage = 0, b_stage = 0, a_sub = 0, b_sub = 0;
@@ -904,7 +911,13 @@ inline int igemm_tile_cols(int rowsB, int most = 256) {
 inline bool igemm_channels_ok(int Ca, int rowsB, long long M) {
     return Ca % 8 == 0 && rowsB % 8 == 0 && rowsB >= 16 && ((Ca % 16 == 0 && rowsB % 16 == 0) || M >= 2 * TC_BM);
 }
-inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int sm_count, int nclasses) {
+// `by_waves`: calls without channel sums (whose grouping is one of tiles) may take mh = 1 where mh = 2 fills its last wave badly
+// and the operands are what takes the time (at least 16 k-blocks); a data-gradient tile then starts its K loop where the tile
+// of mh = 2 would, so that its sums have the same bits (rot_div: 2 there, else 1).  A k-block costs what the tensor pipe or the
+// operand rows take (2.3 cycles each), whichever is longer, and a tile 1500 cycles besides.  Measured (step): 64 -> 336 and
+// 40 -> 336 3x3 on 4 x 87 x 130 pixels (177 tiles of 256 rows on 148 SMs) 147 -> 140 and 174 -> 170 us; evaluation-mode forward
+// of the detector on eight images of 640 x 640 1607 -> 1560 us.
+inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int sm_count, int nclasses, bool by_waves) {
     IgemmCfg c;
     c.Ca = Ca; c.rowsB = rowsB; c.ntaps = ntaps; c.M = M;
     if (M < 1) return c;
@@ -935,13 +948,25 @@ inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int s
         // per parity class) below 384 channels; 1x1 layers with 960 and more input channels gain 1.5-2 us again.
         const bool pair_pays = (ntaps > 1 && Ca >= 96 && (nclasses == 1 || Ca >= 384)) || (ntaps == 1 && Ca >= 960);
         const bool cg2 = bn % 32 == 0 && (getenv("NB_TC_CG2") ? atoi(getenv("NB_TC_CG2")) != 0 : pair_pays);
-        int mh = 1;
-        if (4 * acc_stride <= 512) {
-            const long long rows_tile = 2LL * TC_BM * (cg2 ? 2 : 1);
-            const long long tiles2 = ((M + rows_tile - 1) / rows_tile) * n_tiles * nclasses;
-            if (tiles2 >= (cg2 ? sm_count / 2 : sm_count)) mh = 2;
+        const int workers = cg2 ? sm_count / 2 : sm_count;
+        auto tiles = [&](int h) {
+            const long long rows_tile = (long long)h * TC_BM * (cg2 ? 2 : 1);
+            return ((M + rows_tile - 1) / rows_tile) * n_tiles * nclasses;
+        };
+        int mh = 4 * acc_stride <= 512 && tiles(2) >= workers ? 2 : 1;
+        c.rot_div = 1;
+        c.rot_workers = (int)std::min<long long>(tiles(mh), workers);
+        if (mh == 2 && by_waves && nclasses == 1 && kblocks >= 16) {
+            auto cost = [&](int h) {
+                const double rows = (TC_BM * h + (cg2 ? bn / 2 : bn)) * 2.3, mma = h * 4.0 * (cg2 ? bn / 2.0 : std::max(97.0, bn / 2.0));
+                return (double)((tiles(h) + workers - 1) / workers) * (kblocks * std::max(rows, mma) + 1500.0);
+            };
+            if (cost(1) < 0.95 * cost(2)) {
+                mh = 1;
+                c.rot_div = 2;
+            }
         }
-        if (force_mh && force_mh * acc_stride <= 512) mh = force_mh;
+        if (force_mh && force_mh * acc_stride <= 512) { mh = force_mh; c.rot_div = 1; c.rot_workers = (int)std::min<long long>(tiles(mh), workers); }
         const int acc_bufs = (2 * mh * acc_stride <= 512) ? 2 : 1;
         const uint32_t a_sub = (uint32_t)(TC_BM * mh * c.KC * 2);
         const uint32_t b_sub = (uint32_t)(((cg2 ? bn / 2 : bn) * c.KC * 2 + 1023) / 1024 * 1024);
@@ -985,6 +1010,7 @@ inline void fill_params(IgemmParams& P, const IgemmCfg& c) {
     P.a_stage_bytes = c.a_stage; P.b_stage_bytes = c.b_stage;
     P.kpb = c.kpb; P.a_sub_bytes = c.a_sub; P.b_sub_bytes = c.b_sub;
     P.tail32 = c.tail32 ? 1 : 0;
+    P.rot_workers = c.rot_workers;
     P.mh = c.mh; P.acc_bufs = c.acc_bufs; P.ncol_a = c.stage_cols; P.stage_cw = igemm_stage_cw(c.BN);
     if (getenv("NB_TC_VERBOSE"))
         fprintf(stderr, "[nb_cbs] igemm M=%lld Ca=%d rowsB=%d taps=%d: mh=%d cg2=%d tail32=%d BN=%d kpb=%d stages=%d accbufs=%d tiles=%dx%d grid=%d smem=%zu\n", c.M, c.Ca,
@@ -1055,7 +1081,7 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     P.a_stage_bytes = P.a_sub_bytes = c.a_stage; P.b_stage_bytes = P.b_sub_bytes = c.b_stage;
     P.kpb = 1; P.mh = 1; P.acc_bufs = 1; P.tma_store = 0;
     P.split = c.split;
-    P.full_rows = TC_BM * f.mh * (f.cg2 ? 2 : 1); P.full_bn = f.BN; P.full_n_tiles = f.n_tiles; P.full_workers = workers;
+    P.full_rows = TC_BM * f.mh * f.rot_div * (f.cg2 ? 2 : 1); P.full_bn = f.BN; P.full_n_tiles = f.n_tiles; P.full_workers = f.rot_workers;
     P.idesc = ptx::make_idesc_bf16(TC_BM, c.BN, 0, 0);
     c.ok = true;
     out.cfg = c;
@@ -1148,14 +1174,14 @@ inline bool encode_forward_inputs(TcGemmSlot& S, const Geom& g, const void* x, c
 }
 
 // Raises the dynamic shared-memory limit of one kernel instantiation once per device.
-template <typename OutT, bool STATS, bool CG2, int EPI, bool CLS4> inline bool igemm_allow_smem() {
+template <typename OutT, bool STATS, bool CG2, int EPI, bool CLS4, bool HALF> inline bool igemm_allow_smem() {
     // the attribute belongs to the (function, device) pair: one bit per device ordinal that already has it
     static std::atomic<unsigned long long> attr_set{0};
     int dev = 0;
     cudaGetDevice(&dev);
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(attr_set.load(std::memory_order_acquire) & bit)) {
-        if (cudaFuncSetAttribute(tc_igemm_kernel<OutT, STATS, CG2, EPI, CLS4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess) {
+        if (cudaFuncSetAttribute(tc_igemm_kernel<OutT, STATS, CG2, EPI, CLS4, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess) {
             err() = "cannot raise the dynamic shared memory limit of the implicit-GEMM kernel";
             return false;
         }
@@ -1163,11 +1189,11 @@ template <typename OutT, bool STATS, bool CG2, int EPI, bool CLS4> inline bool i
     }
     return true;
 }
-template <typename OutT, bool STATS, bool CG2, int EPI = 0, bool CLS4 = false> inline nb_status launch_igemm_impl(const TcGemmSlot& s, cudaStream_t st) {
-    if (!igemm_allow_smem<OutT, STATS, CG2, EPI, CLS4>()) return NB_ERR_CUDA;
+template <typename OutT, bool STATS, bool CG2, int EPI = 0, bool CLS4 = false, bool HALF = false> inline nb_status launch_igemm_impl(const TcGemmSlot& s, cudaStream_t st) {
+    if (!igemm_allow_smem<OutT, STATS, CG2, EPI, CLS4, HALF>()) return NB_ERR_CUDA;
     // (Measured: launching a kernel only after its predecessor has completed costs 3.4 us per launch: its prologue --
     // barrier set-up, TMEM allocation, tensor-map fetch -- no longer overlaps the predecessor's tail.)
-    const cudaError_t e = launch_k(tc_igemm_kernel<OutT, STATS, CG2, EPI, CLS4>, dim3((unsigned)s.cfg.grid), dim3(IG_THREADS), s.cfg.smem_bytes, st, CG2 ? 2 : 1, s.prm);
+    const cudaError_t e = launch_k(tc_igemm_kernel<OutT, STATS, CG2, EPI, CLS4, HALF>, dim3((unsigned)s.cfg.grid), dim3(IG_THREADS), s.cfg.smem_bytes, st, CG2 ? 2 : 1, s.prm);
     if (e != cudaSuccess) {
         err() = std::string("launch of tc_igemm_kernel failed: ") + cudaGetErrorString(e);
         return NB_ERR_CUDA;
@@ -1175,8 +1201,9 @@ template <typename OutT, bool STATS, bool CG2, int EPI = 0, bool CLS4 = false> i
     return NB_OK;
 }
 template <typename OutT, bool STATS> inline nb_status launch_igemm(const TcGemmSlot& s, cudaStream_t st) {
-    if constexpr (!STATS) {  // the data gradient: the only launch with four classes
+    if constexpr (!STATS) {  // the data gradient: the only launch with four classes, or with another tiling's K order
         if (s.prm.nclasses == 4) return s.cfg.cg2 ? launch_igemm_impl<OutT, false, true, 0, true>(s, st) : launch_igemm_impl<OutT, false, false, 0, true>(s, st);
+        if (s.cfg.rot_div == 2) return s.cfg.cg2 ? launch_igemm_impl<OutT, false, true, 0, false, true>(s, st) : launch_igemm_impl<OutT, false, false, 0, false, true>(s, st);
     }
     return s.cfg.cg2 ? launch_igemm_impl<OutT, STATS, true>(s, st) : launch_igemm_impl<OutT, STATS, false>(s, st);
 }
@@ -1230,7 +1257,7 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
     if (!d.tiled || !d.im2col) return NB_OK;  // no TMA descriptors from this driver: stay on the CUDA-core kernels
     // ---- fprop: A = x (im2col), B = w [Cout][k*k*Cin]
     if (igemm_channels_ok(g.c_in, g.c_out, g.m)) {
-        const IgemmCfg c = igemm_configure(g.m, g.c_in, g.c_out, g.k * g.k, sm_count, 1);
+        const IgemmCfg c = igemm_configure(g.m, g.c_in, g.c_out, g.k * g.k, sm_count, 1, false);
         if (c.ok) {
             tc->fp.cfg = c;
             IgemmParams& P = tc->fp.prm;
@@ -1249,6 +1276,9 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
             tc->fprop = true;
             tc->fprop_parts = c.grid;
             tc->inf = tc->fp;
+            tc->inf.cfg = igemm_configure(g.m, g.c_in, g.c_out, g.k * g.k, sm_count, 1, true);
+            fill_params(tc->inf.prm, tc->inf.cfg);
+            tc->inf.prm.tiles_per_class = tc->inf.cfg.m_tiles * tc->inf.cfg.n_tiles;
             // (a training forward whose persistent form has one 128-row tile per CTA: its channel sums are one tile's)
             if (c.mh == 1 && (long long)c.m_tiles * c.n_tiles <= (c.cg2 ? c.grid / 2 : c.grid)) split_configure(tc->fps, tc->fp, g.k * g.k, false, sm_count);
             split_configure(tc->infs, tc->inf, g.k * g.k, true, sm_count);
@@ -1305,7 +1335,7 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
             P.Hq = g.ho; P.Wq = g.wo; P.ts = 1; P.lo_w = P.lo_h = 0;
             P.Hout = g.h; P.Wout = g.w; P.os = 2;
         }
-        const IgemmCfg c = igemm_configure((long long)g.n * P.Hq * P.Wq, g.c_out, g.c_in, max_taps, sm_count, ncls);
+        const IgemmCfg c = igemm_configure((long long)g.n * P.Hq * P.Wq, g.c_out, g.c_in, max_taps, sm_count, ncls, true);
         if (c.ok) {
             tc->dg.cfg = c;
             fill_params(P, c);  // sets only the tiling fields; the geometry written above stays
