@@ -818,22 +818,6 @@ def run_e2e(args, layers, blocks, flags, local, dev, dist, world, flops):
 
     from paper_2609_10632_b200 import binding as nb
 
-    host = {}  # per distinct shape: pinned input and output buffers (inputs filled from the device tensors)
-    scratch_bytes = 0
-    h2d = d2h = 0
-    for b in blocks:
-        s = b.shape
-        scratch_bytes = max(scratch_bytes, b.plan.step_host_scratch_bytes())
-        if s.key not in host:
-            pin = lambda t: torch.empty(t.shape, dtype=t.dtype).pin_memory()
-            hin = {k: pin(getattr(b, k)) for k in ("x", "w", "gamma", "beta", "g")}
-            for k, t in hin.items():
-                t.copy_(getattr(b, k))
-            hout = {k: pin(getattr(b, k)) for k in ("a", "dx", "dw", "dgamma", "dbeta")}
-            host[s.key] = (hin, hout)
-        hin, hout = host[s.key]
-        h2d += sum(t.numel() * t.element_size() for t in hin.values())
-        d2h += sum(t.numel() * t.element_size() for t in hout.values())
     # Several streams (--e2e-streams, default 6), each with its own device scratch, take the layers in turn: while one layer computes, the next
     # layer's inputs arrive over PCIe and the previous layer's results leave (the two copy directions run concurrently).
     # Layers of the same shape share a plan and may then be in flight on different streams at once, so the plans of this arm
@@ -844,6 +828,22 @@ def run_e2e(args, layers, blocks, flags, local, dev, dist, world, flops):
     for b in blocks:
         if b.shape.key not in plans:
             plans[b.shape.key] = nb.Plan.for_shape(b.shape, flags=flags | (nb.NB_CBS_FLAG_SEPARATE_FINALIZE if nstreams > 1 else 0), device=local)
+    host = {}  # per distinct shape: pinned input and output buffers (inputs filled from the device tensors)
+    scratch_bytes = 0
+    h2d = d2h = 0
+    for b in blocks:
+        s = b.shape
+        scratch_bytes = max(scratch_bytes, plans[s.key].step_host_scratch_bytes())
+        if s.key not in host:
+            pin = lambda t: torch.empty(t.shape, dtype=t.dtype).pin_memory()
+            hin = {k: pin(getattr(b, k)) for k in ("x", "w", "gamma", "beta", "g")}
+            for k, t in hin.items():
+                t.copy_(getattr(b, k))
+            hout = {k: pin(getattr(b, k)) for k in ("a", "dx", "dw", "dgamma", "dbeta")}
+            host[s.key] = (hin, hout)
+        hin, hout = host[s.key]
+        h2d += sum(t.numel() * t.element_size() for t in hin.values())
+        d2h += sum(t.numel() * t.element_size() for t in hout.values())
     scratches = [torch.empty(scratch_bytes, dtype=torch.uint8, device=dev) for _ in range(nstreams)]
     main = torch.cuda.current_stream()
     streams = [main] if nstreams == 1 else [torch.cuda.Stream(device=dev) for _ in range(nstreams)]

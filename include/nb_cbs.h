@@ -280,8 +280,15 @@ nb_status nb_bn_stats_static(const void* y, int32_t y_dtype, int64_t m, int32_t 
 /* One whole training step of the block from HOST buffers (the end-to-end path of a caller whose data
  * lives in host memory): copies host_x, host_w, host_gamma, host_beta, host_g to the device, runs the
  * forward call and the two backward calls above, and copies a, dx (unless host_dx is NULL), dw, dgamma,
- * dbeta back, all on `stream`; returns after enqueueing (host buffers should be pinned for the copies to
- * be asynchronous, and must stay valid until the stream is synchronised).  device_scratch is a device
+ * dbeta back; returns after enqueueing (host buffers should be pinned for the copies to be asynchronous,
+ * and must stay valid until the stream is synchronised).  The step takes its place on `stream` like any
+ * other call: it starts behind what is queued there, and what is queued there next finds it complete.
+ * The kernels run on `stream`.  The copies of a default plan run on two streams of the plan, one for each
+ * direction, so that they overlap one another; nb_cbs_step_host_scratch_bytes creates them (a plan that
+ * was never asked copies on `stream`).  With NB_CBS_FLAG_SEPARATE_FINALIZE every copy runs on `stream`:
+ * the choice for a caller who keeps several steps in flight on several streams, where the copies of one
+ * step overlap those of another.  When a call fails part of the way, `stream` still waits for what it
+ * has queued.  device_scratch is a device
  * buffer of at least nb_cbs_step_host_scratch_bytes() bytes, 256-byte aligned, owned by the caller; it
  * holds the device copies, the saved tensors and the workspace.  The paper has no counterpart of this
  * entry point; it exists so that the host-to-host cost of the path can be measured. */

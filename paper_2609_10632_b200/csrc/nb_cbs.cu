@@ -16,6 +16,7 @@
 
 #include "common.cuh"
 #include "elementwise.cuh"
+#include "host_step.cuh"
 #include "simt_conv.cuh"
 #include "stem_conv.cuh"
 #include "tc_conv.cuh"
@@ -108,8 +109,16 @@ struct nb_cbs_plan_s {
     unsigned long long dgrad_seq = ~0ull, dgrad_capture = 0;
     cudaStream_t dgrad_stream = nullptr;
     const void* dgrad_dy = nullptr;
-    cudaStream_t copy_in = nullptr, copy_out = nullptr;  // nb_conv_bn_silu_step_host: its copies in either direction, created on first use
-    cudaEvent_t copy_ev[4] = {};
+    // nb_conv_bn_silu_step_host: streams for its copies in either direction, one event per ordering of two of its streams.  A
+    // default plan has them from its first nb_cbs_step_host_scratch_bytes on (its calls follow one another, so that a pair of its
+    // own holds nothing up); an NB_CBS_FLAG_SEPARATE_FINALIZE plan never has, because calls of it may be in flight on several of
+    // the caller's streams, which would all queue in that one pair.  Measured, the detector's 77 layers (3.6 GB in, 3.7 GB out)
+    // with SEPARATE_FINALIZE plans on six streams: 96 ms with copy streams of the plans, 91 ms with one pair for all plans, 86.5 ms
+    // with the copies on the caller's streams; on one stream 118, 118 and 146 ms (a default plan for every layer: 118 ms, on six
+    // streams 90 ms).  One call at a time, default plan: 384 -> 384 1x1 on 16 x 40 x 40 pixels (40 MB each way) 1566 us on the
+    // caller's stream, 1227 us with copy streams; 64 -> 64 3x3 on 2 x 20 x 20 (200 KB) 106 and 85 us.
+    cudaStream_t copy_in = nullptr, copy_out = nullptr;
+    cudaEvent_t copy_ev[3][3] = {};
     double prof_ms[SITE_COUNT] = {};
     long long prof_n[SITE_COUNT] = {};
     size_t fwd_bytes, bwd_bytes;
@@ -160,6 +169,29 @@ struct SiteTimer {
     }
 };
 
+
+// The streams and events of nb_conv_bn_silu_step_host: all of them, or none when one cannot be had (the copies then take the
+// caller's stream, as they do for a plan that nobody has asked for its scratch size).
+void drop_copy_streams(nb_cbs_plan_s* p) {
+    if (p->copy_in) cudaStreamDestroy(p->copy_in);  // (work still queued completes first)
+    if (p->copy_out) cudaStreamDestroy(p->copy_out);
+    p->copy_in = p->copy_out = nullptr;
+    for (auto& row : p->copy_ev)
+        for (cudaEvent_t& e : row) {
+            if (e) cudaEventDestroy(e);
+            e = nullptr;
+        }
+}
+void make_copy_streams(nb_cbs_plan_s* p) {
+    DeviceGuard on_device(p->device);
+    bool ok = cudaStreamCreateWithFlags(&p->copy_in, cudaStreamNonBlocking) == cudaSuccess && cudaStreamCreateWithFlags(&p->copy_out, cudaStreamNonBlocking) == cudaSuccess;
+    for (int copy = HS_IN; copy <= HS_OUT; ++copy)
+        for (cudaEvent_t* e : {&p->copy_ev[HS_CALLER][copy], &p->copy_ev[copy][HS_CALLER]})
+            ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+    if (ok) return;
+    (void)cudaGetLastError();
+    drop_copy_streams(p);
+}
 
 // A launch of the plan's data gradient has just been queued.
 unsigned long long capture_id(cudaStream_t st) {
@@ -695,10 +727,7 @@ nb_status nb_cbs_plan_destroy(nb_cbs_plan p) {
         cudaFree(p->status);
         if (p->ev0) cudaEventDestroy(p->ev0);
         if (p->ev1) cudaEventDestroy(p->ev1);
-        if (p->copy_in) cudaStreamDestroy(p->copy_in);  // (work still queued completes first)
-        if (p->copy_out) cudaStreamDestroy(p->copy_out);
-        for (cudaEvent_t e : p->copy_ev)
-            if (e) cudaEventDestroy(e);
+        drop_copy_streams(p);
         cudaSetDevice(cur);
     }
     delete p;
@@ -1226,12 +1255,47 @@ StepLayout step_layout(const nb_cbs_plan_s* p) {
     L.total = off;
     return L;
 }
+
+// What host_step issues, and on what (host_step.cuh).
+struct HostStepOps {
+    nb_cbs_plan_s* p;
+    const StepLayout& L;
+    char* d;
+    cudaStream_t st[3];  // by HostStepStream
+    void* host[10] = {};  // by HostStepTensor
+    float* f32(size_t off) const { return reinterpret_cast<float*>(d + off); }
+    int order(HostStepStream from, HostStepStream to) {
+        const cudaEvent_t ev = p->copy_ev[from][to];
+        NB_CUDA_CHECK(cudaEventRecord(ev, st[from]));
+        NB_CUDA_CHECK(cudaStreamWaitEvent(st[to], ev, 0));
+        return NB_OK;
+    }
+    int copy(HostStepTensor t, HostStepStream stream) {
+        const size_t off[10] = {L.x, L.w, L.gamma, L.beta, L.g, L.a, L.dx, L.dw, L.dgamma, L.dbeta};
+        const size_t cb = (size_t)p->g.c_out * 4, bytes[10] = {L.nx, L.nw, cb, cb, L.ny_act, L.ny_act, L.nx, L.ndw, cb, cb};
+        if (t < HT_A) NB_CUDA_CHECK(cudaMemcpyAsync(d + off[t], host[t], bytes[t], cudaMemcpyHostToDevice, st[stream]));
+        else NB_CUDA_CHECK(cudaMemcpyAsync(host[t], d + off[t], bytes[t], cudaMemcpyDeviceToHost, st[stream]));
+        return NB_OK;
+    }
+    int forward() {
+        return nb_conv_bn_silu_fwd(p, d + L.x, d + L.w, f32(L.gamma), f32(L.beta), nullptr, nullptr, d + L.y, f32(L.mean), f32(L.invstd), d + L.a, d + L.ws_fwd,
+                                   p->fwd_bytes, st[HS_CALLER]);
+    }
+    int backward_data() {
+        return nb_conv_bn_silu_bwd_data(p, d + L.g, d + L.y, f32(L.mean), f32(L.invstd), f32(L.gamma), f32(L.beta), d + L.w, host[HT_DX] ? d + L.dx : nullptr,
+                                        f32(L.dgamma), f32(L.dbeta), d + L.dy, d + L.ws_bwd, p->bwd_bytes, st[HS_CALLER]);
+    }
+    int backward_weight() {
+        return nb_conv_bn_silu_bwd_weight(p, d + L.x, d + L.dy, f32(L.dw), d + L.ws_bwd, p->bwd_bytes, st[HS_CALLER]);
+    }
+};
 }  // namespace
 
 nb_status nb_cbs_step_host_scratch_bytes(nb_cbs_plan p, size_t* bytes) {
     g_err.clear();
     if (!p || !bytes) return fail(NB_ERR_INVALID_ARG, "NULL argument");
     *bytes = step_layout(p).total;
+    if (p->fuse_finalize && !p->copy_in) make_copy_streams(p);
     return NB_OK;
 }
 
@@ -1246,49 +1310,12 @@ nb_status nb_conv_bn_silu_step_host(nb_cbs_plan p, const void* host_x, const voi
     const StepLayout L = step_layout(p);
     NB_TRY(check_ws(device_scratch, scratch_bytes, L.total));
     DeviceGuard on_device(p->device);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    char* d = static_cast<char*>(device_scratch);
-    const size_t cb = (size_t)p->g.c_out * 4;
-    // PCIe moves data both ways at once: the copies run on two streams of the plan, so that g travels in while a travels
-    // out, and dx goes out while the weight gradient is computed.  On one stream every byte of either direction waits for
-    // every other.  Measured: 384 -> 384 1x1 on 16 x 40 x 40 pixels (40 MB each way) 1548 -> 1230 us (x in, then a and dx out
-    // is what the data dependence leaves), 64 -> 64 3x3 on 2 x 20 x 20 pixels (200 KB) 101 -> 83 us.
-    if (!p->copy_in) NB_CUDA_CHECK(cudaStreamCreateWithFlags(&p->copy_in, cudaStreamNonBlocking));
-    if (!p->copy_out) NB_CUDA_CHECK(cudaStreamCreateWithFlags(&p->copy_out, cudaStreamNonBlocking));
-    for (cudaEvent_t& e : p->copy_ev)
-        if (!e) NB_CUDA_CHECK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    const cudaStream_t in = p->copy_in, out = p->copy_out;
-    // `to` continues behind everything queued on `from` so far
-    auto order = [&](int event, cudaStream_t from, cudaStream_t to) {
-        const cudaError_t e = cudaEventRecord(p->copy_ev[event], from);
-        return e != cudaSuccess ? e : cudaStreamWaitEvent(to, p->copy_ev[event], 0);
-    };
-    NB_CUDA_CHECK(order(0, st, in));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.w, host_w, L.nw, cudaMemcpyHostToDevice, in));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.gamma, host_gamma, cb, cudaMemcpyHostToDevice, in));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.beta, host_beta, cb, cudaMemcpyHostToDevice, in));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.x, host_x, L.nx, cudaMemcpyHostToDevice, in));
-    NB_CUDA_CHECK(order(1, in, st));
-    NB_CUDA_CHECK(cudaMemcpyAsync(d + L.g, host_g, L.ny_act, cudaMemcpyHostToDevice, in));
-    float* gam = reinterpret_cast<float*>(d + L.gamma);
-    float* bet = reinterpret_cast<float*>(d + L.beta);
-    float* mean = reinterpret_cast<float*>(d + L.mean);
-    float* invstd = reinterpret_cast<float*>(d + L.invstd);
-    NB_TRY(nb_conv_bn_silu_fwd(p, d + L.x, d + L.w, gam, bet, nullptr, nullptr, d + L.y, mean, invstd, d + L.a, d + L.ws_fwd, p->fwd_bytes, stream));
-    NB_CUDA_CHECK(order(2, st, out));
-    NB_CUDA_CHECK(cudaMemcpyAsync(host_a, d + L.a, L.ny_act, cudaMemcpyDeviceToHost, out));
-    NB_CUDA_CHECK(order(3, in, st));
-    NB_TRY(nb_conv_bn_silu_bwd_data(p, d + L.g, d + L.y, mean, invstd, gam, bet, d + L.w, host_dx ? d + L.dx : nullptr,
-                                    reinterpret_cast<float*>(d + L.dgamma), reinterpret_cast<float*>(d + L.dbeta), d + L.dy,
-                                    d + L.ws_bwd, p->bwd_bytes, stream));
-    NB_CUDA_CHECK(order(0, st, out));
-    if (host_dx) NB_CUDA_CHECK(cudaMemcpyAsync(host_dx, d + L.dx, L.nx, cudaMemcpyDeviceToHost, out));
-    NB_CUDA_CHECK(cudaMemcpyAsync(host_dgamma, d + L.dgamma, cb, cudaMemcpyDeviceToHost, out));
-    NB_CUDA_CHECK(cudaMemcpyAsync(host_dbeta, d + L.dbeta, cb, cudaMemcpyDeviceToHost, out));
-    NB_TRY(nb_conv_bn_silu_bwd_weight(p, d + L.x, d + L.dy, reinterpret_cast<float*>(d + L.dw), d + L.ws_bwd, p->bwd_bytes, stream));
-    NB_CUDA_CHECK(cudaMemcpyAsync(host_dw, d + L.dw, L.ndw, cudaMemcpyDeviceToHost, st));
-    NB_CUDA_CHECK(order(1, out, st));
-    return NB_OK;
+    HostStepOps ops{p, L, static_cast<char*>(device_scratch), {static_cast<cudaStream_t>(stream), p->copy_in, p->copy_out}};
+    ops.host[HT_X] = const_cast<void*>(host_x); ops.host[HT_W] = const_cast<void*>(host_w); ops.host[HT_G] = const_cast<void*>(host_g);
+    ops.host[HT_GAMMA] = const_cast<float*>(host_gamma); ops.host[HT_BETA] = const_cast<float*>(host_beta);
+    ops.host[HT_A] = host_a; ops.host[HT_DX] = host_dx; ops.host[HT_DW] = host_dw;
+    ops.host[HT_DGAMMA] = host_dgamma; ops.host[HT_DBETA] = host_dbeta;
+    return host_step(ops, p->copy_in != nullptr, host_dx != nullptr);
 }
 
 }  // extern "C"
