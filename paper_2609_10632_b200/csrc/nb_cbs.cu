@@ -555,6 +555,7 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     if (!(d->momentum >= 0.f && d->momentum <= 1.f)) return fail(NB_ERR_INVALID_ARG, "momentum must be in [0,1]");
     const int vec = d->mode == NB_MODE_F32_REF ? 4 : 8;
     if (d->c_out % vec) return fail(NB_ERR_UNSUPPORTED, "c_out=%d must be a multiple of %d in this mode", d->c_out, vec);
+    static_assert(288 * 8 <= SG_REDUCE_MAX * 4, "a block of splitk_fwd_reduce_kernel spans the channels of a row");
     if (d->c_out / vec > 288) return fail(NB_ERR_UNSUPPORTED, "c_out=%d is too large (at most %d channels in this mode)", d->c_out, 288 * vec);
 
     Geom g;

@@ -425,8 +425,11 @@ __global__ void __launch_bounds__(SG_THREADS) simt_gemm_kernel(const TIN* __rest
 
 // out = sum over the slices of a split forward convolution (fp64, slice order), rounded to YT, and with acc.acc != NULL the
 // channel sums of the stored values (a thread keeps one group of four channels, like the elementwise passes).
+// A block is at least one row of channel groups: 288 at the 1152 channels that a plan may have in fp32, 576 at the 2304 of the
+// 16-bit modes.
+constexpr int SG_REDUCE_MAX = 576;
 template <typename YT>
-__global__ void __launch_bounds__(256) splitk_fwd_reduce_kernel(const float* __restrict__ partial, int splits, long long vecs, int C, YT* __restrict__ out, ChanAcc acc) {
+__global__ void __launch_bounds__(SG_REDUCE_MAX) splitk_fwd_reduce_kernel(const float* __restrict__ partial, int splits, long long vecs, int C, YT* __restrict__ out, ChanAcc acc) {
     pdl_launch_dependents();
     pdl_wait();
     extern __shared__ float red[];  // [blockDim.x][4]

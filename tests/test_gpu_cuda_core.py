@@ -4,7 +4,8 @@ channels (no vector loads), every parity class of a stride-2 data gradient, a 1x
 import pytest
 
 from paper_2609_10632_b200 import workloads as wl
-from tests.test_gpu_parity import _compare, _oracle, _run_block
+from tests import parity
+from tests.test_gpu_parity import EPS, _compare, _oracle, _run_block
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +35,28 @@ def test_cuda_core_convolutions_match_oracle(mode, dims):
         assert not out["dx"][:, 1::2].any() and not out["dx"][:, :, 1::2].any()
         out["dx"], ref.dx = out["dx"][:, ::2, ::2], ref.dx[:, ::2, ::2]
     _compare(out, ref, 1 if f32 else 0)
+
+
+WIDE = [("f32", (1, 20, 20, 256, 1152, 3, 1)), ("f32", (1, 10, 11, 32, 1028, 3, 1)), ("bf16", (1, 12, 12, 40, 1280, 3, 1)), ("bf16", (1, 12, 12, 32, 2304, 3, 1))]
+
+
+@pytest.mark.parametrize("mode,dims", WIDE, ids=lambda v: v if isinstance(v, str) else "x".join(map(str, v)))
+def test_forward_slices_of_more_than_1024_channels(mode, dims):
+    """Rows wider than 256 groups of four channels, up to the widest a plan may have: the pass that adds the slices of a split
+    forward convolution has a thread for every group, in training (with the channel sums) and in evaluation mode."""
+    import torch
+
+    import oracle
+    from paper_2609_10632_b200 import binding as nb
+
+    shape = wl.ConvShape("wide", *dims)
+    f32 = mode == "f32"
+    inp, blk, out = _run_block(shape, nb.NB_MODE_F32_REF if f32 else nb.NB_MODE_BF16_TC, cfg_id=43, layer_id=WIDE.index((mode, dims)), affine="random",
+                               flags=0 if f32 else nb.NB_CBS_FLAG_FORCE_SIMT)
+    assert blk.plan.paths["fprop"] == 0
+    _compare(out, _oracle(inp), 1 if f32 else 0)
+    rm, rv, _ = wl.make_eval_stats(shape, 43, 0)
+    up = lambda a: torch.from_numpy(a).to(blk.dev)
+    a, ws = torch.empty_like(blk.a), torch.empty(blk.plan.infer_bytes, dtype=torch.uint8, device=blk.dev)
+    nb.nb_conv_bn_silu_infer(blk.plan, blk.x, blk.w, blk.gamma, blk.beta, up(rm), up(rv), a, ws)
+    parity.check("a_eval", a.double().cpu().numpy(), oracle.cbs_infer(inp.x, inp.w, inp.gamma, inp.beta, rm, rv, shape.stride, EPS), "f32" if f32 else "bf16")
