@@ -438,6 +438,7 @@ SgCfg sg_configure(const Geom& g, int kind, bool f32, int sm_count) {
         if (tiles <= 2 * sm_count) splits = std::max<long long>(1, std::min<long long>(6LL * sm_count / tiles, most));
         const long long flush_free = (KK + 1023) / 1024;
         if (splits < flush_free && (size_t)flush_free * out * 4 <= (size_t)128 << 20) splits = flush_free;
+        splits = std::min<long long>(splits, 65535);  // (slices are gridDim.z: 8 -> 8 1x1 has 65536 of 1024 pixels at 67.1 million)
     }
     c.kchunk = ((KK + splits - 1) / splits + SG_BK - 1) / SG_BK * SG_BK;
     c.splits = (int)((KK + c.kchunk - 1) / c.kchunk);

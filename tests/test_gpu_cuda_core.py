@@ -60,3 +60,26 @@ def test_forward_slices_of_more_than_1024_channels(mode, dims):
     a, ws = torch.empty_like(blk.a), torch.empty(blk.plan.infer_bytes, dtype=torch.uint8, device=blk.dev)
     nb.nb_conv_bn_silu_infer(blk.plan, blk.x, blk.w, blk.gamma, blk.beta, up(rm), up(rv), a, ws)
     parity.check("a_eval", a.double().cpu().numpy(), oracle.cbs_infer(inp.x, inp.w, inp.gamma, inp.beta, rm, rv, shape.stride, EPS), "f32" if f32 else "bf16")
+
+
+def test_weight_gradient_of_more_pixels_than_the_grid_has_slices_for():
+    """8 -> 8 1x1 in fp32 on 64 x 1024 x 1024 pixels: 65536 slices of 1024 pixels would be one more than a grid may have; the
+    kernel takes longer slices (flushed to fp64).  The step against fp64 sums over the kernel's own dy."""
+    import torch
+
+    from paper_2609_10632_b200 import binding as nb
+    from paper_2609_10632_b200.block import CbsBlock
+
+    shape = wl.ConvShape("pixels", 64, 1024, 1024, 8, 8, 1, 1)
+    blk = CbsBlock(shape, mode=nb.NB_MODE_F32_REF)
+    blk.fill_random(5)
+    blk.step()
+    blk.poll()
+    m = shape.m
+    x, dy = blk.x.view(m, 8), blk.dy.view(m, 8)
+    dw = sum(dy[i:i + m // 16].double().t() @ x[i:i + m // 16].double() for i in range(0, m, m // 16))
+    # fp32 sums of up to 1024 products of random sign: 1024 roundings of 2^-24 of partial sums up to 32 products large are 6e-5
+    # of a product's size together, in each of 65536 slices, 1.5e-2 in all; the sum is sqrt(m) = 8192 products large: 2e-6
+    scale = float(dy[:m // 16].double().pow(2).mean().sqrt() * x[:m // 16].double().pow(2).mean().sqrt()) * m ** 0.5
+    err = (blk.dw.view(8, 8).double() - dw).abs().max().item()
+    assert err <= 1e-5 * scale, (err, scale)
