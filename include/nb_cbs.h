@@ -53,8 +53,9 @@
 extern "C" {
 #endif
 
-#define NB_CBS_ABI_VERSION 3u /* 2: adds the evaluation-mode / plain calls (additive); 3: flag 2 is NB_CBS_FLAG_SEPARATE_FINALIZE,
-                                  the grid-barrier test hook is gone with the barriers, nb_cbs_plan_set_bwd_residual is new */
+#define NB_CBS_ABI_VERSION 4u /* 2: adds the evaluation-mode / plain calls (additive); 3: flag 2 is NB_CBS_FLAG_SEPARATE_FINALIZE,
+                                  the grid-barrier test hook is gone with the barriers, nb_cbs_plan_set_bwd_residual is new;
+                                  4: adds nb_conv_bn_silu_bwd (additive) */
 
 typedef int32_t nb_status;
 enum {
@@ -214,6 +215,14 @@ nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan plan, const void* g, const void* 
  * dy is the tensor nb_conv_bn_silu_bwd_data wrote to dy_out (ordering on the stream is the caller's). */
 nb_status nb_conv_bn_silu_bwd_weight(nb_cbs_plan plan, const void* x, const void* dy, float* dw, void* workspace,
                                      size_t workspace_bytes, void* stream);
+
+/* The two backward calls above in one, with the same results: nb_conv_bn_silu_bwd_data, then nb_conv_bn_silu_bwd_weight of
+ * its dy_out.  Both gradients read dy and neither reads what the other writes; the call, which knows that nothing comes
+ * between them, lets the second run beside the first. */
+nb_status nb_conv_bn_silu_bwd(nb_cbs_plan plan, const void* x, const void* g, const void* y_saved, const float* save_mean,
+                              const float* save_invstd, const float* gamma, const float* beta, const void* w, void* dx,
+                              float* dw, float* dgamma, float* dbeta, void* dy_out, void* workspace, size_t workspace_bytes,
+                              void* stream);
 
 /* ---- Evaluation-mode and plain variants of the block (inference; nothing is saved, nothing is updated) ----
  * The paper's reproduction protocol found that validation must normalise with the RUNNING statistics (Table 2 row 9),

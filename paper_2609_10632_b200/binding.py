@@ -24,7 +24,7 @@ NB_CBS_FLAG_SEPARATE_FINALIZE = 2
 EXPORTS = (
     "nb_abi_version", "nb_last_error", "nb_cbs_plan_create", "nb_cbs_plan_destroy", "nb_cbs_out_shape",
     "nb_cbs_workspace_bytes", "nb_cbs_plan_paths", "nb_cbs_poll_status", "nb_conv_bn_silu_fwd", "nb_bn_stats",
-    "nb_conv_bn_silu_bwd_data", "nb_conv_bn_silu_bwd_weight", "nb_cbs_step_host_scratch_bytes",
+    "nb_conv_bn_silu_bwd_data", "nb_conv_bn_silu_bwd_weight", "nb_conv_bn_silu_bwd", "nb_cbs_step_host_scratch_bytes",
     "nb_conv_bn_silu_step_host", "nb_cbs_launch_count", "nb_cbs_profile_enable", "nb_cbs_profile_site_name",
     "nb_cbs_profile_read", "nb_bn_stats_static", "nb_cbs_infer_workspace_bytes", "nb_conv_bn_silu_infer", "nb_conv_bias_act",
     "nb_bn_fold", "nb_sgd_plan_create", "nb_sgd_plan_destroy", "nb_sgd_workspace_bytes", "nb_sgd_upload", "nb_sgd_clip_nesterov_step", "nb_sgd_clip_nesterov_step_scaled",
@@ -90,6 +90,7 @@ def load() -> ctypes.CDLL:
         lib.nb_bn_stats.argtypes = [V, V, c_int32, FP, FP, FP, FP, V, c_size_t, V]
         lib.nb_conv_bn_silu_bwd_data.argtypes = [V, V, V, FP, FP, FP, FP, V, V, FP, FP, V, V, c_size_t, V]
         lib.nb_conv_bn_silu_bwd_weight.argtypes = [V, V, V, FP, V, c_size_t, V]
+        lib.nb_conv_bn_silu_bwd.argtypes = [V, V, V, V, FP, FP, FP, FP, V, V, FP, FP, FP, V, V, c_size_t, V]
         lib.nb_cbs_step_host_scratch_bytes.argtypes = [V, POINTER(c_size_t)]
         lib.nb_conv_bn_silu_step_host.argtypes = [V, V, V, FP, FP, V, V, V, FP, FP, FP, V, c_size_t, V]
         lib.nb_bn_stats_static.argtypes = [V, c_int32, ctypes.c_int64, c_int32, c_float, FP, FP, FP, FP, V]
@@ -297,6 +298,14 @@ def nb_conv_bn_silu_bwd_data(plan: Plan, g, y_saved, save_mean, save_invstd, gam
 def nb_conv_bn_silu_bwd_weight(plan: Plan, x, dy, dw, workspace, stream=None):
     _check(load().nb_conv_bn_silu_bwd_weight(plan.handle, _ptr(x), _ptr(dy), _ptr(dw), _ptr(workspace), _nbytes(workspace),
                                              _stream(stream)))
+
+
+def nb_conv_bn_silu_bwd(plan: Plan, x, g, y_saved, save_mean, save_invstd, gamma, beta, w, dx, dw, dgamma, dbeta, dy_out, workspace,
+                        stream=None):
+    """The data-gradient and the weight-gradient call in one."""
+    _check(load().nb_conv_bn_silu_bwd(plan.handle, _ptr(x), _ptr(g), _ptr(y_saved), _ptr(save_mean), _ptr(save_invstd), _ptr(gamma),
+                                      _ptr(beta), _ptr(w), _ptr(dx), _ptr(dw), _ptr(dgamma), _ptr(dbeta), _ptr(dy_out), _ptr(workspace),
+                                      _nbytes(workspace), _stream(stream)))
 
 
 def nb_conv_bn_silu_infer(plan: Plan, x, w, gamma, beta, running_mean, running_var, a_out, workspace, stream=None):

@@ -65,22 +65,18 @@ class C2fChain:
     def backward(self, stream=None):
         """Expects cv2.g = dL/d out.  Leaves dL/dx in cv1.dx and every block's dw, dgamma, dbeta in the block."""
         c, ct = self.c, self.ctot
-        self.cv2.backward_data(stream)
-        self.cv2.backward_weight(stream)
+        self.cv2.backward(stream)
         for i in reversed(range(self.n)):
             b1, b2 = self.m[i]
             self._add(b2.g, c, self._slice(self.dcat, (2 + i) * c), ct, c, stream=stream)  # dense copy of this part's gradient
-            b2.backward_data(stream)
-            b2.backward_weight(stream)
-            b1.backward_data(stream)
-            b1.backward_weight(stream)
+            b2.backward(stream)
+            b1.backward(stream)
             if self.shortcut:
                 self._add(self._slice(self.dcat, (1 + i) * c), ct, b1.dx, c, c, b=self._slice(self.dcat, (2 + i) * c), ld_b=ct, accumulate=True, stream=stream)
             else:
                 self._add(self._slice(self.dcat, (1 + i) * c), ct, b1.dx, c, c, accumulate=True, stream=stream)
         self._add(self.cv1.g, 2 * c, self._slice(self.dcat, 0), ct, 2 * c, stream=stream)
-        self.cv1.backward_data(stream)
-        self.cv1.backward_weight(stream)
+        self.cv1.backward(stream)
 
     def poll(self):
         for b in self.blocks:
@@ -125,15 +121,13 @@ class SppfChain:
 
     def backward(self, stream=None):
         n, h, w, c = self.dims
-        self.cv2.backward_data(stream)
-        self.cv2.backward_weight(stream)
+        self.cv2.backward(stream)
         for j in range(4):
             nb.nb_slice_add(nb.NB_DTYPE_BF16, self.rows, c, self.dpart[j], c, self._slice(self.dcat, j * c), 4 * c, stream=stream)
         for j in (3, 2, 1):  # part j = pool(part j-1)
             nb.nb_maxpool5_bwd(nb.NB_DTYPE_BF16, n, h, w, c, self.dpart[j], self.idx[j - 1], self.dpart[j - 1], True, stream)
         self.cv1.g = self.dpart[0]
-        self.cv1.backward_data(stream)
-        self.cv1.backward_weight(stream)
+        self.cv1.backward(stream)
 
     def poll(self):
         for b in self.blocks:

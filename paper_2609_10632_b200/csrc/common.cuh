@@ -250,8 +250,9 @@ static __global__ void dgrad_weight_transform_kernel(const __nv_bfloat16* __rest
 // cannot start before dy is complete; and (ii) a weight-gradient kernel that the host knows to be the very next launch on the
 // stream executes its griddepcontrol.wait at its END instead of before its first load.  It still completes after the data
 // gradient, so that "the previous kernel has completed" keeps meaning "all earlier ones have" for everything behind it.
-// The host knows (nb_cbs.cu, follows_dgrad): same plan, stream and dy, and no launch of the library in between.  Anything
-// else that the caller may have queued in between ends completely before the weight gradient starts.
-// Measured: see follows_dgrad.
+// The host knows only where one call of the library queues both (nb_conv_bn_silu_bwd, nb_conv_bias_bwd): between two calls the
+// caller may have queued a kernel that writes dy or x, and a kernel that signals its dependents early at that.
+// Measured (step): 16 -> 88 3x3 f16 on 14 x 55 x 8 pixels 41.2 -> 35.6 us, 336 -> 392 on 21 x 18 53.7 -> 45.4, 40 -> 336 on
+// 4 x 87 x 130 184 -> 177, 384 -> 384 1x1 on 16 x 40 x 40 82.7 -> 80.9, 192 -> 384 stride 2 on 16 x 80 x 80 154 -> 151.
 
 }  // namespace nbcbs

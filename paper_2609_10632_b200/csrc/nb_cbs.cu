@@ -105,10 +105,6 @@ struct nb_cbs_plan_s {
     int stem_dgrad_rows = 0;    // output row pairs per block
     bool profiling = false;  // when set, every kernel site is bracketed by events and the call waits for it
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    // the last data-gradient launch: the library's launch count behind it, its stream, capture and dy (see follows_dgrad)
-    unsigned long long dgrad_seq = ~0ull, dgrad_capture = 0;
-    cudaStream_t dgrad_stream = nullptr;
-    const void* dgrad_dy = nullptr;
     // nb_conv_bn_silu_step_host: streams for its copies in either direction, one event per ordering of two of its streams.  A
     // default plan has them from its first nb_cbs_step_host_scratch_bytes on (its calls follow one another, so that a pair of its
     // own holds nothing up); an NB_CBS_FLAG_SEPARATE_FINALIZE plan never has, because calls of it may be in flight on several of
@@ -191,31 +187,6 @@ void make_copy_streams(nb_cbs_plan_s* p) {
     if (ok) return;
     (void)cudaGetLastError();
     drop_copy_streams(p);
-}
-
-// A launch of the plan's data gradient has just been queued.
-unsigned long long capture_id(cudaStream_t st) {
-    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-    unsigned long long id = 0;
-    if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ~0ull;  // (equal to nothing: see follows_dgrad)
-    }
-    return status == cudaStreamCaptureStatusActive ? id : 0;
-}
-void note_dgrad(nb_cbs_plan_s* p, const void* dy, cudaStream_t st) {
-    p->dgrad_seq = g_launches.load(std::memory_order_relaxed);
-    p->dgrad_stream = st;
-    p->dgrad_dy = dy;
-    p->dgrad_capture = capture_id(st);
-}
-// The weight gradient about to be launched is the library's next launch behind this plan's data gradient of the same dy, on
-// the same stream (and in the same stream capture, if any): it may run beside it (see the end of common.cuh).
-// Measured (step): 16 -> 88 3x3 f16 on 14 x 55 x 8 pixels 41.2 -> 35.6 us, 336 -> 392 on 21 x 18 53.7 -> 45.4, 40 -> 336 on
-// 4 x 87 x 130 184 -> 177, 384 -> 384 1x1 on 16 x 40 x 40 82.7 -> 80.9, 192 -> 384 stride 2 on 16 x 80 x 80 154 -> 151.
-bool follows_dgrad(const nb_cbs_plan_s* p, const void* dy, cudaStream_t st) {
-    return pdl_enabled() && p->dgrad_dy == dy && p->dgrad_stream == st && p->dgrad_seq == g_launches.load(std::memory_order_relaxed) &&
-           p->dgrad_capture != ~0ull && p->dgrad_capture == capture_id(st);
 }
 
 // ---------------------------------------------------------------- elementwise launch helpers
@@ -976,7 +947,7 @@ nb_status nb_conv_bn_silu_infer(nb_cbs_plan p, const void* x, const void* w, con
     if (!p) return fail(NB_ERR_INVALID_ARG, "plan is NULL");
     NB_CHECK_PTR(x); NB_CHECK_PTR(w); NB_CHECK_PTR(gamma); NB_CHECK_PTR(beta); NB_CHECK_PTR(running_mean); NB_CHECK_PTR(running_var);
     NB_CHECK_PTR(a_out);
-    if (p->pitched || p->fwd_res) return fail(NB_ERR_UNSUPPORTED, "the plan has row pitches or a residual set: only the three training calls honour them");
+    if (p->pitched || p->fwd_res) return fail(NB_ERR_UNSUPPORTED, "the plan has row pitches or a residual set: only the training calls honour them");
     NB_TRY(check_ws(workspace, workspace_bytes, p->infer_bytes));
     DeviceGuard on_device(p->device);
     return run_infer(p, x, w, gamma, beta, running_mean, running_var, 1, a_out, static_cast<char*>(workspace), static_cast<cudaStream_t>(stream));
@@ -988,7 +959,7 @@ nb_status nb_conv_bias_act(nb_cbs_plan p, const void* x, const void* w, const fl
     if (!p) return fail(NB_ERR_INVALID_ARG, "plan is NULL");
     NB_CHECK_PTR(x); NB_CHECK_PTR(w); NB_CHECK_PTR(bias, true); NB_CHECK_PTR(out);
     if (act != 0 && act != 1) return fail(NB_ERR_INVALID_ARG, "act must be 0 (none) or 1 (SiLU), got %d", act);
-    if (p->pitched || p->fwd_res) return fail(NB_ERR_UNSUPPORTED, "the plan has row pitches or a residual set: only the three training calls honour them");
+    if (p->pitched || p->fwd_res) return fail(NB_ERR_UNSUPPORTED, "the plan has row pitches or a residual set: only the training calls honour them");
     NB_TRY(check_ws(workspace, workspace_bytes, p->infer_bytes));
     DeviceGuard on_device(p->device);
     return run_infer(p, x, w, nullptr, bias, nullptr, nullptr, act, out, static_cast<char*>(workspace), static_cast<cudaStream_t>(stream));
@@ -1034,6 +1005,52 @@ nb_status nb_bn_stats(nb_cbs_plan p, const void* y, int32_t y_dtype, float* mean
     return run_finalize(p, part, p->ew.blocks_stats, nullptr, nullptr, mean, invstd, nullptr, nullptr, nullptr, nullptr, sum, sumsq, st);
 }
 
+namespace {
+// dx from dy, the last step of a call or in front of the weight gradient.  rearranged: the pass that made dy has rearranged the
+// filter for the tensor-core kernel; else that is done here.
+nb_status run_dgrad(nb_cbs_plan_s* p, const void* dy, const void* w, void* dx, char* ws, bool rearranged, cudaStream_t st) {
+    if (is_f32(p)) return run_simt_dgrad<float>(p, dy, w, dx, ws + p->off_dgpart, st);
+    if (p->stem) {
+        SiteTimer tm(p, SITE_DGRAD, st);
+        return NB_WITH_AT(p, run_stem_dgrad<AT>(p, dy, w, dx, st));
+    }
+    if (p->tc.dgrad) {
+        SiteTimer tm(p, SITE_DGRAD, st);
+        const long long l0 = p->tc.launches;
+        const nb_status ts = tc_dgrad(&p->tc, p->g, dy, w, dx, ws + p->off_wt, p->status, st, rearranged, p->ld_dx, p->dx_accumulate);
+        g_launches.fetch_add((unsigned long long)(p->tc.launches - l0), std::memory_order_relaxed);
+        return ts == NB_OK ? NB_OK : fail(ts, "%s", tc_last_error());
+    }
+    return NB_WITH_AT(p, run_simt_dgrad<AT>(p, dy, w, dx, ws + p->off_dgpart, st));
+}
+
+// overlap: the launch in front of this one on the stream is this layer's data gradient (see the end of common.cuh).  Only a
+// caller that has just queued it itself, in the same call of the library, can say so.
+nb_status run_wgrad(nb_cbs_plan_s* p, const void* x, const void* dy, float* dw, char* ws, bool overlap, cudaStream_t st) {
+    float* partial = reinterpret_cast<float*>(ws + p->off_wgpart);
+    overlap = overlap && pdl_enabled();
+    if (is_f32(p)) return run_simt_wgrad<float>(p, x, dy, dw, partial, overlap, st);
+    if (p->stem) {
+        {
+            SiteTimer tm(p, SITE_WGRAD, st);
+            NB_TRY(NB_WITH_AT(p, run_stem_wgrad<AT>(p, x, dy, partial, overlap, st)));
+        }
+        const size_t elems = (size_t)p->g.c_out * p->g.kdim;
+        SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
+        launch_k(splitk_reduce_tall_kernel, dim3((unsigned)((elems + 31) / 32)), dim3(1024), 0, st, 1, partial, p->stem_wgrad_blocks, elems, dw);
+        return launch_ok("splitk_reduce");
+    }
+    if (p->tc.wgrad) {
+        SiteTimer tm(p, SITE_WGRAD, st);
+        const long long l0 = p->tc.launches;
+        const nb_status ts = tc_wgrad(&p->tc, p->g, x, dy, dw, partial, p->status, st, overlap);
+        g_launches.fetch_add((unsigned long long)(p->tc.launches - l0), std::memory_order_relaxed);
+        return ts == NB_OK ? NB_OK : fail(ts, "%s", tc_last_error());
+    }
+    return NB_WITH_AT(p, run_simt_wgrad<AT>(p, x, dy, dw, partial, overlap, st));
+}
+}  // namespace
+
 nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan p, const void* g, const void* y_saved, const float* save_mean,
                                    const float* save_invstd, const float* gamma, const float* beta, const void* w, void* dx,
                                    float* dgamma, float* dbeta, void* dy_out, void* workspace, size_t workspace_bytes, void* stream) {
@@ -1051,75 +1068,12 @@ nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan p, const void* g, const void* y_s
     float* part = reinterpret_cast<float*>(ws + p->off_bpart);
     if (is_f32(p)) {
         NB_TRY((run_bwd_elementwise<float, float, false>(p, g, y_saved, save_mean, save_invstd, gamma, beta, dgamma, dbeta, dy_out, part, coef, st)));
-        if (!dx) return NB_OK;
-        NB_TRY(run_simt_dgrad<float>(p, dy_out, w, dx, ws + p->off_dgpart, st));
-        note_dgrad(p, dy_out, st);
-        return NB_OK;
+    } else {
+        const bool tc_dg = dx && !p->stem && p->tc.dgrad;  // the finalize kernel also rearranges the filter for the tensor-core dgrad
+        NB_TRY(NB_WITH_AT(p, run_bwd_elementwise<__half, AT, true>(p, g, y_saved, save_mean, save_invstd, gamma, beta, dgamma, dbeta, dy_out, part, coef, st,
+                                                                   tc_dg ? w : nullptr, tc_dg ? ws + p->off_wt : nullptr, tc_dg ? &p->tc.wtp : nullptr)));
     }
-    const bool tc_dg = dx && !p->stem && p->tc.dgrad;  // the finalize kernel also rearranges the filter for the tensor-core dgrad
-    NB_TRY(NB_WITH_AT(p, run_bwd_elementwise<__half, AT, true>(p, g, y_saved, save_mean, save_invstd, gamma, beta, dgamma, dbeta, dy_out, part, coef, st,
-                                                               tc_dg ? w : nullptr, tc_dg ? ws + p->off_wt : nullptr, tc_dg ? &p->tc.wtp : nullptr)));
-    if (!dx) return NB_OK;
-    if (p->stem) {
-        SiteTimer tm(p, SITE_DGRAD, st);
-        NB_TRY(NB_WITH_AT(p, run_stem_dgrad<AT>(p, dy_out, w, dx, st)));
-        note_dgrad(p, dy_out, st);
-        return NB_OK;
-    }
-    if (p->tc.dgrad) {
-        SiteTimer tm(p, SITE_DGRAD, st);
-        const long long l0 = p->tc.launches;
-        const nb_status ts = tc_dgrad(&p->tc, p->g, dy_out, w, dx, ws + p->off_wt, p->status, st, true, p->ld_dx, p->dx_accumulate);
-        g_launches.fetch_add((unsigned long long)(p->tc.launches - l0), std::memory_order_relaxed);
-        if (ts != NB_OK) return fail(ts, "%s", tc_last_error());
-        note_dgrad(p, dy_out, st);
-        return NB_OK;
-    }
-    NB_TRY(NB_WITH_AT(p, run_simt_dgrad<AT>(p, dy_out, w, dx, ws + p->off_dgpart, st)));
-    note_dgrad(p, dy_out, st);
-    return NB_OK;
-}
-
-nb_status nb_conv_bias_bwd(nb_cbs_plan p, const void* x, const void* w, const void* dout, void* dx, float* dw, float* dbias, void* workspace,
-                           size_t workspace_bytes, void* stream) {
-    g_err.clear();
-    if (!p) return fail(NB_ERR_INVALID_ARG, "plan is NULL");
-    NB_CHECK_PTR(x); NB_CHECK_PTR(dout); NB_CHECK_PTR(dw); NB_CHECK_PTR(dx, true); NB_CHECK_PTR(dbias, true);
-    if (dx) NB_CHECK_PTR(w);
-    if (p->pitched || p->ld_dx || p->dx_accumulate || p->fwd_res || p->bwd_gres) return fail(NB_ERR_UNSUPPORTED, "the plan has row pitches, a dx target or a residual set: only the three training calls honour them");
-    NB_TRY(check_ws(workspace, workspace_bytes, p->bwd_bytes));
-    {
-        DeviceGuard on_device(p->device);
-        cudaStream_t st = static_cast<cudaStream_t>(stream);
-        char* ws = static_cast<char*>(workspace);
-        if (dbias) {  // column sums of dout: the statistics kernels with only the raw sum requested
-            float* part = reinterpret_cast<float*>(ws + p->off_bpart);
-            if (is_f32(p)) NB_TRY(run_stats_partial<float>(p, dout, part, st));
-            else NB_TRY(NB_WITH_AT(p, run_stats_partial<AT>(p, dout, part, st)));
-            NB_TRY(run_finalize(p, part, p->ew.blocks_stats, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, dbias, nullptr, st));
-        }
-        if (dx) {
-            if (is_f32(p)) {
-                NB_TRY(run_simt_dgrad<float>(p, dout, w, dx, ws + p->off_dgpart, st));
-                note_dgrad(p, dout, st);
-            } else if (p->stem) {
-                SiteTimer tm(p, SITE_DGRAD, st);
-                NB_TRY(NB_WITH_AT(p, run_stem_dgrad<AT>(p, dout, w, dx, st)));
-                note_dgrad(p, dout, st);
-            } else if (p->tc.dgrad) {
-                SiteTimer tm(p, SITE_DGRAD, st);
-                const long long l0 = p->tc.launches;
-                const nb_status ts = tc_dgrad(&p->tc, p->g, dout, w, dx, ws + p->off_wt, p->status, st, false);  // rearranges the filter itself
-                g_launches.fetch_add((unsigned long long)(p->tc.launches - l0), std::memory_order_relaxed);
-                if (ts != NB_OK) return fail(ts, "%s", tc_last_error());
-                note_dgrad(p, dout, st);
-            } else {
-                NB_TRY(NB_WITH_AT(p, run_simt_dgrad<AT>(p, dout, w, dx, ws + p->off_dgpart, st)));
-                note_dgrad(p, dout, st);
-            }
-        }
-    }
-    return nb_conv_bn_silu_bwd_weight(p, x, dout, dw, workspace, workspace_bytes, stream);
+    return dx ? run_dgrad(p, dy_out, w, dx, ws, true, st) : NB_OK;
 }
 
 nb_status nb_conv_bn_silu_bwd_weight(nb_cbs_plan p, const void* x, const void* dy, float* dw, void* workspace,
@@ -1129,29 +1083,39 @@ nb_status nb_conv_bn_silu_bwd_weight(nb_cbs_plan p, const void* x, const void* d
     NB_CHECK_PTR(x); NB_CHECK_PTR(dy); NB_CHECK_PTR(dw);
     NB_TRY(check_ws(workspace, workspace_bytes, p->bwd_bytes));
     DeviceGuard on_device(p->device);
+    return run_wgrad(p, x, dy, dw, static_cast<char*>(workspace), false, static_cast<cudaStream_t>(stream));
+}
+
+nb_status nb_conv_bn_silu_bwd(nb_cbs_plan p, const void* x, const void* g, const void* y_saved, const float* save_mean,
+                              const float* save_invstd, const float* gamma, const float* beta, const void* w, void* dx, float* dw,
+                              float* dgamma, float* dbeta, void* dy_out, void* workspace, size_t workspace_bytes, void* stream) {
+    g_err.clear();
+    if (!p) return fail(NB_ERR_INVALID_ARG, "plan is NULL");
+    NB_CHECK_PTR(x); NB_CHECK_PTR(dw);  // (the rest by the first of the two)
+    NB_TRY(nb_conv_bn_silu_bwd_data(p, g, y_saved, save_mean, save_invstd, gamma, beta, w, dx, dgamma, dbeta, dy_out, workspace, workspace_bytes, stream));
+    DeviceGuard on_device(p->device);
+    return run_wgrad(p, x, dy_out, dw, static_cast<char*>(workspace), dx != nullptr, static_cast<cudaStream_t>(stream));
+}
+
+nb_status nb_conv_bias_bwd(nb_cbs_plan p, const void* x, const void* w, const void* dout, void* dx, float* dw, float* dbias, void* workspace,
+                           size_t workspace_bytes, void* stream) {
+    g_err.clear();
+    if (!p) return fail(NB_ERR_INVALID_ARG, "plan is NULL");
+    NB_CHECK_PTR(x); NB_CHECK_PTR(dout); NB_CHECK_PTR(dw); NB_CHECK_PTR(dx, true); NB_CHECK_PTR(dbias, true);
+    if (dx) NB_CHECK_PTR(w);
+    if (p->pitched || p->ld_dx || p->dx_accumulate || p->fwd_res || p->bwd_gres) return fail(NB_ERR_UNSUPPORTED, "the plan has row pitches, a dx target or a residual set: only the training calls honour them");
+    NB_TRY(check_ws(workspace, workspace_bytes, p->bwd_bytes));
+    DeviceGuard on_device(p->device);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    float* partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + p->off_wgpart);
-    const bool overlap = follows_dgrad(p, dy, st);
-    if (is_f32(p)) return run_simt_wgrad<float>(p, x, dy, dw, partial, overlap, st);
-    if (p->stem) {
-        {
-            SiteTimer tm(p, SITE_WGRAD, st);
-            NB_TRY(NB_WITH_AT(p, run_stem_wgrad<AT>(p, x, dy, partial, overlap, st)));
-        }
-        const size_t elems = (size_t)p->g.c_out * p->g.kdim;
-        SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
-        launch_k(splitk_reduce_tall_kernel, dim3((unsigned)((elems + 31) / 32)), dim3(1024), 0, st, 1, partial, p->stem_wgrad_blocks, elems, dw);
-        return launch_ok("splitk_reduce");
+    char* ws = static_cast<char*>(workspace);
+    if (dbias) {  // column sums of dout: the statistics kernels with only the raw sum requested
+        float* part = reinterpret_cast<float*>(ws + p->off_bpart);
+        if (is_f32(p)) NB_TRY(run_stats_partial<float>(p, dout, part, st));
+        else NB_TRY(NB_WITH_AT(p, run_stats_partial<AT>(p, dout, part, st)));
+        NB_TRY(run_finalize(p, part, p->ew.blocks_stats, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, dbias, nullptr, st));
     }
-    if (p->tc.wgrad) {
-        SiteTimer tm(p, SITE_WGRAD, st);
-        const long long l0 = p->tc.launches;
-        const nb_status ts = tc_wgrad(&p->tc, p->g, x, dy, dw, partial, p->status, st, overlap);
-        g_launches.fetch_add((unsigned long long)(p->tc.launches - l0), std::memory_order_relaxed);
-        if (ts != NB_OK) return fail(ts, "%s", tc_last_error());
-        return NB_OK;
-    }
-    return NB_WITH_AT(p, run_simt_wgrad<AT>(p, x, dy, dw, partial, overlap, st));
+    if (dx) NB_TRY(run_dgrad(p, dout, w, dx, ws, false, st));
+    return run_wgrad(p, x, dout, dw, ws, dx != nullptr, st);
 }
 
 }  // extern "C"

@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     // the next kernel of the stream may become resident and run its prologue right away (behind a data gradient: once this
-    // kernel's own wait is over, see WgradOverlap)
+    // kernel's own wait is over, see the end of common.cuh)
     if (STATS || EPI) pdl_launch_dependents();
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // warp index in a form the compiler knows to be uniform
     const int total_tiles = p.nclasses * p.tiles_per_class;

@@ -547,14 +547,17 @@ class GraphRunner:
                 blk = self.blocks[o["layer"]]
                 if lanes:
                     stream = lanes.enter(_BACKWARD_READS(blk), _BACKWARD_WRITES(blk) + (getattr(blk, "gres", None),))
-                blk.backward_data(stream)
-                if wgrad_stream is None:
-                    blk.backward_weight(stream)
-                else:
+                if wgrad_stream is not None:
+                    blk.backward_data(stream)
                     ev = torch.cuda.Event()
                     ev.record(torch.cuda.current_stream(self.dev) if stream is None else stream)
                     wgrad_stream.wait_event(ev)
                     blk.backward_weight(wgrad_stream, wgrad_workspace)
+                elif lanes:
+                    blk.backward(stream)
+                else:  # (issued one by one, where the launches are what takes the time: the two calls, for callers that look in between)
+                    blk.backward_data(stream)
+                    blk.backward_weight(stream)
                 src = ins[0]
                 if G[src] is not blk.dx:
                     self._sadd(G[src], blk.dx, self._rows(src), self.shape[src][3], accumulate=self.acc[(oi, 0)], stream=stream, lanes=lanes)
