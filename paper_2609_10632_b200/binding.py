@@ -7,6 +7,7 @@ missing or a call fails, an exception is raised.
 from __future__ import annotations
 
 import ctypes
+import itertools
 import os
 from ctypes import POINTER, Structure, byref, c_char_p, c_float, c_int, c_int32, c_size_t, c_uint32, c_void_p
 
@@ -172,6 +173,9 @@ def nb_abi_version() -> int:
     return int(load().nb_abi_version())
 
 
+_plan_serials = itertools.count()
+
+
 class Plan:
     """Owner of one nb_cbs_plan handle."""
 
@@ -179,6 +183,7 @@ class Plan:
         self.desc = nb_cbs_desc(ctypes.sizeof(nb_cbs_desc), n, h, w, c_in, c_out, ksize, stride, eps, momentum, mode, flags)
         self.handle = c_void_p()
         self.device = device
+        self.serial = next(_plan_serials)  # (a handle is an address, which a later plan may be given again)
         self.revision = 0       # counts the setter calls: what was recorded from calls of this plan is stale after one
         self.profiling = False  # nb_cbs_profile_enable
         _check(load().nb_cbs_plan_create(byref(self.desc), device, byref(self.handle)))

@@ -419,14 +419,14 @@ class GraphRunner:
 
     # ------------------------------------------------------------------ recorded passes
     def _arguments(self, tensors_of, extra):
-        """Everything the calls of a pass are issued with: addresses of the blocks', glue calls' and plain convolutions' tensors
-        and the revision of every plan.  None while a plan is being profiled (its calls wait for their kernels)."""
+        """Everything the calls of a pass are issued with: addresses of the blocks', glue calls' and plain convolutions' tensors,
+        every plan and its revision.  None while a plan is being profiled (its calls wait for their kernels)."""
         if any(b.plan.profiling for b in self.blocks) or any(pl["plan"].profiling for pl in self.plain):
             return None
         key = [t if isinstance(t, int) else _address(t) for b in self.blocks for t in tensors_of(b)]
-        key += [b.plan.revision for b in self.blocks]
+        key += [n for b in self.blocks for n in (b.plan.serial, b.plan.revision)]
         for pl in self.plain:
-            key.append(pl["plan"].revision)
+            key += [pl["plan"].serial, pl["plan"].revision]
             key += [_address(t) for t in pl.values() if isinstance(t, torch.Tensor)]
         for tensors in (self.buf, self.grad, self.idx):
             key += [_address(t) for t in tensors.values()]

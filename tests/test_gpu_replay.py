@@ -76,3 +76,51 @@ def test_replayed_passes_give_the_issued_bits(side):
             torch.cuda.current_stream().wait_stream(second)
     graph.replay()
     assert all(torch.equal(a, b) for a, b in zip(results(), want))
+
+
+def _small_runner():
+    import torch
+
+    from paper_2609_10632_b200.detector import GraphRunner
+
+    ops, layers, outs, plain = wl.detector_graph(1, 64, plain_head=True)
+    run = GraphRunner(ops, layers, outs, plain_layers=plain)
+    run.fill_parameters(seed=3)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    for pl in run.plain:
+        pl["w"].normal_(0.0, 0.05, generator=gen)
+        pl["bias"].normal_(0.0, 0.5, generator=gen)
+    run.buf["img"].uniform_(0.0, 1.0, generator=gen)
+    return run, outs
+
+
+def test_a_plan_that_takes_the_place_of_another_is_issued_and_recorded():
+    """Another plan of the same revision (every setter called as often), here with the statistics finished by kernels of their
+    own: its launches are more.  The old plan stays alive until the end, so that a recording that was replayed by mistake
+    would find its accumulators."""
+    import torch
+
+    from paper_2609_10632_b200 import binding as nb
+
+    run, outs = _small_runner()
+
+    def forward():
+        before = nb.nb_cbs_launch_count()
+        run.forward()
+        torch.cuda.synchronize()
+        return nb.nb_cbs_launch_count() - before, [run.buf[o].clone() for o in outs]
+
+    n, first = forward()
+    assert [forward()[0] for _ in range(2)] == [n, n]
+    k = next(i for i, b in enumerate(run.blocks) if not hasattr(b, "res") and not hasattr(b, "gres"))
+    blk = run.blocks[k]
+    old, new = blk.plan, nb.Plan.for_shape(blk.shape, flags=nb.NB_CBS_FLAG_SEPARATE_FINALIZE)
+    for _ in range(old.revision):
+        new.set_pitches(ld_x=blk.x.stride(-2), ld_a=blk.a.stride(-2), ld_g=blk.g.stride(-2))
+    assert new.revision == old.revision
+    blk.plan = new
+    more = [forward() for _ in range(3)]
+    assert len({m for m, _ in more}) == 1 and more[0][0] > n
+    assert all(torch.equal(a, b) for _, outputs in more[1:] for a, b in zip(outputs, more[0][1]))
+    assert blk.plan is new and old.handle
