@@ -466,17 +466,32 @@ class GraphRunner:
         before = nb.nb_cbs_launch_count()
         with torch.cuda.stream(main):
             graph.capture_begin(capture_error_mode="thread_local")  # (other threads may go on using the GPU)
+            lanes = _Lanes(main, self.dev, spare)
             try:
-                lanes = _Lanes(main, self.dev, spare)
                 issue(main, side if with_side else None, lanes)
                 lanes.finish()
                 if with_side:
                     main.wait_stream(side)
-            finally:
-                graph.capture_end()
+            except BaseException:  # the caller hears of this, and not that a recording was left open
+                self._abandon(graph, main, lanes.streams[1:] + ([side] if with_side else []))
+                raise
+            graph.capture_end()
         rec.launches = nb.nb_cbs_launch_count() - before
         nb.replayed_launches -= rec.launches  # recorded, not launched
         rec.graph = graph
+
+    @staticmethod
+    def _abandon(graph, main, branches):
+        """Ends a recording in which a call has failed (current stream: main), with every branch joined, as it has to be."""
+        try:
+            for st in branches:
+                with torch.cuda.stream(st):
+                    open_ = torch.cuda.is_current_stream_capturing()
+                if open_:
+                    main.wait_stream(st)
+            graph.capture_end()
+        except RuntimeError:
+            pass
 
     # ------------------------------------------------------------------ passes
     def forward(self, stream=None):

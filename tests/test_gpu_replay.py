@@ -124,3 +124,41 @@ def test_a_plan_that_takes_the_place_of_another_is_issued_and_recorded():
     assert len({m for m, _ in more}) == 1 and more[0][0] > n
     assert all(torch.equal(a, b) for _, outputs in more[1:] for a, b in zip(outputs, more[0][1]))
     assert blk.plan is new and old.handle
+
+
+@pytest.mark.parametrize("side", [False, True], ids=["one stream", "weight gradients on a second stream"])
+def test_an_error_in_a_recorded_call_reaches_the_caller(side):
+    """A call that refuses its arguments while the pass is being recorded, with branches open: the caller gets its error, and the
+    runner records and replays again once the cause is gone."""
+    import torch
+
+    from paper_2609_10632_b200 import binding as nb
+
+    run, outs = _small_runner()
+    for name in outs:
+        run.grad[name].normal_()
+    second = torch.cuda.Stream() if side else None
+    ws = torch.empty(max(b.plan.bwd_bytes for b in run.blocks), dtype=torch.uint8, device="cuda") if side else None
+
+    def passes():
+        run.forward()
+        run.backward(wgrad_stream=second, wgrad_workspace=ws)
+
+    passes()
+    torch.cuda.synchronize()
+    want = [run.grad["img"].clone()] + [b.dw.clone() for b in run.blocks]
+    blk = run.blocks[20]
+    good, blk.dy = blk.dy, blk.dy.view(-1)[1:]  # not on a 16-byte boundary
+    for _ in range(3):
+        with pytest.raises(nb.NbError) as ei:  # issued, recorded, recorded again
+            passes()
+        assert ei.value.status == nb.NB_ERR_ALIGNMENT
+    blk.dy = good
+    torch.cuda.synchronize()
+    assert not torch.cuda.is_current_stream_capturing()
+    for _ in range(3):
+        run.grad["img"].zero_()
+        passes()
+        torch.cuda.synchronize()
+        run.poll()
+        assert all(torch.equal(a, b) for a, b in zip([run.grad["img"]] + [b.dw for b in run.blocks], want))
