@@ -136,7 +136,7 @@ nb_status sgd_step_impl(nb_sgd_plan p, void* workspace, size_t workspace_bytes, 
     if (sc) { s.growth_factor = sc->growth_factor; s.backoff_factor = sc->backoff_factor; s.floor_scale = sc->floor_scale; s.growth_interval = sc->growth_interval; }
     for (int i = 0; i < NB_SGD_GROUPS; ++i) { s.lr[i] = hyper->lr[i]; s.wd[i] = hyper->weight_decay[i]; }
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    launch_k(sgd_sqnorm_kernel, dim3((unsigned)p->h.grid), dim3(SGD_THREADS), 0, st, 1, static_cast<const uint8_t*>(ws));
+    launch_k(sgd_sqnorm_kernel, dim3((unsigned)p->h.grid), dim3(SGD_THREADS), 0, st, 1, ws, s.scaler);
     NB_LAUNCH_OK("sgd_sqnorm");
     launch_k(sgd_update_kernel, dim3((unsigned)p->h.grid), dim3(SGD_THREADS), 0, st, 1, ws, s, total_norm);
     NB_LAUNCH_OK("sgd_update");

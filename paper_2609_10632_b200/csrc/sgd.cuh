@@ -35,14 +35,17 @@ __device__ __forceinline__ double block_sum_fixed_order(double v, double* red /*
     return t;  // valid in thread 0
 }
 
+constexpr int SGD_SCALE_AT = 128;  // byte offset in the header block: the loss scale of the step (see sgd_update_kernel)
+
 // partials[b] = sum of g^2 over the chunks of block b (fp32 per thread over at most a few hundred elements, fp64 above).
-__global__ void __launch_bounds__(SGD_THREADS) sgd_sqnorm_kernel(const uint8_t* __restrict__ ws) {
+__global__ void __launch_bounds__(SGD_THREADS) sgd_sqnorm_kernel(uint8_t* __restrict__ ws, const nb_loss_scaler* scaler) {
     pdl_launch_dependents();
     pdl_wait();
+    if (scaler && blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<float*>(ws + SGD_SCALE_AT) = scaler->scale;
     const SgdHeader& H = *reinterpret_cast<const SgdHeader*>(ws);
     const nb_sgd_tensor* T = reinterpret_cast<const nb_sgd_tensor*>(ws + H.off_tensors);
     const SgdChunk* C = reinterpret_cast<const SgdChunk*>(ws + H.off_chunks);
-    double* partials = reinterpret_cast<double*>(const_cast<uint8_t*>(ws) + H.off_partials);
+    double* partials = reinterpret_cast<double*>(ws + H.off_partials);
     __shared__ double red[SGD_THREADS / 32];
     double acc = 0.0;
     for (int c = blockIdx.x; c < H.nchunks; c += gridDim.x) {
@@ -77,7 +80,6 @@ struct SgdScalars {
     float growth_factor, backoff_factor, floor_scale;
     int growth_interval;
 };
-constexpr int SGD_READERS_AT = 128;  // byte offset in the header block: blocks of the update kernel that have read the scaler's state (zero between steps)
 
 __device__ __forceinline__ void sgd_one(float g, float& p, float& b, float coef, float lr, float wd, float mom, bool first) {
     const float d = fmaf(wd, p, g * coef);
@@ -89,8 +91,9 @@ __device__ __forceinline__ void sgd_one(float g, float& p, float& b, float coef,
 // left of them in L2 (126 MB) is their end; parameters and momentum pass through L2 as streams so that they do not push it
 // out, and a chunk's table entries are fetched behind the previous chunk's data.  Measured, the detector's 243 tensors with
 // fp16 copies and the scaler: 162 -> 115 us for the step (5.9 TB/s of 26 bytes per parameter).
-// With a scaler the last block to have read its state writes the state for the next step (no block waits for another);
-// a kernel of its own, whose one thread summed the norm's partials once more, took 30 us after this one.
+// With a scaler the blocks take the scale from the copy that the norm kernel has left in the workspace, and block 0 writes the
+// state for the next step while others are still at work: only the kernel boundaries order the two.  (Read from the state by
+// every block and written by the last to be counted, with the fence that takes: 118 us.)
 __global__ void __launch_bounds__(SGD_THREADS) sgd_update_kernel(uint8_t* __restrict__ ws, SgdScalars hs, float* __restrict__ total_norm_out) {
     pdl_launch_dependents();
     pdl_wait();
@@ -106,33 +109,29 @@ __global__ void __launch_bounds__(SGD_THREADS) sgd_update_kernel(uint8_t* __rest
     const double t = block_sum_fixed_order(acc, red);
     __shared__ int s_skip;
     if (threadIdx.x == 0) {
-        const double inv = hs.scaler ? 1.0 / (double)hs.scaler->scale : 1.0;
+        const double inv = hs.scaler ? 1.0 / (double)*reinterpret_cast<const float*>(ws + SGD_SCALE_AT) : 1.0;
         const double total = sqrt(t) * inv;  // norm of the unscaled gradients; inf or NaN if any gradient element is
         double c = 1.0;
         if (hs.max_norm > 0.f && hs.max_norm < __int_as_float(0x7f800000)) c = fmin((double)hs.max_norm / (total + 1e-6), 1.0);
         s_coef = (float)(c * inv);
         s_skip = (hs.scaler && !isfinite(t)) ? 1 : 0;
         if (blockIdx.x == 0 && total_norm_out) *total_norm_out = (float)total;
-        if (hs.scaler) {
-            int* readers = reinterpret_cast<int*>(ws + SGD_READERS_AT);
-            if (atomicAdd(readers, 1) == (int)gridDim.x - 1) {  // every other block has used the state it read
-                *readers = 0;
-                nb_loss_scaler s = *hs.scaler;
-                if (!isfinite(t)) {
-                    s.scale = fmaxf(s.scale * hs.backoff_factor, hs.floor_scale);
+        if (blockIdx.x == 0 && hs.scaler) {
+            nb_loss_scaler s = *hs.scaler;
+            if (!isfinite(t)) {
+                s.scale = fmaxf(s.scale * hs.backoff_factor, hs.floor_scale);
+                s.growth_tracker = 0;
+                s.skipped = 1;
+            } else {
+                s.skipped = 0;
+                if (++s.growth_tracker >= hs.growth_interval) {
+                    s.scale *= hs.growth_factor;
                     s.growth_tracker = 0;
-                    s.skipped = 1;
-                } else {
-                    s.skipped = 0;
-                    if (++s.growth_tracker >= hs.growth_interval) {
-                        s.scale *= hs.growth_factor;
-                        s.growth_tracker = 0;
-                    }
                 }
-                hs.scaler->scale = s.scale;
-                hs.scaler->growth_tracker = s.growth_tracker;
-                hs.scaler->skipped = s.skipped;
             }
+            hs.scaler->scale = s.scale;
+            hs.scaler->growth_tracker = s.growth_tracker;
+            hs.scaler->skipped = s.skipped;
         }
     }
     __syncthreads();

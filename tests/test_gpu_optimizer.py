@@ -199,3 +199,28 @@ def test_fp16_working_copy():
     torch.cuda.synchronize()
     for p, lp in zip(st.p, st.lp):
         assert torch.equal(lp, p.to(torch.float16))
+
+
+def test_every_block_of_a_scaled_step_uses_the_scale_of_that_step():
+    """The scale doubles at every step, written while blocks of the update are still to come.  Scales are
+    powers of two, so that parameters and momentum have the bits of steps without a scaler; a block that read the scale of the
+    next step would halve its update.  (3 million elements: 735 chunks.)"""
+    import struct
+
+    import torch
+
+    sizes, groups = [2_900_000, 64, 100_001], [0, 1, 2]
+    plain, scaled = State(sizes, groups, cfg_id=37), State(sizes, groups, cfg_id=37)
+    state = torch.zeros(4, dtype=torch.int32, device=plain.p[0].device)
+    state[0] = struct.unpack("i", struct.pack("f", 1024.0))[0]
+    _, grads = wl.make_optimizer_inputs(sizes, 37, 0, 0.3)
+    for d, h in zip(plain.g, grads):
+        d.copy_(torch.from_numpy(h))
+    for k in range(20):
+        for a, b in zip(scaled.g, plain.g):
+            a.copy_(b * 1024.0 * 2.0**k)
+        plain.plan.step(plain.ws, LR, WD, MOM, 1.0, first_step=k == 0)
+        scaled.plan.step_scaled(scaled.ws, state, LR, WD, MOM, 1.0, first_step=k == 0, growth_interval=1)
+        for a, b in zip(plain.p + plain.m, scaled.p + scaled.m):
+            assert torch.equal(a, b), k
+        assert struct.unpack("f", struct.pack("i", int(state[0].item())))[0] == 2048.0 * 2.0**k
