@@ -25,6 +25,7 @@ from the order of the backward pass; zeroed beforehand only if the overwriting c
 """
 from __future__ import annotations
 
+import gc
 from operator import attrgetter
 
 import torch
@@ -464,21 +465,30 @@ class GraphRunner:
         main, side, spare = self._record_streams
         graph = torch.cuda.CUDAGraph()
         before = nb.nb_cbs_launch_count()
+        collecting = gc.isenabled()
+        gc.disable()  # (a collection could free somebody's old CUDA graph, which is not permitted while this thread captures)
+        try:
+            self._capture(graph, issue, main, side if with_side else None, spare)
+        finally:
+            if collecting:
+                gc.enable()
+        rec.launches = nb.nb_cbs_launch_count() - before
+        nb.replayed_launches -= rec.launches  # recorded, not launched
+        rec.graph = graph
+
+    def _capture(self, graph, issue, main, side, spare):
         with torch.cuda.stream(main):
             graph.capture_begin(capture_error_mode="thread_local")  # (other threads may go on using the GPU)
             lanes = _Lanes(main, self.dev, spare)
             try:
-                issue(main, side if with_side else None, lanes)
+                issue(main, side, lanes)
                 lanes.finish()
-                if with_side:
+                if side is not None:
                     main.wait_stream(side)
             except BaseException:  # the caller hears of this, and not that a recording was left open
-                self._abandon(graph, main, lanes.streams[1:] + ([side] if with_side else []))
+                self._abandon(graph, main, lanes.streams[1:] + ([] if side is None else [side]))
                 raise
             graph.capture_end()
-        rec.launches = nb.nb_cbs_launch_count() - before
-        nb.replayed_launches -= rec.launches  # recorded, not launched
-        rec.graph = graph
 
     @staticmethod
     def _abandon(graph, main, branches):

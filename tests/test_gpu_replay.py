@@ -162,3 +162,37 @@ def test_an_error_in_a_recorded_call_reaches_the_caller(side):
         torch.cuda.synchronize()
         run.poll()
         assert all(torch.equal(a, b) for a, b in zip([run.grad["img"]] + [b.dw for b in run.blocks], want))
+
+
+def test_garbage_of_others_does_not_end_a_recording(monkeypatch):
+    """A CUDA graph that nobody holds any more but for a reference cycle, and enough new objects for a collection, in the middle of
+    a recording: freeing the graph there would invalidate the capture."""
+    import gc
+
+    import torch
+
+    run, outs = _small_runner()
+    run.forward()
+    torch.cuda.synchronize()
+    want = [run.buf[o].clone() for o in outs]
+    old, t = torch.cuda.CUDAGraph(), torch.zeros(16, device="cuda")
+    with torch.cuda.graph(old):
+        t.add_(1)
+    old.replay()
+    held, blk = [old], run.blocks[3]
+    del old
+
+    def forward(stream=None, call=blk.forward):
+        cycle = [held.pop()] if held else []
+        cycle.append(cycle)
+        del cycle
+        many = [[] for _ in range(100_000)]
+        call(stream)
+        assert len(many) == 100_000
+
+    monkeypatch.setattr(blk, "forward", forward)
+    assert gc.isenabled()
+    run.forward()
+    assert gc.isenabled() and not held
+    torch.cuda.synchronize()
+    assert all(torch.equal(run.buf[o], a) for o, a in zip(outs, want))
