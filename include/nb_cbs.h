@@ -83,7 +83,9 @@ typedef enum { NB_MODE_BF16_TC = 0, NB_MODE_F32_REF = 1, NB_MODE_F16_TC = 2 } nb
                                      sums to fp64 accumulators with atomics and the pass that follows derives its
                                      coefficients from the totals: the same values, except that a total may differ
                                      in its last fp64 bit with the order of the additions (seen in an fp32 result
-                                     only if the total sits within 2^-50 of a rounding boundary).  No kernel of either
+                                     only if the total sits within 2^-50 of a rounding boundary).  In F32 mode the
+                                     accumulators are fixed-point numbers to which every block sum is added exactly,
+                                     so that results are bit-identical from run to run by default too.  No kernel of either
                                      kind waits for another block or kernel, so calls of different plans may share
                                      the GPU (other streams, other processes) with or without this flag. */
 
@@ -107,8 +109,9 @@ uint32_t nb_abi_version(void);
  * on this thread. */
 const char* nb_last_error(void);
 
-/* Create a plan for one block shape on CUDA device `device`.  Allocates a small (<= 4 KB) device
- * status block; all other memory is the caller's.  Requirements: all extents > 0; ksize in {1,3};
+/* Create a plan for one block shape on CUDA device `device`.  Allocates a small device status block and the
+ * channel accumulators (96 bytes per output channel, 320 in F32 mode, none with
+ * NB_CBS_FLAG_SEPARATE_FINALIZE); all other memory is the caller's.  Requirements: all extents > 0; ksize in {1,3};
  * stride in {1,2}; BF16 mode: c_out % 8 == 0; F32 mode: c_out % 4 == 0; N*Ho*Wo >= 2.
  * Errors: NB_ERR_INVALID_ARG, NB_ERR_UNSUPPORTED, NB_ERR_CUDA (no usable device), NB_ERR_ARCH. */
 nb_status nb_cbs_plan_create(const nb_cbs_desc* desc, int device, nb_cbs_plan* out_plan);

@@ -91,10 +91,10 @@ struct nb_cbs_plan_s {
     long long ld_dx = 0;           // row pitch of dx in the data-gradient call and whether dx is added to (nb_cbs_plan_set_dx_target)
     bool dx_accumulate = false;
     bool pitched = false;
-    // Channel sums go to fp64 accumulators that the consuming pass turns into coefficients itself (ChanAcc); off
-    // (NB_CBS_FLAG_SEPARATE_FINALIZE, fp32 mode): per-block partial sums and separate finalize kernels.
+    // Channel sums go to accumulators that the consuming pass turns into coefficients itself (ChanAcc); off
+    // (NB_CBS_FLAG_SEPARATE_FINALIZE): per-block partial sums and separate finalize kernels.
     bool fuse_finalize = true;
-    double* acc = nullptr;      // device: [acc_copies_f][2][C] forward sums, then [acc_copies_b][2][C] backward sums; zero between calls
+    double* acc = nullptr;      // device: [acc_copies_f][2][C] forward sums, then [acc_copies_b][2][C] backward sums (fp32 mode: 64-bit words); zero between calls
     int acc_copies_f = 0, acc_copies_b = 0;
     bool stem = false;       // 3-channel 3x3 stride-2 first layer: dedicated direct kernels
     int stem_blocks = 0;     // blocks (= partial slices) of the stem wgrad kernel
@@ -622,15 +622,16 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     int cur = 0;
     NB_CUDA_CHECK(cudaGetDevice(&cur));
     cudaError_t ce = cudaSetDevice(device);
-    // one allocation: the status words, then (256-byte aligned) the fp64 channel accumulators
+    // one allocation: the status words, then (256-byte aligned) the channel accumulators
     {
         auto copies = [](const char* name, int dflt) {
             const char* v = getenv(name);
             const int k = v ? atoi(v) : dflt;
             return k < 1 ? 1 : k > 16 ? 16 : k;
         };
-        p->acc_copies_f = p->fuse_finalize ? copies("NB_ACC_COPIES_FWD", 2) : 0;
-        p->acc_copies_b = p->fuse_finalize ? copies("NB_ACC_COPIES_BWD", 4) : 0;
+        const bool exact = d->mode == NB_MODE_F32_REF;
+        p->acc_copies_f = !p->fuse_finalize ? 0 : exact ? EXACT_WORDS : copies("NB_ACC_COPIES_FWD", 2);
+        p->acc_copies_b = !p->fuse_finalize ? 0 : exact ? EXACT_WORDS : copies("NB_ACC_COPIES_BWD", 4);
     }
     const size_t acc_bytes = (size_t)(p->acc_copies_f + p->acc_copies_b) * 2 * g.c_out * sizeof(double);
     if (ce == cudaSuccess) ce = cudaMalloc(&p->status, kStatusBytes + acc_bytes);

@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(SG_THREADS) simt_gemm_kernel(const TIN* __rest
             if (j0 + c >= cols) continue;
             float sum = 0.f;
             for (int r = 0; r < NTY; ++r) sum += red[(r * 2 + which) * BN + c];
-            chan_acc_add(p.acc, g.c_out, which, j0 + c, sum);
+            chan_acc_add<std::is_same<TIN, float>::value>(p.acc, g.c_out, which, j0 + c, sum);
         }
     }
     if (KIND == 2 && p.overlap) pdl_wait();
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(SG_REDUCE_MAX) splitk_fwd_reduce_kernel(const 
         for (int c = tid; c < C; c += blockDim.x) {
             float sum = 0.f;
             for (int r = c / 4; r < (int)blockDim.x; r += cgs) sum += red[r * 4 + (c & 3)];
-            chan_acc_add(acc, C, pass, c, sum);
+            chan_acc_add<std::is_same<YT, float>::value>(acc, C, pass, c, sum);
         }
         __syncthreads();
     }

@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                 const int ld = p.n_tiles * (tm ? ncb : p.ncol_a);
                 const float* base = wstat + (tm ? (size_t)8 * p.n_tiles * p.ncol_a : 0) + (size_t)which * ld + nt * (tm ? ncb : p.ncol_a) + (cc - (tm ? p.ncol_a : 0));
                 const float v = ((base[0] + base[2 * ld]) + base[4 * ld]) + base[6 * ld];
-                if (p.acc.acc) chan_acc_add(p.acc, p.ldo, which, c, v);
+                if (p.acc.acc) chan_acc_add<false>(p.acc, p.ldo, which, c, v);
                 else dst[e] = v;
             }
         }

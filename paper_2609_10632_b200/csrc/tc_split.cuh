@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
                 const int c = e >= p.BN ? e - p.BN : e;
                 if (n_tile * p.BN + c >= p.ldo) continue;
                 const float* b = red + e;
-                chan_acc_add(p.acc, p.ldo, e >= p.BN ? 1 : 0, n_tile * p.BN + c, ((b[0] + b[2 * p.BN]) + b[4 * p.BN]) + b[6 * p.BN]);
+                chan_acc_add<false>(p.acc, p.ldo, e >= p.BN ? 1 : 0, n_tile * p.BN + c, ((b[0] + b[2 * p.BN]) + b[4 * p.BN]) + b[6 * p.BN]);
             }
         }
         if (sat) atomicAdd(p.status + ST_SAT, sat);
