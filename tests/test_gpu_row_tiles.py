@@ -1,5 +1,6 @@
 """Row tiles of 128 instead of 256 pixels where 256 leave the last wave nearly empty (calls without channel sums): the same
-results, in the data gradient to the bit."""
+results, in the data gradient of up to 128 input channels to the bit.  (Elsewhere the forced tiles change the k-block that a tile
+starts its sum with.)"""
 import pytest
 
 from paper_2609_10632_b200 import workloads as wl
@@ -17,24 +18,26 @@ def test_same_bits_as_the_wide_tiles(shape, monkeypatch):
     from paper_2609_10632_b200 import binding as nb
     from paper_2609_10632_b200.block import CbsBlock
 
+    # (statistics in a fixed order, and one forward pass: the two data gradients are taken of the same dy)
+    blk = CbsBlock(wl.ConvShape("rows", *shape, 1), flags=nb.NB_CBS_FLAG_SEPARATE_FINALIZE)
+    blk.fill_random(3)
+    blk.forward()
+    mean, var = torch.zeros(shape[4], device="cuda"), torch.ones(shape[4], device="cuda")
     got = []
     for rows in (None, "2"):
         if rows:
             monkeypatch.setenv("NB_TC_MH", rows)
-        blk = CbsBlock(wl.ConvShape("rows", *shape, 1))
-        blk.fill_random(3)
-        blk.step()
-        mean, var = torch.zeros(shape[4], device="cuda"), torch.ones(shape[4], device="cuda")
+            blk.plan = nb.Plan.for_shape(blk.shape, flags=nb.NB_CBS_FLAG_SEPARATE_FINALIZE)
+            blk.ws = torch.empty(blk.plan.bwd_bytes, dtype=torch.uint8, device="cuda")
+        blk.backward_data()
         ws, out = torch.empty(max(blk.plan.infer_bytes, 256), dtype=torch.uint8, device="cuda"), torch.empty_like(blk.a)
         nb.nb_conv_bn_silu_infer(blk.plan, blk.x, blk.w, blk.gamma, blk.beta, mean, var, out, ws)
-        dx = torch.empty_like(blk.dx)
-        blk.plan.set_pitches()
-        nb.nb_conv_bn_silu_bwd_data(blk.plan, blk.g, blk.y, blk.mean, blk.invstd, blk.gamma, blk.beta, blk.w, dx, blk.dgamma, blk.dbeta, blk.dy, blk.ws)
         blk.poll()
-        got.append((out, dx, blk.dy.clone()))
+        got.append((out, blk.dx.clone(), blk.dy.clone()))
     (a, dx, dy), (a2, dx2, dy2) = got
-    assert (a.float() - a2.float()).norm() <= 1e-3 * a2.float().norm()
-    # (more than 128 columns: 128 rows per tile unless told otherwise as here; the channel sums of two runs may differ in their last bit)
-    if shape[3] <= 128 and torch.equal(dy, dy2):
+    assert torch.equal(dy, dy2)
+    if shape[3] <= 128:
         assert torch.equal(dx, dx2)
-    assert (dx.float() - dx2.float()).norm() <= 1e-3 * dx2.float().norm()
+    # sums in another order, rounded to 16 bits: now and then another way (seen: 9e-5)
+    assert (dx.float() - dx2.float()).norm() <= 4e-4 * dx2.float().norm()
+    assert (a.float() - a2.float()).norm() <= 4e-4 * a2.float().norm()
