@@ -39,7 +39,8 @@
  * its own, with a workspace of its own and ordered after the call that produced dy, it may overlap any other
  * call of this or another plan; and a plan created with NB_CBS_FLAG_SEPARATE_FINALIZE keeps all scratch of a
  * call in the workspace that call was given, so its calls may overlap on different streams when their
- * workspaces differ.  Calls of DIFFERENT plans may always overlap: no kernel waits for another block or kernel.
+ * workspaces differ.  Calls of DIFFERENT plans may always overlap: no kernel waits for
+ * another kernel, nor for a block that is not resident together with its own (a cluster).
  * On invalid arguments nothing is launched and a non-zero status is returned; nb_last_error()
  * then describes the problem.
  */
@@ -86,8 +87,9 @@ typedef enum { NB_MODE_BF16_TC = 0, NB_MODE_F32_REF = 1, NB_MODE_F16_TC = 2 } nb
                                      only if the total sits within 2^-50 of a rounding boundary).  In F32 mode the
                                      accumulators are fixed-point numbers to which every block sum is added exactly,
                                      so that results are bit-identical from run to run by default too.  No kernel of either
-                                     kind waits for another block or kernel, so calls of different plans may share
-                                     the GPU (other streams, other processes) with or without this flag. */
+                                     kind waits for another kernel, nor for a block outside its own cluster, so calls
+                                     of different plans may share the GPU (other streams, other processes) with or
+                                     without this flag. */
 
 typedef struct nb_cbs_desc {
     uint32_t struct_size; /* = sizeof(nb_cbs_desc) */

@@ -25,8 +25,10 @@ enum { ST_ERR = 0, ST_WHERE = 1, ST_DETAIL = 2, ST_SAT = 3, ST_READERS_FWD = 8, 
 // Sites that a give-up is reported from (ST_WHERE): 1-5 the roles of the implicit-GEMM kernel (A producer, accumulator
 // free, operands ready, accumulator ready, B producer), 11-15 the same roles of the weight-gradient kernel.
 
-// Every wait in the library (all of them waits of a CTA on its own mbarriers: no kernel waits for another CTA's or
-// another kernel's flag) is bounded: about two seconds.
+// Every wait on an mbarrier (a CTA's own, on which in a CTA pair its peer arrives too) is bounded: about two seconds.  Nothing
+// else is waited for in a loop: no kernel waits for another kernel's flag, nor for a CTA outside its cluster.  The CTAs of a
+// cluster meet at barrier.cluster, which has no limit and needs none: the cluster is resident as a whole, no CTA waits for
+// anything outside it on the way there, and one that has given up a wait arrives all the same.
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 
 // Records a give-up in a plan's status block (first one wins): error code, site, detail.
@@ -120,12 +122,13 @@ template <typename T> __device__ __forceinline__ void st16_stream(T* p, const Ve
     __stcs(reinterpret_cast<uint4*>(p), *reinterpret_cast<const uint4*>(&r));
 }
 
-// Programmatic dependent launch.  Every kernel starts with pdl_launch_dependents() and executes pdl_wait() before its
-// first access to global memory: the next kernel in the stream may then become resident and run its prologue (barrier
-// set-up, TMEM allocation, descriptor prefetch) while this one drains, and still sees all of its results.  Because every
-// kernel waits before it finishes, completion of the previous kernel implies completion of all earlier ones.  This is
-// safe because no block of any kernel waits for another block: a resident block of the next kernel can delay blocks of
-// this one, never stop them.
+// Programmatic dependent launch.  A kernel signals its dependents with pdl_launch_dependents() when it starts and executes
+// pdl_wait() before its first access to global memory: the next kernel in the stream may then become resident and run its
+// prologue (barrier set-up, TMEM allocation, descriptor prefetch) while this one drains, and still sees all of its results.
+// (Two exceptions, at the end of this file: data gradients signal behind their own wait, and a weight gradient beside one
+// waits at its end.)  Because every kernel waits before it finishes, completion of the previous kernel implies completion of
+// all earlier ones.  This is safe because no block waits for a block outside its own cluster, and a cluster becomes resident as
+// a whole: a resident block of the next kernel can delay blocks of this one, never stop them.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

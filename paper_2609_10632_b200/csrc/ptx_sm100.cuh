@@ -1,7 +1,7 @@
 // Inline-PTX wrappers for the sm_100a features the tensor-core kernels use: mbarrier, TMA (tiled and im2col
 // loads, tiled stores; never multicast), tcgen05 (TMEM allocation, MMA, commit, TMEM loads) and the fences
-// between the generic, async and tensor-core proxies.  Every wait is bounded: it returns false after a fixed
-// number of polls instead of spinning forever.
+// between the generic, async and tensor-core proxies.  Every wait on an mbarrier is bounded: it returns false after a
+// fixed number of polls instead of spinning forever.  (cluster_sync_all is not: see kWaitLimitNs in common.cuh.)
 #pragma once
 #include <cuda.h>
 #include <stdint.h>

@@ -3,7 +3,7 @@
 // products are issued as tcgen05.mma by one thread with fp32 accumulators in TMEM, and whose epilogue (eight warps)
 // reads the accumulators back with tcgen05.ld, converts, stages the tile in shared memory, takes per-channel sums
 // for the batch statistics and hands the rows to TMA stores.  The same kernel computes fprop (A = x, B = w) and dgrad
-// (A = dy, B = the filter rearranged per output-parity class).  No multicast anywhere; every wait is bounded.
+// (A = dy, B = the filter rearranged per output-parity class).  No multicast anywhere; every wait on an mbarrier is bounded.
 #pragma once
 #include <atomic>
 #include <cuda.h>
@@ -1024,7 +1024,7 @@ inline void fill_params(IgemmParams& P, const IgemmCfg& c) {
 // K = 16 step, whichever is longer; then the hand-over and the stores, which the persistent kernel does with TMA and, in the
 // training calls, behind a predecessor that still drains (`eval`: the evaluation-mode call, whose persistent form derives
 // every channel's coefficients in every CTA instead).
-// Measured, evaluation-mode forward of the 77 layers, one image: 1190 -> 590 us; single layers: 288 -> 288 3x3 at 20 x 20
+// Measured, evaluation-mode forward of the 77 layers, one image: 1251 -> 649 us; single layers: 288 -> 288 3x3 at 20 x 20
 // 20.6 -> 7.5 us (8 tiles of 45 k-blocks -> 28 of 9), 192 -> 192 3x3 at 40 x 40 15.1 -> 7.8, 384 -> 384 1x1 at 40 x 40
 // 9.5 -> 5.5; data gradient of 288 -> 288 at 20 x 20 (the whole call) 28.6 -> 16.2.
 inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_taps, bool eval, int sm_count) {

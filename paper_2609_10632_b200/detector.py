@@ -6,9 +6,11 @@ torch allocates the buffers, zeroes gradient accumulators where needed and owns 
 
 A pass is some 200 to 400 kernel launches whose arguments do not change from step to step, and issuing them one by one (2.4 us
 each, plus 2 us for every call's way through Python) takes longer than a small batch takes on the GPU.  From the second pass
-with unchanged arguments on, forward() and backward() therefore replay a CUDA graph recorded from the same calls.  Measured,
-one training iteration at batch 2, 320 x 320: 2.94 ms issued one by one, of which the host alone needs 2.81 ms, and 2.57 ms
-as graphs; at batch 16, 640 x 640: 9.94 and 9.66 ms.  The recording has the dataflow's branches (_Lanes): 2.29 and 9.31 ms.
+with unchanged arguments on, forward() and backward() therefore replay a CUDA graph recorded from the same calls (one graph
+per pass is kept: arguments that alternate are issued every time).  Measured, one training iteration with the update, repeated
+on the same tensors, at batch 2, 320 x 320: 2.78 ms issued one by one, of which the host alone needs 2.68 ms, and 2.54 ms as
+graphs of one branch; at batch 16, 640 x 640: 9.88 and 9.94 ms.  The recording has the dataflow's branches (_Lanes): 2.25 and
+9.35 ms (9.56 ms with tensors that no earlier pass has left in L2).
 
 Every named tensor is an NHWC bf16 tensor, dense or -- with views=True -- a CHANNEL SLICE of a wider buffer (a torch
 view: data_ptr() is the slice's first channel, stride(-2) its row pitch), which the block calls accept through
@@ -82,7 +84,7 @@ class _Lanes:
     branch that ends with one of those; where there is none, as at the detector's six head branches, it opens another.
     The kernels of a small batch leave most SMs idle and are bound by their latency, so that branches beside the longest
     chain of the dataflow (67 of 77 blocks) cost next to nothing.  Measured, forward and backward pass of the detector at batch 2,
-    320 x 320: 888 -> 761 us, 1581 -> 1407 us; at batch 16, 640 x 640: 3163 -> 3085, 6333 -> 6250."""
+    320 x 320: 892 -> 769 us, 1563 -> 1391 us; at batch 16, 640 x 640: 3165 -> 3084, 6687 -> 6270."""
 
     LIMIT = 8  # (the detector opens six)
 

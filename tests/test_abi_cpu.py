@@ -128,9 +128,9 @@ def test_status_codes_of_the_binding_match_the_header():
 
 def test_device_code_reports_give_ups_through_the_named_constant_only():
     """The status word that nb_cbs_poll_status returns is written in ONE place (report_timeout in common.cuh, with
-    NB_ERR_TIMEOUT from the header); no kernel source writes a literal code there.  And no kernel source contains a wait
-    of one block for another (a spin on a global counter or flag): the only bounded waits are those of a CTA on its own
-    mbarriers."""
+    NB_ERR_TIMEOUT from the header); no kernel source writes a literal code there.  And no kernel source contains a spin
+    on a global counter or flag, by which a block could wait for one that is not resident: what is waited for are a CTA's own
+    mbarriers, with a limit, and the other CTAs of its cluster at barrier.cluster."""
     csrc = os.path.join(ROOT, "paper_2609_10632_b200", "csrc")
     writers = []
     for fn in sorted(os.listdir(csrc)):

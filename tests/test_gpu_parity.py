@@ -163,8 +163,8 @@ def test_separate_finalize_kernels_match_oracle(shape):
 
 
 def test_two_plans_on_two_streams():
-    """Calls of different plans may overlap on the GPU: no kernel waits for another block or kernel, so two plans that
-    each hold part of the GPU cannot block each other."""
+    """Calls of different plans may overlap on the GPU: no kernel waits for another kernel or for a block outside its own
+    cluster, so two plans that each hold part of the GPU cannot block each other."""
     import torch
 
     from paper_2609_10632_b200 import binding as nb
