@@ -112,7 +112,7 @@ uint32_t nb_abi_version(void);
 const char* nb_last_error(void);
 
 /* Create a plan for one block shape on CUDA device `device`.  Allocates a small device status block and the
- * channel accumulators (96 bytes per output channel, 320 in F32 mode, none with
+ * channel accumulators (96 bytes per output channel, 320 or 480 in F32 mode, none with
  * NB_CBS_FLAG_SEPARATE_FINALIZE); all other memory is the caller's.  Requirements: all extents > 0; ksize in {1,3};
  * stride in {1,2}; BF16 mode: c_out % 8 == 0; F32 mode: c_out % 4 == 0; N*Ho*Wo >= 2.
  * Errors: NB_ERR_INVALID_ARG, NB_ERR_UNSUPPORTED, NB_ERR_CUDA (no usable device), NB_ERR_ARCH. */

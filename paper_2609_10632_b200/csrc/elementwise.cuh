@@ -218,15 +218,15 @@ template <int V> __device__ __forceinline__ void load_params(const float* __rest
 struct ChanAcc {
     double* acc;   // NULL: the consumer reads coefficients that a finalize kernel has written
     int* readers;
-    int copies;    // (EXACT: EXACT_WORDS, the sets being the words of the sums)
+    int copies;    // (EXACT: EXACT_WORDS for every set, the words of a sum lying where the sets of fp64 sums do)
 };
 
 // A sum of fp32 values as a fixed-point number of 64-bit words: word k counts units of 2^(32 k - 149), so that the 24 bits of
 // a value fall into words k and k + 1, k its exponent / 32.  Integer additions commute: the words are the same whatever order
 // the atomics land in, and the sum has no rounding at all (a word holds 2^31 values).  The last word has a
 // bit for either infinity and for NaN.  Against fp64 sums: two atomics per value instead of one, ten words to read instead of
-// two or four.  Measured (step): 16 -> 32 3x3 on 2 x 32 x 32 pixels 37.9 -> 37.0 us (a lane per sum instead of one for two
-// channels' two sums each), 64 -> 64 on 2 x 40 x 40 57.8 -> 58.7.
+// two or four; measured at exact_apart in nb_cbs.cu (1 to 4 % of a step of up to 60 us, nothing on the smallest and the
+// largest).
 constexpr int EXACT_DIGITS = 9, EXACT_WORDS = EXACT_DIGITS + 1;
 constexpr unsigned long long EXACT_POS_INF = 1, EXACT_NEG_INF = 2, EXACT_NAN = 4;
 __device__ __forceinline__ void exact_add(unsigned long long* word, size_t pitch, float v) {
@@ -255,23 +255,37 @@ __device__ __forceinline__ double exact_total(const unsigned long long (&w)[EXAC
 }
 
 template <bool EXACT> __device__ __forceinline__ void chan_acc_add(const ChanAcc& ca, int C, int which, int c, float v) {
-    if (EXACT) exact_add(reinterpret_cast<unsigned long long*>(ca.acc) + (size_t)which * C + c, (size_t)2 * C, v);
+    if (EXACT) {
+        const size_t set = (size_t)((int)blockIdx.x % (ca.copies / EXACT_WORDS)) * EXACT_WORDS;
+        exact_add(reinterpret_cast<unsigned long long*>(ca.acc) + (set * 2 + which) * C + c, (size_t)2 * C, v);
+    }
     else atomicAdd(ca.acc + ((size_t)((int)blockIdx.x % ca.copies) * 2 + which) * C + c, (double)v);
 }
-// f(c, first total, second total) for every channel (EXACT), by the threads of a block: two neighbouring lanes take a channel's
-// two sums, all words of a sum requested before the first is used, and the even one calls f.
-template <class F> __device__ __forceinline__ void exact_totals(const ChanAcc& ca, int C, F f) {
+// f(c, first total, second total, load(c)) for every channel (EXACT), by the threads of a block, or (CLEAR) of the grid, which
+// then leave the words zero: two neighbouring lanes take a channel's two sums, whatever load reads and all words of a set
+// requested before the first is used, and the even one calls f.
+template <bool CLEAR, class Load, class F> __device__ __forceinline__ void exact_totals(const ChanAcc& ca, int C, Load load, F f) {
     const int threads = (int)blockDim.x & ~1;  // (whole pairs)
     if ((int)threadIdx.x >= threads) return;
 #pragma unroll 1
-    for (int i = (int)threadIdx.x; i < 2 * C; i += threads) {
+    for (int i = (int)threadIdx.x + (CLEAR ? (int)blockIdx.x * threads : 0); i < 2 * C; i += threads * (CLEAR ? (int)gridDim.x : 1)) {
         const int c = i >> 1, which = i & 1;
-        const unsigned long long* const base = reinterpret_cast<const unsigned long long*>(ca.acc) + (size_t)which * C + c;
+        unsigned long long* const base = reinterpret_cast<unsigned long long*>(ca.acc) + (size_t)which * C + c;
+        const auto prm = load(c);
         unsigned long long w[EXACT_WORDS];
 #pragma unroll
         for (int k = 0; k < EXACT_WORDS; ++k) w[k] = __ldcg(base + (size_t)k * 2 * C);
+        for (int set = EXACT_WORDS; set < ca.copies; set += EXACT_WORDS) {
+#pragma unroll
+            for (int k = 0; k < EXACT_WORDS; ++k) {
+                const unsigned long long more = __ldcg(base + (size_t)(set + k) * 2 * C);
+                w[k] = k == EXACT_DIGITS ? w[k] | more : w[k] + more;
+            }
+        }
         const double mine = exact_total(w), other = __shfl_xor_sync(3u << (threadIdx.x & 30u), mine, 1);
-        if (!which) f(c, mine, other);
+        if (!which) f(c, mine, other, prm);
+        if (CLEAR)
+            for (int k = 0; k < ca.copies; ++k) base[(size_t)k * 2 * C] = 0ull;
     }
 }
 // totals of channels c and c + 1 (c even) of both sums; read from L2, where the atomics were performed, with the loads
@@ -332,27 +346,29 @@ struct FwdFin {
     const float *gamma, *beta;
     float *mean, *invstd, *rmean, *rvar;
 };
+__device__ __forceinline__ void fwd_coef_channel(const FwdFin& f, int c, double s, double q, float ga, float be, bool writer, float& scale, float& shift) {
+    const double mu = s * f.inv_m;
+    double var = q * f.inv_m - mu * mu;
+    if (var < 0.0) var = 0.0;
+    const double is = rsqrt_refined(var + (double)f.eps);
+    const double sc = (double)ga * is;
+    scale = (float)sc;
+    shift = (float)((double)be - mu * sc);
+    if (writer) {
+        f.mean[c] = (float)mu;
+        f.invstd[c] = (float)is;
+        if (f.rmean) {
+            f.rmean[c] = (float)((1.0 - (double)f.momentum) * (double)f.rmean[c] + (double)f.momentum * mu);
+            f.rvar[c] = (float)((1.0 - (double)f.momentum) * (double)f.rvar[c] + (double)f.momentum * var * f.unbias);
+        }
+    }
+}
 template <bool EXACT> __device__ __forceinline__ void fwd_coef_from_acc(const ChanAcc& ca, const FwdFin& f, int C, float* s_coef /*[2][C] shared*/) {
     const bool writer = blockIdx.x == 0;
-    auto channel = [&](int c, double s, double q, float ga, float be) {
-        const double mu = s * f.inv_m;
-        double var = q * f.inv_m - mu * mu;
-        if (var < 0.0) var = 0.0;
-        const double is = rsqrt_refined(var + (double)f.eps);
-        const double sc = (double)ga * is;
-        s_coef[c] = (float)sc;
-        s_coef[C + c] = (float)((double)be - mu * sc);
-        if (writer) {
-            f.mean[c] = (float)mu;
-            f.invstd[c] = (float)is;
-            if (f.rmean) {
-                f.rmean[c] = (float)((1.0 - (double)f.momentum) * (double)f.rmean[c] + (double)f.momentum * mu);
-                f.rvar[c] = (float)((1.0 - (double)f.momentum) * (double)f.rvar[c] + (double)f.momentum * var * f.unbias);
-            }
-        }
-    };
+    auto channel = [&](int c, double s, double q, float ga, float be) { fwd_coef_channel(f, c, s, q, ga, be, writer, s_coef[c], s_coef[C + c]); };
     if constexpr (EXACT) {
-        exact_totals(ca, C, [&](int c, double s, double q) { channel(c, s, q, f.gamma[c], f.beta[c]); });
+        exact_totals<false>(ca, C, [&](int c) { return make_float2(f.gamma[c], f.beta[c]); },
+                     [&](int c, double s, double q, float2 p) { channel(c, s, q, p.x, p.y); });
     } else {
         // two channels per thread and round (kept rolled: the fp64 chains must not crowd the registers of the streaming loop)
 #pragma unroll 1
@@ -710,7 +726,8 @@ template <bool EXACT> __device__ __forceinline__ void bwd_coef_from_acc(const Ch
         }
     };
     if constexpr (EXACT) {
-        exact_totals(ca, C, [&](int c, double s0, double s1) { channel(c, s0, s1, f.mean[c], f.invstd[c], f.gamma[c], f.beta[c]); });
+        exact_totals<false>(ca, C, [&](int c) { return make_float4(f.mean[c], f.invstd[c], f.gamma[c], f.beta[c]); },
+                     [&](int c, double s0, double s1, float4 p) { channel(c, s0, s1, p.x, p.y, p.z, p.w); });
     } else {
 #pragma unroll 1
         for (int c = 2 * (int)threadIdx.x; c < C; c += 2 * (int)blockDim.x) {  // two channels per thread and round, see fwd_coef_from_acc
@@ -722,6 +739,28 @@ template <bool EXACT> __device__ __forceinline__ void bwd_coef_from_acc(const Ch
             channel(c + 1, t0.y, t1.y, mu_f.y, is_f.y, ga.y, be.y);
         }
     }
+}
+// The coefficients of an EXACT plan whose words are too many for every block of the consuming pass to read (see exact_apart in
+// nb_cbs.cu): by a kernel of their own, forward and backward, which leaves the words zero.
+__global__ void __launch_bounds__(128) bn_exact_finalize_kernel(ChanAcc ca, int C, FwdFin f, float* __restrict__ scale, float* __restrict__ shift) {
+    pdl_launch_dependents();
+    pdl_wait();
+    exact_totals<true>(ca, C, [&](int c) { return make_float2(f.gamma[c], f.beta[c]); },
+                       [&](int c, double s, double q, float2 p) { fwd_coef_channel(f, c, s, q, p.x, p.y, true, scale[c], shift[c]); });
+}
+__global__ void __launch_bounds__(128) bn_exact_bwd_finalize_kernel(ChanAcc ca, int C, BwdFin f, float* __restrict__ coef /*[4][C]*/) {
+    pdl_launch_dependents();
+    pdl_wait();
+    exact_totals<true>(ca, C, [&](int c) { return make_float4(f.mean[c], f.invstd[c], f.gamma[c], f.beta[c]); },
+                       [&](int c, double s0, double s1, float4 p) {
+                           const BwdCoef k = bwd_coef_channel(p.x, p.y, p.z, p.w, s0, s1, f.inv_m);
+                           coef[c] = k.a;
+                           coef[C + c] = k.b;
+                           coef[2 * C + c] = k.p1;
+                           coef[3 * C + c] = k.p0;
+                           f.dbeta[c] = (float)s0;
+                           f.dgamma[c] = k.dgamma;
+                       });
 }
 // FIN: the coefficients are derived here from the totals in `ca` (dynamic shared memory: 4*C floats); else read from coef.
 // GRES: the incoming gradient g is also the gradient of a residual connection's shortcut: the pass adds it to (or, with

@@ -96,6 +96,11 @@ struct nb_cbs_plan_s {
     bool fuse_finalize = true;
     double* acc = nullptr;      // device: [acc_copies_f][2][C] forward sums, then [acc_copies_b][2][C] backward sums (fp32 mode: 64-bit words); zero between calls
     int acc_copies_f = 0, acc_copies_b = 0;
+    // fp32 mode, whose sums are ten words each: above 160 channels kernels of their own derive the coefficients, below every block
+    // of the consuming pass does.  Measured (step; blocks / kernels, and what fp64 sums took that depended on the order of the
+    // atomics), 2 x 40 x 40 pixels: 64 channels 58.5 / 62.0 us (57.3), 96 81.9 / 84.1 (77.9), 128 85.2 / 86.5 (81.5), 192 53.5 / 52.8
+    // (51.0), 256 58.2 / 56.9 (54.9); 288 on 4 x 20 x 20 271.7 / 265.6 (262.3), 576 on 20 x 20 71.5 / 54.7 (53.5).
+    bool exact_apart = false;
     bool stem = false;       // 3-channel 3x3 stride-2 first layer: dedicated direct kernels
     int stem_blocks = 0;     // blocks (= partial slices) of the stem wgrad kernel
     bool stem_wide = false;  // the stem forward kernel takes 320-pixel strips (wide images)
@@ -303,6 +308,11 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
                  dgamma, dbeta, coef, fin_blocks, static_cast<const __nv_bfloat16*>(w), static_cast<__nv_bfloat16*>(wt), wtp ? *wtp : none);
         NB_LAUNCH_OK("bn_bwd_finalize");
     }
+    if (p->exact_apart) {
+        SiteTimer tm(p, SITE_BWD_FINALIZE, st);
+        launch_k(bn_exact_bwd_finalize_kernel, dim3((unsigned)((2 * C + 127) / 128)), dim3(128), 0, st, 1, ca, C, bf, coef);
+        NB_LAUNCH_OK("bn_exact_bwd_finalize");
+    }
     SiteTimer tm(p, SITE_BWD_DY, st);
     auto go_dy = [&](auto kernel, size_t smem) {
         launch_k(kernel, dim3(e.blocks_dy), dim3(e.tpb), smem, st, 1, static_cast<const AT*>(g), static_cast<const YT*>(y), static_cast<AT*>(dy), e.total_vecs, C, coef,
@@ -313,7 +323,7 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
     if (fuse && p->bwd_gres) {  // (the setter admits this only on plans that take this path)
         if (p->ld_g) one ? go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true, true, true>, coef_smem) : go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true, true>, coef_smem);
         else one ? go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true, true, true>, coef_smem) : go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true, true>, coef_smem);
-    } else if (fuse) {
+    } else if (fuse && !p->exact_apart) {
         if (p->ld_g) one ? go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true, false, true>, coef_smem) : go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, true, true>, coef_smem);
         else one ? go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true, false, true>, coef_smem) : go_dy(bn_silu_bwd_dy_kernel<YT, AT, FAST, false, true>, coef_smem);
     } else {
@@ -450,6 +460,18 @@ nb_status launch_sg(const nb_cbs_plan_s* p, const void* a, const void* b, void* 
     return vec ? launch_sg_tile<KIND, TIN, TO, 64, 32, 4>(p, c, a, b, out, args, st) : launch_sg_tile<KIND, TIN, TO, 64, 32, 1>(p, c, a, b, out, args, st);
 }
 
+// The pass that adds the slices of a split forward convolution: threads and blocks.
+int fwd_reduce_threads(const Geom& g) {
+    const int cgs = g.c_out / 4;
+    return cgs >= 256 ? cgs : 256 / cgs * cgs;
+}
+int fwd_reduce_blocks(const Geom& g, int sm_count) {
+    const int tpb = fwd_reduce_threads(g);
+    return (int)std::min<long long>((g.m * (g.c_out / 4) + tpb - 1) / tpb, (long long)sm_count * 4);
+}
+// Blocks that add to the channel sums of a CUDA-core forward convolution: one per row tile, or those of that pass.
+int simt_fwd_parts(const Geom& g, const SgCfg& c, int sm_count) { return c.splits == 1 ? (int)c.grid.x : fwd_reduce_blocks(g, sm_count); }
+
 // `sums`: with a default plan the channel sums of y go to the plan's accumulators (false: y only, or separate statistics).
 template <typename TIN, typename TOUT>
 nb_status run_simt_fprop(nb_cbs_plan_s* p, const void* x, const void* w, void* y, void* partial, bool sums, cudaStream_t st) {
@@ -462,11 +484,9 @@ nb_status run_simt_fprop(nb_cbs_plan_s* p, const void* x, const void* w, void* y
         NB_TRY((launch_sg<0, TIN, float>(p, x, w, partial, args, st)));
     }
     SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
-    const int cgs = p->g.c_out / 4, tpb = cgs >= 256 ? cgs : 256 / cgs * cgs;
-    const long long vecs = p->g.m * cgs;
-    const long long blocks = std::min<long long>((vecs + tpb - 1) / tpb, (long long)p->sm_count * 4);
-    launch_k(splitk_fwd_reduce_kernel<TOUT>, dim3((unsigned)blocks), dim3(tpb), (size_t)tpb * 16, st, 1, static_cast<const float*>(partial), c.splits, vecs, p->g.c_out,
-             static_cast<TOUT*>(y), ca);
+    const int tpb = fwd_reduce_threads(p->g);
+    launch_k(splitk_fwd_reduce_kernel<TOUT>, dim3((unsigned)fwd_reduce_blocks(p->g, p->sm_count)), dim3(tpb), (size_t)tpb * 16, st, 1, static_cast<const float*>(partial),
+             c.splits, p->g.m * (p->g.c_out / 4), p->g.c_out, static_cast<TOUT*>(y), ca);
     return launch_ok("splitk_fwd_reduce");
 }
 
@@ -630,8 +650,12 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
             return k < 1 ? 1 : k > 16 ? 16 : k;
         };
         const bool exact = d->mode == NB_MODE_F32_REF;
-        p->acc_copies_f = !p->fuse_finalize ? 0 : exact ? EXACT_WORDS : copies("NB_ACC_COPIES_FWD", 2);
+        // (fp32: two sets from 256 adding blocks on: 96 channels on 2 x 40 x 40 81.8 -> 79.7 us, 32 -> 48 1x1 on 16 x 160 x 160
+        // 335 -> 309; below, where they only add to what is read, 16 -> 32 on 2 x 32 x 32 37.7 -> 38.2; four are slower everywhere)
+        const int sets = copies("NB_ACC_COPIES_FWD", simt_fwd_parts(g, p->sg[0], p->sm_count) < 256 ? 1 : 2);
+        p->acc_copies_f = !p->fuse_finalize ? 0 : exact ? EXACT_WORDS * sets : copies("NB_ACC_COPIES_FWD", 2);
         p->acc_copies_b = !p->fuse_finalize ? 0 : exact ? EXACT_WORDS : copies("NB_ACC_COPIES_BWD", 4);
+        p->exact_apart = p->fuse_finalize && exact && g.c_out > 160;
     }
     const size_t acc_bytes = (size_t)(p->acc_copies_f + p->acc_copies_b) * 2 * g.c_out * sizeof(double);
     if (ce == cudaSuccess) ce = cudaMalloc(&p->status, kStatusBytes + acc_bytes);
@@ -895,6 +919,13 @@ nb_status nb_conv_bn_silu_fwd(nb_cbs_plan p, const void* x, const void* w, const
     // when the convolution has left its sums in the accumulators the pass derives mean, invstd, scale and shift from them itself
     const double M = (double)p->g.m;
     const FwdFin fin{1.0 / M, M / (M - 1.0), p->desc.eps, p->desc.momentum, gamma, beta, save_mean, save_invstd, running_mean, running_var};
+    if (p->exact_apart) {
+        SiteTimer tm(p, SITE_FINALIZE, st);
+        const ChanAcc ca{p->acc, nullptr, p->acc_copies_f};
+        launch_k(bn_exact_finalize_kernel, dim3((unsigned)((2 * p->g.c_out + 127) / 128)), dim3(128), 0, st, 1, ca, p->g.c_out, fin, scale, shift);
+        NB_LAUNCH_OK("bn_exact_finalize");
+        finalized = false;  // (the pass reads scale and shift)
+    }
     if (is_f32(p)) return run_apply<float, float, false>(p, y_saved, a_out, scale, shift, st, p->ld_a, p->fwd_res, p->ld_res, finalized ? &fin : nullptr);
     return NB_WITH_AT(p, run_apply<__half, AT, true>(p, y_saved, a_out, scale, shift, st, p->ld_a, p->fwd_res, p->ld_res, finalized ? &fin : nullptr));
 }

@@ -24,22 +24,24 @@ def _f32(v):
     return float(np.float32(v))
 
 
-def test_totals_are_the_sums_without_rounding():
+@pytest.mark.parametrize("h,w,c", [(24, 32, 8), (128, 160, 8), (24, 32, 264), (128, 160, 168)], ids=["", "two sets", "wide", "wide, two sets"])
+def test_totals_are_the_sums_without_rounding(h, w, c):
     """A 1x1 convolution with the identity filter, whose output has one nonzero row in each of six tiles: every tile's sum is that
-    row's value, and the mean is the exact sum of the six over M, rounded once to fp32."""
+    row's value, and the mean is the exact sum of the six over M, rounded once to fp32.  Few and many adding blocks, and few and
+    many channels (whose coefficients a kernel of its own derives); wide rows are also cut into k slices."""
     import torch
 
     from paper_2609_10632_b200 import binding as nb
     from paper_2609_10632_b200.block import CbsBlock
 
-    shape = wl.ConvShape("exact", 1, 24, 32, 8, 8, 1, 1)
+    shape = wl.ConvShape("exact", 1, h, w, c, c, 1, 1)
     blk = CbsBlock(shape, mode=nb.NB_MODE_F32_REF)
     blk.x.zero_()
-    rows = blk.x.view(shape.m, 8)
-    for c, values in enumerate(VALUES):
+    rows = blk.x.view(shape.m, c)
+    for k, values in enumerate(VALUES):
         for t, v in enumerate(values):
-            rows[t * 128 + 17, c] = v
-    blk.w.copy_(torch.eye(8).view(8, 1, 1, 8))
+            rows[t * 128 + 17, k::8] = v
+    blk.w.copy_(torch.eye(c).view(c, 1, 1, c))
     blk.gamma.fill_(1.0)
     blk.beta.zero_()
     mean = None
@@ -48,10 +50,11 @@ def test_totals_are_the_sums_without_rounding():
         blk.poll()
         assert mean is None or np.array_equal(mean, blk.mean.cpu().numpy(), equal_nan=True)
         mean = blk.mean.cpu().numpy()
-    for c, values in enumerate(VALUES):
-        got, want = Fraction(float(mean[c])), sum((Fraction(_f32(v)) for v in values), Fraction(0)) / shape.m
+    for k in range(c):
+        values = VALUES[k % 8]
+        got, want = Fraction(float(mean[k])), sum((Fraction(_f32(v)) for v in values), Fraction(0)) / shape.m
         # one rounding to fp32, behind an fma per word and a product in fp64: a bit more than half a unit in the last place
-        assert abs(got - want) <= abs(want) * Fraction(2) ** -23 + Fraction(2) ** -149, (c, float(got), float(want))
+        assert abs(got - want) <= abs(want) * Fraction(2) ** -23 + Fraction(2) ** -149, (k, float(got), float(want))
 
 
 def test_infinities_and_nan_reach_the_statistics():
@@ -75,7 +78,8 @@ def test_infinities_and_nan_reach_the_statistics():
         np.testing.assert_allclose(blk.mean.cpu().numpy(), want, rtol=1e-7)
 
 
-@pytest.mark.parametrize("dims", [(2, 32, 32, 16, 32, 3, 1), (2, 40, 40, 64, 64, 3, 1), (3, 37, 29, 20, 1028, 1, 1), (4, 60, 60, 32, 48, 3, 2)], ids=str)
+@pytest.mark.parametrize("dims", [(2, 32, 32, 16, 32, 3, 1), (2, 40, 40, 64, 64, 3, 1), (3, 37, 29, 20, 1028, 1, 1), (4, 60, 60, 32, 48, 3, 2),
+                                  (2, 40, 40, 64, 164, 3, 1), (4, 90, 80, 16, 192, 1, 1)], ids=str)
 def test_default_steps_are_the_same_bits_from_run_to_run(dims):
     """Values whose block sums span 2^100, so that fp64 sums would depend on the order of the atomics."""
     import torch
