@@ -461,8 +461,8 @@ class GraphRunner:
 
     def _record(self, rec, issue, with_side):
         if self._record_streams is None:
-            # (priority for the branch that holds the longest chain: 2307 -> 2285 us at batch 2, 320 x 320; given to every
-            # branch it starves the weight gradients, 9.31 -> 9.74 ms at batch 16)
+            # (priority for the branch that holds the longest chain: 2260 -> 2232 us at batch 2, 320 x 320; given to every
+            # branch it starves the weight gradients, 9.46 -> 9.79 ms at batch 16)
             self._record_streams = torch.cuda.Stream(self.dev, priority=-1), torch.cuda.Stream(self.dev), []
         main, side, spare = self._record_streams
         graph = torch.cuda.CUDAGraph()
