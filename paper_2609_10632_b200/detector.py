@@ -28,6 +28,7 @@ from the order of the backward pass; zeroed beforehand only if the overwriting c
 from __future__ import annotations
 
 import gc
+import threading
 from operator import attrgetter
 
 import torch
@@ -76,6 +77,30 @@ def _overlap(a, b):
         d = (b[1] - a[1]) % a[3]
         return d < a[4] or d + b[4] > a[3]
     return True
+
+
+class _NoCollection:
+    """No garbage collection while any thread is in the block: it could free somebody's old CUDA graph, which is not permitted
+    in a thread that captures."""
+
+    def __init__(self):
+        self.lock, self.inside, self.collecting = threading.Lock(), 0, False
+
+    def __enter__(self):
+        with self.lock:
+            if self.inside == 0:
+                self.collecting = gc.isenabled()
+                gc.disable()
+            self.inside += 1
+
+    def __exit__(self, *exc):
+        with self.lock:
+            self.inside -= 1
+            if self.inside == 0 and self.collecting:
+                gc.enable()
+
+
+_no_collection = _NoCollection()
 
 
 class _Lanes:
@@ -467,13 +492,8 @@ class GraphRunner:
         main, side, spare = self._record_streams
         graph = torch.cuda.CUDAGraph()
         before = nb.nb_cbs_launch_count()
-        collecting = gc.isenabled()
-        gc.disable()  # (a collection could free somebody's old CUDA graph, which is not permitted while this thread captures)
-        try:
+        with _no_collection:
             self._capture(graph, issue, main, side if with_side else None, spare)
-        finally:
-            if collecting:
-                gc.enable()
         rec.launches = nb.nb_cbs_launch_count() - before
         nb.replayed_launches -= rec.launches  # recorded, not launched
         rec.graph = graph

@@ -83,6 +83,7 @@ def test_null_plan_arguments(lib):
     assert lib.nb_conv_bn_silu_fwd(None, *([None] * 11), 0, None) == nb.NB_ERR_INVALID_ARG
     assert lib.nb_conv_bn_silu_bwd_data(None, *([None] * 12), 0, None) == nb.NB_ERR_INVALID_ARG
     assert lib.nb_conv_bn_silu_bwd_weight(None, None, None, None, None, 0, None) == nb.NB_ERR_INVALID_ARG
+    assert lib.nb_conv_bn_silu_bwd(None, *([None] * 14), 0, None) == nb.NB_ERR_INVALID_ARG
     assert lib.nb_bn_stats(None, None, 0, None, None, None, None, None, 0, None) == nb.NB_ERR_INVALID_ARG
 
 

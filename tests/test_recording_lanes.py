@@ -47,3 +47,33 @@ def test_branches_keep_the_order_of_conflicting_calls(monkeypatch):
         stream.done.add(i)
     lanes.finish()
     assert main.done == set(range(len(calls))) and len(lanes.streams) == 3
+
+
+def test_no_collection_while_any_recording_is_open():
+    import gc
+    import threading
+
+    assert gc.isenabled()
+    block, opened, leave = detector._NoCollection(), threading.Event(), threading.Event()
+
+    def other():
+        with block:
+            opened.set()
+            leave.wait(10)
+
+    thread = threading.Thread(target=other)
+    with block:
+        thread.start()
+        opened.wait(10)
+        assert not gc.isenabled()
+    assert not gc.isenabled()  # the other thread's recording goes on
+    leave.set()
+    thread.join()
+    assert gc.isenabled()
+    gc.disable()
+    try:
+        with block:
+            pass
+        assert not gc.isenabled()  # left as it was found
+    finally:
+        gc.enable()
