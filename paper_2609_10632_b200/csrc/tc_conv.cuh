@@ -1019,14 +1019,15 @@ inline void fill_params(IgemmParams& P, const IgemmCfg& c) {
 }
 
 // The split form of a launch (tc_split_kernel), where it is the faster one; cfg.ok stays false elsewhere.  `min_taps`: taps of
-// the lightest parity class.  Times in us, fitted to measurements on B200 over the detector's layers at batch 1 (640 x 640)
-// and 2 (320 x 320): a CTA fetches a k-block at about 55 bytes per cycle and the tensor pipe needs max(45, BN / 2) cycles per
-// K = 16 step, whichever is longer; then the hand-over and the stores, which the persistent kernel does with TMA and, in the
-// training calls, behind a predecessor that still drains (`eval`: the evaluation-mode call, whose persistent form derives
-// every channel's coefficients in every CTA instead).
-// Measured, evaluation-mode forward of the 77 layers, one image: 1251 -> 649 us; single layers: 288 -> 288 3x3 at 20 x 20
-// 20.6 -> 7.5 us (8 tiles of 45 k-blocks -> 28 of 9), 192 -> 192 3x3 at 40 x 40 15.1 -> 7.8, 384 -> 384 1x1 at 40 x 40
-// 9.5 -> 5.5; data gradient of 288 -> 288 at 20 x 20 (the whole call) 28.6 -> 16.2.
+// the lightest parity class.  `eval`: the evaluation-mode call, whose K range a cluster may share.  Times in us, fitted to every
+// admissible (tile, cluster) on the detector's layers at batch 1 (640 x 640) and 2 (320 x 320), 830 of them, each between others of
+// its kind: 1.5 to the first operands, 0.147 a k-block whatever the tile's width (its 128 activation rows are written to and read
+// from shared memory once each), 0.018 a column behind the last MMA, 1.05 x the share of the SMs that are taken (more CTAs, more
+// rows through L2), 0.3 where successive launches cannot be on different SMs, and for a cluster the exchange.  The choices are
+// within 1 % of the best ones in sum.  The persistent form: 0.28 a k-block, 6 us besides.
+// Measured, evaluation-mode forward of the 77 layers, one image: 1251 us with the persistent form, 646 with split launches, 530
+// with the epilogue and the choices as they are now; single layers, persistent / split: 288 -> 288 3x3 at 20 x 20 26 / 6.3 (cluster
+// of four, 48 columns), 192 -> 192 3x3 at 40 x 40 14.9 / 6.6, 384 -> 384 1x1 at 40 x 40 9.4 / 4.0.
 inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_taps, bool eval, int sm_count) {
     out = full;
     out.cfg = IgemmCfg();
@@ -1036,10 +1037,11 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     if (getenv("NB_TC_SPLIT") && atoi(getenv("NB_TC_SPLIT")) == 0) return;
     const long long m_tiles = (f.M + TC_BM - 1) / TC_BM;
     if (m_tiles * ncls > sm_count) return;
-    auto kb_time = [](int bn) { return std::max(4.0 * std::max(45.0, bn / 2.0), (TC_BM + bn) * 128 / 55.0) / 1900.0; };
+    // k-blocks of the longest class, a 32-channel one counted as half
+    const double kb_eff = kblocks - (f.tail32 ? 0.5 * f.ntaps : 0.0);
     const int workers = f.cg2 ? f.grid / 2 : f.grid;
     const double full_waves = (double)(((long long)f.m_tiles * f.n_tiles * ncls + workers - 1) / workers);
-    double best = 4.5 + full_waves * (kblocks * f.mh * kb_time(f.BN) + 0.8);
+    double best = 5.2 + full_waves * (kb_eff * f.mh * 0.28 + 0.8);
     const int force_s = getenv("NB_TC_SPLIT_S") ? atoi(getenv("NB_TC_SPLIT_S")) : 0, force_bn = getenv("NB_TC_SPLIT_BN") ? atoi(getenv("NB_TC_SPLIT_BN")) : 0;
     if (force_s || force_bn) best = 1e30;
     int best_bn = 0, best_s = 0;
@@ -1050,7 +1052,7 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
         for (int s = 1; s <= (eval ? 8 : 1) && s <= min_kb; s *= 2) {
             const long long ctas = m_tiles * nt * ncls * s;
             if (ctas > (s == 8 ? sm_count * 6 / 7 : s == 4 ? sm_count * 9 / 10 : sm_count) || (force_s && s != force_s)) continue;
-            const double t = 3.5 + ((kblocks + s - 1) / s) * kb_time(bn) + 0.012 * bn + (s > 1 ? 1.2 : 0.0) + (eval ? 0.0 : 0.5 + 0.023 * bn / s);
+            const double t = 1.5 + 0.147 * kb_eff / s + 0.018 * bn + 1.05 * (double)ctas / sm_count + (2 * ctas > sm_count ? 0.3 : 0.0) + (s > 1 ? 0.8 + 0.011 * bn : 0.0);
             if (t < best) {
                 best = t;
                 best_bn = bn;
@@ -1070,10 +1072,12 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     c.tmem_cols = 32;
     while (c.tmem_cols < best_bn) c.tmem_cols *= 2;
     c.acc_stride = c.tmem_cols;
-    c.stages = std::max(2, std::min(8, (kblocks + best_s - 1) / best_s));
-    const size_t part = (size_t)TC_BM * (best_bn + 4) * 4, fixed = 1024 + 64 + (size_t)8 * 128 * 4 + 512;
+    c.stages = std::max(2, std::min(14, (kblocks + best_s - 1) / best_s));
+    // behind the stages: the shares of a cluster, coefficients, barriers; the training forward stages its rounded rows over the stages
+    const size_t share = best_s > 1 ? (size_t)TC_BM * (best_bn + 4 * SP_PARTS) * 4 : 0, fixed = 1024 + 64 + share + (size_t)2 * 128 * 4 + 512;
     while (c.stages > 2 && fixed + (size_t)c.stages * (c.a_stage + c.b_stage) > kMaxSmem) --c.stages;
-    c.smem_bytes = std::max<size_t>(fixed + std::max(part, (size_t)c.stages * (c.a_stage + c.b_stage)), 120 * 1024);  // > half an SM: one CTA per SM
+    while (best_s > 1 && (size_t)c.stages * (c.a_stage + c.b_stage) < share) ++c.stages;  // (a CTA's own shares lie over its stages)
+    c.smem_bytes = std::max<size_t>(fixed + (size_t)c.stages * (c.a_stage + c.b_stage), 120 * 1024);  // > half an SM: one CTA per SM
     c.grid = (int)(m_tiles * c.n_tiles * ncls * best_s);
     IgemmParams& P = out.prm;
     P.BN = c.BN; P.n_tiles = c.n_tiles; P.m_tiles = c.m_tiles; P.tiles_per_class = c.m_tiles * c.n_tiles;
@@ -1207,24 +1211,32 @@ template <typename OutT, bool STATS> inline nb_status launch_igemm(const TcGemmS
     }
     return s.cfg.cg2 ? launch_igemm_impl<OutT, STATS, true>(s, st) : launch_igemm_impl<OutT, STATS, false>(s, st);
 }
-template <typename OutT, int MODE> inline nb_status launch_split(const TcGemmSlot& s, cudaStream_t st) {
+template <typename OutT, int MODE, int S> inline nb_status launch_split_impl(const TcGemmSlot& s, cudaStream_t st) {
     static std::atomic<unsigned long long> attr_set{0};  // one bit per device ordinal
     int dev = 0;
     cudaGetDevice(&dev);
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(attr_set.load(std::memory_order_acquire) & bit)) {
-        if (cudaFuncSetAttribute(tc_split_kernel<OutT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess) {
+        if (cudaFuncSetAttribute(tc_split_kernel<OutT, MODE, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess) {
             err() = "cannot raise the dynamic shared memory limit of the split implicit-GEMM kernel";
             return NB_ERR_CUDA;
         }
         attr_set.fetch_or(bit, std::memory_order_release);
     }
-    const cudaError_t e = launch_k(tc_split_kernel<OutT, MODE>, dim3((unsigned)s.cfg.grid), dim3(SP_THREADS), s.cfg.smem_bytes, st, s.cfg.split, s.prm);
+    const cudaError_t e = launch_k(tc_split_kernel<OutT, MODE, S>, dim3((unsigned)s.cfg.grid), dim3(SP_THREADS), s.cfg.smem_bytes, st, S, s.prm);
     if (e != cudaSuccess) {
         err() = std::string("launch of tc_split_kernel failed: ") + cudaGetErrorString(e);
         return NB_ERR_CUDA;
     }
     return NB_OK;
+}
+template <typename OutT, int MODE> inline nb_status launch_split(const TcGemmSlot& s, cudaStream_t st) {
+    if constexpr (MODE == 2) {  // (the training calls use clusters of one)
+        if (s.cfg.split == 8) return launch_split_impl<OutT, MODE, 8>(s, st);
+        if (s.cfg.split == 4) return launch_split_impl<OutT, MODE, 4>(s, st);
+        if (s.cfg.split == 2) return launch_split_impl<OutT, MODE, 2>(s, st);
+    }
+    return launch_split_impl<OutT, MODE, 1>(s, st);
 }
 }  // namespace tcdetail
 

@@ -1,15 +1,16 @@
 // Implicit GEMM for layers with few output tiles (one or two images at 40 x 40 and below), sm_100a.
 // The persistent kernel of tc_conv.cuh gives such a layer a handful of CTAs, each of which walks the whole K range alone:
 // 288 -> 288 3x3 on one 20 x 20 image is 8 tiles of 45 k-blocks on 148 SMs, 20 us of one CTA's operand fetches.  Here the
-// K range of a tile is cut over a CLUSTER of 1, 2, 4 or 8 CTAs.  Every CTA accumulates its share in TMEM, leaves it as fp32
-// in its own shared memory, and after one cluster barrier CTA r sums rows [128 r / S, 128 (r + 1) / S) of all S partial
-// tiles through distributed shared memory, in rank order (the same bits every run), applies the epilogue and stores.
+// K range of a tile is cut over a CLUSTER of 1, 2, 4 or 8 CTAs.  Every CTA accumulates its share in TMEM and sends the rows of
+// every rank to that rank's shared memory by bulk copies; CTA r then sums rows [128 r / S, 128 (r + 1) / S) of all S shares in
+// rank order (the same bits every run), applies the epilogue and stores.
 // The training calls use clusters of one (narrow tiles only): the sum of an element then runs over the k-blocks in the order
 // in which the persistent kernel would add them (the same starting k-block), and the channel sums are formed as there, so
 // that the results of a training step do not depend on which of the two kernels a layer gets -- a deep network in training
 // mode turns a difference in the last bit of one layer into percents a few dozen layers on.
-// No block waits for a block outside its cluster.  Bound: latency -- operand fetch to first MMA, the k-blocks of one CTA
-// (a k-block is (128 + BN) 128-byte rows through TMA), accumulator -> shared memory -> peers -> rounding -> store.
+// No block waits for a block outside its cluster.  Bound: latency.  192 -> 192 3x3 on one 40 x 40 image, us behind the end of the
+// launch before: 0.8 until that has reached the CTA, 0.6 until the last CTA runs (an SM holds one), 1.1 to the first operands,
+// 0.15 a k-block (its 128 + BN rows are written to and read from shared memory once each), 0.5 to 0.8 behind the last MMA.
 // The narrow tiles (BN <= 128, often 32 to 64) are part of the same idea: more CTAs, and less to hand over.
 // Measured against the persistent kernel: see split_configure below.
 // Included by tc_conv.cuh (uses its parameter record and bounded-wait helpers).
@@ -18,11 +19,27 @@
 namespace nbcbs {
 
 constexpr int SP_THREADS = 256;
+constexpr int SP_PARTS = SP_THREADS / 128;  // warps that share a quarter's columns (sixteen warps: evaluation of one image 551 -> 563 us)
+// First column of a part's share (whole 16-column pieces) and the part of a column.
+__device__ __forceinline__ int sp_part_lo(int part, int BN) { return part * (BN / 16) / SP_PARTS * 16; }
+__device__ __forceinline__ int sp_part_of(int c, int BN) { return (c / 16 * SP_PARTS + SP_PARTS - 1) / (BN / 16); }
 
-__device__ __forceinline__ float4 ld_dsmem4(uint32_t cluster_addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr) : "memory");
-    return v;
+// `bytes` of this CTA's shared memory to the shared memory of a CTA of the cluster; counted on that CTA's barrier `bar`.
+__device__ __forceinline__ void copy_to_peer(uint32_t dst_cluster, const void* src, uint32_t bytes, uint32_t bar_cluster) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_cluster), "r"(ptx::smem_u32(src)), "r"(bytes),
+                 "r"(bar_cluster)
+                 : "memory");
+}
+__device__ __forceinline__ float tanh_fast(float v) {
+    float t;
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(v));
+    return t;
+}
+// 32 bytes on a 32-byte boundary
+__device__ __forceinline__ void st_global32(void* p, const uint2 (&v)[4]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0].x), "r"(v[0].y), "r"(v[1].x), "r"(v[1].y), "r"(v[2].x), "r"(v[2].y), "r"(v[3].x),
+                 "r"(v[3].y)
+                 : "memory");
 }
 __device__ __forceinline__ void prefetch_tile_2d(const CUtensorMap* m, int c0, int c1) {
     asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1) : "memory");
@@ -30,22 +47,26 @@ __device__ __forceinline__ void prefetch_tile_2d(const CUtensorMap* m, int c0, i
 
 // MODE 0: plain 16-bit output (data gradient; may be pitched, may be added to what the output holds).  MODE 1: training
 // forward (fp16 output, channel sums of the rounded values to the accumulators).  MODE 2: per-channel scale and shift, SiLU.
-template <typename OutT, int MODE>
+// S: CTAs of a cluster (p.split).
+template <typename OutT, int MODE, int S>
 __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_constant__ IgemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* sA = smem;
     uint8_t* sB = sA + (size_t)p.stages * p.a_stage_bytes;
-    float* part = reinterpret_cast<float*>(smem);  // [128][BN + 4] this CTA's share, over the operand stages once they are consumed
-    const int S = p.split, pitch = p.BN + 4;
-    const size_t stage_total = (size_t)p.stages * (p.a_stage_bytes + p.b_stage_bytes), part_total = (size_t)TC_BM * pitch * 4;
-    float* red = reinterpret_cast<float*>(smem + ((stage_total > part_total ? stage_total : part_total) + 15) / 16 * 16);  // MODE 1: channel sums [4][2][BN]; MODE 2: scale, shift [2][BN]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(red + 8 * 128);
+    // S > 1: one slot per rank with that rank's share of this CTA's 128 / S rows, for each part of the columns [rows][columns + 4],
+    // written by the ranks themselves (behind the operand stages, which may still be in use when a peer's share arrives)
+    float* const part = reinterpret_cast<float*>(sB + (size_t)p.stages * p.b_stage_bytes);
+    constexpr int ROWS = TC_BM / S;
+    const int slot = ROWS * (p.BN + 4 * SP_PARTS);
+    float* red = part + (S > 1 ? S * slot : 0);  // MODE 2: scale, shift [2][BN]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(red + 2 * 128);
     uint64_t* full = bars;
     uint64_t* empty = bars + p.stages;
     uint64_t* tfull = empty + p.stages;
     uint64_t* drain = tfull + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    uint64_t* shares = drain + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(shares + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     if (MODE != 0) pdl_launch_dependents();
@@ -73,8 +94,15 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
         }
         ptx::mbar_init(tfull, 1);
         ptx::mbar_init(drain, 1);
+        if (S > 1) ptx::mbar_init(shares, 1);
         *abort_flag = 0;
         ptx::fence_mbar_init();
+        if (S > 1) {
+            int cols = 0;
+            for (int k = 0; k < SP_PARTS; ++k)
+                if (sp_part_lo(k + 1, p.BN) > sp_part_lo(k, p.BN)) cols += sp_part_lo(k + 1, p.BN) - sp_part_lo(k, p.BN) + 4;
+            ptx::mbar_expect_tx(shares, (uint32_t)(TC_BM * cols * 4));
+        }
     }
     if (warp == 2 && lane == 0) {
         ptx::prefetch_tmap(&p.tmB[cls]);
@@ -94,7 +122,10 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    if (S > 1) ptx::cluster_arrive_relaxed();  // (this CTA runs and its barriers are set up: the others may write its shared memory)
     const uint32_t tmem_base = *tmem_slot;
+    // (the producers wait right before their first load; for the others, whose turn comes later, the wait is over by then)
+    if (warp != 0 && warp != 2) pdl_wait();
 
     if (warp == 0 || warp == 2) {
         // ------------------------------------------------------------------ TMA producers: warp 0 feeds A, warp 2 feeds B
@@ -196,138 +227,187 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
             }
         }
     } else if (MODE == 2) {
-        // warps 3-7 meanwhile derive the coefficients of this tile's columns (fp64, like the training-mode finalize)
-        pdl_wait();
+        // the other warps meanwhile derive the coefficients of this tile's columns (fp64, like the training-mode finalize)
         for (int c = (int)threadIdx.x - 96; c < p.BN; c += SP_THREADS - 96) {
             double sc = 0.0, sh = 0.0;
             const int ch = n_tile * p.BN + c;
             if (ch < p.ldo) bn_eval_coef(p.fin_gamma, p.fin_beta, p.fin_rmean, p.fin_rvar, p.fin_eps, ch, sc, sh);
-            red[c] = (float)sc;
-            red[p.BN + c] = (float)sh;
+            const double half = p.epi_act ? 0.5 : 1.0;  // (exact; see finish)
+            red[c] = (float)(sc * half);
+            red[p.BN + c] = (float)(sh * half);
         }
     }
     __syncwarp();
 
-    // ---------------------------------------------------------------------- all eight warps: TMEM -> own shared memory
+    // ---------------------------------------------------------------------- all warps: accumulators -> rounding -> rows
     bool ok = true;
     if (lane == 0) ok = wait_bar(tfull, 0, abort_flag, p.status, 4);
     ok = __syncthreads_and((int)(__shfl_sync(0xffffffffu, (int)ok, 0) != 0)) != 0;
-    if (ok) {
-        ptx::tc_fence_after();
-        const int q = warp & 3;  // TMEM lanes (rows) 32 q .. 32 q + 31; the two warps of a quarter take alternate 16-column pieces
-        float* row = part + (size_t)(q * 32 + lane) * pitch;
-        for (int c = (warp >> 2) * 16; c < p.BN; c += 32) {
-            uint32_t r[16];
-            ptx::tmem_ld_32x32b_x16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c, r);
-            ptx::tmem_ld_wait();
+    const int q = warp & 3, share = warp >> 2, c_lo = sp_part_lo(share, p.BN), nc = sp_part_lo(share + 1, p.BN) - c_lo;  // its rows and columns
+    int sat_bits = 0;
+    // act(v * scale + shift) of four neighbouring columns from c on (MODE 2), rounded and packed.  The coefficients of SiLU are
+    // halved: z * sigmoid(z) = h + h * tanh(h) with h = z / 2.
+    auto finish = [&](const float* v, int c) {
+        float2 a = make_float2(v[0], v[1]), b = make_float2(v[2], v[3]);
+        if (MODE == 2) {
+            const float4 sc = *reinterpret_cast<const float4*>(red + c), sh = *reinterpret_cast<const float4*>(red + p.BN + c);
+            a = fma2(a, make_float2(sc.x, sc.y), make_float2(sh.x, sh.y));
+            b = fma2(b, make_float2(sc.z, sc.w), make_float2(sh.z, sh.w));
+            if (p.epi_act) {
+                a = fma2(a, make_float2(tanh_fast(a.x), tanh_fast(a.y)), a);
+                b = fma2(b, make_float2(tanh_fast(b.x), tanh_fast(b.y)), b);
+            }
+        }
+        return make_uint2(pack2<OutT>(a.x, a.y, &sat_bits), pack2<OutT>(b.x, b.y, &sat_bits));
+    };
+    ptx::tc_fence_after();
+    if constexpr (S == 1) {
+        // MODE 1: the rounded rows for the channel sums, [quarter][32 rows] of BN * 2 + 16 bytes over the consumed operand stages
+        const int srow = p.BN * 2 + 16, squarter = 32 * srow + 32;  // (32 bytes between the quarters: other banks)
+        // A lane stores its row's 32 bytes of a piece at once.  Fewer instructions count most here, since a warp runs this code once:
+        // a [128 x 48] tile leaves 0.75 us behind its last MMA, 1.0 with the rows staged in shared memory for stores of whole
+        // lines, 2.3 when all accumulators went through shared memory to threads of four columns; [128 x 96] 1.4, 1.6 and 4.1.
+        if (ok) {
+            const int grow = m_tile * TC_BM + q * 32 + lane;  // (row counts of the tensor-core path fit 31 bits)
+            bool live = grow < (int)p.M;
+            long long orow = grow;
+            if (MODE == 0 && p.os != 1) {
+                const unsigned t1 = (unsigned)grow / (unsigned)p.Wq, n = t1 / (unsigned)p.Hq;
+                const int oi = (int)(t1 - n * (unsigned)p.Hq) * p.os + p.cls_oa[cls], oj = (grow - (int)t1 * p.Wq) * p.os + p.cls_ob[cls];
+                live = live && oi < p.Hout && oj < p.Wout;  // (odd extents: the grid of an odd parity is longer than the image)
+                orow = ((long long)n * p.Hout + oi) * p.Wout + oj;
+            }
+            OutT* const dst = static_cast<OutT*>(p.out) + orow * p.ld_out + n_tile * p.BN;
+            const bool wide = ((reinterpret_cast<uintptr_t>(p.out) | (uintptr_t)p.ld_out * 2) & 31) == 0;  // (pieces start at multiples of 32 bytes)
+            const int cols = p.ldo - n_tile * p.BN;  // columns of this tile that exist (a multiple of 8)
+            uint8_t* const staged = smem + (size_t)q * squarter + (size_t)lane * srow;
+#pragma unroll 1
+            for (int c = c_lo; c < c_lo + nc; c += 16) {
+                uint32_t r[16];
+                ptx::tmem_ld_32x32b_x16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c, r);
+                ptx::tmem_ld_wait();
+                const int before = sat_bits;
+                uint2 o[4];
 #pragma unroll
-            for (int j = 0; j < 16; j += 4)
-                *reinterpret_cast<float4*>(row + c + j) = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+                for (int j = 0; j < 4; ++j) o[j] = finish(reinterpret_cast<const float*>(r) + 4 * j, c + 4 * j);
+                if (MODE == 1) {
+                    *reinterpret_cast<uint4*>(staged + c * 2) = make_uint4(o[0].x, o[0].y, o[1].x, o[1].y);
+                    *reinterpret_cast<uint4*>(staged + c * 2 + 16) = make_uint4(o[2].x, o[2].y, o[3].x, o[3].y);
+                }
+                if (!live) {
+                    sat_bits = before;
+                    continue;
+                }
+                if (MODE == 0 && p.out_accumulate) {  // the rounded tile is added, as a TMA reduction would
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (c + 4 * j >= cols) break;
+                        const uint2 old = *reinterpret_cast<const uint2*>(dst + c + 4 * j);
+                        const OutT *po = reinterpret_cast<const OutT*>(&old), *pn = reinterpret_cast<const OutT*>(&o[j]);
+                        uint2 sum;
+                        OutT* ps = reinterpret_cast<OutT*>(&sum);
+                        pair_from_f32(ps, add2(pair_to_f32(po), pair_to_f32(pn)));
+                        pair_from_f32(ps + 2, add2(pair_to_f32(po + 2), pair_to_f32(pn + 2)));
+                        o[j] = sum;
+                    }
+                }
+                if (wide && c + 16 <= cols) {
+                    st_global32(dst + c, o);
+                } else {
+                    if (c < cols) *reinterpret_cast<uint4*>(dst + c) = make_uint4(o[0].x, o[0].y, o[1].x, o[1].y);
+                    if (c + 8 < cols) *reinterpret_cast<uint4*>(dst + c + 8) = make_uint4(o[2].x, o[2].y, o[3].x, o[3].y);
+                }
+            }
         }
         ptx::tc_fence_before();
+        __syncthreads();
+        if (MODE == 1 && ok && warp < p.BN / 16) {
+            // channel sums of the rounded values: a lane takes two channels of one quarter's 32 rows, even and odd rows apart, then
+            // the four quarters are added in order (the persistent kernel's grouping; rows past the last pixel are zeros)
+            const int c2 = warp * 8 + (lane & 7), grp = lane >> 3;
+            float2 sa = make_float2(0.f, 0.f), sb = sa, qa = sa, qb = sa;
+            const uint8_t* src = smem + (size_t)grp * squarter + c2 * 4;
+#pragma unroll
+            for (int rr = 0; rr < 32; rr += 2) {
+                const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(src + rr * srow));
+                const float2 f1 = __half22float2(*reinterpret_cast<const __half2*>(src + (rr + 1) * srow));
+                sa = add2(sa, f0);
+                sb = add2(sb, f1);
+                qa = fma2(f0, f0, qa);
+                qb = fma2(f1, f1, qb);
+            }
+            float v[4] = {sa.x + sb.x, sa.y + sb.y, qa.x + qb.x, qa.y + qb.y};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float v1 = __shfl_down_sync(0xffffffffu, v[e], 8), v2 = __shfl_down_sync(0xffffffffu, v[e], 16), v3 = __shfl_down_sync(0xffffffffu, v[e], 24);
+                v[e] = ((v[e] + v1) + v2) + v3;
+            }
+            const int ch = n_tile * p.BN + 2 * c2;
+            if (grp == 0 && ch < p.ldo) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) chan_acc_add<false>(p.acc, p.ldo, e >> 1, ch + (e & 1), v[e]);
+            }
+        }
+    } else {
+        // Every CTA's share of the sums goes to the rank that owns the rows: into this CTA's own shared memory (over the consumed
+        // stages), from there as bulk copies, which a rank counts on its barrier `shares`.  Then each rank adds in rank order.
+        // (Loads of the shares from the peers behind a cluster barrier: 2.4 us for [32 x 96] of four ranks; stores into the peers'
+        // memory, 16 bytes of 32 rows at a time: 1.8 us and a cluster barrier of 1 us.)
+        ptx::cluster_wait();
+        if (ok && nc) {
+            float* const mine = reinterpret_cast<float*>(smem) + TC_BM * (c_lo + 4 * share) + q * 32 * (nc + 4);
+#pragma unroll 1
+            for (int c = 0; c < nc; c += 16) {
+                uint32_t r[16];
+                ptx::tmem_ld_32x32b_x16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(c_lo + c), r);
+                ptx::tmem_ld_wait();
+#pragma unroll
+                for (int j = 0; j < 16; j += 4) *reinterpret_cast<uint4*>(mine + lane * (nc + 4) + c + j) = make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
+            }
+            ptx::fence_async_smem();
+            __syncwarp();
+            constexpr int CHUNK = ROWS < 32 ? ROWS : 32;  // rows of this warp that go to one rank
+            if (lane < 32 / CHUNK) {
+                const int row = q * 32 + lane * CHUNK;
+                const uint32_t to = (uint32_t)(row / ROWS);
+                copy_to_peer(ptx::mapa_u32(ptx::smem_u32(part + (size_t)rank * slot + ROWS * (c_lo + 4 * share) + row % ROWS * (nc + 4)), to), mine + lane * CHUNK * (nc + 4),
+                             (uint32_t)(CHUNK * (nc + 4) * 4), ptx::mapa_u32(ptx::smem_u32(shares), to));
+            }
+        }
+        ptx::tc_fence_before();
+        if (lane == 0 && ok) ok = wait_bar(shares, 0, abort_flag, p.status, 4);
+        ok = __syncthreads_and((int)(__shfl_sync(0xffffffffu, (int)ok, 0) != 0)) != 0;
+        ptx::cluster_arrive_relaxed();
+        if (ok) {
+            // a thread keeps a group of four columns
+            const int groups = p.BN / 4, r0 = (int)threadIdx.x / groups, rp = SP_THREADS / groups, c = ((int)threadIdx.x - r0 * groups) * 4;
+            const int from = sp_part_of(c, p.BN), from_lo = sp_part_lo(from, p.BN), from_pitch = sp_part_lo(from + 1, p.BN) - from_lo + 4;
+            const float* const base = part + ROWS * (from_lo + 4 * from) + c - from_lo;
+            const int row_end = r0 < rp && c < p.ldo - n_tile * p.BN ? min(ROWS, (int)p.M - m_tile * TC_BM - rank * ROWS) : 0;
+            OutT* const dst = static_cast<OutT*>(p.out) + (long long)(m_tile * TC_BM + rank * ROWS) * p.ld_out + n_tile * p.BN + c;
+#pragma unroll 1
+            for (int row = r0; row < row_end; row += rp) {
+                const float* const src = base + row * from_pitch;
+                float4 v[S];
+#pragma unroll
+                for (int j = 0; j < S; ++j) v[j] = *reinterpret_cast<const float4*>(src + (size_t)j * slot);
+#pragma unroll
+                for (int j = 1; j < S; ++j) {
+                    v[0].x += v[j].x;
+                    v[0].y += v[j].y;
+                    v[0].z += v[j].z;
+                    v[0].w += v[j].w;
+                }
+                *reinterpret_cast<uint2*>(dst + (long long)row * p.ld_out) = finish(reinterpret_cast<const float*>(&v[0]), c);
+            }
+        }
     }
-    if (S > 1) ptx::cluster_sync_all(); else __syncthreads();
+    if (sat_bits & (int)0x80008000u) atomicAdd(p.status + ST_SAT, 1);
     if (warp == 1) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
     }
-
-    // ---------------------------------------------------------------------- sum this CTA's rows over the cluster, epilogue, store
-    pdl_wait();
-    if (ok) {
-        const int ng = p.BN / 4, rows = TC_BM / S, rp = SP_THREADS / ng;  // a thread keeps one group of four columns
-        const int gi = (int)threadIdx.x % ng, r0 = (int)threadIdx.x / ng;
-        const int col = n_tile * p.BN + gi * 4;
-        const bool live = r0 < rp && col < p.ldo;
-        const uint32_t part_u32 = ptx::smem_u32(part);
-        float4 sc = make_float4(0.f, 0.f, 0.f, 0.f), sh = sc;
-        if (MODE == 2) {
-            sc = *reinterpret_cast<const float4*>(red + gi * 4);
-            sh = *reinterpret_cast<const float4*>(red + p.BN + gi * 4);
-        }
-        int sat_bits = 0;
-        for (int row = r0; live && row < rows; row += rp) {
-            const int grow = m_tile * TC_BM + rank * rows + row;  // (row counts of the tensor-core path fit 31 bits)
-            if (grow >= (int)p.M) break;
-            const uint32_t at = part_u32 + (uint32_t)(((rank * rows + row) * pitch + gi * 4) * 4);
-            float4 v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j < S) v[j] = S > 1 ? ld_dsmem4(ptx::mapa_u32(at, (uint32_t)j)) : *reinterpret_cast<const float4*>(part + (size_t)row * pitch + gi * 4);
-            float4 a = v[0];
-#pragma unroll
-            for (int j = 1; j < 8; ++j)
-                if (j < S) {
-                    a.x += v[j].x;
-                    a.y += v[j].y;
-                    a.z += v[j].z;
-                    a.w += v[j].w;
-                }
-            if (MODE == 2) {
-                float2 z0 = fma2(make_float2(a.x, a.y), make_float2(sc.x, sc.y), make_float2(sh.x, sh.y));
-                float2 z1 = fma2(make_float2(a.z, a.w), make_float2(sc.z, sc.w), make_float2(sh.z, sh.w));
-                if (p.epi_act) {
-                    z0 = mul2(z0, sigmoid2<true>(z0));
-                    z1 = mul2(z1, sigmoid2<true>(z1));
-                }
-                a = make_float4(z0.x, z0.y, z1.x, z1.y);
-            }
-            uint2 o;
-            o.x = pack2<OutT>(a.x, a.y, &sat_bits);
-            o.y = pack2<OutT>(a.z, a.w, &sat_bits);
-            long long orow = grow;
-            if (p.os != 1) {
-                const unsigned t1 = (unsigned)grow / (unsigned)p.Wq, n = t1 / (unsigned)p.Hq;
-                const int oi = (int)(t1 - n * (unsigned)p.Hq) * p.os + p.cls_oa[cls], oj = (grow - (int)t1 * p.Wq) * p.os + p.cls_ob[cls];
-                if (oi >= p.Hout || oj >= p.Wout) continue;  // (odd extents: the grid of an odd parity is longer than the image)
-                orow = ((long long)n * p.Hout + oi) * p.Wout + oj;
-            }
-            OutT* dst = static_cast<OutT*>(p.out) + orow * p.ld_out + col;
-            if (MODE == 0 && p.out_accumulate) {  // the rounded tile is added, as a TMA reduction would
-                const uint2 old = *reinterpret_cast<const uint2*>(dst);
-                const OutT *po = reinterpret_cast<const OutT*>(&old), *pn = reinterpret_cast<const OutT*>(&o);
-                uint2 sum;
-                OutT* ps = reinterpret_cast<OutT*>(&sum);
-                pair_from_f32(ps, add2(pair_to_f32(po), pair_to_f32(pn)));
-                pair_from_f32(ps + 2, add2(pair_to_f32(po + 2), pair_to_f32(pn + 2)));
-                o = sum;
-            }
-            *reinterpret_cast<uint2*>(dst) = o;
-        }
-        int sat = sat_bits & (int)0x80008000u ? 1 : 0;
-        if (MODE == 1) {
-            // channel sums of the rounded values: a thread takes two channels of 32 rows, even and odd rows apart, then the
-            // four row groups are added in order (the persistent kernel's grouping; rows past the last pixel are zeros)
-            const int c2 = (int)threadIdx.x % (p.BN / 2), grp = (int)threadIdx.x / (p.BN / 2);
-            if (grp < 4) {
-                float2 sa = make_float2(0.f, 0.f), sb = sa, qa = sa, qb = sa;
-                const float* src = part + (size_t)grp * 32 * pitch + 2 * c2;
-#pragma unroll 8
-                for (int rr = 0; rr < 32; rr += 2) {
-                    const float2 a0 = *reinterpret_cast<const float2*>(src + (size_t)rr * pitch), a1 = *reinterpret_cast<const float2*>(src + (size_t)(rr + 1) * pitch);
-                    const uint32_t h0 = pack2<__half>(a0.x, a0.y, nullptr), h1 = pack2<__half>(a1.x, a1.y, nullptr);
-                    const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&h0)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&h1));
-                    sa = add2(sa, f0);
-                    sb = add2(sb, f1);
-                    qa = fma2(f0, f0, qa);
-                    qb = fma2(f1, f1, qb);
-                }
-                const float qx = qa.x + qb.x, qy = qa.y + qb.y;
-                float* dst = red + (size_t)grp * 2 * p.BN + 2 * c2;
-                *reinterpret_cast<float2*>(dst) = make_float2(sa.x + sb.x, sa.y + sb.y);
-                *reinterpret_cast<float2*>(dst + p.BN) = make_float2(qx, qy);
-            }
-            __syncthreads();
-            for (int e = threadIdx.x; e < 2 * p.BN; e += SP_THREADS) {
-                const int c = e >= p.BN ? e - p.BN : e;
-                if (n_tile * p.BN + c >= p.ldo) continue;
-                const float* b = red + e;
-                chan_acc_add<false>(p.acc, p.ldo, e >= p.BN ? 1 : 0, n_tile * p.BN + c, ((b[0] + b[2 * p.BN]) + b[4 * p.BN]) + b[6 * p.BN]);
-            }
-        }
-        if (sat) atomicAdd(p.status + ST_SAT, sat);
-    }
-    if (S > 1) ptx::cluster_sync_all();  // no CTA leaves while a peer may still read its rows
+    if (S > 1) ptx::cluster_wait();  // every rank has its shares: nobody reads this CTA's shared memory any more
 }
 
 }  // namespace nbcbs

@@ -53,3 +53,30 @@ def test_split_launches_match_oracle(dims, split, monkeypatch):
         blk.backward_data()
         torch.cuda.synchronize()
         assert torch.equal(wide, want)
+
+
+@pytest.mark.parametrize("split", [1, 2, 8])
+@pytest.mark.parametrize("cols", [16, 48, 80, 112, 128])
+def test_tile_widths_of_the_evaluation_call(cols, split, monkeypatch):
+    """Every way in which the warps share a tile's columns: one 16-column piece to eight of them, a last tile with padding
+    columns, k ranges of two k-blocks a rank (the fewest operand stages, over which the shares are laid)."""
+    import numpy as np
+    import oracle
+    import torch
+
+    from paper_2609_10632_b200 import binding as nb
+
+    monkeypatch.setenv("NB_TC_SPLIT_S", str(split))
+    monkeypatch.setenv("NB_TC_SPLIT_BN", str(cols))
+    shape = wl.ConvShape("width", 2, 9, 17, 128, 2 * cols - 8 if cols > 16 else 16, 3, 1)
+    inp = wl.make_inputs(shape, 47, cols, bf16=True, affine="random")
+    rm, rv, _ = wl.make_eval_stats(shape, 47, cols)
+    plan = nb.Plan.for_shape(shape, eps=EPS)
+    dev = lambda a, dt=torch.float32: torch.from_numpy(np.ascontiguousarray(a)).to(dt).cuda()
+    x, w = dev(inp.x, torch.bfloat16), dev(inp.w, torch.bfloat16)
+    out = torch.full((shape.n, shape.ho, shape.wo, shape.c_out), 7.0, dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(max(plan.infer_bytes, 256), dtype=torch.uint8, device="cuda")
+    nb.nb_conv_bn_silu_infer(plan, x, w, dev(inp.gamma), dev(inp.beta), dev(rm), dev(rv), out, ws)
+    torch.cuda.synchronize()
+    assert nb.nb_cbs_poll_status(plan) == ""
+    parity.check("a_eval", out.double().cpu().numpy(), oracle.cbs_infer(inp.x, inp.w, inp.gamma, inp.beta, rm, rv, shape.stride, EPS), "bf16")
