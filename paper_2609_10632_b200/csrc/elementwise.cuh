@@ -24,6 +24,14 @@ template <bool FAST> __device__ __forceinline__ float sigmoid_f(float z) {
     }
 }
 
+// SiLU of two values given as halves: z * sigmoid(z) = h + h * tanh(h) with h = z / 2.
+__device__ __forceinline__ float2 silu2_of_half(float2 h) {
+    float2 t;
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t.x) : "f"(h.x));
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t.y) : "f"(h.y));
+    return fma2(h, t, h);
+}
+
 // The same for two values at once, and dz = g * s * (1 + z*(1 - s)) with s = sigmoid(z) (the derivative of SiLU times g);
 // the operations and their order are those of the scalar expressions the passes used to spell out, so the bits agree.
 template <bool FAST> __device__ __forceinline__ float2 sigmoid2(float2 z) {

@@ -108,7 +108,7 @@ template <bool HALF> __device__ __forceinline__ int igemm_first_kblock(const Ige
 }
 
 constexpr int TC_BM = 128;
-constexpr int IG_THREADS = 352;  // implicit-GEMM kernel: the roles below plus a second epilogue team in warps 7-10
+constexpr int IG_THREADS = 384;  // implicit-GEMM kernel: the roles below plus a second epilogue team in warps 7-10 and a second MMA issuer in warp 11
 constexpr int TC_THREADS = 224;  // warp 0: TMA producer for A, warp 1: MMA issuer + TMEM owner, warps 2-5: epilogue, warp 6: TMA producer for B
 
 __device__ __forceinline__ uint64_t global_timer_ns() {
@@ -214,7 +214,7 @@ __device__ __forceinline__ void epi_pass_tma(uint32_t taddr, uint8_t* wrows, int
             for (int j = 0; j < NP; j += 2) {
                 const float4 cf = *reinterpret_cast<const float4*>(coef + j);
                 const float2 z = fma2(make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), make_float2(cf.x, cf.y), make_float2(cf.z, cf.w));
-                const float2 o = mul2(z, sigmoid2<true>(z));
+                const float2 o = silu2_of_half(z);  // (the coefficients are halved)
                 r[j] = __float_as_uint(o.x);
                 r[j + 1] = __float_as_uint(o.y);
             }
@@ -307,8 +307,8 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
     uint64_t* empty = bars + p.stages;    // [stages]
     uint64_t* tfull = empty + p.stages;   // [2]
     uint64_t* tempty = tfull + 2;         // [2]
-    uint64_t* drain = tempty + 2;         // [1]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    uint64_t* drain = tempty + 2;         // [2]
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     // the next kernel of the stream may become resident and run its prologue right away (behind a data gradient: once this
@@ -326,13 +326,14 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
         for (int s = 0; s < p.stages; ++s) {
             ptx::mbar_init(full + s, 2);  // the A and the B producer arrive once each with their byte counts (pairs: rank 0's
                                           // producers announce the bytes of both CTAs, the peer only issues its loads)
-            ptx::mbar_init(empty + s, 1);
+            ptx::mbar_init(empty + s, mh);  // (every issuer commits)
         }
-        ptx::mbar_init(tfull, 1);
-        ptx::mbar_init(tfull + 1, 1);
+        ptx::mbar_init(tfull, mh);
+        ptx::mbar_init(tfull + 1, mh);
         ptx::mbar_init(tempty, CG2 ? 16 : 256);  // pairs: one arrival per epilogue warp of both CTAs
         ptx::mbar_init(tempty + 1, CG2 ? 16 : 256);
         ptx::mbar_init(drain, 1);
+        ptx::mbar_init(drain + 1, 1);
         *abort_flag = 0;
         ptx::fence_mbar_init();
     }
@@ -371,8 +372,9 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
         for (int c = threadIdx.x; c < cols_pad; c += IG_THREADS) {
             double sc = 0.0, sh = 0.0;  // padding columns: zero, so that they cannot count as saturated stores
             if (c < p.ldo) bn_eval_coef(p.fin_gamma, p.fin_beta, p.fin_rmean, p.fin_rvar, p.fin_eps, c, sc, sh);
-            wstat[4 * (c >> 1) + (c & 1)] = (float)sc;
-            wstat[4 * (c >> 1) + 2 + (c & 1)] = (float)sh;
+            const double half = p.epi_act ? 0.5 : 1.0;  // (exact; see silu2_of_half)
+            wstat[4 * (c >> 1) + (c & 1)] = (float)(sc * half);
+            wstat[4 * (c >> 1) + 2 + (c & 1)] = (float)(sh * half);
         }
         __syncthreads();
     }
@@ -475,34 +477,39 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                 }
             }
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer (one thread; in a pair only rank 0)
+    } else if (warp == 1 || warp == 11) {
+        // ------------------------------------------------------------------ MMA issuers (in a pair those of rank 0): warp 1 for the
+        // first 128-row sub-tile, warp 11 for the second.  The operands are always there in time (a wait that finds them takes 105
+        // cycles); what a stage takes is an issuer's instructions: barrier, eight MMAs, commit, 820 cycles for 96 -> 96 channels
+        // 3x3, whose MMAs need 290 to 450.  Hence an issuer for each sub-tile, and the MMAs of a k-block in one block of code.
+        // Measured (step): 96 -> 96 3x3 on 16 x 160 x 160 pixels 367 -> 331 us, on 16 x 80 x 80 130 -> 114, 192 -> 192 on
+        // 16 x 40 x 40 95.5 -> 88 (one sub-tile: the block of code alone), 48 -> 48 on 16 x 160 x 160 207 -> 198.  Testing the next
+        // stage's barrier ahead of the MMAs of this one adds instructions and loses 0.5 to 2 us on the wide layers.
+        const int h = warp == 11 ? 1 : 0;
         const uint32_t leader = ptx::elect_one() ? 1u : 0u;  // the whole warp runs the loop, this lane issues
-        if (rank == 0) {
+        if (rank == 0 && h < mh) {
             int s = 0, acc = 0;
             uint32_t ph = 0, acc_ph = 0;
             bool ok = true;
-            const int ksteps = p.KC / 16, kpb = p.kpb, stages = p.stages;
+            const int kpb = p.kpb, stages = p.stages, kc_per_tap = p.kc_per_tap;
             const uint32_t idesc = p.idesc, acc_stride = (uint32_t)p.acc_stride;
-            const uint64_t a_sub16 = (uint64_t)(p.a_sub_bytes >> 4), b_sub16 = (uint64_t)(p.b_sub_bytes >> 4);
-            const uint64_t a_stage16 = (uint64_t)(p.a_stage_bytes >> 4), b_stage16 = (uint64_t)(p.b_stage_bytes >> 4);
-            const uint64_t a_half16 = (uint64_t)((TC_BM * p.KC * 2) >> 4);  // second 128-row sub-tile inside a k-block of A
+            // descriptors' low words (start address / 16): k-blocks, stages, this issuer's sub-tile of a whole and of a 32-channel k-block
+            const uint32_t a_sub = p.a_sub_bytes >> 4, b_sub = p.b_sub_bytes >> 4, a_stage = p.a_stage_bytes >> 4, b_stage = p.b_stage_bytes >> 4;
+            const uint32_t a_at = (uint32_t)h * ((TC_BM * p.KC * 2) >> 4), a_back = a_at >> 1;
+            const uint64_t da0 = ptx::make_smem_desc(ptx::smem_u32(sA), 16, p.sbo, p.umma_swizzle), db0 = ptx::make_smem_desc(ptx::smem_u32(sB), 16, p.sbo, p.umma_swizzle);
+            const uint32_t a0 = (uint32_t)da0 + a_at, b0 = (uint32_t)db0, hi = (uint32_t)(da0 >> 32);
             // 32-channel k-block: rows of 64 bytes in the 64-byte swizzle; same start address, other stride and swizzle fields
-            const uint64_t tail_flip = ptx::make_smem_desc(0u, 16, p.sbo, p.umma_swizzle) ^ ptx::make_smem_desc(0u, 16, p.sbo >> 1, (uint32_t)ptx::kSwizzle64);
-            const int kc_tail = p.tail32 ? p.kc_per_tap - 1 : -1;
-            const uint64_t da0 = ptx::make_smem_desc(ptx::smem_u32(sA), 16, p.sbo, p.umma_swizzle);
-            const uint64_t db0 = ptx::make_smem_desc(ptx::smem_u32(sB), 16, p.sbo, p.umma_swizzle);
-            const uint32_t empty_u32 = ptx::smem_u32(empty);
-            uint64_t da_s = da0, db_s = db0;  // descriptors of the current stage
-            const int kc_per_tap = p.kc_per_tap;
-            const uint32_t tfull_u32 = ptx::smem_u32(tfull);
+            const uint32_t hi_tail = (uint32_t)(ptx::make_smem_desc(0u, 16, p.sbo >> 1, (uint32_t)ptx::kSwizzle64) >> 32);
+            const int kc_tail = p.tail32 ? kc_per_tap - 1 : -1;
+            uint32_t a_s = a0, b_s = b0;  // those of the current stage
+            const uint32_t empty_u32 = ptx::smem_u32(empty), tfull_u32 = ptx::smem_u32(tfull);
             for (int tile = worker; ok && tile < total_tiles; tile += nworkers) {
                 int cls_mma, lt_mma;
                 igemm_tile_class<CLS4>(p, tile, nworkers, cls_mma, lt_mma);
                 const int kblocks = p.cls_ntaps[cls_mma] * kc_per_tap;
                 if (!wait_bar_fast(tempty + acc, acc_ph ^ 1u, abort_flag, p.status, 2)) break;
                 ptx::tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * mh) * acc_stride;
+                const uint32_t dt = tmem_base + (uint32_t)(acc * mh + h) * acc_stride;
                 uint32_t accumulate = 0;
                 int kc = igemm_first_kblock<HALF>(p, worker, lt_mma, kblocks) % kc_per_tap;  // the producers' starting k-block
                 for (int kb0 = 0; kb0 < kblocks; kb0 += kpb) {
@@ -512,49 +519,23 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                         break;
                     }
                     ptx::tc_fence_after();
-                    uint64_t da = da_s, db = db_s;
+                    uint32_t a = a_s, b = b_s;
                     for (int j = 0; j < nkb; ++j) {
-                        const bool tail = kc == kc_tail;
+                        if (kc == kc_tail) ptx::umma2_if<CG2>(leader, dt, a - a_back, b, hi_tail, idesc, accumulate);
+                        else ptx::umma4_if<CG2>(leader, dt, a, b, hi, idesc, accumulate);
                         if (++kc == kc_per_tap) kc = 0;
-                        for (int h = 0; h < mh; ++h) {
-                            const uint64_t dah = da + (uint64_t)h * a_half16;
-                            const uint32_t dt = d_tmem + (uint32_t)h * acc_stride;
-                            if (tail) {
-                                const uint64_t dat = (da + (uint64_t)h * (a_half16 >> 1)) ^ tail_flip, dbt = db ^ tail_flip;
-                                if (CG2) {
-                                    ptx::umma_f16_cg2_if(leader, dt, dat, dbt, idesc, accumulate);
-                                    ptx::umma_f16_cg2_if(leader, dt, dat + 2, dbt + 2, idesc, 1u);
-                                } else {
-                                    ptx::umma_f16_if(leader, dt, dat, dbt, idesc, accumulate);
-                                    ptx::umma_f16_if(leader, dt, dat + 2, dbt + 2, idesc, 1u);
-                                }
-                            } else if (CG2) {
-                                ptx::umma_f16_cg2_if(leader, dt, dah, db, idesc, accumulate);
-                                ptx::umma_f16_cg2_if(leader, dt, dah + 2, db + 2, idesc, 1u);
-                                ptx::umma_f16_cg2_if(leader, dt, dah + 4, db + 4, idesc, 1u);
-                                ptx::umma_f16_cg2_if(leader, dt, dah + 6, db + 6, idesc, 1u);
-                            } else if (ksteps == 4) {
-                                ptx::umma_f16_if(leader, dt, dah, db, idesc, accumulate);
-                                ptx::umma_f16_if(leader, dt, dah + 2, db + 2, idesc, 1u);
-                                ptx::umma_f16_if(leader, dt, dah + 4, db + 4, idesc, 1u);
-                                ptx::umma_f16_if(leader, dt, dah + 6, db + 6, idesc, 1u);
-                            } else {
-                                for (int k = 0; k < ksteps; ++k)
-                                    ptx::umma_f16_if(leader, dt, dah + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (k | (int)accumulate) ? 1u : 0u);
-                            }
-                        }
                         accumulate = 1u;
-                        da += a_sub16;
-                        db += b_sub16;
+                        a += a_sub;
+                        b += b_sub;
                     }
                     if (CG2) ptx::umma_commit_cg2_mc_if(leader, empty_u32 + 8u * (uint32_t)s, 3); else ptx::umma_commit_u32_if(leader, empty_u32 + 8u * (uint32_t)s);
-                    da_s += a_stage16;
-                    db_s += b_stage16;
+                    a_s += a_stage;
+                    b_s += b_stage;
                     if (++s == stages) {
                         s = 0;
                         ph ^= 1u;
-                        da_s = da0;
-                        db_s = db0;
+                        a_s = a0;
+                        b_s = b0;
                     }
                 }
                 if (!ok) break;
@@ -565,8 +546,8 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                 }
             }
             // Make sure every MMA issued by this thread has retired before TMEM is released.
-            if (CG2) ptx::umma_commit_cg2_if(leader, ptx::smem_u32(drain)); else ptx::umma_commit_u32_if(leader, ptx::smem_u32(drain));
-            for (int i = 0; i < 4000000 && !ptx::mbar_try_wait(drain, 0); ++i) {
+            if (CG2) ptx::umma_commit_cg2_if(leader, ptx::smem_u32(drain + h)); else ptx::umma_commit_u32_if(leader, ptx::smem_u32(drain + h));
+            for (int i = 0; i < 4000000 && !ptx::mbar_try_wait(drain + h, 0); ++i) {
             }
         }
     } else {

@@ -30,11 +30,6 @@ __device__ __forceinline__ void copy_to_peer(uint32_t dst_cluster, const void* s
                  "r"(bar_cluster)
                  : "memory");
 }
-__device__ __forceinline__ float tanh_fast(float v) {
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(v));
-    return t;
-}
 // 32 bytes on a 32-byte boundary
 __device__ __forceinline__ void st_global32(void* p, const uint2 (&v)[4]) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0].x), "r"(v[0].y), "r"(v[1].x), "r"(v[1].y), "r"(v[2].x), "r"(v[2].y), "r"(v[3].x),
@@ -245,8 +240,8 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
     ok = __syncthreads_and((int)(__shfl_sync(0xffffffffu, (int)ok, 0) != 0)) != 0;
     const int q = warp & 3, share = warp >> 2, c_lo = sp_part_lo(share, p.BN), nc = sp_part_lo(share + 1, p.BN) - c_lo;  // its rows and columns
     int sat_bits = 0;
-    // act(v * scale + shift) of four neighbouring columns from c on (MODE 2), rounded and packed.  The coefficients of SiLU are
-    // halved: z * sigmoid(z) = h + h * tanh(h) with h = z / 2.
+    // act(v * scale + shift) of four neighbouring columns from c on (MODE 2), rounded and packed.  (With SiLU the
+    // coefficients are halved.)
     auto finish = [&](const float* v, int c) {
         float2 a = make_float2(v[0], v[1]), b = make_float2(v[2], v[3]);
         if (MODE == 2) {
@@ -254,8 +249,8 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
             a = fma2(a, make_float2(sc.x, sc.y), make_float2(sh.x, sh.y));
             b = fma2(b, make_float2(sc.z, sc.w), make_float2(sh.z, sh.w));
             if (p.epi_act) {
-                a = fma2(a, make_float2(tanh_fast(a.x), tanh_fast(a.y)), a);
-                b = fma2(b, make_float2(tanh_fast(b.x), tanh_fast(b.y)), b);
+                a = silu2_of_half(a);
+                b = silu2_of_half(b);
             }
         }
         return make_uint2(pack2<OutT>(a.x, a.y, &sat_bits), pack2<OutT>(b.x, b.y, &sat_bits));
