@@ -490,35 +490,68 @@ nb_status run_simt_fprop(nb_cbs_plan_s* p, const void* x, const void* w, void* y
     return launch_ok("splitk_fwd_reduce");
 }
 
-template <typename TIN>
-nb_status run_simt_dgrad(nb_cbs_plan_s* p, const void* dy, const void* w, void* dx, void* partial, cudaStream_t st) {
+unsigned splitk_reduce_blocks(size_t elems, int sm_count) { return (unsigned)std::min<size_t>((elems / 4 + 255) / 256 + 1, (size_t)sm_count * 8); }
+template <typename TIN> nb_status simt_dgrad_conv(nb_cbs_plan_s* p, const void* dy, const void* w, void* dx, void* partial, cudaStream_t st) {
     const SgCfg& c = p->sg[1];
     const SgArgs args{p->g, c.kchunk, false, ChanAcc{nullptr, nullptr, 1}, 0};
-    {
-        SiteTimer tm(p, SITE_DGRAD, st);
-        if (c.splits == 1) return launch_sg<1, TIN, TIN>(p, dy, w, dx, args, st);
-        NB_TRY((launch_sg<1, TIN, float>(p, dy, w, partial, args, st)));
-    }
+    SiteTimer tm(p, SITE_DGRAD, st);
+    if (c.splits == 1) return launch_sg<1, TIN, TIN>(p, dy, w, dx, args, st);
+    return launch_sg<1, TIN, float>(p, dy, w, partial, args, st);
+}
+template <typename TIN>
+nb_status run_simt_dgrad(nb_cbs_plan_s* p, const void* dy, const void* w, void* dx, void* partial, cudaStream_t st) {
+    NB_TRY(simt_dgrad_conv<TIN>(p, dy, w, dx, partial, st));
+    const SgCfg& c = p->sg[1];
+    if (c.splits == 1) return NB_OK;
     const size_t elems = (size_t)p->g.n * p->g.h * p->g.w * p->g.c_in;
     SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
-    const unsigned blocks = (unsigned)std::min<size_t>((elems / 4 + 255) / 256 + 1, (size_t)p->sm_count * 8);
-    launch_k(splitk_reduce_kernel<TIN, true>, dim3(blocks), dim3(256), 0, st, 1, static_cast<const float*>(partial), c.splits, elems, static_cast<TIN*>(dx));
+    launch_k(splitk_reduce_kernel<TIN, true>, dim3(splitk_reduce_blocks(elems, p->sm_count)), dim3(256), 0, st, 1, static_cast<const float*>(partial), c.splits, elems, static_cast<TIN*>(dx));
     return launch_ok("splitk_reduce");
 }
 
 template <typename TIN>
-nb_status run_simt_wgrad(nb_cbs_plan_s* p, const void* x, const void* dy, float* dw, float* partial, bool overlap, cudaStream_t st) {
+nb_status simt_wgrad_conv(nb_cbs_plan_s* p, const void* x, const void* dy, float* dw, float* partial, bool overlap, cudaStream_t st) {
     const SgCfg& c = p->sg[2];
     const SgArgs args{p->g, c.kchunk, false, ChanAcc{nullptr, nullptr, 1}, overlap ? 1 : 0};
-    {
-        SiteTimer tm(p, SITE_WGRAD, st);
-        NB_TRY((launch_sg<2, TIN, float>(p, dy, x, c.splits == 1 ? dw : partial, args, st)));
-        if (c.splits == 1) return NB_OK;
-    }
+    SiteTimer tm(p, SITE_WGRAD, st);
+    return launch_sg<2, TIN, float>(p, dy, x, c.splits == 1 ? dw : partial, args, st);
+}
+template <typename TIN>
+nb_status run_simt_wgrad(nb_cbs_plan_s* p, const void* x, const void* dy, float* dw, float* partial, bool overlap, cudaStream_t st) {
+    NB_TRY(simt_wgrad_conv<TIN>(p, x, dy, dw, partial, overlap, st));
+    const SgCfg& c = p->sg[2];
+    if (c.splits == 1) return NB_OK;
     const size_t elems = (size_t)p->g.c_out * p->g.kdim;
     SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
     if (c.splits >= 96) launch_k(splitk_reduce_tall_kernel, dim3((unsigned)((elems + 31) / 32)), dim3(1024), 0, st, 1, partial, c.splits, elems, dw);
-    else launch_k(splitk_reduce_kernel<float>, dim3((unsigned)std::min<size_t>((elems / 4 + 255) / 256 + 1, (size_t)p->sm_count * 8)), dim3(256), 0, st, 1, partial, c.splits, elems, dw);
+    else launch_k(splitk_reduce_kernel<float>, dim3(splitk_reduce_blocks(elems, p->sm_count)), dim3(256), 0, st, 1, partial, c.splits, elems, dw);
+    return launch_ok("splitk_reduce");
+}
+
+// Both gradients of a layer on the CUDA cores: the convolutions beside each other (the weight gradient is the very next launch
+// behind the data gradient, see the end of common.cuh), then the slices of both in one launch.  With the data gradient's slices
+// added in between, its convolution and the weight gradient followed one another, two launches more in a row.
+template <typename TIN>
+nb_status run_simt_grads(nb_cbs_plan_s* p, const void* x, const void* dy, const void* w, void* dx, float* dw, void* dgpart, float* wgpart, cudaStream_t st) {
+    const SgCfg &d = p->sg[1], &c = p->sg[2];
+    NB_TRY(simt_dgrad_conv<TIN>(p, dy, w, dx, dgpart, st));
+    NB_TRY(simt_wgrad_conv<TIN>(p, x, dy, dw, wgpart, pdl_enabled(), st));
+    const size_t elems1 = (size_t)p->g.n * p->g.h * p->g.w * p->g.c_in, elems2 = (size_t)p->g.c_out * p->g.kdim;
+    const bool both = d.splits > 1 && c.splits > 1 && c.splits < 96;
+    SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
+    if (both) {
+        const unsigned b1 = splitk_reduce_blocks(elems1, p->sm_count), b2 = splitk_reduce_blocks(elems2, p->sm_count);
+        launch_k(splitk_reduce_both_kernel<TIN>, dim3(b1 + b2), dim3(256), 0, st, 1, static_cast<const float*>(dgpart), d.splits, elems1, static_cast<TIN*>(dx), (int)b1,
+                 static_cast<const float*>(wgpart), c.splits, elems2, dw);
+        return launch_ok("splitk_reduce_both");
+    }
+    if (d.splits > 1) {
+        launch_k(splitk_reduce_kernel<TIN>, dim3(splitk_reduce_blocks(elems1, p->sm_count)), dim3(256), 0, st, 1, static_cast<const float*>(dgpart), d.splits, elems1, static_cast<TIN*>(dx));
+        NB_LAUNCH_OK("splitk_reduce");
+    }
+    if (c.splits >= 96) launch_k(splitk_reduce_tall_kernel, dim3((unsigned)((elems2 + 31) / 32)), dim3(1024), 0, st, 1, wgpart, c.splits, elems2, dw);
+    else if (c.splits > 1) launch_k(splitk_reduce_kernel<float>, dim3(splitk_reduce_blocks(elems2, p->sm_count)), dim3(256), 0, st, 1, wgpart, c.splits, elems2, dw);
+    else return NB_OK;
     return launch_ok("splitk_reduce");
 }
 
@@ -1083,18 +1116,16 @@ nb_status run_wgrad(nb_cbs_plan_s* p, const void* x, const void* dy, float* dw, 
 }
 }  // namespace
 
-nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan p, const void* g, const void* y_saved, const float* save_mean,
-                                   const float* save_invstd, const float* gamma, const float* beta, const void* w, void* dx,
-                                   float* dgamma, float* dbeta, void* dy_out, void* workspace, size_t workspace_bytes, void* stream) {
-    g_err.clear();
+namespace {
+// dgamma, dbeta and dy, and the checks of the data-gradient call; its convolution follows
+nb_status run_bwd_head(nb_cbs_plan p, const void* g, const void* y_saved, const float* save_mean, const float* save_invstd, const float* gamma, const float* beta,
+                       const void* w, void* dx, float* dgamma, float* dbeta, void* dy_out, void* workspace, size_t workspace_bytes, cudaStream_t st) {
     if (!p) return fail(NB_ERR_INVALID_ARG, "plan is NULL");
     NB_CHECK_PTR(g); NB_CHECK_PTR(y_saved); NB_CHECK_PTR(save_mean); NB_CHECK_PTR(save_invstd);
     NB_CHECK_PTR(gamma); NB_CHECK_PTR(beta); NB_CHECK_PTR(dgamma); NB_CHECK_PTR(dbeta); NB_CHECK_PTR(dy_out);
     NB_CHECK_PTR(dx, true);
     if (dx) NB_CHECK_PTR(w);
     NB_TRY(check_ws(workspace, workspace_bytes, p->bwd_bytes));
-    DeviceGuard on_device(p->device);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     char* ws = static_cast<char*>(workspace);
     float* coef = reinterpret_cast<float*>(ws + p->off_coef);
     float* part = reinterpret_cast<float*>(ws + p->off_bpart);
@@ -1105,7 +1136,19 @@ nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan p, const void* g, const void* y_s
         NB_TRY(NB_WITH_AT(p, run_bwd_elementwise<__half, AT, true>(p, g, y_saved, save_mean, save_invstd, gamma, beta, dgamma, dbeta, dy_out, part, coef, st,
                                                                    tc_dg ? w : nullptr, tc_dg ? ws + p->off_wt : nullptr, tc_dg ? &p->tc.wtp : nullptr)));
     }
-    return dx ? run_dgrad(p, dy_out, w, dx, ws, true, st) : NB_OK;
+    return NB_OK;
+}
+}  // namespace
+
+nb_status nb_conv_bn_silu_bwd_data(nb_cbs_plan p, const void* g, const void* y_saved, const float* save_mean,
+                                   const float* save_invstd, const float* gamma, const float* beta, const void* w, void* dx,
+                                   float* dgamma, float* dbeta, void* dy_out, void* workspace, size_t workspace_bytes, void* stream) {
+    g_err.clear();
+    if (!p) return fail(NB_ERR_INVALID_ARG, "plan is NULL");
+    DeviceGuard on_device(p->device);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    NB_TRY(run_bwd_head(p, g, y_saved, save_mean, save_invstd, gamma, beta, w, dx, dgamma, dbeta, dy_out, workspace, workspace_bytes, st));
+    return dx ? run_dgrad(p, dy_out, w, dx, static_cast<char*>(workspace), true, st) : NB_OK;
 }
 
 nb_status nb_conv_bn_silu_bwd_weight(nb_cbs_plan p, const void* x, const void* dy, float* dw, void* workspace,
@@ -1124,9 +1167,17 @@ nb_status nb_conv_bn_silu_bwd(nb_cbs_plan p, const void* x, const void* g, const
     g_err.clear();
     if (!p) return fail(NB_ERR_INVALID_ARG, "plan is NULL");
     NB_CHECK_PTR(x); NB_CHECK_PTR(dw);  // (the rest by the first of the two)
-    NB_TRY(nb_conv_bn_silu_bwd_data(p, g, y_saved, save_mean, save_invstd, gamma, beta, w, dx, dgamma, dbeta, dy_out, workspace, workspace_bytes, stream));
     DeviceGuard on_device(p->device);
-    return run_wgrad(p, x, dy_out, dw, static_cast<char*>(workspace), dx != nullptr, static_cast<cudaStream_t>(stream));
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    NB_TRY(run_bwd_head(p, g, y_saved, save_mean, save_invstd, gamma, beta, w, dx, dgamma, dbeta, dy_out, workspace, workspace_bytes, st));
+    char* ws = static_cast<char*>(workspace);
+    if (dx && !p->stem && !p->tc.dgrad && !p->tc.wgrad) {
+        float* wgpart = reinterpret_cast<float*>(ws + p->off_wgpart);
+        if (is_f32(p)) return run_simt_grads<float>(p, x, dy_out, w, dx, dw, ws + p->off_dgpart, wgpart, st);
+        return NB_WITH_AT(p, run_simt_grads<AT>(p, x, dy_out, w, dx, dw, ws + p->off_dgpart, wgpart, st));
+    }
+    if (dx) NB_TRY(run_dgrad(p, dy_out, w, dx, ws, true, st));
+    return run_wgrad(p, x, dy_out, dw, ws, dx != nullptr, st);
 }
 
 nb_status nb_conv_bias_bwd(nb_cbs_plan p, const void* x, const void* w, const void* dout, void* dx, float* dw, float* dbias, void* workspace,

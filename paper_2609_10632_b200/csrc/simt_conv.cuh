@@ -470,16 +470,12 @@ __global__ void __launch_bounds__(SG_REDUCE_MAX) splitk_fwd_reduce_kernel(const 
 // Eight slices are loaded before any is added so that a thread keeps eight independent 16-byte loads in flight:
 // the kernel is tiny and otherwise bound by one memory latency per slice.
 // LATE: the last launch of a data gradient (it signals its dependents behind its own wait: see the end of common.cuh).
-template <typename TO, bool LATE = false>
-__global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restrict__ partial, int splits, size_t elems, TO* __restrict__ out) {
-    if (!LATE) pdl_launch_dependents();
-    pdl_wait();
-    if (LATE) pdl_launch_dependents();
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
+// (thread `at` of `stride` threads)
+template <typename TO> __device__ __forceinline__ void splitk_reduce(const float* __restrict__ partial, int splits, size_t elems, TO* __restrict__ out, size_t at, size_t stride) {
     if ((elems & 3) == 0) {
         const size_t nv = elems >> 2;
         const float4* p4 = reinterpret_cast<const float4*>(partial);
-        for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += stride) {
+        for (size_t v = at; v < nv; v += stride) {
             double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
             for (int z0 = 0; z0 < splits; z0 += 8) {
                 float4 a[8];
@@ -503,12 +499,29 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
             }
         }
     } else {
-        for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < elems; e += stride) {
+        for (size_t e = at; e < elems; e += stride) {
             double s = 0.0;
             for (int z = 0; z < splits; ++z) s += (double)partial[(size_t)z * elems + e];
             out[e] = from_f32<TO>((float)s);
         }
     }
+}
+template <typename TO, bool LATE = false>
+__global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restrict__ partial, int splits, size_t elems, TO* __restrict__ out) {
+    if (!LATE) pdl_launch_dependents();
+    pdl_wait();
+    if (LATE) pdl_launch_dependents();
+    splitk_reduce(partial, splits, elems, out, (size_t)blockIdx.x * blockDim.x + threadIdx.x, (size_t)gridDim.x * blockDim.x);
+}
+// The slices of a data gradient (the first `blocks1` blocks) and of the weight gradient beside it, in one launch.
+template <typename TO>
+__global__ void __launch_bounds__(256) splitk_reduce_both_kernel(const float* __restrict__ partial1, int splits1, size_t elems1, TO* __restrict__ out1, int blocks1,
+                                                                 const float* __restrict__ partial2, int splits2, size_t elems2, float* __restrict__ out2) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int b = (int)blockIdx.x;
+    if (b < blocks1) splitk_reduce(partial1, splits1, elems1, out1, (size_t)b * blockDim.x + threadIdx.x, (size_t)blocks1 * blockDim.x);
+    else splitk_reduce(partial2, splits2, elems2, out2, (size_t)(b - blocks1) * blockDim.x + threadIdx.x, (size_t)((int)gridDim.x - blocks1) * blockDim.x);
 }
 
 // The same sum for many slices of few elements (the first layer's weight gradient: ~1200 slices of 1296 values): a block of
