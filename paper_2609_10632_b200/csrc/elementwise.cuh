@@ -869,12 +869,13 @@ __device__ __forceinline__ double ld_dsmem_f64(uint32_t cluster_addr) {
     return v;
 }
 // Dynamic shared memory: fp64 sums [2][C / slabs], coefficients [4][C / slabs], then red [2][blockDim.x * V] and part [2 C].
-inline size_t bwd_small_smem(int C, int slabs, int tpb, int vec) { return (size_t)(C / slabs) * 32 + ((size_t)2 * tpb * vec + 2 * C) * 4; }
+// wc: channels of a slab, units: row blocks of a CTA, threads of a CTA
+inline size_t bwd_small_smem(int wc, int units, int threads, int vec) { return (size_t)wc * 32 + ((size_t)2 * threads * vec + 2 * units * wc) * 4; }
 template <typename YT, typename AT, bool FAST, bool PITCHED, bool GRES>
 __global__ void __launch_bounds__(288, 1) bn_silu_bwd_small_kernel(const AT* __restrict__ g, const YT* __restrict__ y, AT* __restrict__ dy, long long rows,
                                                                    int C, BwdFin fin, const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wt,
                                                                    WtParams wtp, long long ld_g, AT* __restrict__ gres, long long ld_gres, int gres_add,
-                                                                   int slabs, int cluster, int row_blocks) {
+                                                                   int slabs, int units, int cluster, int row_blocks) {
     pdl_launch_dependents();
     pdl_wait();
     const int slab = (int)blockIdx.x / cluster, q = (int)blockIdx.x % cluster;
@@ -886,13 +887,13 @@ __global__ void __launch_bounds__(288, 1) bn_silu_bwd_small_kernel(const AT* __r
     static_assert(V == Vec16<AT>::N, "g and y must have the same element size");
     extern __shared__ __align__(16) float small_smem[];
     const int tid = threadIdx.x, tpb = blockDim.x;
-    const int cgs = C / V, R = tpb / cgs, wv = cgs / slabs, wc = wv * V;  // vectors and channels of the slab
+    const int cgs = C / V, wv = cgs / slabs, wc = wv * V, R = tpb / (units * wv);  // vectors and channels of the slab, rows of a row block
     double* const s_tot = reinterpret_cast<double*>(small_smem);          // [2][wc]
     float* const s_coef = small_smem + 4 * wc;                            // [4][wc]
     float* const red = s_coef + 4 * wc;                                   // [2][tpb * V]
-    float* const part = red + 2 * tpb * V;                                // [2][slabs][wc]
+    float* const part = red + 2 * tpb * V;                                // [2][units][wc]
     const int jl = tid / (R * wv), rem = tid % (R * wv), cg = rem % wv;
-    const int block = q * slabs + jl;                                     // of the reduce kernel's grid
+    const int block = q * units + jl, uc = units * wc;                    // of the reduce kernel's grid
     const long long row0 = (long long)block * R + rem / wv, row_step = (long long)row_blocks * R;
     const int ch = (slab * wv + cg) * V;
     auto has = [&](int u) { return block < row_blocks && row0 + u * row_step < rows; };
@@ -936,19 +937,19 @@ __global__ void __launch_bounds__(288, 1) bn_silu_bwd_small_kernel(const AT* __r
         }
     }
     __syncthreads();
-    for (int e = tid; e < 2 * C; e += tpb) {  // the sums of every row block of this CTA (zero past the last)
-        const int pass = e >= C ? 1 : 0, k = e - pass * C, bl = k / wc, c = k - bl * wc;
+    for (int e = tid; e < 2 * uc; e += tpb) {  // the sums of every row block of this CTA (zero past the last)
+        const int pass = e >= uc ? 1 : 0, k = e - pass * uc, bl = k / wc, c = k - bl * wc;
         const float* const src = red + (pass * tpb + bl * R * wv) * V + c;
         float acc = 0.f;
         for (int r = 0; r < R; ++r) acc += src[r * wc];
-        part[e] = q * slabs + bl < row_blocks ? acc : 0.f;
+        part[e] = q * units + bl < row_blocks ? acc : 0.f;
     }
     __syncthreads();
     for (int e = tid; e < 2 * wc; e += tpb) {
         const int pass = e >= wc ? 1 : 0;
-        const float* const src = part + pass * C + (e - pass * wc);
+        const float* const src = part + pass * uc + (e - pass * wc);
         double t = 0.0;
-        for (int bl = 0; bl < slabs; ++bl) t += (double)src[bl * wc];
+        for (int bl = 0; bl < units; ++bl) t += (double)src[bl * wc];
         s_tot[e] = t;
     }
     __syncthreads();  // (the cluster barrier wants whole warps)
@@ -957,11 +958,20 @@ __global__ void __launch_bounds__(288, 1) bn_silu_bwd_small_kernel(const AT* __r
     for (int c = tid; c < wc; c += tpb) {
         double s0 = 0.0, s1 = 0.0;
         if (cluster > 1) {
-            for (int k = 0; k < cluster; ++k) {
-                const uint32_t peer = ptx::mapa_u32(tot, (uint32_t)k);
-                s0 += ld_dsmem_f64(peer + 8u * (uint32_t)c);
-                s1 += ld_dsmem_f64(peer + 8u * (uint32_t)(wc + c));
-            }
+            double t0[8], t1[8];  // (all peers asked before the first answer is used)
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (k < cluster) {
+                    const uint32_t peer = ptx::mapa_u32(tot, (uint32_t)k);
+                    t0[k] = ld_dsmem_f64(peer + 8u * (uint32_t)c);
+                    t1[k] = ld_dsmem_f64(peer + 8u * (uint32_t)(wc + c));
+                }
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (k < cluster) {
+                    s0 += t0[k];
+                    s1 += t1[k];
+                }
         } else {
             s0 = s_tot[c];
             s1 = s_tot[wc + c];

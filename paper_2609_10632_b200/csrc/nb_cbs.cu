@@ -57,7 +57,7 @@ struct EwCfg {  // launch geometry of the [M][C] passes
     int blocks_reduce, blocks_map;  // stats / backward-reduce grids (they size the partial buffers) and apply / dy grids
     int blocks_stats, blocks_apply, blocks_dy;
     int wave_reduce;  // resident blocks of the backward-reduce kernel on the whole device
-    int slabs, slab_ctas;  // both backward passes in one launch: channel slabs (0: two launches) and CTAs of a slab
+    int slabs, slab_ctas, slab_units, slab_threads;  // both backward passes in one launch: channel slabs (0: two launches), CTAs of a slab, row blocks and threads of a CTA
 };
 
 }  // namespace
@@ -262,10 +262,10 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
         const int rows_grid = e.slabs * e.slab_ctas, tiles = wtp && wt ? wt_num_tiles(*wtp) : 0;
         const int wt_ctas = (std::min(tiles, 4 * p->sm_count) + e.slab_ctas - 1) / e.slab_ctas * e.slab_ctas;
         auto go = [&](auto kernel) {
-            launch_k(kernel, dim3(rows_grid + wt_ctas), dim3(e.tpb), bwd_small_smem(C, e.slabs, e.tpb, e.vec), st, e.slab_ctas, static_cast<const AT*>(g),
+            launch_k(kernel, dim3(rows_grid + wt_ctas), dim3(e.slab_threads), bwd_small_smem(C / e.slabs, e.slab_units, e.slab_threads, e.vec), st, e.slab_ctas, static_cast<const AT*>(g),
                      static_cast<const YT*>(y), static_cast<AT*>(dy), p->g.m, C, bf, static_cast<const __nv_bfloat16*>(w), static_cast<__nv_bfloat16*>(wt), wtp ? *wtp : none,
                      p->ld_g ? p->ld_g : (long long)C, static_cast<AT*>(p->bwd_gres), p->ld_gres ? p->ld_gres : (long long)C, p->gres_add ? 1 : 0,
-                     e.slabs, e.slab_ctas, e.blocks_reduce);
+                     e.slabs, e.slab_units, e.slab_ctas, e.blocks_reduce);
         };
         if (p->bwd_gres) p->ld_g ? go(bn_silu_bwd_small_kernel<YT, AT, FAST, true, true>) : go(bn_silu_bwd_small_kernel<YT, AT, FAST, false, true>);
         else p->ld_g ? go(bn_silu_bwd_small_kernel<YT, AT, FAST, true, false>) : go(bn_silu_bwd_small_kernel<YT, AT, FAST, false, false>);
@@ -656,18 +656,24 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
         e.blocks_map = std::max(e.blocks_apply, e.blocks_dy);
         // Both backward passes in one launch (16-bit modes), where a thread of the reduction has at most eight vectors and its
         // blocks fit, by channel slabs, into clusters of eight CTAs (at most 48 KB of shared memory with the filter tile, which
-        // needs no opt-in): the fewest slabs, hence the widest pieces of a row.  Above 24 row blocks the pieces get narrow and
-        // the eight vectors of a thread, one after the other, take as long as the launch saved: detector iteration at batch 2,
-        // 320 x 320 with at most 0 / 8 / 16 / 24 / 40 row blocks 2282 / 2284 / 2268 / 2237 / 2245 us.  The fp32 mode, whose
-        // sigmoid is an exponential and a division, loses 2 us (16 -> 32 on 2 x 32 x 32 pixels 38.1 -> 40.3).
+        // needs no opt-in).  A CTA takes as few row blocks as eight CTAs allow, and as narrow a slab as leaves it 96 threads: the
+        // work is a few row blocks of 256 threads with eight vectors each, and more SMs share it that way.  Above 24 row blocks the
+        // eight vectors of a thread, one after the other, take as long as the launch saved: detector iteration at batch 2,
+        // 320 x 320 with at most 0 / 8 / 16 / 24 / 40 row blocks 2282 / 2284 / 2268 / 2237 / 2245 us.  At least 256 / 128 / 96 / 64 /
+        // 48 threads, the same iteration: 2117 / 2096 / 2049 / 2049 / 2081 us.  The fp32 mode, whose sigmoid is an exponential and
+        // a division, loses 2 us (16 -> 32 on 2 x 32 x 32 pixels 38.1 -> 40.3).
         e.slabs = 0;
         const bool forbidden = getenv("NB_EW_SLABS") && atoi(getenv("NB_EW_SLABS")) == 0;
         if (p->fuse_finalize && !forbidden && d->mode != NB_MODE_F32_REF && e.blocks_reduce <= 24 && (long long)e.blocks_reduce * e.tpb * 8 >= e.total_vecs)
-            for (int sl = 1; sl <= e.cgs && !e.slabs; ++sl)
-                if (e.cgs % sl == 0 && (e.blocks_reduce + sl - 1) / sl <= 8 && bwd_small_smem(g.c_out, sl, e.tpb, vec) <= 40 * 1024) {
-                    e.slabs = sl;
-                    e.slab_ctas = (e.blocks_reduce + sl - 1) / sl;
-                }
+            for (int sl = 1; sl <= e.cgs; ++sl) {
+                const int units = (e.blocks_reduce + 7) / 8, threads = e.tpb / sl * units;
+                if (e.cgs % sl || units > sl || bwd_small_smem(g.c_out / sl, units, threads, vec) > 40 * 1024) continue;
+                if (e.slabs && threads < 96) break;
+                e.slabs = sl;
+                e.slab_units = units;
+                e.slab_threads = threads;
+                e.slab_ctas = (e.blocks_reduce + units - 1) / units;
+            }
     }
 
     for (int kind = 0; kind < 3; ++kind) p->sg[kind] = sg_configure(g, kind, d->mode == NB_MODE_F32_REF, p->sm_count);
