@@ -281,7 +281,11 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
         if (fuse) {
             fb.w = static_cast<const __nv_bfloat16*>(w); fb.wt = wtp ? static_cast<__nv_bfloat16*>(wt) : nullptr;
         }
-        const bool deep = 2 * e.blocks_reduce <= p->sm_count;  // at most every second SM has rows
+        // At most two blocks of rows an SM, whose threads have at most eight vectors: all of them asked for at once, with the
+        // registers that takes.  Measured (step), one block for at most every second SM / two for every SM: 72 -> 136 3x3 on
+        // 3 x 53 x 75 pixels (93 blocks) 58.9 / 55.5 us, 192 -> 192 on 4 x 40 x 40 50.5 / 46.9, 288 -> 288 on 16 x 20 x 20 80.1 / 78.0,
+        // 96 -> 96 on 2 x 80 x 80 43.2 / 40.0, on 16 x 40 x 40 (150 blocks) 60.6 / 59.8.
+        const bool deep = e.blocks_reduce <= 2 * p->sm_count && (long long)e.blocks_reduce * e.tpb * 8 >= e.total_vecs;
         const size_t red_smem = std::max((size_t)2 * e.tpb * e.vec * sizeof(float), deep ? (size_t)0 : (size_t)EW_RING * 2 * e.tpb * 16);
         // A small activation needs few blocks, a large filter many: every block takes two filter tiles, blocks without
         // rows of their own take nothing else (288 -> 288 3x3 on one 20 x 20 image has 405 tiles and 8 blocks of rows:
