@@ -109,7 +109,6 @@ template <bool HALF> __device__ __forceinline__ int igemm_first_kblock(const Ige
 
 constexpr int TC_BM = 128;
 constexpr int IG_THREADS = 384;  // implicit-GEMM kernel: the roles below plus a second epilogue team in warps 7-10 and a second MMA issuer in warp 11
-constexpr int TC_THREADS = 224;  // warp 0: TMA producer for A, warp 1: MMA issuer + TMEM owner, warps 2-5: epilogue, warp 6: TMA producer for B
 
 __device__ __forceinline__ uint64_t global_timer_ns() {
     uint64_t t;
@@ -144,8 +143,8 @@ __device__ __forceinline__ bool wait_bar_fast(uint64_t* bar, uint32_t parity, vo
     return __all_sync(0xffffffffu, ok) != 0;
 }
 
-__device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-// The same over the 256 threads of the implicit-GEMM kernel's two epilogue teams.
+// Barriers over the 256 threads of a kernel's two epilogue teams, the second with the AND of a predicate, so that all of them take
+// the same decision.
 __device__ __forceinline__ void epi2_bar_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ bool epi2_bar_and(bool ok) {
     uint32_t r;
@@ -161,22 +160,6 @@ __device__ __forceinline__ bool epi2_bar_and(bool ok) {
         : "memory");
     return r != 0;
 }
-// Barrier over the 128 epilogue threads that also ANDs a predicate, so that all of them take the same decision.
-__device__ __forceinline__ bool epi_bar_and(bool ok) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t"
-        ".reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.and.pred q, 1, 128, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t"
-        "}\n"
-        : "=r"(r)
-        : "r"((uint32_t)ok)
-        : "memory");
-    return r != 0;
-}
-
 template <typename OutT> __device__ __forceinline__ uint32_t pack2(float a, float b, int* sat);
 template <> __device__ __forceinline__ uint32_t pack2<__nv_bfloat16>(float a, float b, int*) {
     __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
@@ -1608,7 +1591,7 @@ inline nb_status tc_wgrad(TcPlan* tc, const Geom& g, const void* x, const void* 
             }
             rows_attr_set.fetch_or(bit, std::memory_order_release);
         }
-        launch_k(tc_wgrad_rows_kernel, dim3(tc->wr_grid), dim3(TC_THREADS), tc->wr_smem, st, 1, R);
+        launch_k(tc_wgrad_rows_kernel, dim3(tc->wr_grid), dim3(WG_THREADS), tc->wr_smem, st, 1, R);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) { err() = std::string("launch of tc_wgrad_rows_kernel failed: ") + cudaGetErrorString(e); return NB_ERR_CUDA; }
         tc->launches += 1;
@@ -1647,7 +1630,7 @@ inline nb_status tc_wgrad(TcPlan* tc, const Geom& g, const void* x, const void* 
         }
         attr_set.fetch_or(bit, std::memory_order_release);
     }
-    launch_k(tc_wgrad_kernel, dim3(tc->wg_grid), dim3(TC_THREADS), tc->wg_smem, st, 1, P);
+    launch_k(tc_wgrad_kernel, dim3(tc->wg_grid), dim3(WG_THREADS), tc->wg_smem, st, 1, P);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { err() = std::string("launch of tc_wgrad_kernel failed: ") + cudaGetErrorString(e); return NB_ERR_CUDA; }
     tc->launches += 1;

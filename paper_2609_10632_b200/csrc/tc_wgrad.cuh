@@ -10,6 +10,11 @@
 
 namespace nbcbs {
 
+// warp 0: TMA producer of x, warp 1: MMA issuer and TMEM owner, warp 6: TMA producer of dy, warps 2-5 and 7-10: the epilogue, which
+// nothing overlaps (weight-gradient call with four / eight warps there: 384 -> 384 1x1 on 16 x 40 x 40 pixels 18.2 / 17.3 us, 192 -> 384 3x3
+// stride 2 on 16 x 80 x 80 35.0 / 33.5, 288 -> 288 3x3 on 16 x 20 x 20 20.3 / 19.5, 72 -> 136 on 3 x 53 x 75 14.5 / 13.9).
+constexpr int WG_THREADS = 352;
+
 struct WgradParams {
     CUtensorMap tmA;  // im2col map over x [N][H][W][Cin], 64 channels x KP pixels per load
     CUtensorMap tmB;  // tiled map over dy [M][Cout], 64 channels x KP pixels per load
@@ -32,7 +37,7 @@ struct WgradParams {
     uint16_t off_w[9], off_h[9];
 };
 
-__global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_constant__ WgradParams p) {
+__global__ void __launch_bounds__(WG_THREADS, 1) tc_wgrad_kernel(const __grid_constant__ WgradParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* sA = smem;
@@ -195,13 +200,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
             }
         }
     } else {
-        // ------------------------------------------------------------------ epilogue (warps 2-5)
-        const int lane_group = warp & 3;
+        // ------------------------------------------------------------------ epilogue (warps 2-5 and 7-10)
+        const int lane_group = warp & 3, team = warp >= 7 ? 1 : 0;  // the teams take alternate 16-column pieces
         const int row = lane_group * 32 + lane;
         bool ok = true;
         if (nchunks > 0 && lane == 0) ok = wait_bar(tfull, 0, abort_flag, p.status, 13);
         ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-        ok = epi_bar_and(ok);
+        ok = epi2_bar_and(ok);
         if (ok) ptx::tc_fence_after();
         for (int h = 0; ok && h < p.mh; ++h) {
             // accumulator row -> (tap, channel): rows come in blocks of 64 channels
@@ -212,7 +217,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_kernel(const __grid_co
             const int kidx = tap * p.c_in + c;  // position inside dw[c'][:]
             const uint32_t taddr = tmem_base + ((uint32_t)(lane_group * 32) << 16) + (uint32_t)(h * p.acc_stride);
             float* dst = p.out + (size_t)split * p.c_out * p.kdim;
-            for (int c0 = 0; c0 < p.BN && n_tile * p.BN + c0 < p.c_out; c0 += 16) {  // (the last tile may reach past the channel count)
+            for (int c0 = 16 * team; c0 < p.BN && n_tile * p.BN + c0 < p.c_out; c0 += 32) {  // (the last tile may reach past the channel count)
                 uint32_t r[16];
                 if (nchunks > 0) {
                     ptx::tmem_ld_32x32b_x16(taddr + (uint32_t)c0, r);
@@ -267,7 +272,7 @@ struct WgradRowsParams {
     int overlap;  // see WgradParams
 };
 
-__global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_rows_kernel(const __grid_constant__ WgradRowsParams p) {
+__global__ void __launch_bounds__(WG_THREADS, 1) tc_wgrad_rows_kernel(const __grid_constant__ WgradRowsParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* sA = smem;
@@ -424,13 +429,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_rows_kernel(const __gr
             }
         }
     } else {
-        // ------------------------------------------------------------------ epilogue (warps 2-5)
-        const int lane_group = warp & 3;
+        // ------------------------------------------------------------------ epilogue (warps 2-5 and 7-10)
+        const int lane_group = warp & 3, team = warp >= 7 ? 1 : 0;  // the teams take alternate 16-column pieces
         const int row = lane_group * 32 + lane;
         bool ok = true;
         if (nrows > 0 && lane == 0) ok = wait_bar(tfull, 0, abort_flag, p.status, 19);
         ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-        ok = epi_bar_and(ok);
+        ok = epi2_bar_and(ok);
         if (ok) ptx::tc_fence_after();
         for (int a = 0; ok && a < nacc; ++a) {
             // accumulator row -> block (r, channel block, s) -> position inside dw[c'][:]
@@ -441,7 +446,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_wgrad_rows_kernel(const __gr
             const int kidx = (r * 3 + sft) * p.c_in + c;
             const uint32_t taddr = tmem_base + ((uint32_t)(lane_group * 32) << 16) + (uint32_t)(a * p.acc_stride);
             float* dst = p.out + (size_t)split * p.c_out * p.kdim;
-            for (int c0 = 0; c0 < p.BN && n_tile * p.BN + c0 < p.c_out; c0 += 16) {  // (the last tile may reach past the channel count)
+            for (int c0 = 16 * team; c0 < p.BN && n_tile * p.BN + c0 < p.c_out; c0 += 32) {  // (the last tile may reach past the channel count)
                 uint32_t rr[16];
                 if (nrows > 0) {
                     ptx::tmem_ld_32x32b_x16(taddr + (uint32_t)c0, rr);
