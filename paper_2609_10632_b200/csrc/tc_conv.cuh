@@ -988,11 +988,15 @@ inline void fill_params(IgemmParams& P, const IgemmCfg& c) {
 // its kind: 1.5 to the first operands, 0.147 a k-block whatever the tile's width (its 128 activation rows are written to and read
 // from shared memory once each), 0.018 a column behind the last MMA, 1.05 x the share of the SMs that are taken (more CTAs, more
 // rows through L2), 0.3 where successive launches cannot be on different SMs, and for a cluster the exchange.  The choices are
-// within 1 % of the best ones in sum.  The persistent form: 0.28 a k-block, 6 us besides.
+// within 1 % of the best ones in sum.  The persistent form: 0.28 a k-block, 6 us besides.  Tiles of more than 128 columns (one CTA)
+// serve layers whose persistent form has one such tile a CTA; forward / data-gradient / evaluation call, persistent -> split: 288 ->
+// 288 3x3 on 16 x 20 x 20 pixels 25.1 -> 20.3 / 32.6 -> 28.5 / 20.8 -> 15.5 us, 64 -> 144 3x3 on 4 x 64 x 64 14.1 -> 12.2 / - / 9.6 -> 6.7, 256 ->
+// 176 1x1 on 2 x 80 x 80 12.7 -> 11.0 / - / 8.0 -> 6.3.  Not so with padding columns in a training call (72 -> 136 3x3 on 3 x 53 x 75
+// forward 18.5 -> 19.1) nor above 160 columns in a data gradient (208 -> 192 3x3 on 8 x 40 x 40 31.4 -> 33.4).
 // Measured, evaluation-mode forward of the 77 layers, one image: 1251 us with the persistent form, 646 with split launches, 530
 // with the epilogue and the choices as they are now; single layers, persistent / split: 288 -> 288 3x3 at 20 x 20 26 / 6.3 (cluster
 // of four, 48 columns), 192 -> 192 3x3 at 40 x 40 14.9 / 6.6, 384 -> 384 1x1 at 40 x 40 9.4 / 4.0.
-inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_taps, bool eval, int sm_count) {
+inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_taps, bool eval, int sm_count, int most_cols = 256) {
     out = full;
     out.cfg = IgemmCfg();
     out.a_ptr = out.b_ptr = out.out_ptr = nullptr;
@@ -1009,14 +1013,15 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     const int force_s = getenv("NB_TC_SPLIT_S") ? atoi(getenv("NB_TC_SPLIT_S")) : 0, force_bn = getenv("NB_TC_SPLIT_BN") ? atoi(getenv("NB_TC_SPLIT_BN")) : 0;
     if (force_s || force_bn) best = 1e30;
     int best_bn = 0, best_s = 0;
-    for (int nt = (f.rowsB + 127) / 128; nt <= (f.rowsB + 15) / 16; ++nt) {
+    for (int nt = (f.rowsB + 255) / 256; nt <= (f.rowsB + 15) / 16; ++nt) {
         const int bn = ((f.rowsB + nt - 1) / nt + 15) / 16 * 16;
         if ((f.rowsB + bn - 1) / bn != nt || (force_bn && bn != force_bn)) continue;
         if (!eval && f.BN % bn) continue;  // a tile lies within one tile of the persistent form
-        for (int s = 1; s <= (eval ? 8 : 1) && s <= min_kb; s *= 2) {
+        if (bn > most_cols || (!eval && bn > 128 && f.rowsB % bn)) continue;
+        for (int s = 1; s <= (eval && bn <= 128 ? 8 : 1) && s <= min_kb; s *= 2) {
             const long long ctas = m_tiles * nt * ncls * s;
             if (ctas > (s == 8 ? sm_count * 6 / 7 : s == 4 ? sm_count * 9 / 10 : sm_count) || (force_s && s != force_s)) continue;
-            const double t = 1.5 + 0.147 * kb_eff / s + 0.018 * bn + 1.05 * (double)ctas / sm_count + (2 * ctas > sm_count ? 0.3 : 0.0) + (s > 1 ? 0.8 + 0.011 * bn : 0.0);
+            const double t = 1.5 + 0.147 * std::max(1.0, (TC_BM + bn) / 256.0) * kb_eff / s + 0.018 * bn + 1.05 * (double)ctas / sm_count + (2 * ctas > sm_count ? 0.3 : 0.0) + (s > 1 ? 0.8 + 0.011 * bn : 0.0);
             if (t < best) {
                 best = t;
                 best_bn = bn;
@@ -1038,7 +1043,7 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     c.acc_stride = c.tmem_cols;
     c.stages = std::max(2, std::min(14, (kblocks + best_s - 1) / best_s));
     // behind the stages: the shares of a cluster, coefficients, barriers; the training forward stages its rounded rows over the stages
-    const size_t share = best_s > 1 ? (size_t)TC_BM * (best_bn + 4 * SP_PARTS) * 4 : 0, fixed = 1024 + 64 + share + (size_t)2 * 128 * 4 + 512;
+    const size_t share = best_s > 1 ? (size_t)TC_BM * (best_bn + 4 * SP_PARTS) * 4 : 0, fixed = 1024 + 64 + share + (size_t)2 * 256 * 4 + 512;
     while (c.stages > 2 && fixed + (size_t)c.stages * (c.a_stage + c.b_stage) > kMaxSmem) --c.stages;
     while (best_s > 1 && (size_t)c.stages * (c.a_stage + c.b_stage) < share) ++c.stages;  // (a CTA's own shares lie over its stages)
     c.smem_bytes = std::max<size_t>(fixed + (size_t)c.stages * (c.a_stage + c.b_stage), 120 * 1024);  // > half an SM: one CTA per SM
@@ -1321,7 +1326,7 @@ inline nb_status tc_plan_init_impl(TcPlan* tc, const Geom& g, bool enable, int s
             W.nclasses = ncls;
             tc->wt_bytes = off * 2;
             tc->dgrad = true;
-            split_configure(tc->dgs, tc->dg, ncls == 4 ? 1 : g.k * g.k, false, sm_count);
+            split_configure(tc->dgs, tc->dg, ncls == 4 ? 1 : g.k * g.k, false, sm_count, 160);
         }
     }
     // ---- wgrad: A = x (im2col, MN-major), B = dy (MN-major), reduction over pixels with split-K

@@ -11,7 +11,7 @@
 // No block waits for a block outside its cluster.  Bound: latency.  192 -> 192 3x3 on one 40 x 40 image, us behind the end of the
 // launch before: 0.8 until that has reached the CTA, 0.6 until the last CTA runs (an SM holds one), 1.1 to the first operands,
 // 0.15 a k-block (its 128 + BN rows are written to and read from shared memory once each), 0.5 to 0.8 behind the last MMA.
-// The narrow tiles (BN <= 128, often 32 to 64) are part of the same idea: more CTAs, and less to hand over.
+// The narrow tiles (often 32 to 64 columns) are part of the same idea: more CTAs, and less to hand over.
 // Measured against the persistent kernel: see split_configure below.
 // Included by tc_conv.cuh (uses its parameter record and bounded-wait helpers).
 #pragma once
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
     constexpr int ROWS = TC_BM / S;
     const int slot = ROWS * (p.BN + 4 * SP_PARTS);
     float* red = part + (S > 1 ? S * slot : 0);  // MODE 2: scale, shift [2][BN]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(red + 2 * 128);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(red + 2 * 256);
     uint64_t* full = bars;
     uint64_t* empty = bars + p.stages;
     uint64_t* tfull = empty + p.stages;
@@ -316,10 +316,10 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
         }
         ptx::tc_fence_before();
         __syncthreads();
-        if (MODE == 1 && ok && warp < p.BN / 16) {
+        for (int piece = warp; MODE == 1 && ok && piece < p.BN / 16; piece += SP_THREADS / 32) {
             // channel sums of the rounded values: a lane takes two channels of one quarter's 32 rows, even and odd rows apart, then
             // the four quarters are added in order (the persistent kernel's grouping; rows past the last pixel are zeros)
-            const int c2 = warp * 8 + (lane & 7), grp = lane >> 3;
+            const int c2 = piece * 8 + (lane & 7), grp = lane >> 3;
             float2 sa = make_float2(0.f, 0.f), sb = sa, qa = sa, qb = sa;
             const uint8_t* src = smem + (size_t)grp * squarter + c2 * 4;
 #pragma unroll
