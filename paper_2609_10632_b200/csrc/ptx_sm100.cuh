@@ -327,42 +327,6 @@ __device__ __forceinline__ void umma_f16_cg2_if(uint32_t issue, uint32_t tmem_d,
                  "r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
                  : "memory");
 }
-// Four (two) MMAs along K, 32 bytes of a row each: the descriptors' low words are given, their high words are the same.  One block:
-// a predicate, a 32-bit addition and the instruction for each, where four calls also test their flags and add 64-bit descriptors.
-#define NB_UMMA4(CG)                                                                                            \
-    asm volatile(NB_PRED_OPEN                                                                                   \
-                 ".reg .pred p;\n\t.reg .b32 l, r;\n\t.reg .b64 a, b;\n\t"                                \
-                 "setp.ne.b32 p, %6, 0;\n\t"                                                                  \
-                 "mov.b64 a, {%2, %4};\n\tmov.b64 b, {%3, %4};\n\t"                                         \
-                 "@q tcgen05.mma.cta_group::" CG ".kind::f16 [%1], a, b, %5, p;\n\t"                          \
-                 "setp.eq.b32 p, 0, 0;\n\t"                                                                   \
-                 "add.u32 l, %2, 2;\n\tadd.u32 r, %3, 2;\n\tmov.b64 a, {l, %4};\n\tmov.b64 b, {r, %4};\n\t" \
-                 "@q tcgen05.mma.cta_group::" CG ".kind::f16 [%1], a, b, %5, p;\n\t"                          \
-                 "add.u32 l, %2, 4;\n\tadd.u32 r, %3, 4;\n\tmov.b64 a, {l, %4};\n\tmov.b64 b, {r, %4};\n\t" \
-                 "@q tcgen05.mma.cta_group::" CG ".kind::f16 [%1], a, b, %5, p;\n\t"                          \
-                 "add.u32 l, %2, 6;\n\tadd.u32 r, %3, 6;\n\tmov.b64 a, {l, %4};\n\tmov.b64 b, {r, %4};\n\t" \
-                 "@q tcgen05.mma.cta_group::" CG ".kind::f16 [%1], a, b, %5, p;\n\t}\n" ::"r"(issue),        \
-                 "r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)                        \
-                 : "memory")
-#define NB_UMMA2(CG)                                                                                            \
-    asm volatile(NB_PRED_OPEN                                                                                   \
-                 ".reg .pred p;\n\t.reg .b32 l, r;\n\t.reg .b64 a, b;\n\t"                                \
-                 "setp.ne.b32 p, %6, 0;\n\t"                                                                  \
-                 "mov.b64 a, {%2, %4};\n\tmov.b64 b, {%3, %4};\n\t"                                         \
-                 "@q tcgen05.mma.cta_group::" CG ".kind::f16 [%1], a, b, %5, p;\n\t"                          \
-                 "setp.eq.b32 p, 0, 0;\n\t"                                                                   \
-                 "add.u32 l, %2, 2;\n\tadd.u32 r, %3, 2;\n\tmov.b64 a, {l, %4};\n\tmov.b64 b, {r, %4};\n\t" \
-                 "@q tcgen05.mma.cta_group::" CG ".kind::f16 [%1], a, b, %5, p;\n\t}\n" ::"r"(issue),        \
-                 "r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)                        \
-                 : "memory")
-template <bool CG2> __device__ __forceinline__ void umma4_if(uint32_t issue, uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate) {
-    if (CG2) NB_UMMA4("2"); else NB_UMMA4("1");
-}
-template <bool CG2> __device__ __forceinline__ void umma2_if(uint32_t issue, uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate) {
-    if (CG2) NB_UMMA2("2"); else NB_UMMA2("1");
-}
-#undef NB_UMMA4
-#undef NB_UMMA2
 __device__ __forceinline__ void umma_commit_u32_if(uint32_t issue, uint32_t bar) {
     asm volatile(NB_PRED_OPEN "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n\t}\n" ::"r"(issue), "r"(bar) : "memory");
 }

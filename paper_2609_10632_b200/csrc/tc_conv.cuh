@@ -464,9 +464,9 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
         // ------------------------------------------------------------------ MMA issuers (in a pair those of rank 0): warp 1 for the
         // first 128-row sub-tile, warp 11 for the second.  The operands are always there in time (a wait that finds them takes 105
         // cycles); what a stage takes is an issuer's instructions: barrier, eight MMAs, commit, 820 cycles for 96 -> 96 channels
-        // 3x3, whose MMAs need 290 to 450.  Hence an issuer for each sub-tile, and the MMAs of a k-block in one block of code.
-        // Measured (step): 96 -> 96 3x3 on 16 x 160 x 160 pixels 367 -> 331 us, on 16 x 80 x 80 130 -> 114, 192 -> 192 on
-        // 16 x 40 x 40 95.5 -> 88 (one sub-tile: the block of code alone), 48 -> 48 on 16 x 160 x 160 207 -> 198.  Testing the next
+        // 3x3, whose MMAs need 290 to 450.  Hence an issuer for each sub-tile, and 32-bit arithmetic for the descriptors.
+        // Measured (step): 96 -> 96 3x3 on 16 x 160 x 160 pixels 367 -> 328 us, on 16 x 80 x 80 130 -> 113, 192 -> 192 on
+        // 16 x 40 x 40 95.5 -> 88 (one sub-tile: shorter code alone), 48 -> 48 on 16 x 160 x 160 207 -> 198.  Testing the next
         // stage's barrier ahead of the MMAs of this one adds instructions and loses 0.5 to 2 us on the wide layers.
         const int h = warp == 11 ? 1 : 0;
         const uint32_t leader = ptx::elect_one() ? 1u : 0u;  // the whole warp runs the loop, this lane issues
@@ -504,8 +504,24 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
                     ptx::tc_fence_after();
                     uint32_t a = a_s, b = b_s;
                     for (int j = 0; j < nkb; ++j) {
-                        if (kc == kc_tail) ptx::umma2_if<CG2>(leader, dt, a - a_back, b, hi_tail, idesc, accumulate);
-                        else ptx::umma4_if<CG2>(leader, dt, a, b, hi, idesc, accumulate);
+                        const bool tail = kc == kc_tail;
+                        const uint32_t al = tail ? a - a_back : a, hh = tail ? hi_tail : hi;
+                        const uint64_t da = ((uint64_t)hh << 32) | al, db = ((uint64_t)hh << 32) | b;
+                        if (CG2) {
+                            ptx::umma_f16_cg2_if(leader, dt, da, db, idesc, accumulate);
+                            ptx::umma_f16_cg2_if(leader, dt, da + 2, db + 2, idesc, 1u);
+                            if (!tail) {
+                                ptx::umma_f16_cg2_if(leader, dt, da + 4, db + 4, idesc, 1u);
+                                ptx::umma_f16_cg2_if(leader, dt, da + 6, db + 6, idesc, 1u);
+                            }
+                        } else {
+                            ptx::umma_f16_if(leader, dt, da, db, idesc, accumulate);
+                            ptx::umma_f16_if(leader, dt, da + 2, db + 2, idesc, 1u);
+                            if (!tail) {
+                                ptx::umma_f16_if(leader, dt, da + 4, db + 4, idesc, 1u);
+                                ptx::umma_f16_if(leader, dt, da + 6, db + 6, idesc, 1u);
+                            }
+                        }
                         if (++kc == kc_per_tap) kc = 0;
                         accumulate = 1u;
                         a += a_sub;
