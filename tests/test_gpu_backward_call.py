@@ -13,7 +13,10 @@ SHAPES = [  # mode, (n, h, w, c_in, c_out, k, stride)
     ("bf16", (2, 64, 96, 3, 48, 3, 2)),      # first layer
     ("bf16", (2, 13, 9, 16, 16, 1, 2)),      # data gradient on the CUDA cores, weight gradient on the tensor cores
     ("f32", (2, 40, 40, 64, 64, 3, 1)),      # slices, and the pass that adds them, last in the data gradient
-    ("f32", (1, 9, 7, 8, 12, 3, 1)),
+    ("f32", (1, 9, 7, 8, 12, 3, 1)),         # one slice each: nothing is added
+    ("f32", (2, 32, 32, 16, 32, 3, 1)),      # slices of both, added in one launch
+    ("f32", (4, 80, 80, 16, 16, 1, 1)),      # 200 slices of the weight gradient, one of the data gradient
+    ("f32", (1, 24, 20, 3, 16, 3, 2)),       # element counts that are not multiples of four
 ]
 IDS = ["-".join((m, "x".join(map(str, d)))) for m, d in SHAPES]
 

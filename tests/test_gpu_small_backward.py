@@ -75,3 +75,16 @@ def _against_fp64(blk):
     dy = gamma * invstd * (dz - dbeta / m - xhat * dgamma / m)
     for name, got, want in (("dbeta", blk.dbeta, dbeta), ("dgamma", blk.dgamma, dgamma), ("dy", blk.dy.reshape(m, c), dy)):
         parity.check(name, d(got).cpu().numpy(), want.cpu().numpy(), "bf16")
+
+
+@pytest.mark.parametrize("blocks", [74, 75, 148, 149, 296, 297])
+def test_reduction_at_its_block_counts(blocks):
+    """All eight vectors of a thread at once up to two blocks an SM, a ring of three beyond; the last block one image row short."""
+    from paper_2609_10632_b200 import binding as nb
+    from paper_2609_10632_b200.block import CbsBlock
+
+    blk = CbsBlock(wl.ConvShape("blocks", 1, 16 * blocks - 1, 16, 16, 64, 1, 1), mode=nb.NB_MODE_BF16_TC)  # 256 rows a block
+    blk.fill_random(blocks)
+    blk.step()
+    blk.poll()
+    _against_fp64(blk)

@@ -56,7 +56,7 @@ def test_split_launches_match_oracle(dims, split, monkeypatch):
 
 
 @pytest.mark.parametrize("split", [1, 2, 8])
-@pytest.mark.parametrize("cols", [16, 48, 80, 112, 128])
+@pytest.mark.parametrize("cols", [16, 48, 80, 112, 128, 144, 208, 256])
 def test_tile_widths_of_the_evaluation_call(cols, split, monkeypatch):
     """Every way in which the warps share a tile's columns: one 16-column piece to eight of them, a last tile with padding
     columns, k ranges of two k-blocks a rank (the fewest operand stages, over which the shares are laid)."""
@@ -80,3 +80,24 @@ def test_tile_widths_of_the_evaluation_call(cols, split, monkeypatch):
     torch.cuda.synchronize()
     assert nb.nb_cbs_poll_status(plan) == ""
     parity.check("a_eval", out.double().cpu().numpy(), oracle.cbs_infer(inp.x, inp.w, inp.gamma, inp.beta, rm, rv, shape.stride, EPS), "bf16")
+
+
+@pytest.mark.parametrize("dims,cols", [((2, 20, 20, 288, 288, 3, 1), 144), ((1, 33, 31, 64, 144, 3, 1), 144), ((4, 13, 9, 256, 176, 1, 1), 176),
+                                       ((2, 17, 19, 40, 256, 3, 1), 256), ((1, 40, 40, 192, 192, 3, 1), 16), ((3, 11, 9, 96, 192, 3, 2), 48)],
+                         ids=lambda v: str(v) if isinstance(v, int) else "x".join(map(str, v)))
+def test_training_calls_have_the_bits_of_the_persistent_form(dims, cols, monkeypatch):
+    import torch
+
+    from paper_2609_10632_b200.block import CbsBlock
+
+    got = []
+    for split in ("0", "1"):
+        monkeypatch.setenv("NB_TC_SPLIT", split)
+        if split == "1":
+            monkeypatch.setenv("NB_TC_SPLIT_BN", str(cols))
+        blk = CbsBlock(wl.ConvShape("bits", *dims), eps=EPS)
+        blk.fill_random(3)
+        blk.step()
+        blk.poll()
+        got.append(blk)
+    assert all(torch.equal(getattr(got[0], k), getattr(got[1], k)) for k in ("y", "mean", "invstd", "dx"))
