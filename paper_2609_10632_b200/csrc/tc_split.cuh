@@ -398,6 +398,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
         }
     }
     if (sat_bits & (int)0x80008000u) atomicAdd(p.status + ST_SAT, 1);
+    __syncwarp();  // (what follows wants whole warps)
     if (warp == 1) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
