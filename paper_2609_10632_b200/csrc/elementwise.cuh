@@ -556,10 +556,16 @@ struct BwdFused {
     __nv_bfloat16* wt;
 };
 // `row_blocks` blocks walk the tensor (the sums are grouped by them); blocks past those only rearrange filter tiles.
-// DEEP: for small tensors, whose threads have at most eight vectors each and whose blocks do not fill the device: all of them
-// are on their way before the parameters are used (a small tensor's pass is one memory latency per step of this loop), with
-// the registers that takes; the additions and their order are the same.
-template <typename YT, typename AT, bool FAST, bool PITCHED = false, bool DEEP = false>
+// DEEP: for tensors whose threads have at most eight vectors each and whose blocks are all resident: all vectors are on their way
+// before the parameters are used (a small tensor's pass is one memory latency per step of this loop), with the registers that
+// takes; the additions and their order are the same.  1: up to one block an SM.  2: up to two of at most 256 threads, so at most
+// 128 registers: the bf16 form takes 129 with indices of 64 bits and 128 with indices of 32 (the tensor has fewer than 2^20 vectors).
+// A launch bound that forces the count costs 0.2 to 0.3 us a call, since the compiler then asks for some of the vectors later.
+// Up to one block an SM the second block's room does harm: blocks become resident while the pass before still runs, wherever it leaves
+// room, and pile up two to an SM beside idle ones.  Form 1 / 2 in bf16, us a step: 72 -> 136 3x3 on 3 x 53 x 75 pixels (100 blocks)
+// 55.1 / 57.6, 192 -> 192 3x3 on 4 x 40 x 40 (80) 43.5 / 45.4.  (Form 2 with half an SM's shared memory, one block an SM by that:
+// 55.2 and 43.5, but then no block fits beside a weight gradient's: detector iteration at batch 2, 320 x 320 2036 -> 2044 us.)
+template <typename YT, typename AT, bool FAST, bool PITCHED = false, int DEEP = 0>
 __global__ void __launch_bounds__(288, DEEP ? 1 : 3) bn_silu_bwd_reduce_kernel(const AT* __restrict__ g, const YT* __restrict__ y,
                                                                   long long total_vecs, int C, const float* __restrict__ mean,
                                                                   const float* __restrict__ invstd, const float* __restrict__ gamma,
@@ -593,12 +599,14 @@ __global__ void __launch_bounds__(288, DEEP ? 1 : 3) bn_silu_bwd_reduce_kernel(c
     constexpr int D = DEEP ? 8 : 1;
     Vec16<YT> qyd[D];
     Vec16<AT> qgd[D];
+    using Index = std::conditional_t<DEEP == 2, int, long long>;
+    const Index first = (Index)v0, step = (Index)stride, total = (Index)total_vecs;
     if (DEEP && has_rows) {
 #pragma unroll
         for (int u = 0; u < D; ++u)
-            if (v0 + u * stride < total_vecs) {
-                qyd[u] = ld16(y + (v0 + u * stride) * V);
-                qgd[u] = ld16(g + og + u * og_step);
+            if (first + u * step < total) {
+                qyd[u] = ld16(y + (first + u * step) * V);
+                qgd[u] = ld16(PITCHED || DEEP == 1 ? g + og + u * og_step : g + (first + u * step) * V);
             }
     }
     float2 a[V / 2], b[V / 2], sb[V / 2], sy[V / 2];
@@ -628,7 +636,7 @@ __global__ void __launch_bounds__(288, DEEP ? 1 : 3) bn_silu_bwd_reduce_kernel(c
         if (has_rows) {
 #pragma unroll
             for (int u = 0; u < D; ++u)
-                if (v0 + u * stride < total_vecs) add_vec(qyd[u], qgd[u]);
+                if (first + u * step < total) add_vec(qyd[u], qgd[u]);
         }
     } else {
         uint4* const ring = reinterpret_cast<uint4*>(red) + tid;  // [EW_RING][2][blockDim.x] vectors, in the space of the block's reduction below

@@ -56,7 +56,8 @@ struct EwCfg {  // launch geometry of the [M][C] passes
     long long total_vecs;
     int blocks_reduce, blocks_map;  // stats / backward-reduce grids (they size the partial buffers) and apply / dy grids
     int blocks_stats, blocks_apply, blocks_dy;
-    int wave_reduce;  // resident blocks of the backward-reduce kernel on the whole device
+    int wave_reduce;  // resident blocks of the backward-reduce kernel (ring form) on the whole device
+    int wave_deep;  // the same of the form that asks for all vectors of a thread at once, at most two an SM
     int slabs, slab_ctas, slab_units, slab_threads;  // both backward passes in one launch: channel slabs (0: two launches), CTAs of a slab, row blocks and threads of a CTA
 };
 
@@ -281,23 +282,27 @@ nb_status run_bwd_elementwise(nb_cbs_plan_s* p, const void* g, const void* y, co
         if (fuse) {
             fb.w = static_cast<const __nv_bfloat16*>(w); fb.wt = wtp ? static_cast<__nv_bfloat16*>(wt) : nullptr;
         }
-        // At most two blocks of rows an SM, whose threads have at most eight vectors: all of them asked for at once, with the
-        // registers that takes.  Measured (step), one block for at most every second SM / two for every SM: 72 -> 136 3x3 on
-        // 3 x 53 x 75 pixels (93 blocks) 58.9 / 55.5 us, 192 -> 192 on 4 x 40 x 40 50.5 / 46.9, 288 -> 288 on 16 x 20 x 20 80.1 / 78.0,
-        // 96 -> 96 on 2 x 80 x 80 43.2 / 40.0, on 16 x 40 x 40 (150 blocks) 60.6 / 59.8.
-        const bool deep = e.blocks_reduce <= 2 * p->sm_count && (long long)e.blocks_reduce * e.tpb * 8 >= e.total_vecs;
-        const size_t red_smem = std::max((size_t)2 * e.tpb * e.vec * sizeof(float), deep ? (size_t)0 : (size_t)EW_RING * 2 * e.tpb * 16);
         // A small activation needs few blocks, a large filter many: every block takes two filter tiles, blocks without
         // rows of their own take nothing else (288 -> 288 3x3 on one 20 x 20 image has 405 tiles and 8 blocks of rows:
-        // 61 us when those 8 rearranged the filter alone).
+        // 61 us when those 8 rearranged the filter alone).  As many as three an SM, also where two blocks of rows fit one: with at most
+        // two, 512 -> 512 3x3 on 16 x 20 x 20 takes 48.6 instead of 46.8 us (backward data call), on 4 x 20 x 20 29.7 instead of 28.5.
         int blocks = e.blocks_reduce;
         if (fb.wt) blocks = std::max(blocks, std::min(e.wave_reduce, (wt_num_tiles(*wtp) + 1) / 2));
+        // All vectors of a thread at once where those are at most eight and the blocks of rows, at most two an SM, are resident together.
+        // Measured (backward data call, us; blocks in brackets), ring / all at once: 288 -> 576 1x1 on 16 x 20 x 20 pixels (267)
+        // 23.4 / 21.1, 576 -> 384 1x1 there (160) 23.0 / 22.0, 96 -> 96 1x1 on 21 x 40 x 40 (200) 20.5 / 18.8, on 222 x 224 (296)
+        // 23.4 / 22.5, 64 -> 256 1x1 on 4 x 56 x 56 (196) 18.1 / 16.5, 288 -> 288 3x3 on 16 x 20 x 20 (115) 29.8 / 29.0.  With one register
+        // too many for the second block on an SM the first five took 24.3, 23.8, 20.3, 23.7 and 18.5.  The form for one block an SM not
+        // where filter tiles make more than two turns of them (512 -> 512 3x3 on 4 x 20 x 20, 50 + 394 blocks: 32.8 instead of 28.3).
+        const bool deep = e.blocks_reduce <= e.wave_deep && (long long)e.blocks_reduce * e.tpb * 8 >= e.total_vecs;
+        const bool deep1 = deep && e.blocks_reduce <= p->sm_count && blocks <= 2 * p->sm_count;
+        const size_t red_smem = std::max((size_t)2 * e.tpb * e.vec * sizeof(float), deep ? (size_t)0 : (size_t)EW_RING * 2 * e.tpb * 16);
         auto go = [&](auto kernel, long long ld) {
             launch_k(kernel, dim3(blocks), dim3(e.tpb), red_smem, st, 1, static_cast<const AT*>(g), static_cast<const YT*>(y), e.total_vecs, C, mean, invstd,
                      gamma, beta, partials, fb, wtp ? *wtp : none, ld, e.blocks_reduce);
         };
-        if (p->ld_g) deep ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true, true>, p->ld_g) : go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true>, p->ld_g);
-        else deep ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false, true>, (long long)C) : go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false>, (long long)C);
+        if (p->ld_g) deep1 ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true, 1>, p->ld_g) : deep ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true, 2>, p->ld_g) : go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, true>, p->ld_g);
+        else deep1 ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false, 1>, (long long)C) : deep ? go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false, 2>, (long long)C) : go(bn_silu_bwd_reduce_kernel<YT, AT, FAST, false>, (long long)C);
         NB_LAUNCH_OK("bn_silu_bwd_reduce");
     }
     if (!fuse) {
@@ -627,33 +632,39 @@ nb_status nb_cbs_plan_create(const nb_cbs_desc* d, int device, nb_cbs_plan* out)
     // the grouping of the additions is part of the results' last bits, and stays), one in the maps, whose threads would
     // otherwise chain memory latencies: 16 -> 32 on 2 x 32 x 32 pixels, 36.3 -> 34.0 us for the step's kernels against four.
     {
-        e.wave_reduce = 0;
-        auto wave = [&](const void* fn, size_t dyn_smem, int min_vecs, int* resident = nullptr) {
+        auto resident = [&](const void* fn, size_t dyn_smem) {
             int occ = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, e.tpb, dyn_smem) != cudaSuccess || occ < 1) {
                 cudaGetLastError();
                 occ = 1;
             }
-            const long long cap = (long long)p->sm_count * occ;
-            if (resident) *resident = (int)cap;
-            return (int)std::max<long long>(1, std::min<long long>((max_blocks + min_vecs - 1) / min_vecs, cap));
+            return p->sm_count * occ;
+        };
+        auto wave = [&](const void* fn, size_t dyn_smem, int min_vecs) {
+            return (int)std::max<long long>(1, std::min<long long>((max_blocks + min_vecs - 1) / min_vecs, resident(fn, dyn_smem)));
         };
         const size_t red_smem = (size_t)e.tpb * vec * sizeof(float);
+        auto reduce = [&](auto ring, auto deep, auto deep_pitched) {
+            const size_t ring_smem = std::max(2 * red_smem, (size_t)EW_RING * 2 * e.tpb * 16);
+            e.blocks_reduce = wave((const void*)ring, ring_smem, 8);
+            e.wave_reduce = resident((const void*)ring, ring_smem);
+            e.wave_deep = std::min({2 * p->sm_count, resident((const void*)deep, 2 * red_smem), resident((const void*)deep_pitched, 2 * red_smem)});
+        };
         // the passes that derive their coefficients from the accumulators keep them in dynamic shared memory
         const size_t apply_smem = p->fuse_finalize ? (size_t)2 * g.c_out * sizeof(float) : 0, dy_smem = p->fuse_finalize ? (size_t)4 * g.c_out * sizeof(float) : 0;
         if (d->mode == NB_MODE_F32_REF) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<float>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<float, float, false>, std::max(2 * red_smem, (size_t)EW_RING * 2 * e.tpb * 16), 8, &e.wave_reduce);
+            reduce(bn_silu_bwd_reduce_kernel<float, float, false>, bn_silu_bwd_reduce_kernel<float, float, false, false, 2>, bn_silu_bwd_reduce_kernel<float, float, false, true, 2>);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<float, float, false, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<float, float, false, false, true>, dy_smem, 1);
         } else if (d->mode == NB_MODE_F16_TC) {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __half, true>, std::max(2 * red_smem, (size_t)EW_RING * 2 * e.tpb * 16), 8, &e.wave_reduce);
+            reduce(bn_silu_bwd_reduce_kernel<__half, __half, true>, bn_silu_bwd_reduce_kernel<__half, __half, true, false, 2>, bn_silu_bwd_reduce_kernel<__half, __half, true, true, 2>);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __half, true, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __half, true, false, true>, dy_smem, 1);
         } else {
             e.blocks_stats = wave((const void*)bn_stats_partial_kernel<__half>, red_smem, 4);
-            e.blocks_reduce = wave((const void*)bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, std::max(2 * red_smem, (size_t)EW_RING * 2 * e.tpb * 16), 8, &e.wave_reduce);
+            reduce(bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true>, bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true, false, 2>, bn_silu_bwd_reduce_kernel<__half, __nv_bfloat16, true, true, 2>);
             e.blocks_apply = wave((const void*)bn_silu_apply_kernel<__half, __nv_bfloat16, true, true, false, false, true>, apply_smem, 1);
             e.blocks_dy = wave((const void*)bn_silu_bwd_dy_kernel<__half, __nv_bfloat16, true, false, true>, dy_smem, 1);
         }

@@ -88,3 +88,63 @@ def test_reduction_at_its_block_counts(blocks):
     blk.step()
     blk.poll()
     _against_fp64(blk)
+
+
+@pytest.mark.parametrize("blocks", [148, 149])
+def test_reduction_of_rows_wider_than_256_threads(blocks):
+    """2056 channels are a row of 257 threads: all vectors at once up to one block an SM."""
+    from paper_2609_10632_b200.block import CbsBlock
+
+    blk = CbsBlock(wl.ConvShape("wide", 1, blocks, 8, 16, 2056, 1, 1))  # eight rows a block
+    blk.fill_random(blocks)
+    blk.step()
+    blk.poll()
+    _against_fp64(blk)
+
+
+def test_reduction_with_all_vectors_at_once_is_one_wave_of_blocks(tmp_path):
+    """With all vectors of a thread in registers, the blocks of the backward reduction are on the device together: one an SM in the
+    first form, two in the second.  Registers, shared memory and shape of every launch as the profiler reports them."""
+    import json
+
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+
+    from paper_2609_10632_b200 import binding as nb
+    from paper_2609_10632_b200.block import CbsBlock
+
+    prop = torch.cuda.get_device_properties(0)
+    sms, sm_smem = prop.multi_processor_count, prop.shared_memory_per_multiprocessor
+    blks = []
+    for mode, rows in ((nb.NB_MODE_BF16_TC, 256), (nb.NB_MODE_F16_TC, 256), (nb.NB_MODE_F32_REF, 128)):  # rows a block
+        for blocks in (sms, sms + 1, 2 * sms):
+            for pitched in (False, True):
+                blk = CbsBlock(wl.ConvShape("wave", 1, rows // 16 * blocks - 1, 16, 16, 64, 1, 1), mode=mode)
+                blk.fill_random(3)
+                if pitched:
+                    wide = torch.zeros(*blk.g.shape[:-1], 72, dtype=blk.g.dtype, device="cuda")
+                    blk.plan.set_pitches(ld_g=72)
+                    blk.g = wide[..., 8:]
+                blk.step()
+                blks.append((blocks, blk))
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        for _, blk in blks:
+            blk.step()
+        torch.cuda.synchronize()
+    prof.export_chrome_trace(str(tmp_path / "trace.json"))
+    events = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
+    events = sorted((e for e in events if e.get("cat") == "kernel" and "bn_silu_bwd_reduce_kernel<" in e["name"]), key=lambda e: e["ts"])
+    if not events:
+        pytest.skip("the profiler delivers no launches here")
+    assert len(events) == len(blks)
+    for (blocks, _), e in zip(blks, events):
+        a = e["args"]
+        assert a["grid"][0] == blocks
+        warps = -(-a["block"][0] // 32)
+        registers = warps * 32 * (-(-a["registers per thread"] // 8) * 8)
+        smem = a["shared memory"] + 1024  # (what the system keeps of each block)
+        resident = min(65536 // registers, 64 // warps, sm_smem // smem)
+        assert blocks <= resident * sms, (e["name"], a)
+    forms = [e["name"].split(">(")[0].rsplit(", ", 1)[1] for e in events]
+    assert forms == ["1" if blocks <= sms else "2" for blocks, _ in blks]
