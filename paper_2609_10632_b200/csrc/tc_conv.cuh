@@ -1075,7 +1075,7 @@ inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_tap
     c.ok = true;
     out.cfg = c;
     if (getenv("NB_TC_VERBOSE"))
-        fprintf(stderr, "[nb_cbs] split igemm M=%lld Ca=%d rowsB=%d taps=%d classes=%d: BN=%d S=%d stages=%d tiles=%dx%d grid=%d est %.1f us\n", c.M, c.Ca, c.rowsB, c.ntaps, ncls,
+        fprintf(stderr, "[nb_cbs] split igemm%s M=%lld Ca=%d rowsB=%d taps=%d classes=%d: BN=%d S=%d stages=%d tiles=%dx%d grid=%d est %.1f us\n", eval ? " (evaluation)" : "", c.M, c.Ca, c.rowsB, c.ntaps, ncls,
                 c.BN, c.split, c.stages, c.m_tiles, c.n_tiles, c.grid, best);
 }
 

@@ -1,6 +1,8 @@
 """The split-K cluster form of the implicit GEMM (layers with few output tiles) with every cluster size forced: k-blocks that
 do not divide evenly, a 32-channel tail k-block, ragged rows, padded columns, the parity classes of a stride-2 data gradient
-with odd extents, and a data gradient added into a channel slice."""
+with odd extents, and a data gradient added into a channel slice (the training calls use clusters of one alone).  Each test makes sure that its plans have this form."""
+import re
+
 import pytest
 
 from paper_2609_10632_b200 import workloads as wl
@@ -8,6 +10,16 @@ from tests import parity
 from tests.test_gpu_parity import EPS, _compare, _oracle, _run_block
 
 pytestmark = pytest.mark.gpu
+
+LINE = re.compile(r"split igemm( \(evaluation\))? M=(\d+) Ca=(\d+) rowsB=(\d+) .*BN=(\d+) S=(\d+) stages=(\d+)")
+
+
+def _chosen(capfd):
+    """The split launches that the plans created since the last look have chosen (their lines under NB_TC_VERBOSE):
+    (evaluation call?, channels of the A operand, rows of the B operand, tile columns, cluster size, operand stages)."""
+    found = LINE.findall(capfd.readouterr().err)
+    return [(bool(ev), int(ca), int(rows), int(cols), int(size), int(stages)) for ev, _, ca, rows, cols, size, stages in found]
+
 
 SHAPES = [
     (1, 20, 20, 192, 192, 3, 1),  # 27 k-blocks, four row tiles
@@ -20,7 +32,7 @@ SHAPES = [
 
 @pytest.mark.parametrize("split", [1, 2, 4, 8])
 @pytest.mark.parametrize("dims", SHAPES, ids=lambda d: "x".join(map(str, d)))
-def test_split_launches_match_oracle(dims, split, monkeypatch):
+def test_split_launches_match_oracle(dims, split, monkeypatch, capfd):
     import oracle
     import torch
 
@@ -28,9 +40,14 @@ def test_split_launches_match_oracle(dims, split, monkeypatch):
     from paper_2609_10632_b200.block import CbsBlock
 
     monkeypatch.setenv("NB_TC_SPLIT_S", str(split))
+    monkeypatch.setenv("NB_TC_VERBOSE", "1")
     shape = wl.ConvShape("split", *dims)
     mode = nb.NB_MODE_F16_TC if split == 2 else nb.NB_MODE_BF16_TC
     inp, blk, out = _run_block(shape, mode, cfg_id=43, layer_id=SHAPES.index(dims), affine="random")
+    evaluation = (True, shape.c_in, shape.c_out, split)
+    training = [(False, shape.c_in, shape.c_out, 1), (False, shape.c_out, shape.c_in, 1)]  # forward, data gradient
+    chosen = [(ev, ca, rows, size) for ev, ca, rows, _, size, _ in _chosen(capfd)]
+    assert sorted(chosen) == sorted([evaluation] + (training if split == 1 else []))
     _compare(out, _oracle(inp), 0)
     again = CbsBlock(shape, mode=mode, eps=EPS)
     again.upload(inp)
@@ -55,22 +72,19 @@ def test_split_launches_match_oracle(dims, split, monkeypatch):
         assert torch.equal(wide, want)
 
 
-@pytest.mark.parametrize("split", [1, 2, 8])
-@pytest.mark.parametrize("cols", [16, 48, 80, 112, 128, 144, 208, 256])
-def test_tile_widths_of_the_evaluation_call(cols, split, monkeypatch):
-    """Every way in which the warps share a tile's columns: one 16-column piece to eight of them, a last tile with padding
-    columns, k ranges of two k-blocks a rank (the fewest operand stages, over which the shares are laid)."""
+WIDTHS = [16, 48, 80, 112, 128, 144, 208, 256]
+
+
+def _evaluate(shape, seed):
+    """One evaluation call of a fresh plan against the oracle."""
     import numpy as np
     import oracle
     import torch
 
     from paper_2609_10632_b200 import binding as nb
 
-    monkeypatch.setenv("NB_TC_SPLIT_S", str(split))
-    monkeypatch.setenv("NB_TC_SPLIT_BN", str(cols))
-    shape = wl.ConvShape("width", 2, 9, 17, 128, 2 * cols - 8 if cols > 16 else 16, 3, 1)
-    inp = wl.make_inputs(shape, 47, cols, bf16=True, affine="random")
-    rm, rv, _ = wl.make_eval_stats(shape, 47, cols)
+    inp = wl.make_inputs(shape, 47, seed, bf16=True, affine="random")
+    rm, rv, _ = wl.make_eval_stats(shape, 47, seed)
     plan = nb.Plan.for_shape(shape, eps=EPS)
     dev = lambda a, dt=torch.float32: torch.from_numpy(np.ascontiguousarray(a)).to(dt).cuda()
     x, w = dev(inp.x, torch.bfloat16), dev(inp.w, torch.bfloat16)
@@ -82,15 +96,42 @@ def test_tile_widths_of_the_evaluation_call(cols, split, monkeypatch):
     parity.check("a_eval", out.double().cpu().numpy(), oracle.cbs_infer(inp.x, inp.w, inp.gamma, inp.beta, rm, rv, shape.stride, EPS), "bf16")
 
 
+@pytest.mark.parametrize("cols,split", [(c, s) for c in WIDTHS for s in (1, 2, 8) if s == 1 or c <= 128])
+def test_tile_widths_of_the_evaluation_call(cols, split, monkeypatch, capfd):
+    """Every way in which the warps share a tile's columns: one 16-column piece to sixteen of them (clusters: to eight), a last
+    tile with padding columns."""
+    monkeypatch.setenv("NB_TC_SPLIT_S", str(split))
+    monkeypatch.setenv("NB_TC_SPLIT_BN", str(cols))
+    monkeypatch.setenv("NB_TC_VERBOSE", "1")
+    shape = wl.ConvShape("width", 2, 9, 17, 128, 2 * cols - 8 if cols > 16 else 16, 3, 1)
+    _evaluate(shape, cols)
+    assert [c[3:5] for c in _chosen(capfd) if c[0]] == [(cols, split)]
+
+
+@pytest.mark.parametrize("cols", [112, 128])
+@pytest.mark.parametrize("per_rank", [1, 2])
+@pytest.mark.parametrize("split", [2, 4, 8])
+def test_short_k_ranges_of_a_cluster(split, per_rank, cols, monkeypatch, capfd):
+    """One and two k-blocks a rank.  Two operand stages are the fewest; a rank lays its 128 x (columns + 8) sums over them before
+    it hands them out, which fits exactly at 112 columns and takes a third stage at 128."""
+    monkeypatch.setenv("NB_TC_SPLIT_S", str(split))
+    monkeypatch.setenv("NB_TC_SPLIT_BN", str(cols))
+    monkeypatch.setenv("NB_TC_VERBOSE", "1")
+    shape = wl.ConvShape("short", 2, 9, 17, 64 * split * per_rank, cols, 1, 1)
+    _evaluate(shape, 300 + cols)
+    assert [c[3:] for c in _chosen(capfd) if c[0]] == [(cols, split, 2 if cols == 112 else 3)]
+
+
 @pytest.mark.parametrize("dims,cols", [((2, 20, 20, 288, 288, 3, 1), 144), ((1, 33, 31, 64, 144, 3, 1), 144), ((4, 13, 9, 256, 176, 1, 1), 176),
-                                       ((2, 17, 19, 40, 256, 3, 1), 256), ((1, 40, 40, 192, 192, 3, 1), 16), ((3, 11, 9, 96, 192, 3, 2), 48)],
+                                       ((2, 17, 19, 40, 256, 3, 1), 256), ((1, 40, 40, 192, 192, 3, 1), 32), ((3, 11, 9, 96, 192, 3, 2), 48)],
                          ids=lambda v: str(v) if isinstance(v, int) else "x".join(map(str, v)))
-def test_training_calls_have_the_bits_of_the_persistent_form(dims, cols, monkeypatch):
+def test_training_calls_have_the_bits_of_the_persistent_form(dims, cols, monkeypatch, capfd):
     import torch
 
     from paper_2609_10632_b200.block import CbsBlock
 
     got = []
+    monkeypatch.setenv("NB_TC_VERBOSE", "1")
     for split in ("0", "1"):
         monkeypatch.setenv("NB_TC_SPLIT", split)
         if split == "1":
@@ -100,4 +141,6 @@ def test_training_calls_have_the_bits_of_the_persistent_form(dims, cols, monkeyp
         blk.step()
         blk.poll()
         got.append(blk)
+        chosen = [c[1:4] for c in _chosen(capfd) if not c[0]]
+        assert {c[2] for c in chosen} == ({cols} if split == "1" else set())
     assert all(torch.equal(getattr(got[0], k), getattr(got[1], k)) for k in ("y", "mean", "invstd", "dx"))
