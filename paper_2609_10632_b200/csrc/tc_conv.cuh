@@ -262,8 +262,8 @@ __device__ __forceinline__ void epi_pass_tma(uint32_t taddr, uint8_t* wrows, int
             *ps = a2;
             *pq = b2;
         }
-        __syncwarp();  // staged rows read before the next pass overwrites them
     }
+    __syncwarp();  // staged rows read before the next pass overwrites them; its accumulator loads want the whole warp
 }
 
 // CG2 = the CTAs run as pairs (clusters of two): rank 0 issues tcgen05.mma.cta_group::2 with M = 256; each CTA owns 128
@@ -735,6 +735,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
         // the staging rows must have been read before this CTA's shared memory is released; the writes themselves are
         // complete when the grid is (a kernel boundary orders them like any other store)
         if (store_pending && lane == 0) ptx::tma_store_wait_read<0>();
+        __syncwarp();
         if (STATS) {
             epi2_bar_sync();  // all eight warps' running sums are final
             // channel c of the layer sits in team (c % BN >= ncol_a) at index (c / BN) * (team's columns) + its column there
@@ -754,6 +755,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
         }
         if (sat) atomicAdd(p.status + ST_SAT, sat);
     }
+    __syncwarp();  // (the cluster barrier and the release of TMEM want whole warps)
     ptx::tc_fence_before();
     if (CG2) ptx::cluster_sync_all(); else __syncthreads();  // pairs: neither CTA may leave while the other still uses its memory
     if (warp == 1) {

@@ -231,10 +231,12 @@ __global__ void __launch_bounds__(WG_THREADS, 1) tc_wgrad_kernel(const __grid_co
                     for (int j = 0; j < 16; ++j)
                         if (j < 8 || n_tile * p.BN + c0 + 8 < p.c_out) dst[(size_t)(n_tile * p.BN + c0 + j) * p.kdim + kidx] = __uint_as_float(r[j]);
                 }
+                __syncwarp();  // (the next accumulator load wants the whole warp)
             }
         }
     }
     if (p.overlap) pdl_wait();
+    __syncwarp();  // (the release of TMEM wants a whole warp)
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -460,10 +462,12 @@ __global__ void __launch_bounds__(WG_THREADS, 1) tc_wgrad_rows_kernel(const __gr
                     for (int j = 0; j < 16; ++j)
                         if (j < 8 || n_tile * p.BN + c0 + 8 < p.c_out) dst[(size_t)(n_tile * p.BN + c0 + j) * p.kdim + kidx] = __uint_as_float(rr[j]);
                 }
+                __syncwarp();  // (the next accumulator load wants the whole warp)
             }
         }
     }
     if (p.overlap) pdl_wait();
+    __syncwarp();  // (the release of TMEM wants a whole warp)
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 1) {

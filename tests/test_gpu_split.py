@@ -144,3 +144,18 @@ def test_training_calls_have_the_bits_of_the_persistent_form(dims, cols, monkeyp
         chosen = [c[1:4] for c in _chosen(capfd) if not c[0]]
         assert {c[2] for c in chosen} == ({cols} if split == "1" else set())
     assert all(torch.equal(getattr(got[0], k), getattr(got[1], k)) for k in ("y", "mean", "invstd", "dx"))
+
+
+@pytest.mark.parametrize("dims", [(1, 3, 11, 96, 96, 3, 1), (1, 7, 5, 96, 96, 3, 2), (1, 17, 17, 72, 80, 3, 1), (2, 9, 16, 40, 80, 3, 1)], ids=lambda d: "x".join(map(str, d)))
+@pytest.mark.parametrize("split", ["0", "1"])
+def test_warps_of_which_some_rows_do_not_exist(split, dims, monkeypatch, capfd):
+    """Accumulator rows past the last pixel, outside an odd parity class or past the last input channel of a tap, in a warp whose
+    other rows are stored, with several pieces of columns a warp: the rows that exist are right in every piece."""
+    monkeypatch.setenv("NB_TC_SPLIT", split)
+    monkeypatch.setenv("NB_TC_SPLIT_S", "1")
+    monkeypatch.setenv("NB_TC_SPLIT_BN", str((dims[4] + 15) // 16 * 16))
+    monkeypatch.setenv("NB_TC_VERBOSE", "1")
+    inp, blk, out = _run_block(wl.ConvShape("edge", *dims), 0, cfg_id=53, layer_id=dims[3], affine="random")
+    assert blk.plan.paths == {"fprop": 1, "dgrad": 1, "wgrad": 1}
+    assert any(not c[0] for c in _chosen(capfd)) == (split == "1")
+    _compare(out, _oracle(inp), 0)
