@@ -913,7 +913,8 @@ inline IgemmCfg igemm_configure(long long M, int Ca, int rowsB, int ntaps, int s
     const int kblocks = ntaps * ((Ca + c.KC - 1) / c.KC);
     const int force_bn = getenv("NB_TC_BN") ? atoi(getenv("NB_TC_BN")) : 0;
     const int force_kpb = getenv("NB_TC_KPB") ? atoi(getenv("NB_TC_KPB")) : 0;
-    const int force_mh = getenv("NB_TC_MH") ? atoi(getenv("NB_TC_MH")) : 0;
+    int force_mh = getenv("NB_TC_MH") ? atoi(getenv("NB_TC_MH")) : 0;
+    if (force_mh < 1 || force_mh > 2) force_mh = 0;  // (one MMA issuer for each sub-tile, and there are two: with three no stage would ever be free again)
     // Rules distilled from sweeps over the detector's layer shapes on B200: the widest N tile that divides the channel
     // count wins everywhere (fewer shared-memory bytes written and read per flop); pairing two 128-row blocks per tile
     // (mh = 2) pays only while two accumulator sets still fit in TMEM (N <= 128) and there are enough tiles for every SM;

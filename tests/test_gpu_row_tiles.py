@@ -41,3 +41,21 @@ def test_same_bits_as_the_wide_tiles(shape, monkeypatch):
     # sums in another order, rounded to 16 bits: now and then another way (seen: 9e-5)
     assert (dx.float() - dx2.float()).norm() <= 4e-4 * dx2.float().norm()
     assert (a.float() - a2.float()).norm() <= 4e-4 * a2.float().norm()
+
+
+@pytest.mark.parametrize("rows", ["-1", "0", "3", "4", "16"])
+def test_forced_sub_tiles_are_one_or_two(rows, monkeypatch, capfd):
+    """Anything else asked for leaves the choice as it is (the kernel has two MMA issuers)."""
+    import re
+
+    from paper_2609_10632_b200 import binding as nb
+
+    monkeypatch.setenv("NB_TC_VERBOSE", "1")
+    shape = wl.ConvShape("rows", 2, 40, 40, 64, 16, 3, 1)
+    lines = []
+    for forced in (None, rows):
+        if forced:
+            monkeypatch.setenv("NB_TC_MH", forced)
+        nb.Plan.for_shape(shape)
+        lines.append(re.findall(r"\] igemm .*", capfd.readouterr().err))
+    assert len(lines[0]) >= 2 and lines[0] == lines[1]
