@@ -546,21 +546,22 @@ nb_status run_simt_grads(nb_cbs_plan_s* p, const void* x, const void* dy, const 
     NB_TRY(simt_dgrad_conv<TIN>(p, dy, w, dx, dgpart, st));
     NB_TRY(simt_wgrad_conv<TIN>(p, x, dy, dw, wgpart, pdl_enabled(), st));
     const size_t elems1 = (size_t)p->g.n * p->g.h * p->g.w * p->g.c_in, elems2 = (size_t)p->g.c_out * p->g.kdim;
-    const bool both = d.splits > 1 && c.splits > 1 && c.splits < 96;
-    SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
-    if (both) {
+    if (d.splits > 1 && c.splits > 1 && c.splits < 96) {
         const unsigned b1 = splitk_reduce_blocks(elems1, p->sm_count), b2 = splitk_reduce_blocks(elems2, p->sm_count);
+        SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
         launch_k(splitk_reduce_both_kernel<TIN>, dim3(b1 + b2), dim3(256), 0, st, 1, static_cast<const float*>(dgpart), d.splits, elems1, static_cast<TIN*>(dx), (int)b1,
                  static_cast<const float*>(wgpart), c.splits, elems2, dw);
         return launch_ok("splitk_reduce_both");
     }
     if (d.splits > 1) {
+        SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
         launch_k(splitk_reduce_kernel<TIN>, dim3(splitk_reduce_blocks(elems1, p->sm_count)), dim3(256), 0, st, 1, static_cast<const float*>(dgpart), d.splits, elems1, static_cast<TIN*>(dx));
         NB_LAUNCH_OK("splitk_reduce");
     }
+    if (c.splits == 1) return NB_OK;
+    SiteTimer tm(p, SITE_SPLITK_REDUCE, st);
     if (c.splits >= 96) launch_k(splitk_reduce_tall_kernel, dim3((unsigned)((elems2 + 31) / 32)), dim3(1024), 0, st, 1, wgpart, c.splits, elems2, dw);
-    else if (c.splits > 1) launch_k(splitk_reduce_kernel<float>, dim3(splitk_reduce_blocks(elems2, p->sm_count)), dim3(256), 0, st, 1, wgpart, c.splits, elems2, dw);
-    else return NB_OK;
+    else launch_k(splitk_reduce_kernel<float>, dim3(splitk_reduce_blocks(elems2, p->sm_count)), dim3(256), 0, st, 1, wgpart, c.splits, elems2, dw);
     return launch_ok("splitk_reduce");
 }
 

@@ -87,3 +87,22 @@ def test_weight_gradient_sees_what_is_written_between_the_calls(mode, dims):
         blk.backward_weight()
         blk.poll()
         assert torch.equal(blk.dw, want)
+
+
+@pytest.mark.parametrize("mode,dims", [c for c in SHAPES if c[0] == "f32"], ids=[i for i in IDS if i.startswith("f32")])
+def test_profile_counts_the_launches_that_add_slices(mode, dims):
+    """The one call reports as many launches at the site of the slices as it makes, in particular none where nothing is added."""
+    from paper_2609_10632_b200 import binding as nb
+
+    blk = _block(mode, dims)
+
+    def sites(call):
+        nb.nb_cbs_profile_enable(blk.plan, True)  # (clears the counts)
+        before = nb.nb_cbs_launch_count()
+        call()
+        return nb.nb_cbs_launch_count() - before, nb.nb_cbs_profile_read(blk.plan)["wgrad_splitk_reduce"][1]
+
+    launches2, two = sites(lambda: (blk.backward_data(), blk.backward_weight()))
+    launches1, one = sites(blk.backward)
+    assert launches2 - launches1 == two - one
+    assert (one > 0) == (two > 0)
