@@ -870,8 +870,8 @@ __global__ void __launch_bounds__(288, 3) bn_silu_bwd_dy_kernel(const AT* __rest
 // Where the reduction's threads have at most eight vectors each and few blocks, the two passes are two memory latencies, a
 // launch and a trip of the sums through the fp64 accumulators, with nothing busy.  Here g and y stay in registers between
 // them and the sums travel through distributed shared memory: the channels are cut into `slabs` (clusters of at most eight
-// CTAs that need nothing from one another), and CTA q of a slab's cluster does the slab's share of the `slabs` row blocks
-// from q * slabs on.  The additions and their grouping in fp32 are those of the reduce kernel, the block sums are added in
+// CTAs that need nothing from one another), and CTA q of a slab's cluster does the slab's share of the `units` row blocks
+// from q * units on.  The additions and their grouping in fp32 are those of the reduce kernel, the block sums are added in
 // fp64 as there, and dz is computed anew from the same coefficients as in the dy kernel, so the results are too.
 // CTAs past the slabs rearrange filter tiles.
 // Bound: latency (loads, two cluster barriers, the fp64 chain of a channel).  Measured (step): 336 -> 392 3x3 on 21 x 18 pixels
@@ -881,7 +881,7 @@ __device__ __forceinline__ double ld_dsmem_f64(uint32_t cluster_addr) {
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(cluster_addr) : "memory");
     return v;
 }
-// Dynamic shared memory: fp64 sums [2][C / slabs], coefficients [4][C / slabs], then red [2][blockDim.x * V] and part [2 C].
+// Dynamic shared memory: fp64 sums [2][wc], coefficients [4][wc], then red [2][threads * V] and part [2][units][wc].
 // wc: channels of a slab, units: row blocks of a CTA, threads of a CTA
 inline size_t bwd_small_smem(int wc, int units, int threads, int vec) { return (size_t)wc * 32 + ((size_t)2 * threads * vec + 2 * units * wc) * 4; }
 template <typename YT, typename AT, bool FAST, bool PITCHED, bool GRES>

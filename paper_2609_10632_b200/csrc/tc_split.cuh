@@ -4,10 +4,10 @@
 // K range of a tile is cut over a CLUSTER of 1, 2, 4 or 8 CTAs.  Every CTA accumulates its share in TMEM and sends the rows of
 // every rank to that rank's shared memory by bulk copies; CTA r then sums rows [128 r / S, 128 (r + 1) / S) of all S shares in
 // rank order (the same bits every run), applies the epilogue and stores.
-// The training calls use clusters of one (narrow tiles only): the sum of an element then runs over the k-blocks in the order
-// in which the persistent kernel would add them (the same starting k-block), and the channel sums are formed as there, so
-// that the results of a training step do not depend on which of the two kernels a layer gets -- a deep network in training
-// mode turns a difference in the last bit of one layer into percents a few dozen layers on.
+// The training calls use clusters of one (tiles of up to 256 columns, 160 in the data gradient): the sum of an element then
+// runs over the k-blocks in the order in which the persistent kernel would add them (the same starting k-block), and the
+// channel sums are formed as there, so that the results of a training step do not depend on which of the two kernels a layer
+// gets -- a deep network in training mode turns a difference in the last bit of one layer into percents a few dozen layers on.
 // No block waits for a block outside its cluster.  Bound: latency.  192 -> 192 3x3 on one 40 x 40 image, us behind the end of the
 // launch before: 0.8 until that has reached the CTA, 0.6 until the last CTA runs (an SM holds one), 1.1 to the first operands,
 // 0.15 a k-block (its 128 + BN rows are written to and read from shared memory once each), 0.5 to 0.8 behind the last MMA.

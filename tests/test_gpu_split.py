@@ -122,10 +122,12 @@ def test_short_k_ranges_of_a_cluster(split, per_rank, cols, monkeypatch, capfd):
     assert [c[3:] for c in _chosen(capfd) if c[0]] == [(cols, split, 2 if cols == 112 else 3)]
 
 
-@pytest.mark.parametrize("dims,cols", [((2, 20, 20, 288, 288, 3, 1), 144), ((1, 33, 31, 64, 144, 3, 1), 144), ((4, 13, 9, 256, 176, 1, 1), 176),
-                                       ((2, 17, 19, 40, 256, 3, 1), 256), ((1, 40, 40, 192, 192, 3, 1), 32), ((3, 11, 9, 96, 192, 3, 2), 48)],
-                         ids=lambda v: str(v) if isinstance(v, int) else "x".join(map(str, v)))
-def test_training_calls_have_the_bits_of_the_persistent_form(dims, cols, monkeypatch, capfd):
+@pytest.mark.parametrize("dims,cols,calls", [  # the calls whose channel count has such a tile; the other one stays on the persistent kernel
+    ((2, 20, 20, 288, 288, 3, 1), 144, "both"), ((1, 40, 40, 192, 192, 3, 1), 32, "both"), ((3, 11, 9, 96, 192, 3, 2), 48, "both"),
+    ((1, 33, 31, 64, 144, 3, 1), 144, "forward"), ((4, 13, 9, 256, 176, 1, 1), 176, "forward"), ((2, 17, 19, 40, 256, 3, 1), 256, "forward"),
+    ((1, 33, 31, 144, 64, 3, 1), 144, "data gradient"), ((2, 17, 19, 160, 40, 3, 1), 160, "data gradient")],
+    ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_training_calls_have_the_bits_of_the_persistent_form(dims, cols, calls, monkeypatch, capfd):
     import torch
 
     from paper_2609_10632_b200.block import CbsBlock
@@ -141,8 +143,9 @@ def test_training_calls_have_the_bits_of_the_persistent_form(dims, cols, monkeyp
         blk.step()
         blk.poll()
         got.append(blk)
-        chosen = [c[1:4] for c in _chosen(capfd) if not c[0]]
-        assert {c[2] for c in chosen} == ({cols} if split == "1" else set())
+        forward, data = (dims[3], dims[4], cols), (dims[4], dims[3], cols)
+        expect = {"0": [], "1": {"both": [forward, data], "forward": [forward], "data gradient": [data]}[calls]}[split]
+        assert sorted(c[1:4] for c in _chosen(capfd) if not c[0]) == sorted(expect)
     assert all(torch.equal(getattr(got[0], k), getattr(got[1], k)) for k in ("y", "mean", "invstd", "dx"))
 
 
