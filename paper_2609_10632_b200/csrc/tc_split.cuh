@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
 #pragma unroll 1
             for (int c = c_lo; c < c_lo + nc; c += 16) {
                 uint32_t r[16];
+                __syncwarp();  // (lanes without a row have left the last round early)
                 ptx::tmem_ld_32x32b_x16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c, r);
                 ptx::tmem_ld_wait();
                 const int before = sat_bits;
@@ -289,30 +290,29 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
                     *reinterpret_cast<uint4*>(staged + c * 2) = make_uint4(o[0].x, o[0].y, o[1].x, o[1].y);
                     *reinterpret_cast<uint4*>(staged + c * 2 + 16) = make_uint4(o[2].x, o[2].y, o[3].x, o[3].y);
                 }
-                if (live) {
-                    if (MODE == 0 && p.out_accumulate) {  // the rounded tile is added, as a TMA reduction would
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if (c + 4 * j >= cols) break;
-                            const uint2 old = *reinterpret_cast<const uint2*>(dst + c + 4 * j);
-                            const OutT *po = reinterpret_cast<const OutT*>(&old), *pn = reinterpret_cast<const OutT*>(&o[j]);
-                            uint2 sum;
-                            OutT* ps = reinterpret_cast<OutT*>(&sum);
-                            pair_from_f32(ps, add2(pair_to_f32(po), pair_to_f32(pn)));
-                            pair_from_f32(ps + 2, add2(pair_to_f32(po + 2), pair_to_f32(pn + 2)));
-                            o[j] = sum;
-                        }
-                    }
-                    if (wide && c + 16 <= cols) {
-                        st_global32(dst + c, o);
-                    } else {
-                        if (c < cols) *reinterpret_cast<uint4*>(dst + c) = make_uint4(o[0].x, o[0].y, o[1].x, o[1].y);
-                        if (c + 8 < cols) *reinterpret_cast<uint4*>(dst + c + 8) = make_uint4(o[2].x, o[2].y, o[3].x, o[3].y);
-                    }
-                } else {
+                if (!live) {
                     sat_bits = before;
+                    continue;
                 }
-                __syncwarp();  // (the next accumulator load wants the whole warp)
+                if (MODE == 0 && p.out_accumulate) {  // the rounded tile is added, as a TMA reduction would
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (c + 4 * j >= cols) break;
+                        const uint2 old = *reinterpret_cast<const uint2*>(dst + c + 4 * j);
+                        const OutT *po = reinterpret_cast<const OutT*>(&old), *pn = reinterpret_cast<const OutT*>(&o[j]);
+                        uint2 sum;
+                        OutT* ps = reinterpret_cast<OutT*>(&sum);
+                        pair_from_f32(ps, add2(pair_to_f32(po), pair_to_f32(pn)));
+                        pair_from_f32(ps + 2, add2(pair_to_f32(po + 2), pair_to_f32(pn + 2)));
+                        o[j] = sum;
+                    }
+                }
+                if (wide && c + 16 <= cols) {
+                    st_global32(dst + c, o);
+                } else {
+                    if (c < cols) *reinterpret_cast<uint4*>(dst + c) = make_uint4(o[0].x, o[0].y, o[1].x, o[1].y);
+                    if (c + 8 < cols) *reinterpret_cast<uint4*>(dst + c + 8) = make_uint4(o[2].x, o[2].y, o[3].x, o[3].y);
+                }
             }
         }
         ptx::tc_fence_before();
