@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(IG_THREADS, 1) tc_igemm_kernel(const __grid_co
         // first 128-row sub-tile, warp 11 for the second.  The operands are always there in time (a wait that finds them takes 105
         // cycles); what a stage takes is an issuer's instructions: barrier, eight MMAs, commit, 820 cycles for 96 -> 96 channels
         // 3x3, whose MMAs need 290 to 450.  Hence an issuer for each sub-tile, and 32-bit arithmetic for the descriptors.
-        // Measured (step): 96 -> 96 3x3 on 16 x 160 x 160 pixels 367 -> 328 us, on 16 x 80 x 80 130 -> 113, 192 -> 192 on
+        // Measured (step): 96 -> 96 3x3 on 16 x 160 x 160 pixels 367 -> 330 us, on 16 x 80 x 80 130 -> 113, 192 -> 192 on
         // 16 x 40 x 40 95.5 -> 88 (one sub-tile: shorter code alone), 48 -> 48 on 16 x 160 x 160 207 -> 198.  Testing the next
         // stage's barrier ahead of the MMAs of this one adds instructions and loses 0.5 to 2 us on the wide layers.
         const int h = warp == 11 ? 1 : 0;
@@ -1014,9 +1014,9 @@ inline void fill_params(IgemmParams& P, const IgemmCfg& c) {
 // 288 3x3 on 16 x 20 x 20 pixels 25.1 -> 20.3 / 32.6 -> 28.5 / 20.8 -> 15.5 us, 64 -> 144 3x3 on 4 x 64 x 64 14.1 -> 12.2 / - / 9.6 -> 6.7, 256 ->
 // 176 1x1 on 2 x 80 x 80 12.7 -> 11.0 / - / 8.0 -> 6.3.  Not so with padding columns in a training call (72 -> 136 3x3 on 3 x 53 x 75
 // forward 18.5 -> 19.1) nor above 160 columns in a data gradient (208 -> 192 3x3 on 8 x 40 x 40 31.4 -> 33.4).
-// Measured, evaluation-mode forward of the 77 layers, one image: 1251 us with the persistent form, 646 with split launches, 530
-// with the epilogue and the choices as they are now; single layers, persistent / split: 288 -> 288 3x3 at 20 x 20 26 / 6.3 (cluster
-// of four, 48 columns), 192 -> 192 3x3 at 40 x 40 14.9 / 6.6, 384 -> 384 1x1 at 40 x 40 9.4 / 4.0.
+// Measured, evaluation-mode forward of the 77 layers, one image: 1251 us with the persistent form, 646 with split launches, 557
+// with the epilogue and the choices as they are now; single layers repeated in a graph, persistent / split: 288 -> 288 3x3 at
+// 20 x 20 18.6 / 6.7 (cluster of four, 48 columns), 192 -> 192 3x3 at 40 x 40 13.6 / 6.9, 384 -> 384 1x1 at 40 x 40 8.1 / 4.5.
 inline void split_configure(TcGemmSlot& out, const TcGemmSlot& full, int min_taps, bool eval, int sm_count, int most_cols = 256) {
     out = full;
     out.cfg = IgemmCfg();
