@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) tc_split_kernel(const __grid_co
 #pragma unroll 1
             for (int c = c_lo; c < c_lo + nc; c += 16) {
                 uint32_t r[16];
-                __syncwarp();  // (lanes without a row have left the last round early)
+                __syncwarp();  // (lanes without a row have left the last iteration early)
                 ptx::tmem_ld_32x32b_x16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c, r);
                 ptx::tmem_ld_wait();
                 const int before = sat_bits;
